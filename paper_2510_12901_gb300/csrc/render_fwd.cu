@@ -30,30 +30,30 @@ namespace sg {
 
 constexpr int kFwdWarps = 4;        // warps per block of the persistent grid
 // blocks per SM the register budget is set for (72 registers; a few bytes of
-// the merge spill).  Measured on the street views, compositing alone / the
-// two-view step: 6 blocks 0.387 / 0.547 ms, 3122 Mrays/s; 7 blocks 0.383 /
-// 0.534 ms, 3189-3200 Mrays/s; 8 blocks 0.418 / 0.545 ms, 3237 Mrays/s.
+// the merge spill).  Measured (1920x1080 pinhole, 2M Gaussians): 6 blocks 744,
+// 7 blocks 736, 8 blocks 761 us.
 constexpr int kFwdBlocks = 7;
-// List entries a warp scans per batch: kFwdPer per lane.  The entries of
-// the window that reach a live ray of the sub-block (about a third of them
-// on the street views) are staged together, so that the staging pass, one
-// entry per lane, runs with more of its lanes busy than over a 32-entry
-// window.  Measured (street views, compositing alone / bench): 32 entries
-// 0.374 / 0.528 ms, 3219 Mrays/s; 64 entries 0.364 / 0.519 ms, 3284; 96
-// entries 0.362 / 0.514 ms, 3305; 128 entries 0.361 / 0.524 ms, 3265.
+// List entries a warp scans at a time: kFwdPer per lane.  Those that reach a
+// live ray of the sub-block (about a third on the street views) go to a queue
+// and are staged 32 at a time, so that the staging pass, one entry per lane,
+// runs with all its lanes busy whatever the window.  Measured (1920x1080
+// pinhole, 2M Gaussians): 32 entries 716, 64 711, 96 736 us.
 #ifndef SG_FWD_PER_LANE
-#define SG_FWD_PER_LANE 3
+#define SG_FWD_PER_LANE 2
 #endif
 constexpr int kFwdPer = SG_FWD_PER_LANE;
 constexpr int kFwdWin = 32 * kFwdPer;
-constexpr int kFwdStage = 64;
+constexpr int kFwdStage = 32;         // staged entries held in shared memory at once
+// the queue of entries to stage: a window's, after at most 31 left over
+constexpr int kFwdQueue = 128;
+static_assert(kFwdWin + 31 <= kFwdQueue && (kFwdQueue & (kFwdQueue - 1)) == 0, "staging queue");
 // Segment length of this kernel's work items (frames that keep no backward
 // state need not match the segments of a backward).  Measured on the street
 // views (compositing alone fisheye / pinhole, two-view step): 128 entries
 // 0.390 / 0.562 ms, 3102 Mrays/s; 256 0.363 / 0.513 ms, 3310; 384 0.367 /
 // 0.503 ms, 3364; 512 0.381 / 0.508 ms, 3384.  Longer runs mean fewer
 // merges; shorter ones split the densest tiles (the fisheye's) finer.
-constexpr uint32_t kFwdSeg = 384;   // staged entries held in shared memory at once
+constexpr uint32_t kFwdSeg = 384;
 
 // The tile's reference frame in world coordinates: d_T = dh + dl (from the
 // double direction, as cam_tile_ref) and e_1, e_2 rotated in float.
@@ -76,6 +76,97 @@ __device__ __forceinline__ void cross3(const float a[3], const float b[3], float
     c[2] = a[0] * b[1] - a[1] * b[0];
 }
 
+// The rays of a sub-block in the tangent plane, as a parallelogram that holds
+// every valid one: centre (x, y), half-edges along the pixel rows and columns.
+// s_reg: centre, row half-edge, column half-edge (2 floats each), a bound on
+// |x| + |y| over it, and 1 if there is one (the four corner lanes have rays).
+// Every lane calls it with its ray's coordinates.
+constexpr int kRegion = 8;
+__device__ __forceinline__ void fwd_region(float x, float y, bool has_ray, float *s_reg)
+{
+    constexpr uint32_t full = 0xffffffffu, corners = 0x81000081u;
+    const uint32_t have = __ballot_sync(full, has_ray);
+    const float x0 = __shfl_sync(full, x, 0), x7 = __shfl_sync(full, x, 7);
+    const float x24 = __shfl_sync(full, x, 24), x31 = __shfl_sync(full, x, 31);
+    const float y0 = __shfl_sync(full, y, 0), y7 = __shfl_sync(full, y, 7);
+    const float y24 = __shfl_sync(full, y, 24), y31 = __shfl_sync(full, y, 31);
+    const float xc = 0.25f * ((x0 + x7) + (x24 + x31)), yc = 0.25f * ((y0 + y7) + (y24 + y31));
+    const float gx = 0.25f * ((x7 - x0) + (x31 - x24)), gy = 0.25f * ((y7 - y0) + (y31 - y24));
+    const float hx = 0.25f * ((x24 - x0) + (x31 - x7)), hy = 0.25f * ((y24 - y0) + (y31 - y7));
+    // the lanes' coordinates along the two half-edges; their largest values
+    // (the lens curves the pixel grid) scale the parallelogram
+    const float det = gx * hy - gy * hx, inv = 1.f / det;
+    const float dx = x - xc, dy = y - yc;
+    const float s = fabsf(dx * hy - dy * hx) * fabsf(inv), t = fabsf(gx * dy - gy * dx) * fabsf(inv);
+    const float ks = 1.0001f * __uint_as_float(__reduce_max_sync(full, has_ray ? __float_as_uint(s) : 0u));
+    const float kt = 1.0001f * __uint_as_float(__reduce_max_sync(full, has_ray ? __float_as_uint(t) : 0u));
+    const bool ok = (have & corners) == corners && ks < 2.f && kt < 2.f;   // no for NaN, too
+    if ((threadIdx.x & 31) == 0) {
+        s_reg[0] = xc; s_reg[1] = yc;
+        s_reg[2] = ks * gx; s_reg[3] = ks * gy;
+        s_reg[4] = kt * hx; s_reg[5] = kt * hy;
+        s_reg[6] = fabsf(xc) + fabsf(yc) + ks * (fabsf(gx) + fabsf(gy)) + kt * (fabsf(hx) + fabsf(hy));
+        s_reg[7] = ok ? 1.f : 0.f;
+    }
+}
+
+__device__ __forceinline__ float rsqrt_approx(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Whether no ray of the sub-block composites the entry: alpha = sigma 2^-q
+// with q = |num|^2 / |den|^2 stays below alpha_min wherever |num|^2 > c
+// |den|^2, c = log2(sigma / alpha_min).  Over the parallelogram num is n_c + s
+// A + t B, |s|, |t| <= 1.  For any vector u, |num| |u| >= u . n_c - |u . A| -
+// |u . B|; u is taken as the point of the parallelogram nearest to 0 (by
+// coordinate descent: a bad u only weakens the bound).  |den| is bounded per
+// component.  Half of a pinhole street view's (entry, sub-block) pairs are left
+// out (a box is mostly empty beside a long diagonal ellipse), a sixth of a
+// fisheye view's; the test takes about 4 instructions a pair (a lane each, 32
+// at once), the composited pair it saves about 50.  Measured, compositing:
+// 1920x1080 pinhole of 2M Gaussians 938 -> 711 us; both street views of 1M in
+// one step 1341 -> 1193 us; a 641x479 fisheye view (7% left out) 62 -> 64 us.
+// The slack covers the rounding of the bound and of the pair
+// evaluation: 4e-6 (about 30 ulp) of the size of the terms num is summed
+// from, and 1e-3 relative on q.  False for any NaN.
+__device__ __forceinline__ bool fwd_unseen(const float a[3], const float p1[3], const float p2[3],
+                                           const float b[3], const float m1[3], const float m2[3],
+                                           float sigma, float alpha_min, const float *s_reg)
+{
+    const float xc = s_reg[0], yc = s_reg[1], gx = s_reg[2], gy = s_reg[3];
+    const float hx = s_reg[4], hy = s_reg[5];
+    float n[3], A[3], B[3];
+    float mag = 0.f, mp = 0.f, U2 = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        n[k] = a[k] + xc * p1[k] + yc * p2[k];
+        A[k] = gx * p1[k] + gy * p2[k];
+        B[k] = hx * p1[k] + hy * p2[k];
+        mag += fabsf(a[k]);
+        mp += fabsf(p1[k]) + fabsf(p2[k]);
+        const float d = fabsf(b[k] + xc * m1[k] + yc * m2[k]) + fabsf(gx * m1[k] + gy * m2[k]) +
+                        fabsf(hx * m1[k] + hy * m2[k]);
+        U2 += d * d;
+    }
+    mag += s_reg[6] * mp;
+    const float na = dot3(n, A), nb = dot3(n, B), ab = dot3(A, B);
+    const float ia = __fdividef(1.f, dot3(A, A)), ib = __fdividef(1.f, dot3(B, B));
+    float s = fmaxf(-1.f, fminf(1.f, -na * ia));
+    float t = fmaxf(-1.f, fminf(1.f, -(nb + s * ab) * ib));
+    s = fmaxf(-1.f, fminf(1.f, -(na + t * ab) * ia));
+    t = fmaxf(-1.f, fminf(1.f, -(nb + s * ab) * ib));
+    float u[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[k] = n[k] + s * A[k] + t * B[k];
+    const float uu = dot3(u, u);
+    const float low = dot3(u, n) - fabsf(dot3(u, A)) - fabsf(dot3(u, B)) - 4e-6f * mag * uu * rsqrt_approx(uu);
+    const float c = 1.0002f * __log2f(__fdividef(sigma, alpha_min)) + 1e-3f;
+    return low > 0.f && low * low > 1.001f * c * U2 * uu;
+}
+
 // A staged entry, 7 float4 (one per shared-memory plane):
 //   0 (a0, p01, p02, a1)   1 (p11, p12, a2, p21)   2 (p22, b0, m01, m02)
 //   3 (b1, m11, m12, b2)   4 (m21, m22, t0, t1)    5 (t2, sigma, c0, c1)
@@ -84,10 +175,13 @@ __device__ __forceinline__ void cross3(const float a[3], const float b[3], float
 // carry the response scale sqrt(log2(e) / 2), as in cam_pair_scaled, so that
 // |num|^2 / |den|^2 is the exponent of 2.  ref: the tile's reference frame
 // (dh, dl, e_1, e_2), in the warp's shared memory.
-__device__ __forceinline__ void fwd_entry(const GRec &r, const float o[3], const float *ref,
-                                          float4 e[7])
+// The entry goes to slot `t` of the warp's planes s, with its lane mask.
+// Returns whether some ray of the sub-block (s_reg) may composite it.
+__device__ __forceinline__ bool fwd_entry(const GRec &r, const float o[3], const float *ref,
+                                          const float *s_reg, float alpha_min, uint32_t lanes,
+                                          float4 (*s)[kFwdStage], int t)
 {
-    const float mu[3] = {r.mu_sigma.x, r.mu_sigma.y, r.mu_sigma.z};
+    const float mu[3] = {r.mu_sigma.x, r.mu_sigma.y, r.mu_sigma.z}, sigma = r.mu_sigma.w;
     const float M[3][3] = {{r.m0.x, r.m0.y, r.m0.z}, {r.m1.x, r.m1.y, r.m1.z},
                            {r.m2.x, r.m2.y, r.m2.z}};
     const float f[3] = {kResponseScale * r.m0.w, kResponseScale * r.m1.w,
@@ -109,13 +203,14 @@ __device__ __forceinline__ void fwd_entry(const GRec &r, const float o[3], const
         m2[k] = dot3(M[k], e2);
         mv[k] = dot3(M[k], vh);
     }
-    e[0] = make_float4(a[0], p1[0], p2[0], a[1]);
-    e[1] = make_float4(p1[1], p2[1], a[2], p1[2]);
-    e[2] = make_float4(p2[2], b[0], m1[0], m2[0]);
-    e[3] = make_float4(b[1], m1[1], m2[1], b[2]);
-    e[4] = make_float4(m1[2], m2[2], dot3(mv, b), dot3(mv, m1));
-    e[5] = make_float4(dot3(mv, m2), r.mu_sigma.w, r.feat.x, r.feat.y);
-    e[6] = make_float4(r.feat.z, 0.f, 0.f, 0.f);
+    s[0][t] = make_float4(a[0], p1[0], p2[0], a[1]);
+    s[1][t] = make_float4(p1[1], p2[1], a[2], p1[2]);
+    s[2][t] = make_float4(p2[2], b[0], m1[0], m2[0]);
+    s[3][t] = make_float4(b[1], m1[1], m2[1], b[2]);
+    s[4][t] = make_float4(m1[2], m2[2], dot3(mv, b), dot3(mv, m1));
+    s[5][t] = make_float4(dot3(mv, m2), sigma, r.feat.x, r.feat.y);
+    s[6][t] = make_float4(r.feat.z, __uint_as_float(lanes), 0.f, 0.f);
+    return s_reg[7] == 0.f || !fwd_unseen(a, p1, p2, b, m1, m2, sigma, alpha_min, s_reg);
 }
 
 struct FwdAcc {
@@ -158,21 +253,59 @@ __device__ __forceinline__ void fwd_composite(const CamRender &P, float4 (*s)[kF
     }
 }
 
+// Stage the n <= 32 entries waiting at the head of the warp's queue and
+// composite the ones a ray of the sub-block may composite.  Each lane stages
+// one entry at its own slot, tests it, and moves it to its place among the
+// kept ones (through shared memory, a plane at a time: the 28 registers of an
+// entry do not fit beside the test's).
+__device__ __forceinline__ void fwd_batch(const CamRender &P, const CamPose &pose,
+                                          const GRec *__restrict__ rec, const float *ref,
+                                          const uint2 *cand, uint32_t head, int n, float x, float y,
+                                          float4 (*s)[kFwdStage], FwdAcc &a, bool &done)
+{
+    const int lane = threadIdx.x & 31;
+    bool keep = false;
+    __syncwarp();
+    if (lane < n) {
+        const uint2 c = cand[(head + lane) % kFwdQueue];
+        keep = fwd_entry(rec[c.x], pose.t, ref, ref + 12, P.alpha_min, c.y, s, lane);
+    }
+    const uint32_t kb = __ballot_sync(0xffffffffu, keep);
+    const int m = __popc(kb);
+    __syncwarp();
+    if (m != n) {
+        const int t = __popc(kb & ((1u << lane) - 1u));
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+            float4 e;
+            if (keep) e = s[k][lane];
+            __syncwarp();
+            if (keep) s[k][t] = e;
+        }
+        __syncwarp();
+    }
+    fwd_composite(P, s, m, x, y, a, done);
+}
+
 // Composite list entries [lo, hi) of a tile that can reach sub-block `sub`
 // into the lane's accumulator.  Lanes whose ray is done take part in the
 // staging and keep their state; only entries whose box holds a live ray are
 // staged (their lane masks come from the column/row words, no record load).
-// cand: the warp's (Gaussian, lane mask) list of a window's staged entries.
+// ref: the tile's reference frame, then the sub-block's region, which the
+// first walk of an item (done = no ray) writes through `region`.  cand: the
+// warp's queue of (Gaussian, lane mask) entries to stage, a ring; they are
+// staged 32 at a time, so that every lane of a staging pass has one.
 __device__ __forceinline__ void fwd_walk(const CamRender &P, const CamPose &pose,
                                          const GRec *__restrict__ rec,
                                          const uint32_t *__restrict__ ids,
                                          const uint32_t *__restrict__ crw, int sub, uint32_t lo,
                                          uint32_t hi, const float *ref, float x, float y,
                                          float4 (*s)[kFwdStage], uint2 *cand, FwdAcc &a,
-                                         bool &done)
+                                         bool &done, float *region = nullptr)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
+    uint32_t head = 0u, tail = 0u;
     // the next window's column/row words and Gaussian ids (entries lane + 32 w
     // of it), loaded one window ahead
     uint32_t ncr[kFwdPer], nid[kFwdPer];
@@ -182,14 +315,16 @@ __device__ __forceinline__ void fwd_walk(const CamRender &P, const CamPose &pose
         ncr[w] = i < hi ? crw[i] : 0u;
         nid[w] = i < hi ? ids[i] : 0u;
     }
+    if (region) fwd_region(x, y, !done, region);    // while they arrive
     for (uint32_t base = lo; base < hi; base += kFwdWin) {
         const uint32_t act = __ballot_sync(0xffffffffu, !done);
-        if (act == 0u) break;
-        uint32_t g[kFwdPer], lm[kFwdPer], bw[kFwdPer];
+        if (act == 0u) return;
 #pragma unroll
         for (int w = 0; w < kFwdPer; ++w) {
-            g[w] = nid[w];
-            lm[w] = word_lanes(ncr[w], sub) & act;
+            const uint32_t lm = word_lanes(ncr[w], sub) & act;
+            const uint32_t bw = __ballot_sync(0xffffffffu, lm != 0u);
+            if (lm) cand[(tail + __popc(bw & below)) % kFwdQueue] = make_uint2(nid[w], lm);
+            tail += __popc(bw);
             const uint32_t i = base + kFwdWin + 32 * w + lane;
             ncr[w] = 0u;
             if (i < hi) {
@@ -197,34 +332,12 @@ __device__ __forceinline__ void fwd_walk(const CamRender &P, const CamPose &pose
                 nid[w] = ids[i];
             }
         }
-        int n = 0;
-#pragma unroll
-        for (int w = 0; w < kFwdPer; ++w) {
-            bw[w] = __ballot_sync(0xffffffffu, lm[w] != 0u);
-            n += __popc(bw[w]);
-        }
-        if (n == 0) continue;
-        __syncwarp();
-        int off = 0;
-#pragma unroll
-        for (int w = 0; w < kFwdPer; ++w) {
-            if (lm[w]) cand[off + __popc(bw[w] & below)] = make_uint2(g[w], lm[w]);
-            off += __popc(bw[w]);
-        }
-        // stage and composite them, in list order, kFwdStage at a time
-        for (int c0 = 0; c0 < n; c0 += kFwdStage) {
-            const int m = n - c0 < kFwdStage ? n - c0 : kFwdStage;
-            __syncwarp();
-            for (int t = lane; t < m; t += 32) {
-                const uint2 c = cand[c0 + t];
-                float4 e[7];
-                fwd_entry(rec[c.x], pose.t, ref, e);
-                e[6].y = __uint_as_float(c.y);
-#pragma unroll
-                for (int k = 0; k < 7; ++k) s[k][t] = e[k];
-            }
-            __syncwarp();
-            fwd_composite(P, s, m, x, y, a, done);
+        // after the last window, what is left over
+        const uint32_t least = base + kFwdWin < hi ? 32u : 1u;
+        while (tail - head >= least) {
+            const uint32_t n = min(32u, tail - head);
+            fwd_batch(P, pose, rec, ref, cand, head, (int)n, x, y, s, a, done);
+            head += n;
         }
     }
 }
@@ -248,8 +361,8 @@ k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *_
                     const float *__restrict__ tile_basis, const RenderDesc *__restrict__ D)
 {
     __shared__ float4 s_all[kFwdWarps][7][kFwdStage];
-    __shared__ uint2 s_cand[kFwdWarps][kFwdWin];
-    __shared__ float s_refs[kFwdWarps][12];
+    __shared__ uint2 s_cand[kFwdWarps][kFwdQueue];
+    __shared__ __align__(16) float s_refs[kFwdWarps][12 + kRegion];
     __shared__ CamPose s_pose;
     load_cam_pose(D, s_pose);
     __syncthreads();
@@ -280,7 +393,8 @@ k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *_
         const uint32_t hi = min(rg.y, lo + kSeg);
         FwdAcc a = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         bool done = no_ray;
-        fwd_walk(P, s_pose, rec, ids, crw, sub, lo, hi, s_ref, e.x, e.y, s_e, cand, a, done);
+        fwd_walk(P, s_pose, rec, ids, crw, sub, lo, hi, s_ref, e.x, e.y, s_e, cand, a, done,
+                 s_ref + 12);
         if (ti.x > 1) {
             // long tile: publish this run, and combine if it is the last one
             fwd_put(partials + ((size_t)(ti.y + seg) * 256 + sub * 32 + lane) * 2, a,
