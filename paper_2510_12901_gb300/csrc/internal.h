@@ -320,9 +320,17 @@ constexpr WorkSize work_size(int64_t units, int64_t n_pairs, uint32_t seg_len, i
 // 8-bit passes: digit counts and offsets (256 per pass), per-pass tile
 // tickets, and the look-back words (256 per tile of kRadixTile pairs and pass).
 #ifndef SG_RADIX_TILE
-#define SG_RADIX_TILE 8192
+#define SG_RADIX_TILE 4096
 #endif
 constexpr int kRadixTile = SG_RADIX_TILE;
+// First key bit of pass p of a sort of bits [begin, end): the bits split
+// evenly over the passes (of at most 8 each), so that no pass has more
+// digits, and shorter runs of one digit, than it needs.
+__host__ __device__ constexpr int radix_bit(int begin, int end, int p)
+{
+    const int passes = (end - begin + 7) / 8;
+    return begin + (end - begin) * p / passes;
+}
 constexpr int64_t radix_scratch_words(int64_t n_max, int passes)
 {
     const int64_t tiles = (n_max + kRadixTile - 1) / kRadixTile;
@@ -331,7 +339,7 @@ constexpr int64_t radix_scratch_words(int64_t n_max, int passes)
 // The depth stage's scratch (fr.hist): the radix scratch of its 4 passes,
 // then two tickets and a 64-bit look-back word per tile of kChainTile
 // entries for each of its two chained scans.
-constexpr int kChainTile = 4096;
+constexpr int kChainTile = 2048;
 constexpr int64_t depth_stage_words(int64_t n)
 {
     return radix_scratch_words(n, 4) + 2 * (2 + 2 * ((n + kChainTile - 1) / kChainTile));
@@ -341,9 +349,10 @@ sg_status radix_prepare(int64_t n_max, int passes, Frame &fr, cudaStream_t st, u
 // Stable sort of up to n pairs (*d_n of them) by key bits [begin_bit,
 // end_bit); the digit counts are in the scratch that radix_prepare returned.
 // site: SG_LOOKBACK_DEPTH_SORT or SG_LOOKBACK_TILE_SORT (the test hook's site).
+// keep_keys = false: only the values are needed (keys[*result_buf] is stale).
 sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n,
                            const uint32_t *d_n, int begin_bit, int end_bit, Frame &fr,
-                           cudaStream_t st, int *result_buf, int site);
+                           cudaStream_t st, int *result_buf, int site, bool keep_keys = true);
 // The depth stage: the Gaussians with a non-zero tile count sorted by depth
 // (keys/vals[*result_buf]: depth bits, ids), d_scal[0] = their number,
 // d_offsets = exclusive scan of their tile counts in that order, d_scal[1]

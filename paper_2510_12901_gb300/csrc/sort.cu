@@ -30,33 +30,10 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v)
     return v;
 }
 
-// Block-wide exclusive scan of one value per thread; returns the exclusive
-// prefix and writes the block total to *total.
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *s_warp, uint32_t *total)
-{
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    uint32_t inc = warp_incl_scan(v);
-    if (lane == 31) s_warp[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t w = lane < nw ? s_warp[lane] : 0u;
-        uint32_t wi = warp_incl_scan(w);
-        if (lane < nw) s_warp[lane] = wi - w;
-        if (lane == nw - 1) s_warp[32] = wi;
-    }
-    __syncthreads();
-    uint32_t r = s_warp[warp] + inc - v;
-    *total = s_warp[32];
-    __syncthreads();
-    return r;
-}
-
 // ------------------------------------------------------------------ radix sort
 // Lanes of the warp holding the same 8-bit digit as this one, among lanes
 // with a key (valid): one ballot per bit, each lane keeping the lanes that
 // agree with it on that bit.  A lane without a key is in no lane's set.
-// (Nine ballots take less time here than __match_any_sync: the depth stage
-// went from 0.144 to 0.127 ms per view.)
 __device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid)
 {
     uint32_t peers = __ballot_sync(0xffffffffu, valid);
@@ -69,29 +46,55 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid)
     return peers;
 }
 
-// Stable LSD radix sort of (key, value) pairs, 8-bit digits, one kernel per
-// digit pass with decoupled look-back (the "onesweep" scheme):
+// Stable LSD radix sort of (key, value) pairs, digits of at most 8 bits, one
+// kernel per digit pass with decoupled look-back (the "onesweep" scheme):
 //   1. the kernel that writes the keys counts the digits of every pass
 //      (k_compact_depth, k_bin) into scratch that radix_prepare zeroed;
-//   2. per pass, the exclusive scan of its 256 counts gives the first
+//   2. per pass, the exclusive scan of its digit counts gives the first
 //      output position of each digit (every block of the pass scans them);
 //   3. k_onesweep, per pass: a block takes the next tile of kRadixTile pairs
 //      (an atomic ticket, so tiles are taken in order), ranks them stably
-//      (each warp owns kRadixItems x 32 consecutive pairs, ranks among equal
-//      digits from per-bit ballots), publishes its per-digit counts, and
-//      walks back over earlier tiles' published counts, kLbBatch tiles per
-//      round of loads, until it meets an inclusive prefix; then it
-//      publishes its own inclusive prefix and scatters.
-// A tile only waits for tiles taken before it, whose blocks are running;
-// every such wait is bounded, and a wait that runs out sets *err.
+//      (each warp owns kRadixItems x 32 consecutive pairs), publishes its
+//      per-digit counts, orders its pairs by digit in shared memory, and walks back over
+//      earlier tiles' published counts until it meets an inclusive prefix;
+//      then it publishes its own and writes its pairs out.
+// A tile only waits for tiles taken before it, whose blocks are running and
+// which publish their counts before they wait themselves; every such wait is
+// bounded, and a wait that runs out sets *err.
+//
+// A pass moves 16 bytes a pair, all in L2 at the sizes of a frame: it is
+// bound by the latency of its stages and by L2 transactions.  Hence
+//   - tiles of 4096 pairs (512 threads, two blocks an SM: three spill), so
+//     that 0.7M pairs fill the chip;
+//   - equal digits found by an atomicOr of lane bits into the digit's word
+//     (8 ballots a pair took the six passes of a 1M view from 89 to 97 us);
+//   - a look-back that reads 32 tiles' words a round, four digits a load, in
+//     eight groups of threads: the tiles of a launch all publish at about the
+//     same time, so a walk of 8 words a round was a chain of tiles / 8 rounds
+//     of L2 latency.  More words a round cost more than they save (64: 103
+//     us): reading words that are not yet published delays their writers;
+//   - pairs written from shared memory in digit order, consecutive threads to
+//     consecutive addresses within a digit (a scattered 4-byte write is an L2
+//     transaction of its own).
+// Measured, the six passes of a frame (four over the visible Gaussians, two
+// over the pairs), against tiles of 8192 ranked by ballots, eight words a
+// round and scattered writes: 150k Gaussians 85 -> 45 us, 1M (1.5M pairs) 120
+// -> 87 us, 2M (3.9M pairs) 242 -> 149 us.
 #ifndef SG_RADIX_THREADS
-#define SG_RADIX_THREADS 1024
+#define SG_RADIX_THREADS 512
 #endif
-constexpr int kRadixThreads = SG_RADIX_THREADS;   // >= 256: one digit per thread below 256
+constexpr int kRadixThreads = SG_RADIX_THREADS;
 constexpr int kRadixItems = kRadixTile / kRadixThreads;
-static_assert(kRadixThreads >= 256 && kRadixItems * kRadixThreads == kRadixTile,
-              "radix tile layout");
 constexpr int kRadixWarps = kRadixThreads / 32;
+constexpr int kLbGroups = kRadixThreads / 64;        // threads per four digits in the look-back
+#ifndef SG_LB_BATCH
+#define SG_LB_BATCH 4
+#endif
+constexpr int kLbBatch = SG_LB_BATCH;                // earlier tiles a thread reads a round
+static_assert(kRadixThreads % 256 == 0 && kRadixItems * kRadixThreads == kRadixTile &&
+                  kRadixTile <= 65535 && kRadixWarps * 256 <= kRadixTile, "radix tile layout");
+static_assert(kLbGroups * 256 * sizeof(uint32_t) <= kRadixWarps * 256 * sizeof(uint16_t),
+              "look-back sums in the counts' place");
 constexpr uint32_t kLbAgg = 1u << 30, kLbPre = 2u << 30, kLbCount = (1u << 30) - 1u;
 // Polling rounds a look-back wait makes before it gives up (about a second
 // on an idle GPU).  Test hook: the tile whose look-back words the kernels
@@ -108,108 +111,193 @@ __device__ __forceinline__ int64_t held_tile(int site)
     return *(volatile int *)&g_hold_site == site ? (int64_t) * (volatile long long *)&g_hold_tile
                                                  : (int64_t)-1;
 }
-#ifndef SG_LB_BATCH
-#define SG_LB_BATCH 8
-#endif
-constexpr int kLbBatch = SG_LB_BATCH;   // earlier tiles' words loaded per look-back round
 
-__global__ void __launch_bounds__(kRadixThreads)
+// Exclusive scans of two values per thread over the block's first 256
+// threads (the others pass anything); every thread of the block calls it.
+__device__ __forceinline__ uint2 excl_scan2_256(uint32_t a, uint32_t b, uint2 *s_w)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t ia = warp_incl_scan(a), ib = warp_incl_scan(b);
+    if (lane == 31 && warp < 8) s_w[warp] = make_uint2(ia, ib);
+    __syncthreads();
+    uint2 r = make_uint2(ia - a, ib - b);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        const uint2 t = s_w[w];
+        if (w < warp) { r.x += t.x; r.y += t.y; }
+    }
+    return r;
+}
+
+// Four digits' look-back words of a tile (16-byte aligned), past the L1.
+__device__ __forceinline__ uint4 load_words(const uint32_t *p)
+{
+    uint4 w;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w)
+                 : "l"(p)
+                 : "memory");
+    return w;
+}
+
+__device__ __forceinline__ bool published(const uint4 &w)
+{
+    constexpr uint32_t f = kLbAgg | kLbPre;
+    return (w.x & f) && (w.y & f) && (w.z & f) && (w.w & f);
+}
+
+__global__ void __launch_bounds__(kRadixThreads, 2)
 k_onesweep(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
            uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out,
            const uint32_t *__restrict__ d_n, int shift, uint32_t mask,
            const uint32_t *__restrict__ hist, uint32_t *__restrict__ lookback,
            uint32_t *__restrict__ ticket, uint32_t *__restrict__ err, int site)
 {
-    __shared__ uint32_t s_cnt[kRadixWarps][256];
-    __shared__ uint32_t s_pre[256];
-    __shared__ uint32_t s_warp[33];
+    // the warps' digit counts, then the look-back groups' sums
+    __shared__ __align__(16) union {
+        uint16_t cnt[kRadixWarps][256];
+        uint32_t far[kLbGroups][256];
+    } S;
+    __shared__ __align__(16) uint32_t s_key[kRadixTile], s_val[kRadixTile];
+    __shared__ uint32_t s_start[256], s_pre[256];
+    __shared__ uint2 s_w[8];
     __shared__ uint32_t s_tile;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < kRadixWarps * 256; i += kRadixThreads) (&s_cnt[0][0])[i] = 0;
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t == 0) s_tile = atomicAdd(ticket, 1u);
+    const int64_t n = *d_n;
+    const uint32_t h = t < 256 ? hist[t] : 0u;
+    const int64_t held = held_tile(site);
+    const uint32_t max_spins = g_lb_spins;
+    for (int i = t; i < kRadixWarps * 128; i += kRadixThreads) ((uint32_t *)&S.cnt[0][0])[i] = 0u;
+    for (int i = t; i < kRadixWarps * 64; i += kRadixThreads)
+        reinterpret_cast<uint4 *>(s_key)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     const uint32_t tile = s_tile;
-    const int64_t n = *d_n;
     const int64_t base = (int64_t)tile * kRadixTile;
     if (base >= n) return;     // so is every later tile: nobody waits for this one
-    // the first output position of this thread's digit (threads < 256): the
-    // exclusive scan of the pass's digit counts, done by every block
-    uint32_t dig_total;
-    const uint32_t dig_off =
-        block_excl_scan(threadIdx.x < 256 ? hist[threadIdx.x] : 0u, s_warp, &dig_total);
-    uint32_t k[kRadixItems], v[kRadixItems], d[kRadixItems], rk[kRadixItems];
+    const int cnt = n - base < kRadixTile ? (int)(n - base) : kRadixTile;
+    const int w0 = warp * 32 * kRadixItems + lane;      // the thread's first pair in the tile
+    uint32_t k[kRadixItems], v[kRadixItems];
+#pragma unroll
+    for (int r = 0; r < kRadixItems; ++r) k[r] = w0 + 32 * r < cnt ? keys_in[base + w0 + 32 * r] : 0u;
+#pragma unroll
+    for (int r = 0; r < kRadixItems; ++r) v[r] = w0 + 32 * r < cnt ? vals_in[base + w0 + 32 * r] : 0u;
+    // ranks among the warp's earlier pairs of the same digit (the words of
+    // lane bits lie where the ordered keys will)
+    uint16_t rk[kRadixItems];
 #pragma unroll
     for (int r = 0; r < kRadixItems; ++r) {
-        const int64_t idx = base + (int64_t)warp * 32 * kRadixItems + r * 32 + lane;
-        const bool in = idx < n;
-        k[r] = in ? keys_in[idx] : 0u;
-        v[r] = in ? vals_in[idx] : 0u;
-        d[r] = in ? (k[r] >> shift) & mask : 0xffffffffu;
-        const uint32_t peers = digit_peers(d[r], in);
-        const uint32_t below = __popc(peers & ((1u << lane) - 1u));
-        const uint32_t before = in ? s_cnt[warp][d[r]] : 0u;
-        rk[r] = before + below;
+        const bool in = w0 + 32 * r < cnt;
+        const uint32_t d = (k[r] >> shift) & mask;
+        uint32_t *m = s_key + warp * 256;
+        if (in) atomicOr(&m[d], 1u << lane);
         __syncwarp();
-        if (in && lane == __ffs(peers) - 1) s_cnt[warp][d[r]] = before + __popc(peers);
+        const uint32_t peers = in ? m[d] : 0u;
+        const uint32_t before = in ? S.cnt[warp][d] : 0u;
+        rk[r] = (uint16_t)(before + __popc(peers & ((1u << lane) - 1u)));
+        __syncwarp();
+        if (in && lane == __ffs(peers) - 1) {
+            S.cnt[warp][d] = (uint16_t)(before + __popc(peers));
+            m[d] = 0u;
+        }
         __syncwarp();
     }
     __syncthreads();
-    if (threadIdx.x < 256) {
-        // one digit per thread: offsets of the warps within the tile, the
-        // tile's count, then the look-back for the pairs of earlier tiles
-        const uint32_t dg = threadIdx.x;
-        uint32_t run = 0;
+    // one digit per thread: the warps' offsets within the digit and the
+    // tile's count, published at once
+    const bool publish = (int64_t)tile != held;
+    uint32_t run = 0u;
+    if (t < 256) {
+        uint32_t c[kRadixWarps];
+#pragma unroll
+        for (int w = 0; w < kRadixWarps; ++w) c[w] = S.cnt[w][t];
 #pragma unroll
         for (int w = 0; w < kRadixWarps; ++w) {
-            const uint32_t c = s_cnt[w][dg];
-            s_cnt[w][dg] = run;
-            run += c;
+            S.cnt[w][t] = (uint16_t)run;
+            run += c[w];
         }
-        volatile uint32_t *lb = lookback;
-        const bool publish = (int64_t)tile != held_tile(site);
-        const uint32_t max_spins = g_lb_spins;
-        if (publish) lb[(int64_t)tile * 256 + dg] = (tile == 0 ? kLbPre : kLbAgg) | run;
-        uint32_t excl = 0, spins = 0;
-        int64_t t = (int64_t)tile - 1;
-        while (t >= 0) {
-            // the words of tiles t, t-1, .. at once (before tile 0: an empty
-            // inclusive prefix); take them in order up to an inclusive prefix
-            // or up to one not yet published, which the next round reloads
-            uint32_t w[kLbBatch];
-#pragma unroll
-            for (int k = 0; k < kLbBatch; ++k)
-                w[k] = t - k >= 0 ? (uint32_t)lb[(t - k) * 256 + dg] : (uint32_t)kLbPre;
-            int took = 0;
-            bool pre = false, wait = false;
-#pragma unroll
-            for (int k = 0; k < kLbBatch; ++k) {
-                if (pre || wait) continue;
-                if (w[k] & (kLbAgg | kLbPre)) {
-                    excl += w[k] & kLbCount;
-                    pre = (w[k] & kLbPre) != 0u;
-                    ++took;
-                } else {
-                    wait = true;
-                }
-            }
-            if (pre) break;
-            t -= took;
-            if (took == 0 && ++spins > max_spins) {   // gave up: flag it, leave the order wrong
-                atomicOr(err, kStatusLookback);
-                break;
-            }
-        }
-        if (tile > 0 && publish) lb[(int64_t)tile * 256 + dg] = kLbPre | (excl + run);
-        s_pre[dg] = dig_off + excl;
+        if (publish)
+            ((volatile uint32_t *)lookback)[(int64_t)tile * 256 + t] =
+                (tile == 0 ? kLbPre : kLbAgg) | run;
     }
+    // first position of the digit in the tile and in the pass's output
+    const uint2 first = excl_scan2_256(run, h, s_w);
+    if (t < 256) s_start[t] = first.x;
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < kRadixItems; ++r) {
-        const int64_t idx = base + (int64_t)warp * 32 * kRadixItems + r * 32 + lane;
-        if (idx < n) {
-            const uint32_t pos = s_pre[d[r]] + s_cnt[warp][d[r]] + rk[r];
-            keys_out[pos] = k[r];
-            vals_out[pos] = v[r];
+        if (w0 + 32 * r < cnt) {
+            const uint32_t d = (k[r] >> shift) & mask;
+            const uint32_t q = s_start[d] + S.cnt[warp][d] + rk[r];
+            s_key[q] = k[r];
+            s_val[q] = v[r];
+        }
+    }
+    __syncthreads();
+    // look-back: thread (group g, digits 4 q .. 4 q + 3) sums the words of the
+    // kLbBatch tiles before hi - g kLbBatch, up to the first inclusive prefix
+    uint32_t excl = 0u;
+    bool done = tile == 0;
+    const int q = t & 63, g = t >> 6;
+    const bool used = 4u * q <= mask;
+    for (int64_t hi = tile; hi > 0; hi -= kLbGroups * kLbBatch) {
+        const int64_t h0 = hi - 1 - g * kLbBatch;
+        const uint32_t *words = lookback + h0 * 256 + 4 * q;
+        if (used) {
+            uint4 w[kLbBatch], sum = make_uint4(0u, 0u, 0u, 0u);
+            uint32_t spins = 0, found = 0u;
+#pragma unroll
+            for (int i = 0; i < kLbBatch; ++i)      // before tile 0: an empty inclusive prefix
+                w[i] = h0 - i >= 0 ? load_words(words - 256 * i)
+                                   : make_uint4(kLbPre, kLbPre, kLbPre, kLbPre);
+#pragma unroll
+            for (int i = 0; i < kLbBatch; ++i) {
+                if (found == 15u) continue;
+                while (!published(w[i])) {       // only these words are read again
+                    if (++spins > max_spins) {   // gave up: flag it, leave the order wrong
+                        atomicOr(err, kStatusLookback);
+                        w[i] = make_uint4(kLbPre, kLbPre, kLbPre, kLbPre);
+                        break;
+                    }
+                    w[i] = load_words(words - 256 * i);
+                }
+                if (!(found & 1u)) sum.x += w[i].x & kLbCount;
+                if (!(found & 2u)) sum.y += w[i].y & kLbCount;
+                if (!(found & 4u)) sum.z += w[i].z & kLbCount;
+                if (!(found & 8u)) sum.w += w[i].w & kLbCount;
+                found |= (w[i].x >> 31) | (w[i].y >> 31) << 1 | (w[i].z >> 31) << 2 |
+                         (w[i].w >> 31) << 3;
+            }
+            sum.x |= (found & 1u) << 31;
+            sum.y |= (found & 2u) << 30;
+            sum.z |= (found & 4u) << 29;
+            sum.w |= (found & 8u) << 28;
+            *reinterpret_cast<uint4 *>(&S.far[g][4 * q]) = sum;
+        }
+        __syncthreads();
+        const bool walk = t < 256 && !done;
+        if (walk) {
+#pragma unroll
+            for (int i = 0; i < kLbGroups; ++i) {
+                const uint32_t x = t <= (int)mask ? S.far[i][t] : kLbPre;
+                if (!done) excl += x & kLbCount;
+                done = done || (x & kLbPre) != 0u;
+            }
+            if (done && publish)
+                ((volatile uint32_t *)lookback)[(int64_t)tile * 256 + t] = kLbPre | (excl + run);
+        }
+        if (!__syncthreads_or(t < 256 && !done)) break;
+    }
+    if (t < 256) s_pre[t] = first.y + excl - first.x;
+    __syncthreads();
+    // the digit's pairs of this tile follow one another in the output; after a
+    // wait gave up the counts may not match the pairs: nothing past the end
+    for (int i = t; i < cnt; i += kRadixThreads) {
+        const uint32_t key = s_key[i];
+        const uint32_t pos = s_pre[(key >> shift) & mask] + i;
+        if (pos < n) {
+            if (keys_out) keys_out[pos] = key;
+            vals_out[pos] = s_val[i];
         }
     }
 }
@@ -231,7 +319,7 @@ sg_status radix_prepare(int64_t n_max, int passes, Frame &fr, cudaStream_t st, u
 
 sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
                            const uint32_t *d_n, int begin_bit, int end_bit, Frame &fr,
-                           cudaStream_t st, int *result_buf, int site)
+                           cudaStream_t st, int *result_buf, int site, bool keep_keys)
 {
     *result_buf = 0;
     if (n_max <= 0 || end_bit <= begin_bit) return SG_OK;
@@ -247,10 +335,11 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
     uint32_t *err = (uint32_t *)fr.scalars.p + kScalStatus;
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
-        const int b = begin_bit + 8 * p;
-        const int bits = end_bit - b < 8 ? end_bit - b : 8;
+        const int b = radix_bit(begin_bit, end_bit, p);
+        const int bits = radix_bit(begin_bit, end_bit, p + 1) - b;
+        uint32_t *keys_out = p == passes - 1 && !keep_keys ? nullptr : keys[cur ^ 1];
         k_onesweep<<<(unsigned)tiles, kRadixThreads, 0, st>>>(
-            keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], d_n, b, (1u << bits) - 1u,
+            keys[cur], vals[cur], keys_out, vals[cur ^ 1], d_n, b, (1u << bits) - 1u,
             hist + 256 * p, lookback + (int64_t)p * tiles * 256, tickets + p, err, site);
         SG_LAUNCHED();
         cur ^= 1;
@@ -270,47 +359,96 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
 //     histograms of the four radix passes over their keys;
 //   k_pair_offsets: in depth order, the exclusive scan of the tile counts
 //     count[ids[i]] (gathered as it goes) into pair offsets, and the total.
+// Both are bound by latency (a few MB, in L2).  The compaction publishes its
+// tile's total before it counts digits, with plain shared-memory atomics
+// (ballots over 64 digits a thread held the publication back): 26 -> 11 us at
+// 1M Gaussians, 41 -> 17 us at 2M, tiles of 2048 so that 1M give every SM
+// three blocks.  The offsets gather a 4-byte count per Gaussian (one L1 request
+// each, about 5 us at 1.5M) and take tiles of 8192, whose shorter look-back
+// chain is worth more than the fuller chip: at 1M 9.7 us (4096: 14, 2048: 17),
+// at 2M 16 us.  One warp walks back, 32 words a round: 128 words a round or
+// all warps reading took 11 -> 12 and 14 -> 17 us.
 constexpr int kChainThreads = 256;
 constexpr int kChainWarps = kChainThreads / 32;
 constexpr int kChainChunks = kChainTile / kChainThreads;   // 32-entry chunks per warp
-static_assert(kChainChunks * kChainThreads == kChainTile && kChainChunks == 16, "chain tile");
+#ifndef SG_OFF_CHUNKS
+#define SG_OFF_CHUNKS 32
+#endif
+constexpr int kOffChunks = SG_OFF_CHUNKS;                  // of a tile of k_pair_offsets
+constexpr int kOffTile = kOffChunks * kChainThreads;
+static_assert(kOffTile >= kChainTile, "look-back words sized by kChainTile");
+static_assert(kChainChunks * kChainThreads == kChainTile && kChainWarps == 8, "chain tile");
 constexpr unsigned long long kChAgg = 1ull << 62, kChPre = 2ull << 62,
                              kChCount = (1ull << 62) - 1ull;
 
-// Exclusive prefix of tile `tile` (total `total`) from the earlier tiles'
-// words, 32 of them per round; warp 0 runs it and every lane returns it.  A
-// wait that runs out sets *err (the prefix is then wrong, never unbounded).
-__device__ unsigned long long chain_lookback(unsigned long long *lb, int64_t tile,
-                                             unsigned long long total, uint32_t *err, int site)
+constexpr int kChainBatch = 1;     // earlier tiles' words a lane of the walking warp loads a round
+
+struct ChainShared {
+    unsigned long long excl;
+    uint32_t warp[kChainWarps];
+    uint32_t tile;
+};
+
+// Publish the tile's total (thread 0).
+__device__ __forceinline__ void chain_publish(unsigned long long *lb, int64_t tile,
+                                              unsigned long long total, bool publish)
 {
-    const int lane = threadIdx.x & 31;
-    volatile unsigned long long *v = lb;
-    const bool publish = tile != held_tile(site);
-    const uint32_t max_spins = g_lb_spins;
-    if (lane == 0 && publish) v[tile] = (tile == 0 ? kChPre : kChAgg) | total;
-    unsigned long long excl = 0;
-    uint32_t spins = 0;
-    int64_t t = tile - 1;
-    while (t >= 0) {
-        const int64_t tt = t - lane;
-        const unsigned long long w = tt >= 0 ? v[tt] : (unsigned long long)kChPre;   // before tile 0: empty prefix
-        const uint32_t np = __ballot_sync(0xffffffffu, (w & (kChAgg | kChPre)) == 0ull);
-        const uint32_t pre = __ballot_sync(0xffffffffu, (w & kChPre) != 0ull);
-        const int fnp = np ? __ffs(np) - 1 : 32, fp = pre ? __ffs(pre) - 1 : 32;
-        const int take = fp < fnp ? fp + 1 : fnp;   // lanes [0, take) are summed
-        unsigned long long c = lane < take ? (w & kChCount) : 0ull;
+    if (threadIdx.x == 0 && publish)
+        ((volatile unsigned long long *)lb)[tile] = (tile == 0 ? kChPre : kChAgg) | total;
+}
+
+// Exclusive prefix of tile `tile` (whose total is published) from the earlier
+// tiles' words; every thread of the block calls it and gets it, warp 0 walks
+// (more threads reading words not yet published slow their writers down).  A
+// wait that runs out sets *err (the prefix is then wrong, never unbounded).
+__device__ __forceinline__ unsigned long long chain_lookback(unsigned long long *lb, int64_t tile,
+                                                             unsigned long long total,
+                                                             bool publish, uint32_t *err,
+                                                             ChainShared &S)
+{
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        volatile unsigned long long *v = lb;
+        const uint32_t max_spins = g_lb_spins;
+        unsigned long long excl = 0;
+        uint32_t spins = 0;
+        bool found = false;
+        for (int64_t hi = tile; hi > 0 && !found; hi -= 32 * kChainBatch) {
+            unsigned long long w[kChainBatch];
 #pragma unroll
-        for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        excl += c;
-        if (fp < fnp) break;
-        t -= take;
-        if (take == 0 && ++spins > max_spins) {   // gave up: flag it
-            if (lane == 0) atomicOr(err, kStatusLookback);
-            break;
+            for (int i = 0; i < kChainBatch; ++i) {
+                const int64_t tt = hi - 1 - 32 * i - lane;
+                // before tile 0: an empty inclusive prefix
+                w[i] = tt >= 0 ? v[tt] : (unsigned long long)kChPre;
+            }
+#pragma unroll
+            for (int i = 0; i < kChainBatch; ++i) {
+                if (found) continue;
+                const int64_t tt = hi - 1 - 32 * i - lane;
+                while ((w[i] & (kChAgg | kChPre)) == 0ull) {
+                    if (++spins > max_spins) {   // gave up: flag it
+                        atomicOr(err, kStatusLookback);
+                        w[i] = kChPre;
+                        break;
+                    }
+                    w[i] = v[tt];
+                }
+                const uint32_t pre = __ballot_sync(0xffffffffu, (w[i] & kChPre) != 0ull);
+                const int last = pre ? __ffs(pre) - 1 : 31;     // lanes [0, last] are summed
+                unsigned long long c = lane <= last ? (w[i] & kChCount) : 0ull;
+#pragma unroll
+                for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                excl += c;
+                found = pre != 0u;
+            }
+        }
+        if (lane == 0) {
+            if (tile > 0 && publish) v[tile] = kChPre | (excl + total);
+            S.excl = excl;
         }
     }
-    if (lane == 0 && tile > 0 && publish) v[tile] = kChPre | (excl + total);
-    return excl;
+    __syncthreads();
+    return S.excl;
 }
 
 __global__ void __launch_bounds__(kChainThreads)
@@ -321,16 +459,15 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
                 uint32_t *__restrict__ err)
 {
     __shared__ uint32_t s_h[4][256];
-    __shared__ uint32_t s_warp[kChainWarps];
-    __shared__ uint32_t s_tile;
+    __shared__ ChainShared S;
     for (int i = threadIdx.x; i < 4 * 256; i += kChainThreads) (&s_h[0][0])[i] = 0;
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    if (threadIdx.x == 0) S.tile = atomicAdd(ticket, 1u);
     __syncthreads();
-    const int64_t tile = s_tile;
+    const int64_t tile = S.tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // warp w owns kChainChunks x 32 consecutive entries of the tile
     const int64_t wbase = tile * kChainTile + (int64_t)warp * 32 * kChainChunks;
-    uint32_t cnt[kChainChunks], bal[kChainChunks], key[kChainChunks];
+    uint32_t bal[kChainChunks], key[kChainChunks], cnt[kChainChunks];
 #pragma unroll
     for (int r = 0; r < kChainChunks; ++r) {
         const int64_t i = wbase + r * 32 + lane;
@@ -340,28 +477,29 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
     uint32_t wtot = 0;
 #pragma unroll
     for (int r = 0; r < kChainChunks; ++r) {
-        const bool ok = cnt[r] > 0u;
-        bal[r] = __ballot_sync(0xffffffffu, ok);
+        bal[r] = __ballot_sync(0xffffffffu, cnt[r] > 0u);
         wtot += __popc(bal[r]);
+    }
+    if (lane == 0) S.warp[warp] = wtot;
+    __syncthreads();
+    uint32_t before = 0, total = 0;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const uint32_t d = ok ? (key[r] >> (8 * p)) & 255u : 0xffffffffu;
-            const uint32_t peers = digit_peers(d, ok);
-            if (ok && lane == __ffs(peers) - 1) atomicAdd(&s_h[p][d], (uint32_t)__popc(peers));
-        }
+    for (int w = 0; w < kChainWarps; ++w) {
+        const uint32_t c = S.warp[w];
+        before += w < warp ? c : 0u;
+        total += c;
     }
-    if (lane == 0) s_warp[warp] = wtot;
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t v = lane < kChainWarps ? s_warp[lane] : 0u;
-        const uint32_t inc = warp_incl_scan(v);
-        const uint32_t total = __shfl_sync(0xffffffffu, inc, kChainWarps - 1);
-        const uint32_t excl = (uint32_t)chain_lookback(lb, tile, total, err, SG_LOOKBACK_COMPACT);
-        if (lane < kChainWarps) s_warp[lane] = excl + inc - v;
-        if (lane == 0 && tile == ntiles - 1) *d_nvalid = excl + total;
-    }
-    __syncthreads();
-    uint32_t pos = s_warp[warp];
+    const bool publish = tile != held_tile(SG_LOOKBACK_COMPACT);
+    chain_publish(lb, tile, total, publish);
+    // the digit counts, while earlier tiles publish
+#pragma unroll
+    for (int r = 0; r < kChainChunks; ++r)
+        if (cnt[r] > 0u)
+#pragma unroll
+            for (int p = 0; p < 4; ++p) atomicAdd(&s_h[p][(key[r] >> (8 * p)) & 255u], 1u);
+    const uint32_t excl = (uint32_t)chain_lookback(lb, tile, total, publish, err, S);
+    if (threadIdx.x == 0 && tile == ntiles - 1) *d_nvalid = excl + total;
+    uint32_t pos = excl + before;
 #pragma unroll
     for (int r = 0; r < kChainChunks; ++r) {
         if ((bal[r] >> lane) & 1u) {
@@ -371,6 +509,7 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
         }
         pos += __popc(bal[r]);
     }
+    __syncthreads();
     for (int i = threadIdx.x; i < 4 * 256; i += kChainThreads) {
         const uint32_t c = (&s_h[0][0])[i];
         if (c) atomicAdd(&hist[i], c);
@@ -383,56 +522,58 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
                uint32_t *__restrict__ d_total, unsigned long long *__restrict__ lb,
                uint32_t *__restrict__ ticket, uint32_t *__restrict__ err)
 {
-    __shared__ uint32_t s_warp[kChainWarps];
-    __shared__ uint32_t s_tile;
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
-    __syncthreads();
-    const int64_t tile = s_tile;
+    __shared__ ChainShared S;
+    if (threadIdx.x == 0) S.tile = atomicAdd(ticket, 1u);
     const int64_t nv = *d_nvalid;
-    const int64_t ntiles = (nv + kChainTile - 1) / kChainTile;
+    __syncthreads();
+    const int64_t tile = S.tile;
+    const int64_t ntiles = (nv + kOffTile - 1) / kOffTile;
     if (nv == 0) {
         if (tile == 0 && threadIdx.x == 0) *d_total = 0u;
         return;
     }
     if (tile >= ntiles) return;   // so is every later tile: nobody waits for this one
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t wbase = tile * kChainTile + (int64_t)warp * 32 * kChainChunks;
-    uint32_t c[kChainChunks];
+    const int64_t wbase = tile * kOffTile + (int64_t)warp * 32 * kOffChunks;
+    uint32_t c[kOffChunks];
 #pragma unroll
-    for (int r = 0; r < kChainChunks; ++r) {
+    for (int r = 0; r < kOffChunks; ++r) {
         const int64_t i = wbase + r * 32 + lane;
         c[r] = i < nv ? ids[i] : 0xffffffffu;
     }
     // an id is outside 0..n-1 only after a look-back wait of the depth sort
     // gave up (err set, the sort's output partly unwritten): count it as 0
 #pragma unroll
-    for (int r = 0; r < kChainChunks; ++r) c[r] = (int64_t)c[r] < n ? count[c[r]] : 0u;
+    for (int r = 0; r < kOffChunks; ++r) c[r] = (int64_t)c[r] < n ? count[c[r]] : 0u;
     uint32_t run = 0;   // the warp's entries before chunk r
 #pragma unroll
-    for (int r = 0; r < kChainChunks; ++r) {
+    for (int r = 0; r < kOffChunks; ++r) {
         const uint32_t inc = warp_incl_scan(c[r]);
         const uint32_t v = c[r];
         c[r] = run + inc - v;
         run += __shfl_sync(0xffffffffu, inc, 31);
     }
-    if (lane == 0) s_warp[warp] = run;
+    if (lane == 0) S.warp[warp] = run;
     __syncthreads();
-    if (warp == 0) {
-        const uint32_t v = lane < kChainWarps ? s_warp[lane] : 0u;
-        const uint32_t inc = warp_incl_scan(v);
-        const uint32_t total = __shfl_sync(0xffffffffu, inc, kChainWarps - 1);
-        const unsigned long long excl = chain_lookback(lb, tile, total, err, SG_LOOKBACK_OFFSETS);
-        if (lane < kChainWarps) s_warp[lane] = (uint32_t)excl + inc - v;
-        if (lane == 0 && tile == ntiles - 1) {
-            // saturated, so that a total of 2^32 pairs or more reads as an overflow
-            const unsigned long long tot = excl + total;
-            *d_total = tot > 0xffffffffull ? 0xffffffffu : (uint32_t)tot;
-        }
-    }
-    __syncthreads();
-    const uint32_t pre = s_warp[warp];
+    uint32_t before = 0;
+    unsigned long long total = 0;
 #pragma unroll
-    for (int r = 0; r < kChainChunks; ++r) {
+    for (int w = 0; w < kChainWarps; ++w) {
+        const uint32_t x = S.warp[w];
+        before += w < warp ? x : 0u;
+        total += x;
+    }
+    const bool publish = tile != held_tile(SG_LOOKBACK_OFFSETS);
+    chain_publish(lb, tile, total, publish);
+    const unsigned long long excl = chain_lookback(lb, tile, total, publish, err, S);
+    if (threadIdx.x == 0 && tile == ntiles - 1) {
+        // saturated, so that a total of 2^32 pairs or more reads as an overflow
+        const unsigned long long tot = excl + total;
+        *d_total = tot > 0xffffffffull ? 0xffffffffu : (uint32_t)tot;
+    }
+    const uint32_t pre = (uint32_t)excl + before;
+#pragma unroll
+    for (int r = 0; r < kOffChunks; ++r) {
         const int64_t i = wbase + r * 32 + lane;
         if (i < nv) offsets[i] = pre + c[r];
     }
@@ -465,10 +606,11 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     k_compact_depth<<<(unsigned)ntiles, kChainThreads, 0, st>>>(
         d_count, d_depth, n, ntiles, keys[0], vals[0], d_scal, hist, chain + 2, tickets, err);
     SG_LAUNCHED();
+    // (only the ids of the sorted order are read again)
     if ((s = radix_sort_pairs(keys, vals, n, d_scal, 0, 32, fr, st, result_buf,
-                              SG_LOOKBACK_DEPTH_SORT)) != SG_OK)
+                              SG_LOOKBACK_DEPTH_SORT, false)) != SG_OK)
         return s;
-    k_pair_offsets<<<(unsigned)ntiles, kChainThreads, 0, st>>>(
+    k_pair_offsets<<<(unsigned)((n + kOffTile - 1) / kOffTile), kChainThreads, 0, st>>>(
         vals[*result_buf], d_count, n, d_scal, d_offsets, d_scal + 1, chain + 2 + ntiles,
         tickets + 1, err);
     SG_LAUNCHED();
@@ -552,8 +694,8 @@ k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
         if (hist) {
             // the digit counts of every tile-sort pass
             for (int p = 0; p < passes; ++p) {
-                const int bits = end_bit - 8 * p < 8 ? end_bit - 8 * p : 8;
-                const uint32_t dg = (key >> (8 * p)) & ((1u << bits) - 1u);
+                const int b = radix_bit(0, end_bit, p), bits = radix_bit(0, end_bit, p + 1) - b;
+                const uint32_t dg = (key >> b) & ((1u << bits) - 1u);
                 const uint32_t peers = digit_peers(dg, in);
                 if (in && (t & 31) == __ffs(peers) - 1) atomicAdd(&s_h[p][dg], (uint32_t)__popc(peers));
             }
