@@ -250,6 +250,7 @@ static sg_status frame_prepare(Frame &fr, int64_t n, int64_t nrays, int64_t ntil
         SG_ENS(fr.dvals[i], sizeof(uint32_t) * (n > 0 ? n : 1));
     }
     SG_ENS(fr.offsets, sizeof(uint32_t) * (n > 0 ? n : 1));
+    SG_ENS(fr.owner, sizeof(uint32_t) * bin_owner_words(n));
     SG_ENS(fr.ranges, sizeof(uint2) * (ntiles > 0 ? ntiles : 1));
     SG_ENS(fr.ray_state, sizeof(float4) * (nrays > 0 ? nrays : 1));
     SG_ENS(fr.ray_feat, sizeof(float4) * (nrays > 0 ? nrays : 1));
@@ -363,7 +364,7 @@ static sg_status bin_and_sort(Frame &fr, int64_t n, int ntx, int64_t ntiles, int
     if (K > 0 && (s = radix_prepare(K, (bits + 7) / 8, fr, st, &hist, 0)) != SG_OK) return s;
     const uint32_t *err = sc + kScalStatus;
     s = bin_pairs((const uint32_t *)fr.dvals[fr.depth_buf].p, (const uint32_t *)fr.offsets.p, sc,
-                  (const int4 *)fr.tiles.p, ntx, wrap, K, pk[0], pv[0], st, err, hist, bits);
+                  (const int4 *)fr.tiles.p, ntx, wrap, K, pk[0], pv[0], st, err, fr.owner, hist, bits);
     if (s != SG_OK) return s;
     int pb = 0;
     s = radix_sort_pairs(pk, pv, K, sc + 1, 0, bits, fr, st, &pb, SG_LOOKBACK_TILE_SORT);
@@ -371,11 +372,13 @@ static sg_status bin_and_sort(Frame &fr, int64_t n, int ntx, int64_t ntiles, int
     fr.pair_buf = pb;
     if (fr.kind == 1) {   // LiDAR lists also get their per-item ray masks
         const Lidar &L = static_cast<const sg_lidar_s *>(fr.sensor)->l;
-        const size_t by = sizeof(uint32_t) * (size_t)(K > 0 ? K : 1) * L.max_items_per_tile;
+        // planes a multiple of 4 long: four pairs' masks are written as 16 bytes
+        fr.lmask_stride = (K + 3) / 4 * 4;
+        const size_t by =
+            sizeof(uint32_t) * (size_t)(K > 0 ? fr.lmask_stride : 1) * L.max_items_per_tile;
         if ((s = ensure(fr.lmask, by)) != SG_OK) return s;
-        fr.lmask_stride = K;
         s = lidar_tile_ranges(pk[pb], sc + 1, K, (uint2 *)fr.ranges.p, ntiles, st, err, pv[pb],
-                              (const float4 *)fr.rect.p, L, (uint32_t *)fr.lmask.p);
+                              (const float4 *)fr.rect.p, L, (uint32_t *)fr.lmask.p, fr.lmask_stride);
     } else {   // camera lists also get their column/row words
         if ((s = ensure(fr.submask, 4 * (size_t)(K > 0 ? K : 1))) != SG_OK) return s;
         s = tile_ranges(pk[pb], sc + 1, K, (uint2 *)fr.ranges.p, ntiles, st, err, pv[pb],
@@ -1079,6 +1082,7 @@ sg_status sg_workspace_bytes(sg_scene scene, int sensor_kind, int64_t n_rays, si
     // covariance, depth keys and ids (x2), offsets
     const size_t g[] = {sizeof(GRec), 16, 16, 4, 4, 8, 16, 4, 4, 4, 4, 4};
     for (size_t by : g) b += grown(by * (size_t)n);
+    b += grown(sizeof(uint32_t) * (size_t)bin_owner_words(n));
     // per ray: state, features, contributor count; per unit: ranges, order
     b += grown(16 * (size_t)nr) * 2 + grown(4 * (size_t)nr);
     b += grown(8 * (size_t)units) + grown(4 * (size_t)units);

@@ -140,12 +140,14 @@ struct LidarItem {       // one warp of LiDAR rendering
 // The ray slots of a LiDAR work item, factorised: slot k holds the ray of
 // column col0 + s (bit k of col_bits[s]) and of the beam at elevation
 // beam_el[j] (bit k of beam_bits[j]); empty slots are in no mask.
-struct LidarItemRays {
-    int ncols, nbeams;
+// (16-byte aligned and read in fours: an absent column or beam has no bits.)
+static_assert(kLidarColsMax == 4, "columns are read as one float4");
+struct __align__(16) LidarItemRays {
     float col_az[kLidarColsMax];
     uint32_t col_bits[kLidarColsMax];
     float beam_el[32];
     uint32_t beam_bits[32];
+    int ncols, nbeams;
 };
 
 struct Lidar {
@@ -205,6 +207,7 @@ struct Frame {
     Buf rec, rect, tiles, depth, count, mean2d, cov2d;
     // depth sort / offsets
     Buf dkeys[2], dvals[2], offsets, hist;
+    Buf owner;        // owner of the first pair of each binning block
     // pairs; LiDAR: per (work item of the pair's tile, pair) the 32-bit mask
     // of the item's rays inside the Gaussian's box, planes of lmask_stride
     Buf pkeys[2], pvals[2], ranges, order, submask, lmask;
@@ -344,6 +347,11 @@ constexpr int64_t depth_stage_words(int64_t n)
 {
     return radix_scratch_words(n, 4) + 2 * (2 + 2 * ((n + kChainTile - 1) / kChainTile));
 }
+// Pairs per binning block, and the entries of the table of their first
+// pairs' owners (blocks beyond it search the offsets): 32 pairs a Gaussian
+// and two million more.
+constexpr int kBinChunk = 2048;
+constexpr int64_t bin_owner_words(int64_t n) { return n / 64 + 1024; }
 sg_status radix_prepare(int64_t n_max, int passes, Frame &fr, cudaStream_t st, uint32_t **hist,
                         int64_t extra);
 // Stable sort of up to n pairs (*d_n of them) by key bits [begin_bit,
@@ -365,7 +373,7 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
 // status word (nothing is written once it is set).
 sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint32_t *d_nvalid,
                     const int4 *d_tiles, int ntx, int wrap_x, int64_t cap, uint32_t *d_keys,
-                    uint32_t *d_vals, cudaStream_t st, const uint32_t *d_err,
+                    uint32_t *d_vals, cudaStream_t st, const uint32_t *d_err, const Buf &owner,
                     uint32_t *d_hist = nullptr, int end_bit = 0);
 // Per-tile ranges of the sorted pairs; with d_mask (camera lists), also the
 // per-pair sub-block masks (d_ids, d_rects, ntx: the pairs' Gaussians, the
@@ -375,12 +383,14 @@ sg_status tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max
                       const uint32_t *d_ids = nullptr, const float4 *d_rects = nullptr,
                       int ntx = 0, uint32_t *d_words = nullptr);
 // LiDAR lists: ranges, and for every pair and every work item of its tile
-// the item's rays inside the Gaussian's extent box (lmask[k * K_max + i]
-// for the k-th item of the tile, by the compositing's own float test).
+// the item's rays inside the Gaussian's extent box (lmask[k * stride + i]
+// for the k-th item of the tile, by the compositing's own float test; stride
+// a multiple of 4).
 sg_status lidar_tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max,
                             uint2 *d_ranges, int64_t ntiles, cudaStream_t st,
                             const uint32_t *d_err, const uint32_t *d_ids,
-                            const float4 *d_rects, const Lidar &L, uint32_t *d_lmask);
+                            const float4 *d_rects, const Lidar &L, uint32_t *d_lmask,
+                            int64_t lmask_stride);
 sg_status clamp_pairs(uint32_t *d_K, int64_t cap, uint32_t *d_dropped, cudaStream_t st);
 
 // project.cu
@@ -436,7 +446,7 @@ namespace sg {
 template <class Fn> inline void for_each_buf(Frame &f, Fn fn)
 {
     Buf *bufs[] = {&f.rec, &f.rect, &f.tiles, &f.depth, &f.count, &f.mean2d, &f.cov2d,
-                   &f.dkeys[0], &f.dkeys[1], &f.dvals[0], &f.dvals[1], &f.offsets, &f.hist,
+                   &f.dkeys[0], &f.dkeys[1], &f.dvals[0], &f.dvals[1], &f.offsets, &f.hist, &f.owner,
                    &f.pkeys[0], &f.pkeys[1], &f.pvals[0], &f.pvals[1], &f.ranges, &f.order, &f.submask,
                    &f.lmask, &f.camwork,
                    &f.partials, &f.ray_state, &f.n_contrib, &f.ray_feat, &f.gacc, &f.scalars,

@@ -35,6 +35,7 @@ constexpr size_t kStBytes = kStRec + 3 * kStG16 + kStG8 +       // rec, rect, ti
                             2 * kStG4 +                          // depth, count
                             4 * kStG4 +                          // depth-sort keys/values x2
                             kStG4 +                              // offsets
+                            al(4 * bin_owner_words(kStMaxGauss)) + // binning blocks' owners
                             4 * kStP4 +                          // pair keys/values x2
                             kStHist +
                             al(8 * kStMaxTiles) + al(4 * kStMaxTiles) +  // ranges, order
@@ -135,6 +136,7 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
         carve(fr.dvals[i], cur, kStG4);
     }
     carve(fr.offsets, cur, kStG4);
+    carve(fr.owner, cur, al(4 * bin_owner_words(kStMaxGauss)));
     for (int i = 0; i < 2; ++i) {
         carve(fr.pkeys[i], cur, kStP4);
         carve(fr.pvals[i], cur, kStP4);
@@ -202,7 +204,8 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
     if (K > 0 && (s = radix_prepare(K, (bits + 7) / 8, fr, st, &hist, 0)) != SG_OK) return s;
     const uint32_t *err = scal + kScalStatus;
     if ((s = bin_pairs(dv[rb], (const uint32_t *)fr.offsets.p, scal, (const int4 *)fr.tiles.p,
-                       c.ntx, 0, K, pk[0], pv[0], st, err, hist, bits)) != SG_OK)
+                       c.ntx, 0, K, pk[0], pv[0], st, err, fr.owner, hist, bits)) !=
+        SG_OK)
         return s;
     int pb = 0;
     if ((s = radix_sort_pairs(pk, pv, K, scal + 1, 0, bits, fr, st, &pb,

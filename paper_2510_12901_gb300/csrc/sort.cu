@@ -364,20 +364,19 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
 // (ballots over 64 digits a thread held the publication back): 26 -> 11 us at
 // 1M Gaussians, 41 -> 17 us at 2M, tiles of 2048 so that 1M give every SM
 // three blocks.  The offsets gather a 4-byte count per Gaussian (one L1 request
-// each, about 5 us at 1.5M) and take tiles of 8192, whose shorter look-back
-// chain is worth more than the fuller chip: at 1M 9.7 us (4096: 14, 2048: 17),
-// at 2M 16 us.  One warp walks back, 32 words a round: 128 words a round or
+// each, about 5 us at 1.5M) and take tiles of 8192 above 256k Gaussians, whose
+// shorter look-back chain is worth more than the fuller chip (at 1M 12 us; 4096
+// 16, 2048 19), and of 2048 below, where the chain is short (150k: the stage 52
+// us, 56 with 8192).  One warp walks back, 32 words a round: 128 words a round or
 // all warps reading took 11 -> 12 and 14 -> 17 us.
 constexpr int kChainThreads = 256;
 constexpr int kChainWarps = kChainThreads / 32;
 constexpr int kChainChunks = kChainTile / kChainThreads;   // 32-entry chunks per warp
-#ifndef SG_OFF_CHUNKS
-#define SG_OFF_CHUNKS 32
-#endif
-constexpr int kOffChunks = SG_OFF_CHUNKS;                  // of a tile of k_pair_offsets
-constexpr int kOffTile = kOffChunks * kChainThreads;
-static_assert(kOffTile >= kChainTile, "look-back words sized by kChainTile");
-static_assert(kChainChunks * kChainThreads == kChainTile && kChainWarps == 8, "chain tile");
+// Chunks of a tile of k_pair_offsets, and the scene size up to which its tiles
+// are small.
+constexpr int kOffSmall = 8, kOffLarge = 32;
+constexpr int64_t kOffSmallN = 262144;
+static_assert(kOffSmall >= kChainChunks, "look-back words sized by kChainTile");
 constexpr unsigned long long kChAgg = 1ull << 62, kChPre = 2ull << 62,
                              kChCount = (1ull << 62) - 1ull;
 
@@ -516,12 +515,15 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
     }
 }
 
+template <int kOffChunks>
 __global__ void __launch_bounds__(kChainThreads)
 k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ count, int64_t n,
                const uint32_t *__restrict__ d_nvalid, uint32_t *__restrict__ offsets,
                uint32_t *__restrict__ d_total, unsigned long long *__restrict__ lb,
-               uint32_t *__restrict__ ticket, uint32_t *__restrict__ err)
+               uint32_t *__restrict__ ticket, uint32_t *__restrict__ err,
+               uint32_t *__restrict__ owner, int64_t owner_cap)
 {
+    constexpr int kOffTile = kOffChunks * kChainThreads;
     __shared__ ChainShared S;
     if (threadIdx.x == 0) S.tile = atomicAdd(ticket, 1u);
     const int64_t nv = *d_nvalid;
@@ -575,7 +577,19 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
 #pragma unroll
     for (int r = 0; r < kOffChunks; ++r) {
         const int64_t i = wbase + r * 32 + lane;
-        if (i < nv) offsets[i] = pre + c[r];
+        // the next entry's offset: the entry's pairs are [off, next)
+        uint32_t next = __shfl_down_sync(0xffffffffu, c[r], 1);
+        const uint32_t chunk_end =
+            r + 1 < kOffChunks ? __shfl_sync(0xffffffffu, c[r + 1 < kOffChunks ? r + 1 : r], 0) : run;
+        if (lane == 31) next = chunk_end;
+        if (i < nv) {
+            const uint64_t off = pre + c[r], end = off + (next - c[r]);
+            offsets[i] = (uint32_t)off;
+            // the binning blocks whose first pair is one of them
+            for (uint64_t b = (off + kBinChunk - 1) / kBinChunk;
+                 b * kBinChunk < end && (int64_t)b < owner_cap; ++b)
+                owner[b] = (uint32_t)i;
+        }
     }
 }
 
@@ -610,9 +624,12 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     if ((s = radix_sort_pairs(keys, vals, n, d_scal, 0, 32, fr, st, result_buf,
                               SG_LOOKBACK_DEPTH_SORT, false)) != SG_OK)
         return s;
-    k_pair_offsets<<<(unsigned)((n + kOffTile - 1) / kOffTile), kChainThreads, 0, st>>>(
+    const bool small = n <= kOffSmallN;
+    const int64_t off_tile = (int64_t)kChainThreads * (small ? kOffSmall : kOffLarge);
+    auto k_off = small ? k_pair_offsets<kOffSmall> : k_pair_offsets<kOffLarge>;
+    k_off<<<(unsigned)((n + off_tile - 1) / off_tile), kChainThreads, 0, st>>>(
         vals[*result_buf], d_count, n, d_scal, d_offsets, d_scal + 1, chain + 2 + ntiles,
-        tickets + 1, err);
+        tickets + 1, err, (uint32_t *)fr.owner.p, (int64_t)(fr.owner.bytes / 4));
     SG_LAUNCHED();
     return SG_OK;
 }
@@ -625,27 +642,45 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
 // the caller learns of them from the dropped-pairs count).
 // Balanced by pairs: block b writes pairs [b C, (b + 1) C) of the
 // depth-ordered expansion (C = kBinChunk; pair p belongs to the valid
-// Gaussian k with offsets[k] <= p < offsets[k + 1]).  The block first finds
-// the owner of its first pair by a cooperative search over the offsets
-// (256 samples per round), loads the offsets and ids of the at most C + 1
-// Gaussians its pairs can belong to, then every thread places its pairs
-// (owner by binary search in shared memory, tile from the owner's range).
+// Gaussian k with offsets[k] <= p < offsets[k + 1]).  The owner of its first
+// pair is in the table that k_pair_offsets wrote (beyond the table, a
+// cooperative search over the offsets, 256 samples per round).  The block
+// loads the at most C + 1 Gaussians its pairs can belong to, marks each one's
+// first pair, and a running maximum over the pairs gives every pair its
+// owner; a thread takes four consecutive pairs and writes them as 16 bytes.
 // A Gaussian that covers thousands of tiles is spread over many blocks.
-constexpr int kBinThreads = 256;
+// Bound by instructions and the latency of its loads (8 bytes a pair to L2):
+// a search in shared memory, two integer divisions and 16 digit ballots a
+// pair took 26 us for 1.5M pairs and 60 us for 3.9M; now 17 and 34 us (blocks
+// of 1024 pairs and 256 threads: 19 and 35).
+constexpr int kBinThreads = 512;
 constexpr int kBinPasses = 3;         // tile ids up to 24 bits when k_bin counts the digits
-constexpr int kBinChunk = 1024;
+static_assert(kBinChunk == 4 * kBinThreads, "four pairs a thread");
+
+__device__ __forceinline__ int pmod_i(int a, int n)
+{
+    const int m = a % n;
+    return m < 0 ? m + n : m;
+}
 
 __global__ void __launch_bounds__(kBinThreads)
 k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
       const uint32_t *__restrict__ d_scal, const int4 *__restrict__ tiles, int ntx, int wrap_x,
       uint32_t cap, uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
-      uint32_t *__restrict__ hist, int end_bit, const uint32_t *__restrict__ err)
+      uint32_t *__restrict__ hist, int end_bit, const uint32_t *__restrict__ err,
+      const uint32_t *__restrict__ owner, int64_t owner_cap)
 {
+    // per Gaussian of the block: first pair, id, tile columns (first, count),
+    // tile rows (first, last); per pair: its owner, where it is the first
     __shared__ uint32_t s_off[kBinChunk + 1], s_id[kBinChunk + 1];
+    __shared__ uint2 s_rg[kBinChunk + 1];
+    __shared__ __align__(8) uint16_t s_own[kBinChunk];
+    __shared__ uint32_t s_max[kBinThreads / 32];
     __shared__ uint32_t s_h[kBinPasses][256];
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int passes = (end_bit + 7) / 8;
     for (int i = t; i < kBinPasses * 256; i += kBinThreads) (&s_h[0][0])[i] = 0u;
+    for (int i = t; i < kBinChunk / 2; i += kBinThreads) reinterpret_cast<uint32_t *>(s_own)[i] = 0u;
     const int64_t nvalid = d_scal[0];
     const int64_t K = min((int64_t)d_scal[1], (int64_t)cap);
     const int64_t p0 = (int64_t)blockIdx.x * kBinChunk;
@@ -655,53 +690,91 @@ k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
     const int64_t p1 = min(K, p0 + kBinChunk);
     // the owner of p0: the largest k with offsets[k] <= p0 (offsets[0] = 0,
     // strictly increasing: every valid Gaussian has a pair)
-    int64_t lo = 0, hi = nvalid;
-    while (hi - lo > 1) {
-        const int64_t step = (hi - lo + kBinThreads - 1) / kBinThreads;
-        const int64_t idx = lo + t * step;
-        const bool le = idx < hi && (int64_t)offsets[idx] <= p0;
-        const int c = __syncthreads_count(le);
-        lo = lo + (int64_t)(c - 1) * step;
-        hi = min(hi, lo + step);
+    int64_t k0 = 0;
+    if ((int64_t)blockIdx.x < owner_cap) {
+        k0 = owner[blockIdx.x];
+    } else {
+        int64_t hi = nvalid;
+        while (hi - k0 > 1) {
+            const int64_t step = (hi - k0 + kBinThreads - 1) / kBinThreads;
+            const int64_t idx = k0 + t * step;
+            const bool le = idx < hi && (int64_t)offsets[idx] <= p0;
+            const int c = __syncthreads_count(le);
+            k0 = k0 + (int64_t)(c - 1) * step;
+            hi = min(hi, k0 + step);
+        }
     }
-    const int64_t k0 = lo;
     const int nk = (int)min((int64_t)kBinChunk + 1, nvalid - k0);
-    for (int i = t; i < nk; i += kBinThreads) {
-        s_off[i] = offsets[k0 + i];
-        s_id[i] = ids[k0 + i];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kBinChunk / kBinThreads + 1; ++r) {
+        const int i = r * kBinThreads + t;
+        if (i >= nk) continue;
+        const uint32_t off = offsets[k0 + i], g = ids[k0 + i];
+        if ((int64_t)off >= p1) continue;
+        const int4 q = tiles[g];
+        s_off[i] = off;
+        s_id[i] = g;
+        const int x = wrap_x ? pmod_i(q.x, ntx) : q.x;
+        s_rg[i] = make_uint2((uint32_t)x | (uint32_t)(q.y - q.x + 1) << 16,
+                             (uint32_t)q.z | (uint32_t)q.w << 16);
+        if ((int64_t)off >= p0) s_own[off - p0] = (uint16_t)i;
     }
     __syncthreads();
-    for (int r0 = 0; r0 < kBinChunk; r0 += kBinThreads) {
-        const int64_t pos = p0 + r0 + t;
-        const bool in = pos < p1;
-        uint32_t key = 0u;
-        if (in) {
-            int a = 0, b = nk;             // the last j with s_off[j] <= pos
-            while (b - a > 1) {
-                const int m = (a + b) >> 1;
-                if ((int64_t)s_off[m] <= pos) a = m; else b = m;
-            }
-            const uint32_t g = s_id[a];
-            const int4 r = tiles[g];
-            const uint32_t local = (uint32_t)(pos - s_off[a]), w = (uint32_t)(r.y - r.x + 1);
-            const int ty = min(r.w, r.z + (int)(local / w));   // within the range, always
-            int x = r.x + (int)(local % w);
-            if (wrap_x) { x %= ntx; if (x < 0) x += ntx; }
-            key = (uint32_t)(ty * ntx + x);
-            keys[pos] = key;
-            vals[pos] = g;
-        }
-        if (hist) {
-            // the digit counts of every tile-sort pass
-            for (int p = 0; p < passes; ++p) {
-                const int b = radix_bit(0, end_bit, p), bits = radix_bit(0, end_bit, p + 1) - b;
-                const uint32_t dg = (key >> b) & ((1u << bits) - 1u);
-                const uint32_t peers = digit_peers(dg, in);
-                if (in && (t & 31) == __ffs(peers) - 1) atomicAdd(&s_h[p][dg], (uint32_t)__popc(peers));
-            }
+    // the owners, as local indices, of pairs p0 + 4 t ..
+    const ushort4 o = *reinterpret_cast<const ushort4 *>(s_own + 4 * t);
+    uint32_t m[4] = {o.x, max((uint32_t)o.x, (uint32_t)o.y), o.z, o.w};
+    m[2] = max(m[2], m[1]);
+    m[3] = max(m[3], m[2]);
+    uint32_t inc = m[3];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc = max(inc, x);
+    }
+    uint32_t before = __shfl_up_sync(0xffffffffu, inc, 1);
+    if (lane == 0) before = 0u;
+    if (lane == 31) s_max[warp] = inc;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kBinThreads / 32; ++w)
+        if (w < warp) before = max(before, s_max[w]);
+    uint32_t key[4], val[4];
+    const int64_t pos0 = p0 + 4 * t;
+    const int nin = p1 - pos0 >= 4 ? 4 : (int)max((int64_t)0, p1 - pos0);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const uint32_t j = max(before, m[e]);
+        const uint2 rg = s_rg[j];
+        const int w = (int)(rg.x >> 16), local = (int)((uint32_t)(pos0 + e) - s_off[j]);
+        // local / w (both below 2^24): the float quotient is off by one at most
+        int row = (int)__fdividef((float)local, (float)w), col = local - row * w;
+        if (col < 0) { --row; col += w; }
+        else if (col >= w) { ++row; col -= w; }
+        const int ty = min((int)(rg.y >> 16), (int)(rg.y & 0xffffu) + row);
+        int x = (int)(rg.x & 0xffffu) + col;
+        if (wrap_x && x >= ntx) x -= ntx;
+        key[e] = (uint32_t)(ty * ntx + x);
+        val[e] = s_id[j];
+    }
+    if (nin == 4) {
+        *reinterpret_cast<uint4 *>(keys + pos0) = make_uint4(key[0], key[1], key[2], key[3]);
+        *reinterpret_cast<uint4 *>(vals + pos0) = make_uint4(val[0], val[1], val[2], val[3]);
+    } else {
+        for (int e = 0; e < nin; ++e) {
+            keys[pos0 + e] = e == 0 ? key[0] : e == 1 ? key[1] : key[2];
+            vals[pos0 + e] = e == 0 ? val[0] : e == 1 ? val[1] : val[2];
         }
     }
     if (hist) {
+        // the digit counts of every tile-sort pass
+        for (int p = 0; p < passes; ++p) {
+            const int b = radix_bit(0, end_bit, p);
+            const uint32_t mask = (1u << (radix_bit(0, end_bit, p + 1) - b)) - 1u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (e < nin) atomicAdd(&s_h[p][(key[e] >> b) & mask], 1u);
+        }
         __syncthreads();
         for (int i = t; i < passes * 256; i += kBinThreads) {
             const uint32_t c = (&s_h[0][0])[i];
@@ -712,8 +785,8 @@ k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
 
 sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint32_t *d_nvalid,
                     const int4 *d_tiles, int ntx, int wrap_x, int64_t cap, uint32_t *d_keys,
-                    uint32_t *d_vals, cudaStream_t st, const uint32_t *d_err, uint32_t *d_hist,
-                    int end_bit)
+                    uint32_t *d_vals, cudaStream_t st, const uint32_t *d_err, const Buf &owner,
+                    uint32_t *d_hist, int end_bit)
 {
     if (cap <= 0) return SG_OK;
     if (d_hist && (end_bit < 1 || end_bit > 8 * kBinPasses)) {
@@ -722,7 +795,7 @@ sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint
     }
     k_bin<<<(unsigned)((cap + kBinChunk - 1) / kBinChunk), kBinThreads, 0, st>>>(
         d_ids, d_offsets, d_nvalid, d_tiles, ntx, wrap_x, (uint32_t)cap, d_keys, d_vals, d_hist,
-        end_bit, d_err);
+        end_bit, d_err, (const uint32_t *)owner.p, (int64_t)(owner.bytes / 4));
     SG_LAUNCHED();
     return SG_OK;
 }
@@ -736,36 +809,53 @@ sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint
 // entry that no live ray of its sub-block can see and loads no box.  After a
 // look-back wait gave up (*err) the pairs may hold stale tile ids: every
 // range stays empty (zeroed before the launch).
-// Each thread takes kRangePer consecutive pairs, their loads (keys, ids,
-// then the boxes by id) issued together, so that a thread waits for two
-// rounds of loads for all of them.
+// Each thread takes kRangePer consecutive pairs (16-byte loads of keys and
+// ids; the lists' buffers are 256-byte aligned), the boxes' loads issued
+// together.  The columns whose centre c + 1/2 is in [lo, hi] are the run from
+// ceil(lo - 1/2) to floor(hi - 1/2): the subtraction is exact in float for
+// 1/2 <= lo < 2^23, rounds to a value with the same ceiling below 1/2 (every
+// lo <= 1/2 starts at column 0), and an image has no columns beyond 2^14.
+// Measured: 16 comparisons a side took 20 us for 1.5M pairs and 45 us for
+// 3.9M; now 11 and 22.
 constexpr int kRangePer = 4;
 
-template <bool kMask>
-__global__ void __launch_bounds__(256)
-k_ranges(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K,
-         uint2 *__restrict__ ranges, const uint32_t *__restrict__ ids,
-         const float4 *__restrict__ rects, int ntx, uint32_t *__restrict__ mask,
-         const uint32_t *__restrict__ err)
+// Bits of the kTile centres first + 1/2 .. first + kTile - 1/2 in [lo, hi].
+__device__ __forceinline__ uint32_t centre_bits(float lo, float hi, int first)
 {
-    const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRangePer;
-    const int64_t K = *d_K;
-    if (i0 >= K || *err) return;
-    uint32_t t[kRangePer], id[kRangePer];
-    float4 rc[kRangePer];
+    const float f = (float)first;
+    const int a = (int)fmaxf(0.f, fminf((float)kTile, ceilf(lo - 0.5f) - f));
+    const int b = (int)fmaxf(-1.f, fminf((float)(kTile - 1), floorf(hi - 0.5f) - f));
+    return (0xffffu << a) & (0xffffu >> (kTile - 1 - b));
+}
+
+// Quotient and remainder of t < 2^24 by n, inv = 1 / n rounded: the float
+// quotient is off by one at most.
+__device__ __forceinline__ void div_small(uint32_t t, int n, float inv, int &q, int &r)
+{
+    q = (int)((float)t * inv);
+    r = (int)t - q * n;
+    if (r < 0) { --q; r += n; }
+    else if (r >= n) { ++q; r -= n; }
+}
+
+__device__ __forceinline__ void load4(const uint32_t *__restrict__ p, int64_t i, int64_t n,
+                                      uint32_t v[kRangePer])
+{
+    if (i + kRangePer <= n) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(p + i);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else {
 #pragma unroll
-    for (int j = 0; j < kRangePer; ++j) {
-        const bool in = i0 + j < K;
-        t[j] = in ? keys[i0 + j] : 0u;
-        if (kMask) id[j] = in ? ids[i0 + j] : 0u;
+        for (int j = 0; j < kRangePer; ++j) v[j] = i + j < n ? p[i + j] : 0u;
     }
+}
+
+// The ends of the tiles' runs among a thread's pairs [i0, i0 + kRangePer).
+__device__ __forceinline__ void write_ranges(const uint32_t *__restrict__ keys, int64_t i0, int64_t K,
+                                             const uint32_t t[kRangePer], uint2 *__restrict__ ranges)
+{
     const uint32_t before = i0 > 0 ? keys[i0 - 1] : 0u;
     const uint32_t after = i0 + kRangePer < K ? keys[i0 + kRangePer] : 0u;
-    if (kMask) {
-#pragma unroll
-        for (int j = 0; j < kRangePer; ++j)
-            if (i0 + j < K) rc[j] = rects[id[j]];   // the extent box, 16 B per Gaussian
-    }
 #pragma unroll
     for (int j = 0; j < kRangePer; ++j) {
         const int64_t i = i0 + j;
@@ -774,17 +864,44 @@ k_ranges(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K,
         const uint32_t right = j + 1 < kRangePer ? t[j + 1] : after;
         if (i == 0 || left != t[j]) ranges[t[j]].x = (uint32_t)i;
         if (i == K - 1 || right != t[j]) ranges[t[j]].y = (uint32_t)(i + 1);
-        if (kMask) {
-            const int tx = (int)(t[j] % (uint32_t)ntx), ty = (int)(t[j] / (uint32_t)ntx);
-            uint32_t cols = 0, rows = 0;
+    }
+}
+
+template <bool kMask>
+__global__ void __launch_bounds__(256)
+k_ranges(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K,
+         uint2 *__restrict__ ranges, const uint32_t *__restrict__ ids,
+         const float4 *__restrict__ rects, int ntx, float inv_ntx, uint32_t *__restrict__ mask,
+         const uint32_t *__restrict__ err)
+{
+    const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRangePer;
+    const int64_t K = *d_K;
+    if (i0 >= K || *err) return;
+    uint32_t t[kRangePer], id[kRangePer];
+    load4(keys, i0, K, t);
+    float4 rc[kRangePer];
+    if (kMask) {
+        load4(ids, i0, K, id);
 #pragma unroll
-            for (int c = 0; c < kTile; ++c) {
-                const float x = (float)(tx * kTile + c) + 0.5f;
-                const float y = (float)(ty * kTile + c) + 0.5f;
-                cols |= (uint32_t)(x >= rc[j].x && x <= rc[j].y) << c;
-                rows |= (uint32_t)(y >= rc[j].z && y <= rc[j].w) << c;
-            }
-            mask[i] = cols | (rows << 16);
+        for (int j = 0; j < kRangePer; ++j)      // the extent box, 16 B per Gaussian
+            rc[j] = i0 + j < K ? rects[id[j]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    write_ranges(keys, i0, K, t, ranges);
+    if (kMask) {
+        uint32_t m[kRangePer];
+#pragma unroll
+        for (int j = 0; j < kRangePer; ++j) {
+            int tx, ty;
+            div_small(t[j], ntx, inv_ntx, ty, tx);
+            m[j] = centre_bits(rc[j].x, rc[j].y, tx * kTile) |
+                   centre_bits(rc[j].z, rc[j].w, ty * kTile) << 16;
+        }
+        if (i0 + kRangePer <= K) {
+            *reinterpret_cast<uint4 *>(mask + i0) = make_uint4(m[0], m[1], m[2], m[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < kRangePer; ++j)
+                if (i0 + j < K) mask[i0 + j] = m[j];
         }
     }
 }
@@ -797,64 +914,109 @@ sg_status tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max
     if (K_max == 0) return SG_OK;
     const unsigned grid = (unsigned)((K_max + 256 * kRangePer - 1) / (256 * kRangePer));
     if (d_words)
-        k_ranges<true><<<grid, 256, 0, st>>>(d_keys, d_K, d_ranges, d_ids, d_rects, ntx, d_words,
-                                             d_err);
+        k_ranges<true><<<grid, 256, 0, st>>>(d_keys, d_K, d_ranges, d_ids, d_rects, ntx,
+                                             1.f / (float)ntx, d_words, d_err);
     else
-        k_ranges<false><<<grid, 256, 0, st>>>(d_keys, d_K, d_ranges, nullptr, nullptr, 0, nullptr,
-                                              d_err);
+        k_ranges<false><<<grid, 256, 0, st>>>(d_keys, d_K, d_ranges, nullptr, nullptr, 0, 0.f,
+                                              nullptr, d_err);
     SG_LAUNCHED();
     return SG_OK;
 }
 
 // LiDAR lists: per-tile ranges, and per pair the ray masks of the work
-// items of its tile (k-th item of the tile: lmask[k * K_max + i]), so that
+// items of its tile (k-th item of the tile: lmask[k * stride + i]), so that
 // the compositing walks skip entries that reach none of their rays without
 // loading their records.  A ray is in the box iff its column's azimuth (the
 // alias nearest the box centre) and its beam's elevation are, so the mask
 // takes one test per column and one per beam of the item.  Both the forward
 // and the backward walks read these masks, so they take the same decisions.
-__global__ void k_ranges_lidar(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K,
-                               int64_t K_max, uint2 *__restrict__ ranges,
-                               const uint32_t *__restrict__ ids, const float4 *__restrict__ rects,
-                               const uint2 *__restrict__ tile_items,
-                               const LidarItemRays *__restrict__ tab,
-                               uint32_t *__restrict__ lmask, const uint32_t *__restrict__ err)
+// Four consecutive pairs a thread, loaded together; lists are sorted by tile,
+// so that the four mostly share one and each table entry is loaded once for
+// them.  Measured (2M Gaussians, 3.7M pairs): one pair a thread 43 us, now 36
+// (38 with the table read word by word).
+__global__ void __launch_bounds__(256)
+k_ranges_lidar(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K, int64_t stride,
+               uint2 *__restrict__ ranges, const uint32_t *__restrict__ ids,
+               const float4 *__restrict__ rects, const uint2 *__restrict__ tile_items,
+               const LidarItemRays *__restrict__ tab, uint32_t *__restrict__ lmask,
+               const uint32_t *__restrict__ err)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRangePer;
     const int64_t K = *d_K;
-    if (i >= K || *err) return;
-    const uint32_t t = keys[i];
-    if (i == 0 || keys[i - 1] != t) ranges[t].x = (uint32_t)i;
-    if (i == K - 1 || keys[i + 1] != t) ranges[t].y = (uint32_t)(i + 1);
-    const float4 rc = rects[ids[i]];
-    const float cx = 0.5f * (rc.x + rc.y);
-    const uint2 ti = tile_items[t];
-    for (uint32_t k = 0; k < ti.y; ++k) {
-        const LidarItemRays &R = tab[ti.x + k];
-        uint32_t mc = 0u, me = 0u;
-        for (int s = 0; s < R.ncols; ++s) {
-            const float az = R.col_az[s];
-            const float ra = az + 360.f * rintf((cx - az) * (1.f / 360.f));
-            mc |= (ra >= rc.x && ra <= rc.y) ? R.col_bits[s] : 0u;
+    if (i0 >= K || *err) return;
+    const int np = K - i0 < kRangePer ? (int)(K - i0) : kRangePer;
+    uint32_t t[kRangePer], id[kRangePer];
+    load4(keys, i0, K, t);
+    load4(ids, i0, K, id);
+    float4 rc[kRangePer];
+    float cx[kRangePer];
+#pragma unroll
+    for (int j = 0; j < kRangePer; ++j)
+        rc[j] = j < np ? rects[id[j]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    write_ranges(keys, i0, K, t, ranges);
+#pragma unroll
+    for (int j = 0; j < kRangePer; ++j) cx[j] = 0.5f * (rc[j].x + rc[j].y);
+    // runs [j0, j1) of the pairs that share a tile (all four, mostly)
+    for (int j0 = 0; j0 < np;) {
+        const uint32_t tile = j0 == 0 ? t[0] : j0 == 1 ? t[1] : j0 == 2 ? t[2] : t[3];
+        int j1 = j0 + 1;
+#pragma unroll
+        for (int j = 1; j < kRangePer; ++j)
+            if (j == j1 && j < np && t[j] == tile) j1 = j + 1;
+        const uint2 ti = tile_items[tile];
+        for (uint32_t k = 0; k < ti.y; ++k) {
+            const LidarItemRays &R = tab[ti.x + k];
+            uint32_t mc[kRangePer] = {0u, 0u, 0u, 0u}, me[kRangePer] = {0u, 0u, 0u, 0u};
+            const float4 az4 = *reinterpret_cast<const float4 *>(R.col_az);
+            const uint4 cb4 = *reinterpret_cast<const uint4 *>(R.col_bits);
+            const float az[4] = {az4.x, az4.y, az4.z, az4.w};
+            const uint32_t cb[4] = {cb4.x, cb4.y, cb4.z, cb4.w};     // 0: no such column
+            const int nbeams = R.nbeams;
+#pragma unroll
+            for (int s = 0; s < kLidarColsMax; ++s) {
+#pragma unroll
+                for (int j = 0; j < kRangePer; ++j) {
+                    const float ra = az[s] + 360.f * rintf((cx[j] - az[s]) * (1.f / 360.f));
+                    mc[j] |= (ra >= rc[j].x && ra <= rc[j].y) ? cb[s] : 0u;
+                }
+            }
+            for (int b0 = 0; b0 < nbeams; b0 += 4) {
+                const float4 el4 = *reinterpret_cast<const float4 *>(R.beam_el + b0);
+                const uint4 bb4 = *reinterpret_cast<const uint4 *>(R.beam_bits + b0);
+                const float el[4] = {el4.x, el4.y, el4.z, el4.w};
+                const uint32_t bb[4] = {bb4.x, bb4.y, bb4.z, bb4.w};  // 0: no such beam
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+#pragma unroll
+                    for (int j = 0; j < kRangePer; ++j)
+                        me[j] |= (el[b] >= rc[j].z && el[b] <= rc[j].w) ? bb[b] : 0u;
+            }
+            uint32_t *out = lmask + (int64_t)k * stride + i0;
+            if (j0 == 0 && j1 == kRangePer) {
+                *reinterpret_cast<uint4 *>(out) =
+                    make_uint4(mc[0] & me[0], mc[1] & me[1], mc[2] & me[2], mc[3] & me[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < kRangePer; ++j)
+                    if (j >= j0 && j < j1) out[j] = mc[j] & me[j];
+            }
         }
-        for (int j = 0; j < R.nbeams; ++j) {
-            const float el = R.beam_el[j];
-            me |= (el >= rc.z && el <= rc.w) ? R.beam_bits[j] : 0u;
-        }
-        lmask[(int64_t)k * K_max + i] = mc & me;
+        j0 = j1;
     }
 }
 
 sg_status lidar_tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max,
                             uint2 *d_ranges, int64_t ntiles, cudaStream_t st,
                             const uint32_t *d_err, const uint32_t *d_ids,
-                            const float4 *d_rects, const Lidar &L, uint32_t *d_lmask)
+                            const float4 *d_rects, const Lidar &L, uint32_t *d_lmask,
+                            int64_t lmask_stride)
 {
     SG_CUDA(cudaMemsetAsync(d_ranges, 0, sizeof(uint2) * ntiles, st));
     if (K_max == 0) return SG_OK;
-    k_ranges_lidar<<<(unsigned)((K_max + 255) / 256), 256, 0, st>>>(
-        d_keys, d_K, K_max, d_ranges, d_ids, d_rects, L.d_tile_items, L.d_item_ray_tab, d_lmask,
-        d_err);
+    const unsigned grid = (unsigned)((K_max + 256 * kRangePer - 1) / (256 * kRangePer));
+    k_ranges_lidar<<<grid, 256, 0, st>>>(
+        d_keys, d_K, lmask_stride, d_ranges, d_ids, d_rects, L.d_tile_items, L.d_item_ray_tab,
+        d_lmask, d_err);
     SG_LAUNCHED();
     return SG_OK;
 }

@@ -24,9 +24,11 @@ def _expected(tiles, depth, count, ntx):
     return tile[order].astype(np.uint32), ids[owner][order].astype(np.uint32)
 
 
-# tiles of 2048 (compaction), 4096 (radix passes) and 8192 (offsets) entries;
+# tiles of 2048 (compaction, offsets up to 262144 Gaussians), 4096 (radix passes)
+# and 8192 (offsets above) entries;
 # 32 of them a look-back round
-@pytest.mark.parametrize("n", [1, 2, 2047, 2049, 4096, 4097, 8193, 66000, 135000, 300001])
+@pytest.mark.parametrize("n", [1, 2, 2047, 2049, 4096, 4097, 8193, 66000, 135000, 262144,
+                               300001])
 @pytest.mark.parametrize("ties", [False, True])
 @pytest.mark.parametrize("w,h", [(16, 16), (64, 64), (1030, 517)])
 def test_pair_list_order(n, ties, w, h):
@@ -57,3 +59,27 @@ def test_pair_list_order(n, ties, w, h):
     per = np.bincount(tile, minlength=len(r))
     assert np.array_equal(r[:, 1] - r[:, 0], per)
     assert np.array_equal(r[per > 0, 0], (np.cumsum(per) - per)[per > 0])
+
+
+def test_more_pairs_than_the_owner_table():
+    """A few Gaussians over every tile of a large image: binning blocks beyond
+    the table of first owners search the offsets for theirs."""
+    import torch
+    from paper_2510_12901_gb300 import simgut as sg, synthetic as syn
+    n = 403
+    sc = syn.tiny_scene(seed=43, n=n)
+    sc.means[:] = np.random.default_rng(44).uniform(-0.5, 0.5, (n, 3)) + [0.0, 8.0, 0.0]
+    sc.log_scales[:] = np.log(4.0)
+    cam = dataclasses.replace(syn.tiny_camera(), width=2000, height=2041, fx=900.0, fy=900.0,
+                              cx=1000.0, cy=1020.0)
+    S, C, fr = sg.Scene(sc), sg.Camera(cam), sg.Frame()
+    sg.sg_frame_set_backward_state(fr.handle, 0)
+    sg.render_camera(S, C, cam.c2w, frame=fr)
+    torch.cuda.synchronize()
+    sg.sg_frame_status(fr.handle)
+    tile, ids = _expected(fr.field(sg.FIELD_TILES, np.int32, 4),
+                          fr.field(sg.FIELD_DEPTH, np.float32),
+                          fr.field(sg.FIELD_COUNT, np.uint32), 125)
+    assert len(ids) > 2048 * (n // 64 + 1024)
+    assert np.array_equal(fr.field(sg.FIELD_PAIR_TILES, np.uint32), tile)
+    assert np.array_equal(fr.field(sg.FIELD_PAIR_IDS, np.uint32), ids)
