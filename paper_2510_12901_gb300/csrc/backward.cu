@@ -15,17 +15,33 @@
 // where U comes from the ray's saved final (F, Z, W) and U_{<=i} is the
 // prefix sum up to and including entry i; T_{i+1} = T_i (1 - alpha_i) is
 // the forward's own product.  The closest approach gives the geometric
-// gradients in a stable form: with q* = M (o + tau d - mu) = (num x den) /
-// |den|^2 (the closest point in the Gaussian's frame, no cancellation) and
-// p = M^-1 q* = M^T diag(s^2) q*,
-//   dD^2/dM = 2 q* p^T,          dD^2/dmu = -2 M^T q*,
-//   dtau/dM = -(den p^T + q* d^T) / |den|^2,   dtau/dmu = M^T den / |den|^2
-// (envelope theorem at tau_max).  Per staged entry the 16 partials dL/dM
-// (9), dL/dmu (3), dL/dsigma, dL/dfeature (3) are summed over the warp by a
-// transposing butterfly (16 shuffles) and added with 16 float atomics.  A
-// last per-Gaussian kernel maps them to the raw parameters (M = S^-1 R^T, R
-// of the normalised quaternion, SH colour at the direction from the camera
-// to the mean).
+// gradients in a stable form: with q = M (o + tau d - mu) = (num x den) /
+// |den|^2 (the closest point in the Gaussian's frame, no cancellation),
+// p = M^-1 q and d = M^-1 den (envelope theorem at tau_max),
+//   dD^2/dM = 2 q p^T,                        dD^2/dmu = -2 M^T q,
+//   dtau/dM = -(den p^T + q d^T) / |den|^2,   dtau/dmu = M^T den / |den|^2.
+// Every term of dL/dM is a product of q and den times M^-T, so with a = 2
+// dL/dD^2, b = (dL/dtau) / |den|^2 and u = a q - b den,
+//   dL/dM = S M^-T,  S = sum (u q^T - b q den^T)  (symmetric),
+//   dL/dmu = -M^T sum u:
+// 13 sums a Gaussian (6 of S, 3 of u, sum x / sigma for dL/dsigma, 3 of the
+// features) that need neither M^-1 nor the ray's direction.  A last
+// per-Gaussian kernel maps them to the raw parameters (M = S^-1 R^T, R of the
+// normalised quaternion, SH colour at the direction from the camera to the
+// mean).
+//
+// Two phases per 16 staged entries.  Lanes are rays first: each walks the
+// entries in list order, as the forward, and leaves two numbers per pair in
+// shared memory, w = alpha T and x = alpha dL/dalpha (0 where alpha is clamped
+// or the pair does not composite).  Then lanes are entries (two lanes each,
+// half of the rays a lane): each evaluates its pairs' num and den again and
+// adds the 13 terms in registers.  One shuffle a sum joins the two halves and
+// four 16-byte atomics a Gaussian add them to its row.  The kernels are bound
+// by instructions: summing 16 components over the warp for every (entry,
+// warp), 16 shuffles with their selects and 16 atomics, and forming p and d
+// per pair (three divisions) took about 280 instructions an entry, the second
+// evaluation takes 75.  Measured: the 1M-Gaussian fisheye view 826 -> 594 us,
+// the 2M-Gaussian LiDAR sweep 620 -> 410 us.
 #include <math.h>
 
 #include "pairs.cuh"
@@ -33,104 +49,99 @@
 
 namespace sg {
 
-constexpr int kG = 16;          // accumulated partials per Gaussian
-constexpr int kBwWarps = 4;     // warps per block of the persistent backward grids
+constexpr int kG = 16;          // floats per Gaussian in the accumulator (13 used)
+constexpr int kBwBatch = 16;    // staged entries a phase takes
+constexpr int kBwQueue = 64;    // entries waiting to be staged: a window's, after at most 31
+constexpr int kBwWarps = 4;     // warps per block of the camera's persistent grid
+constexpr int kBwCamBlocks = 5;  // its blocks per SM (4: 648 us, 6: 633)
+constexpr int kBwWarpsPosed = 2;   // of LiDAR's and the rolling shutter's (13 KB a warp; 3: 422 us)
 
-__device__ __forceinline__ float warp_sum(float v)
+// A ray's walk over its composited entries.
+struct RayGrad {
+    float gQ[5];     // dL/d(F0, F1, F2, Z, W)
+    float T, U, Ut;  // transmittance and gQ . Q before the entry, gQ . Q of the ray
+};
+
+// Front-to-back step of one composited entry with features q: returns (w, x).
+__device__ __forceinline__ float2 ray_step(RayGrad &r, const PairEval &pe, const float q[3])
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    const float w = pe.alpha * r.T;
+    const float gq = r.gQ[0] * q[0] + r.gQ[1] * q[1] + r.gQ[2] * q[2] + r.gQ[3] * pe.tau + r.gQ[4];
+    const float Ua = r.U + gq * w, om = 1.f - pe.alpha;
+    const float dLda = gq * r.T - __fdividef(r.Ut - Ua, om);
+    r.U = Ua;
+    r.T = r.T * om;
+    return make_float2(w, pe.clamped ? 0.f : dLda * pe.alpha);
 }
 
-// Gradient partials of one composited pair.
-//   Mr: rows of M; d: ray direction; dLdD2, dLdtau: upstream.
-__device__ __forceinline__ void pair_geometry_grads(const float Mr[9], const PairEval &pe,
-                                                    const float d[3], float dLdD2, float dLdtau,
-                                                    float g[kG])
+// The sums of one Gaussian.
+struct GaussSums {
+    float S[6];      // 00 01 02 11 12 22
+    float u[3];
+    float x;
+    float F[3];
+};
+
+__device__ __forceinline__ void clear(GaussSums &g)
 {
-    // q* = (num x den) * inv
-    const float *n = pe.n, *e = pe.e;
-    const float qs[3] = {(n[1] * e[2] - n[2] * e[1]) * pe.inv, (n[2] * e[0] - n[0] * e[2]) * pe.inv,
-                         (n[0] * e[1] - n[1] * e[0]) * pe.inv};
-    // p = M^-1 q* = sum_k s_k^2 q*_k M_k,  s_k^2 = 1 / |M_k|^2
-    float p[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) g.S[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) g.u[k] = g.F[k] = 0.f;
+    g.x = 0.f;
+}
+
+// Add one pair: num scaled by 1 / nscale, den, (w, x) and the ray's upstream
+// (gF, gZ).
+__device__ __forceinline__ void add_pair(GaussSums &g, const float n[3], const float e[3],
+                                         float nscale, float2 wx, const float gF[3], float gZ)
+{
+    const float inv = __fdividef(1.f, e[0] * e[0] + e[1] * e[1] + e[2] * e[2]);
+    const float c = inv * nscale;
+    const float q[3] = {(n[1] * e[2] - n[2] * e[1]) * c, (n[2] * e[0] - n[0] * e[2]) * c,
+                        (n[0] * e[1] - n[1] * e[0]) * c};
+    // a = 2 dL/dD^2 = -x (dalpha/dD^2 = -alpha / 2); b = gZ w / |den|^2
+    const float b = gZ * wx.x * inv;
+    float u[3], bq[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float *Mk = Mr + 3 * k;
-        const float s2 = 1.f / (Mk[0] * Mk[0] + Mk[1] * Mk[1] + Mk[2] * Mk[2]);
-        const float c = s2 * qs[k];
-        p[0] += c * Mk[0];
-        p[1] += c * Mk[1];
-        p[2] += c * Mk[2];
+        u[k] = -(wx.y * q[k] + b * e[k]);
+        bq[k] = b * q[k];
+        g.u[k] += u[k];
+        g.F[k] += gF[k] * wx.x;
     }
-    const float a2 = 2.f * dLdD2, ti = dLdtau * pe.inv;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-            g[3 * k + j] = a2 * qs[k] * p[j] - ti * (e[k] * p[j] + qs[k] * d[j]);
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-        g[9 + j] = -a2 * (Mr[j] * qs[0] + Mr[3 + j] * qs[1] + Mr[6 + j] * qs[2]) +
-                   ti * (Mr[j] * e[0] + Mr[3 + j] * e[1] + Mr[6 + j] * e[2]);
+    g.x += wx.y;
+    g.S[0] += u[0] * q[0] - bq[0] * e[0];
+    g.S[1] += u[0] * q[1] - bq[0] * e[1];
+    g.S[2] += u[0] * q[2] - bq[0] * e[2];
+    g.S[3] += u[1] * q[1] - bq[1] * e[1];
+    g.S[4] += u[1] * q[2] - bq[1] * e[2];
+    g.S[5] += u[2] * q[2] - bq[2] * e[2];
 }
 
-// Front-to-back step for one composited entry: returns the partials.
-//   q = (f0, f1, f2): features; gQ: upstream of (F0, F1, F2, Z, W);
-//   T: transmittance before the entry (updated to after it); U: gQ . Q
-//   before the entry (updated); Ut: gQ . Q of the whole ray.
-__device__ __forceinline__ void composite_grads(const PairEval &pe, float sigma, const float q[3],
-                                                const float gQ[5], float &T, float &U, float Ut,
-                                                const float Mr[9], const float d[3], float g[kG])
+// Join the halves of an entry's rays (lanes L and L ^ 16) and add the sums to
+// the Gaussian's row: S 0..5, u 6..8, sum x / sigma 9, F 10..12.  Every lane
+// calls it; `use`: the entry has a composited pair.
+__device__ __forceinline__ void add_sums(GaussSums &g, float sigma, bool use, float *row)
 {
-    const float w = pe.alpha * T;
-    const float gq = gQ[0] * q[0] + gQ[1] * q[1] + gQ[2] * q[2] + gQ[3] * pe.tau + gQ[4];
-    const float Ua = U + gq * w;
-    const float dLda = gq * T - (Ut - Ua) / (1.f - pe.alpha);
-    U = Ua;
-    T = T * (1.f - pe.alpha);
-    const float dLdtau = gQ[3] * w;
-    float dLdD2 = 0.f;
-    g[12] = 0.f;
-    if (!pe.clamped) {
-        g[12] = dLda * pe.rho;                       // d alpha / d sigma = rho
-        dLdD2 = dLda * sigma * pe.rho * -0.5f;       // d alpha / d D^2
-    }
-    g[13] = gQ[0] * w;
-    g[14] = gQ[1] * w;
-    g[15] = gQ[2] * w;
-    pair_geometry_grads(Mr, pe, d, dLdD2, dLdtau, g);
-}
-
-// Sum g[16] over the warp and add it to acc[0..15]: a butterfly that halves
-// the vector at each of the first four levels (8 + 4 + 2 + 1 shuffles) and
-// leaves lane L with component 8 b4 + 4 b3 + 2 b2 + b1 (b = bits of L)
-// summed over 16 lanes; the last shuffle adds the other half.
-__device__ __forceinline__ void warp_reduce_add16(const float g[kG], float *acc)
-{
-    const int lane = threadIdx.x & 31;
-    const bool h1 = lane & 16, h2 = lane & 8, h3 = lane & 4, h4 = lane & 2;
-    float a8[8], a4[4], a2[2];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const float mine = h1 ? g[8 + k] : g[k], other = h1 ? g[k] : g[8 + k];
-        a8[k] = mine + __shfl_xor_sync(0xffffffffu, other, 16);
-    }
+    for (int k = 0; k < 6; ++k) g.S[k] += __shfl_xor_sync(0xffffffffu, g.S[k], 16);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float mine = h2 ? a8[4 + k] : a8[k], other = h2 ? a8[k] : a8[4 + k];
-        a4[k] = mine + __shfl_xor_sync(0xffffffffu, other, 8);
+    for (int k = 0; k < 3; ++k) {
+        g.u[k] += __shfl_xor_sync(0xffffffffu, g.u[k], 16);
+        g.F[k] += __shfl_xor_sync(0xffffffffu, g.F[k], 16);
     }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float mine = h3 ? a4[2 + k] : a4[k], other = h3 ? a4[k] : a4[2 + k];
-        a2[k] = mine + __shfl_xor_sync(0xffffffffu, other, 4);
+    g.x += __shfl_xor_sync(0xffffffffu, g.x, 16);
+    if (!use) return;
+    if (threadIdx.x & 16) {
+        atomicAdd(reinterpret_cast<float4 *>(row) + 2,
+                  make_float4(g.u[2], __fdividef(g.x, sigma), g.F[0], g.F[1]));
+        atomicAdd(row + 12, g.F[2]);
+    } else {
+        atomicAdd(reinterpret_cast<float4 *>(row), make_float4(g.S[0], g.S[1], g.S[2], g.S[3]));
+        atomicAdd(reinterpret_cast<float4 *>(row) + 1,
+                  make_float4(g.S[4], g.S[5], g.u[0], g.u[1]));
     }
-    float a1 = (h4 ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, h4 ? a2[0] : a2[1], 2);
-    a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
-    const int comp = (h1 ? 8 : 0) + (h2 ? 4 : 0) + (h3 ? 2 : 0) + (h4 ? 1 : 0);
-    if (!(lane & 1) && a1 != 0.f) atomicAdd(acc + comp, a1);
 }
 
 // Upstream of (F0, F1, F2, Z, W) for a camera ray from dL/d(rgb, alpha,
@@ -147,10 +158,118 @@ __device__ __forceinline__ void camera_gQ(const float *g_rgb, const float *g_alp
     gQ[4] = ga - (W > 0.f ? gd * Z / (W * W) : 0.f);
 }
 
+// The start of a segment's walk: the state the forward's merge left before it
+// (partial slot of two float4), the ray's totals and its upstream gQ.
+__device__ __forceinline__ void start_ray(RayGrad &r, const float4 *slot, const float gQ[5],
+                                          const float4 F, float Z, float W)
+{
+    float Q[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    r.T = 1.f;
+    if (slot) {
+        const float4 u = slot[0], v = slot[1];
+        Q[0] = u.x; Q[1] = u.y; Q[2] = u.z; Q[3] = v.x; Q[4] = u.w;
+        r.T = v.y;
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) r.gQ[k] = gQ[k];
+    r.Ut = gQ[0] * F.x + gQ[1] * F.y + gQ[2] * F.z + gQ[3] * Z + gQ[4] * W;
+    r.U = gQ[0] * Q[0] + gQ[1] * Q[1] + gQ[2] * Q[2] + gQ[3] * Q[3] + gQ[4] * Q[4];
+}
+
+// Push the window's entries that reach a lane of `act` to the warp's queue.
+__device__ __forceinline__ void push(uint2 *cand, uint32_t *cpos, uint32_t &tail, uint32_t gid,
+                                     uint32_t lanes, uint32_t pos)
+{
+    const uint32_t bal = __ballot_sync(0xffffffffu, lanes != 0u);
+    if (lanes) {
+        const uint32_t at =
+            (tail + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))) % kBwQueue;
+        cand[at] = make_uint2(gid, lanes);
+        cpos[at] = pos;
+    }
+    tail += __popc(bal);
+}
+
 // ------------------------------------------------------------------ camera
-// Six blocks per SM (80 registers, 20 bytes spilled): the differentiable
-// street step 4.64 -> 4.60 ms against five at 96 registers.
-__global__ void __launch_bounds__(32 * kBwWarps, 6)
+struct BwCam {                     // a warp's shared memory
+    float4 e[8][32];               // staged entries (cam_entry's planes 0..7)
+    float2 wx[kBwBatch][33];       // (w, x) per (entry, ray); rows an odd number of banks apart
+    float4 ray[2][32];             // (dd, gZ), (gF, 0)
+    uint2 cand[kBwQueue];          // waiting: (Gaussian, lane mask)
+    uint32_t cpos[kBwQueue];       // and list position
+    uint32_t pos[32], lanes[32], gid[32];
+    float ref[6];
+};
+
+// Stage the n <= 32 entries at the queue's head and add their gradients.
+__device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose,
+                                         const GRec *__restrict__ rec, BwCam &S, uint32_t head,
+                                         int n, const float dh[3], const float dl[3],
+                                         const float dd[3], uint32_t last, RayGrad &r,
+                                         float *__restrict__ gacc)
+{
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane < n) {
+        const uint2 c = S.cand[(head + lane) % kBwQueue];
+        float4 ent[9];
+        cam_entry(rec[c.x], pose.t, dh, dl, ent, kResponseScale);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) S.e[k][lane] = ent[k];
+        S.lanes[lane] = c.y;
+        S.pos[lane] = S.cpos[(head + lane) % kBwQueue];
+        S.gid[lane] = c.x;
+    }
+    __syncwarp();
+    for (int b0 = 0; b0 < n; b0 += kBwBatch) {
+        const int nb = min(kBwBatch, n - b0);
+        uint32_t used = 0u;        // entries with a composited pair
+        for (int j = 0; j < nb; ++j) {
+            const int i = b0 + j;
+            PairEval pe;
+            bool ok = cam_pair_scaled(S.e[0][i], S.e[1][i], S.e[2][i], S.e[3][i], S.e[4][i],
+                                      S.e[5][i], S.e[6][i], (S.lanes[i] >> lane) & 1u, dd,
+                                      P.alpha_min, P.alpha_max, pe);
+            ok = ok && S.pos[i] <= last;
+            float2 wx = make_float2(0.f, 0.f);
+            if (ok) {
+                const float4 col = S.e[7][i];
+                const float q[3] = {col.x, col.y, col.z};
+                wx = ray_step(r, pe, q);
+            }
+            S.wx[j][lane] = wx;
+            used |= (__any_sync(0xffffffffu, ok) ? 1u : 0u) << j;
+        }
+        __syncwarp();
+        if (used == 0u) continue;
+        // lanes as entries: lane & 15 of the batch, rays 16 (lane >> 4) ..
+        const int j = lane & 15, i = b0 + j, r0 = lane & 16;
+        const bool use = (used >> j) & 1u;
+        GaussSums g;
+        clear(g);
+        const int il = use ? i : b0;
+        const float4 q0 = S.e[0][il], q1 = S.e[1][il], q2 = S.e[2][il];
+        const float4 m0 = S.e[3][il], m1 = S.e[4][il], m2 = S.e[5][il];
+#pragma unroll 4
+        for (int k = 0; k < 16; ++k) {
+            const float4 d = S.ray[0][r0 + k], f = S.ray[1][r0 + k];
+            const float2 wx = use ? S.wx[j][r0 + k] : make_float2(0.f, 0.f);
+            if (wx.x == 0.f) continue;      // not composited
+            const float num[3] = {q0.w + q0.x * d.x + q0.y * d.y + q0.z * d.z,
+                                  q1.w + q1.x * d.x + q1.y * d.y + q1.z * d.z,
+                                  q2.w + q2.x * d.x + q2.y * d.y + q2.z * d.z};
+            const float den[3] = {m0.w + m0.x * d.x + m0.y * d.y + m0.z * d.z,
+                                  m1.w + m1.x * d.x + m1.y * d.y + m1.z * d.z,
+                                  m2.w + m2.x * d.x + m2.y * d.y + m2.z * d.z};
+            const float gF[3] = {f.x, f.y, f.z};
+            add_pair(g, num, den, 1.f / kResponseScale, wx, gF, d.w);
+        }
+        add_sums(g, S.e[6][il].w, use, gacc + (int64_t)S.gid[il] * kG);
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(32 * kBwWarps, kBwCamBlocks)
 k_backward_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
                   const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
                   const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
@@ -162,15 +281,12 @@ k_backward_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__r
                   const float *__restrict__ g_alpha, const float *__restrict__ g_depth,
                   float *__restrict__ gacc)
 {
-    __shared__ float4 s_all[kBwWarps][8][32];
-    __shared__ uint32_t s_pos[kBwWarps][32], s_lanes[kBwWarps][32], s_gid[kBwWarps][32];
-    __shared__ float s_refs[kBwWarps][6];
+    __shared__ BwCam s_all[kBwWarps];
     __shared__ CamPose s_pose;
     load_cam_pose(D, s_pose);
     __syncthreads();
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    float4(*s_e)[32] = s_all[wib];
-    float *s_ref = s_refs[wib];
+    const int lane = threadIdx.x & 31;
+    BwCam &S = s_all[threadIdx.x >> 5];
     const uint32_t n_items = counts[0];
     while (true) {
         uint32_t item = 0;
@@ -191,97 +307,110 @@ k_backward_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__r
         const uint2 rg = ranges[tile];
         const uint32_t lo = rg.x + (uint32_t)seg * kSegLen;
         uint32_t hi = min(rg.y, lo + kSegLen);
-        uint32_t lim = rg.x + last;                    // entries idx < lim may contribute
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lim = max(lim, __shfl_xor_sync(0xffffffffu, lim, o));
-        hi = min(hi, lim);
+        // entries idx < rg.x + last may contribute
+        hi = min(hi, rg.x + __reduce_max_sync(0xffffffffu, last));
         if (hi <= lo) continue;                        // nothing of this segment composited
-        if (lane == 0) cam_tile_ref(s_pose, tile_dir, tile, s_ref);
+        if (lane == 0) cam_tile_ref(s_pose, tile_dir, tile, S.ref);
         __syncwarp();
-        const float dh[3] = {s_ref[0], s_ref[1], s_ref[2]};
-        const float dl[3] = {s_ref[3], s_ref[4], s_ref[5]};
-        float dd[3], d[3];
+        const float dh[3] = {S.ref[0], S.ref[1], S.ref[2]};
+        const float dl[3] = {S.ref[3], S.ref[4], S.ref[5]};
+        float dd[3];
         cam_ray_offset(s_pose, e, dd);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) d[i] = dh[i] + dd[i];
-        // state before the segment, upstream, totals
-        float T = 1.f, Qp[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        if (seg > 0) {
-            const float4 *pq = partials + ((size_t)(ti.y + seg) * 256 + sub * 32 + lane) * 2;
-            const float4 u = pq[0], v = pq[1];
-            Qp[0] = u.x; Qp[1] = u.y; Qp[2] = u.z; Qp[3] = v.x; Qp[4] = u.w;
-            T = v.y;
+        RayGrad r;
+        {
+            float gQ[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            float4 st = make_float4(0.f, 0.f, 0.f, 0.f), F = st;
+            if (ray_ok) {
+                st = ray_state[pidx];
+                F = ray_feat[pidx];
+                camera_gQ(g_rgb, g_alpha, g_depth, pidx, st.y, st.z, gQ);
+            }
+            start_ray(r, seg > 0 ? partials + ((size_t)(ti.y + seg) * 256 + sub * 32 + lane) * 2 : nullptr,
+                      gQ, F, st.z, st.y);
         }
-        float gQ[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, Ut = 0.f, U = 0.f;
-        if (ray_ok) {
-            const float4 st = ray_state[pidx], F = ray_feat[pidx];
-            camera_gQ(g_rgb, g_alpha, g_depth, pidx, st.y, st.z, gQ);
-            Ut = gQ[0] * F.x + gQ[1] * F.y + gQ[2] * F.z + gQ[3] * st.z + gQ[4] * st.y;
-            U = gQ[0] * Qp[0] + gQ[1] * Qp[1] + gQ[2] * Qp[2] + gQ[3] * Qp[3] + gQ[4] * Qp[4];
-        }
-        // the next batch's column/row word and id, loaded one batch ahead
-        uint32_t ncr = 0u, nid = 0u;
+        S.ray[0][lane] = make_float4(dd[0], dd[1], dd[2], r.gQ[3]);
+        S.ray[1][lane] = make_float4(r.gQ[0], r.gQ[1], r.gQ[2], 0.f);
+        // the next window's column/row word and id, loaded one window ahead
+        uint32_t ncr = 0u, nid = 0u, head = 0u, tail = 0u;
         if (lo + lane < hi) {
             ncr = crw[lo + lane];
             nid = ids[lo + lane];
         }
         for (uint32_t base = lo; base < hi; base += 32) {
-            // lanes whose composited entries reach this batch: an entry that
+            // lanes whose composited entries reach this window: an entry that
             // reaches none of them contributes to no ray and is not staged
             const uint32_t act = __ballot_sync(0xffffffffu, rg.x + last > base);
             const uint32_t idx = base + lane;
-            const uint32_t g = nid;
-            const uint32_t lm = word_lanes(ncr, sub) & act;
-            const bool ov = lm != 0u;
+            push(S.cand, S.cpos, tail, nid, word_lanes(ncr, sub) & act, idx + 1 - rg.x);
+            ncr = 0u;
             if (idx + 32 < hi) {
                 ncr = crw[idx + 32];
                 nid = ids[idx + 32];
-            } else {
-                ncr = 0u;
             }
-            const uint32_t bal = __ballot_sync(0xffffffffu, ov);
-            if (bal == 0u) continue;
-            __syncwarp();
-            if (ov) {
-                const int pos = __popc(bal & ((1u << lane) - 1u));
-                float4 ent[9];
-                cam_entry(rec[g], s_pose.t, dh, dl, ent, kResponseScale);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) s_e[k][pos] = ent[k];
-                s_lanes[wib][pos] = lm;
-                s_pos[wib][pos] = idx + 1 - rg.x;
-                s_gid[wib][pos] = g;
-            }
-            __syncwarp();
-            const int n = __popc(bal);
-            for (int j = 0; j < n; ++j) {
-                PairEval pe;
-                bool ok = cam_pair_scaled(s_e[0][j], s_e[1][j], s_e[2][j], s_e[3][j], s_e[4][j],
-                                          s_e[5][j], s_e[6][j], (s_lanes[wib][j] >> lane) & 1u, dd,
-                                          P.alpha_min, P.alpha_max, pe);
-                ok = ok && s_pos[wib][j] <= last;
-                if (!__any_sync(0xffffffffu, ok)) continue;
-                float g[kG];
-#pragma unroll
-                for (int k = 0; k < kG; ++k) g[k] = 0.f;
-                if (ok) {
-                    const float4 m0 = s_e[3][j], m1 = s_e[4][j], m2 = s_e[5][j];
-                    const float Mr[9] = {m0.x, m0.y, m0.z, m1.x, m1.y, m1.z, m2.x, m2.y, m2.z};
-                    const float4 col = s_e[7][j];
-                    const float q[3] = {col.x, col.y, col.z};
-                    composite_grads(pe, s_e[6][j].w, q, gQ, T, U, Ut, Mr, d, g);
-                }
-                warp_reduce_add16(g, gacc + (int64_t)s_gid[wib][j] * kG);
+            const uint32_t least = base + 32 < hi ? 32u : 1u;     // at the end, what is left
+            while (tail - head >= least) {
+                const uint32_t n = min(32u, tail - head);
+                bw_batch(P, s_pose, rec, S, head, (int)n, dh, dl, dd, last, r, gacc);
+                head += n;
             }
         }
         __syncwarp();
     }
 }
 
+// ------------------------------------------------------------------ posed rays
+// LiDAR items and rolling-shutter sub-blocks, whose rays lie in up to four
+// slots (columns, pixel rows) with a pose each: entries are staged as by the
+// forward (lidar_entry), 16 at a time, two lanes an entry, each for two of its
+// slots.
+struct BwPosed {                   // a warp's shared memory
+    float4 s[(3 * 32 + kBwBatch * kLidEntryStride + 31) / 32][32];
+    float2 wx[kBwBatch][33];
+    float4 ray[3][32];             // (dd, gZ), (d, slot), (gF, 0)
+    uint2 cand[kBwQueue];
+    uint32_t cpos[kBwQueue];
+    uint32_t pos[kBwBatch], lanes[kBwBatch], gid[kBwBatch];
+};
+
+__device__ __forceinline__ void posed_stage(const GRec *__restrict__ rec, BwPosed &S, uint32_t head,
+                                            int n, const float *poses, int first, int slots,
+                                            const float dh[3], const float dl[3])
+{
+    const int lane = threadIdx.x & 31, j = lane & 15, half = lane >> 4;
+    __syncwarp();
+    if (j < n) {
+        const uint2 c = S.cand[(head + j) % kBwQueue];
+        lidar_entry_slots(rec[c.x], poses, first, 2 * half, min(slots, 2 * half + 2), dh, dl, S.s, j);
+        if (half == 0) {
+            S.lanes[j] = c.y;
+            S.pos[j] = S.cpos[(head + j) % kBwQueue];
+            S.gid[j] = c.x;
+        }
+    }
+    __syncwarp();
+}
+
+// Phase 2 of one pair: entry j, ray k (rows of M in m).
+__device__ __forceinline__ void posed_pair(GaussSums &g, BwPosed &S, int j, int k, const float4 m[3],
+                                           float2 wx)
+{
+    if (wx.x == 0.f) return;     // not composited
+    const float4 a = S.ray[0][k], d = S.ray[1][k], f = S.ray[2][k];
+    const int sl = __float_as_int(d.w);
+    const float4 q0 = lid_col(S.s, j, 0, sl), q1 = lid_col(S.s, j, 1, sl), q2 = lid_col(S.s, j, 2, sl);
+    const float num[3] = {q0.w + q0.x * a.x + q0.y * a.y + q0.z * a.z,
+                          q1.w + q1.x * a.x + q1.y * a.y + q1.z * a.z,
+                          q2.w + q2.x * a.x + q2.y * a.y + q2.z * a.z};
+    float den[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) den[i] = m[i].x * d.x + m[i].y * d.y + m[i].z * d.z;
+    const float gF[3] = {f.x, f.y, f.z};
+    add_pair(g, num, den, 1.f, wx, gF, a.w);
+}
+
 // ------------------------------------------------------------------ rolling shutter
-// The camera backward with a pose per pixel row: the rolling-shutter
-// forward's staging (row slots as LiDAR columns) and ray set-up.
-__global__ void __launch_bounds__(32 * kBwWarps, 4)
+// The camera backward with a pose per pixel row.
+__global__ void __launch_bounds__(32 * kBwWarpsPosed)
 k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
                      const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
                      const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
@@ -293,10 +422,9 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
                      const float *__restrict__ g_alpha, const float *__restrict__ g_depth,
                      float *__restrict__ gacc)
 {
-    __shared__ float4 s_all[kBwWarps][kLidPlanes][32];
-    __shared__ uint32_t s_pos[kBwWarps][32], s_lanes[kBwWarps][32], s_gid[kBwWarps][32];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    float4(*s)[32] = s_all[wib];
+    __shared__ BwPosed s_all[kBwWarpsPosed];
+    const int lane = threadIdx.x & 31;
+    BwPosed &S = s_all[threadIdx.x >> 5];
     const uint32_t n_items = counts[0];
     while (true) {
         uint32_t item = 0;
@@ -317,10 +445,7 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
         const uint2 rg = ranges[tile];
         const uint32_t lo = rg.x + (uint32_t)seg * kSegLen;
         uint32_t hi = min(rg.y, lo + kSegLen);
-        uint32_t lim = rg.x + last;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lim = max(lim, __shfl_xor_sync(0xffffffffu, lim, o));
-        hi = min(hi, lim);
+        hi = min(hi, rg.x + __reduce_max_sync(0xffffffffu, last));
         if (hi <= lo) continue;
         const int nrows = min(4, P.H - sby);
         const int row = py < P.H ? py : sby;
@@ -330,21 +455,22 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
             const double *u = tile_dir + 3 * tile;
             sensor_ray(poses + 12 * sby, u[0], u[1], u[2], poses + 12 * row, e, dh, dl, dd, d);
         }
-        float T = 1.f, Qp[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        if (seg > 0) {
-            const float4 *pq = partials + ((size_t)(ti.y + seg) * 256 + sub * 32 + lane) * 2;
-            const float4 u = pq[0], v = pq[1];
-            Qp[0] = u.x; Qp[1] = u.y; Qp[2] = u.z; Qp[3] = v.x; Qp[4] = u.w;
-            T = v.y;
+        RayGrad r;
+        {
+            float gQ[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            float4 st = make_float4(0.f, 0.f, 0.f, 0.f), F = st;
+            if (ray_ok) {
+                st = ray_state[pidx];
+                F = ray_feat[pidx];
+                camera_gQ(g_rgb, g_alpha, g_depth, pidx, st.y, st.z, gQ);
+            }
+            start_ray(r, seg > 0 ? partials + ((size_t)(ti.y + seg) * 256 + sub * 32 + lane) * 2 : nullptr,
+                      gQ, F, st.z, st.y);
         }
-        float gQ[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, Ut = 0.f, U = 0.f;
-        if (ray_ok) {
-            const float4 st = ray_state[pidx], F = ray_feat[pidx];
-            camera_gQ(g_rgb, g_alpha, g_depth, pidx, st.y, st.z, gQ);
-            Ut = gQ[0] * F.x + gQ[1] * F.y + gQ[2] * F.z + gQ[3] * st.z + gQ[4] * st.y;
-            U = gQ[0] * Qp[0] + gQ[1] * Qp[1] + gQ[2] * Qp[2] + gQ[3] * Qp[3] + gQ[4] * Qp[4];
-        }
-        uint32_t ncr = 0u, nid = 0u;    // the next batch's, one batch ahead
+        S.ray[0][lane] = make_float4(dd[0], dd[1], dd[2], r.gQ[3]);
+        S.ray[1][lane] = make_float4(d[0], d[1], d[2], __int_as_float(row - sby));
+        S.ray[2][lane] = make_float4(r.gQ[0], r.gQ[1], r.gQ[2], 0.f);
+        uint32_t ncr = 0u, nid = 0u, head = 0u, tail = 0u;    // as in k_backward_camera
         if (lo + lane < hi) {
             ncr = crw[lo + lane];
             nid = ids[lo + lane];
@@ -352,42 +478,44 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
         for (uint32_t base = lo; base < hi; base += 32) {
             const uint32_t act = __ballot_sync(0xffffffffu, rg.x + last > base);
             const uint32_t idx = base + lane;
-            const uint32_t g = nid;
-            const uint32_t lm = word_lanes(ncr, sub) & act;
+            push(S.cand, S.cpos, tail, nid, word_lanes(ncr, sub) & act, idx + 1 - rg.x);
+            ncr = 0u;
             if (idx + 32 < hi) {
                 ncr = crw[idx + 32];
                 nid = ids[idx + 32];
-            } else {
-                ncr = 0u;
             }
-            const uint32_t bal = __ballot_sync(0xffffffffu, lm != 0u);
-            if (bal == 0u) continue;
-            __syncwarp();
-            if (lm) {
-                const int pos = __popc(bal & ((1u << lane) - 1u));
-                lidar_entry(rec[g], poses, sby, nrows, dh, dl, s, pos);
-                s_lanes[wib][pos] = lm;
-                s_pos[wib][pos] = idx + 1 - rg.x;
-                s_gid[wib][pos] = g;
-            }
-            __syncwarp();
-            const int cnt = __popc(bal);
-            for (int j = 0; j < cnt; ++j) {
-                PairEval pe;
-                bool ok = lidar_pair_in(s, j, sb, (s_lanes[wib][j] >> lane) & 1u, dd, d,
-                                        P.alpha_min, P.alpha_max, pe);
-                ok = ok && s_pos[wib][j] <= last;
-                if (!__any_sync(0xffffffffu, ok)) continue;
-                float gg[kG];
-#pragma unroll
-                for (int k = 0; k < kG; ++k) gg[k] = 0.f;
-                if (ok) {
-                    const float4 m0 = s[0][j], m1 = s[1][j], m2 = s[2][j];
-                    const float Mr[9] = {m0.x, m0.y, m0.z, m1.x, m1.y, m1.z, m2.x, m2.y, m2.z};
-                    const float q[3] = {m1.w, m2.w, lid_u(s, j, sb).w};
-                    composite_grads(pe, m0.w, q, gQ, T, U, Ut, Mr, d, gg);
+            const uint32_t least = base + 32 < hi ? (uint32_t)kBwBatch : 1u;
+            while (tail - head >= least) {
+                const int nb = (int)min((uint32_t)kBwBatch, tail - head);
+                posed_stage(rec, S, head, nb, poses, sby, nrows, dh, dl);
+                head += nb;
+                uint32_t used = 0u;
+                for (int j = 0; j < nb; ++j) {
+                    PairEval pe;
+                    bool ok = lidar_pair_in(S.s, j, sb, (S.lanes[j] >> lane) & 1u, dd, d,
+                                            P.alpha_min, P.alpha_max, pe);
+                    ok = ok && S.pos[j] <= last;
+                    float2 wx = make_float2(0.f, 0.f);
+                    if (ok) {
+                        const float q[3] = {S.s[1][j].w, S.s[2][j].w, lid_u(S.s, j, sb).w};
+                        wx = ray_step(r, pe, q);
+                    }
+                    S.wx[j][lane] = wx;
+                    used |= (__any_sync(0xffffffffu, ok) ? 1u : 0u) << j;
                 }
-                warp_reduce_add16(gg, gacc + (int64_t)s_gid[wib][j] * kG);
+                __syncwarp();
+                if (used == 0u) continue;
+                const int j = lane & 15, r0 = lane & 16;
+                const bool use = (used >> j) & 1u;
+                const int jl = use ? j : 0;
+                const float4 m[3] = {S.s[0][jl], S.s[1][jl], S.s[2][jl]};
+                GaussSums g;
+                clear(g);
+#pragma unroll 2
+                for (int k = 0; k < 16; ++k)
+                    posed_pair(g, S, jl, r0 + k, m,
+                               use ? S.wx[j][r0 + k] : make_float2(0.f, 0.f));
+                add_sums(g, m[0].w, use, gacc + (int64_t)S.gid[jl] * kG);
             }
         }
         __syncwarp();
@@ -395,7 +523,10 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
 }
 
 // ------------------------------------------------------------------ LiDAR
-__global__ void __launch_bounds__(32 * kBwWarps)
+// Phase 1 by column groups, as the forward (the lanes of one column walk the
+// entries whose box holds a ray of it, side by side with the other columns');
+// phase 2 over the rays in each entry's own box (6 of 32 on the street sweep).
+__global__ void __launch_bounds__(32 * kBwWarpsPosed)
 k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
                  const uint32_t *__restrict__ item_rays, const float4 *__restrict__ ray_e,
                  const double *__restrict__ item_u, const float *__restrict__ poses,
@@ -410,10 +541,9 @@ k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
                  const float *__restrict__ g_int, const float *__restrict__ g_drop,
                  const float *__restrict__ g_alpha, float *__restrict__ gacc)
 {
-    __shared__ float4 s_all[kBwWarps][kLidPlanes][32];
-    __shared__ uint32_t s_gid[kBwWarps][32], s_lanes[kBwWarps][32], s_pos[kBwWarps][32];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    float4(*s)[32] = s_all[wib];
+    __shared__ BwPosed s_all[kBwWarpsPosed];
+    const int lane = threadIdx.x & 31;
+    BwPosed &S = s_all[threadIdx.x >> 5];
     const uint32_t n_work = counts[0];
     while (true) {
         uint32_t wi = 0;
@@ -431,43 +561,43 @@ k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
         const uint2 rg = ranges[it.tile];
         const uint32_t lo = rg.x + seg * kSegLen;
         uint32_t hi = min(rg.y, lo + kSegLen);
-        uint32_t lim = rg.x + last;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lim = max(lim, __shfl_xor_sync(0xffffffffu, lim, o));
-        hi = min(hi, lim);
+        hi = min(hi, rg.x + __reduce_max_sync(0xffffffffu, last));
         if (hi <= lo) continue;
         const int c = valid ? (int)(ray % (uint32_t)P.n_cols) : it.col0;
         const int sb = 3 + 4 * (c - it.col0);
+        const uint32_t gm = __match_any_sync(0xffffffffu, sb);   // lanes of this lane's column
         float dh[3], dl[3], dd[3], d[3];
         lidar_ray(it, item_u, item_id, poses, ray_e[it.ray_off + lane], c, dh, dl, dd, d);
         // the item's ray masks of the list entries (the forward's own)
         const uint32_t *lm = lmask + (int64_t)(item_id - (int)tile_items[it.tile].x) * lmask_stride;
-        float T = 1.f, Qp[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        if (seg > 0) {
-            const float4 *pq = partials + ((size_t)(ui.y + seg) * 32 + lane) * 2;
-            const float4 u = pq[0], v = pq[1];
-            Qp[0] = u.x; Qp[1] = u.y; Qp[2] = u.z; Qp[3] = v.x; Qp[4] = u.w;
-            T = v.y;
+        RayGrad r;
+        {
+            float gQ[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            float4 st = make_float4(0.f, 0.f, 0.f, 0.f), F = st;
+            if (valid) {
+                st = ray_state[ray];
+                F = ray_feat[ray];
+                const float W = st.y, Z = st.z, drop = st.w;
+                const float gr = g_range ? g_range[ray] : 0.f;
+                const float gi = g_int ? g_int[ray] : 0.f;
+                const float gp = g_drop ? g_drop[ray] : 0.f;
+                const float ga = g_alpha ? g_alpha[ray] : 0.f;
+                // drop = softmax(F1, F2)[drop] = 1 / (1 + exp(F1 - F2))
+                const float dd_ = drop * (1.f - drop);
+                gQ[0] = gi;
+                gQ[1] = -gp * dd_;
+                gQ[2] = gp * dd_;
+                gQ[3] = W > 0.f ? gr / W : 0.f;
+                gQ[4] = ga - (W > 0.f ? gr * Z / (W * W) : 0.f);
+            }
+            start_ray(r, seg > 0 ? partials + ((size_t)(ui.y + seg) * 32 + lane) * 2 : nullptr, gQ, F,
+                      st.z, st.y);
         }
-        float gQ[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, Ut = 0.f, U = 0.f;
-        if (valid) {
-            const float4 st = ray_state[ray], F = ray_feat[ray];
-            const float W = st.y, Z = st.z, drop = st.w;
-            const float gr = g_range ? g_range[ray] : 0.f;
-            const float gi = g_int ? g_int[ray] : 0.f;
-            const float gp = g_drop ? g_drop[ray] : 0.f;
-            const float ga = g_alpha ? g_alpha[ray] : 0.f;
-            // drop = softmax(F1, F2)[drop] = 1 / (1 + exp(F1 - F2))
-            const float dd_ = drop * (1.f - drop);
-            gQ[0] = gi;
-            gQ[1] = -gp * dd_;
-            gQ[2] = gp * dd_;
-            gQ[3] = W > 0.f ? gr / W : 0.f;
-            gQ[4] = ga - (W > 0.f ? gr * Z / (W * W) : 0.f);
-            Ut = gQ[0] * F.x + gQ[1] * F.y + gQ[2] * F.z + gQ[3] * Z + gQ[4] * W;
-            U = gQ[0] * Qp[0] + gQ[1] * Qp[1] + gQ[2] * Qp[2] + gQ[3] * Qp[3] + gQ[4] * Qp[4];
-        }
-        uint32_t nid = 0u, nm = 0u;   // one batch ahead
+        __syncwarp();
+        S.ray[0][lane] = make_float4(dd[0], dd[1], dd[2], r.gQ[3]);
+        S.ray[1][lane] = make_float4(d[0], d[1], d[2], __int_as_float(c - it.col0));
+        S.ray[2][lane] = make_float4(r.gQ[0], r.gQ[1], r.gQ[2], 0.f);
+        uint32_t nid = 0u, nm = 0u, head = 0u, tail = 0u;   // one window ahead
         if (lo + lane < hi) {
             nid = ids[lo + lane];
             nm = lm[lo + lane];
@@ -475,301 +605,415 @@ k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
         for (uint32_t base = lo; base < hi; base += 32) {
             const uint32_t act = __ballot_sync(0xffffffffu, rg.x + last > base);
             const uint32_t idx = base + lane;
-            const uint32_t g = nid;
-            const uint32_t m = nm & act;
+            push(S.cand, S.cpos, tail, nid, nm & act, idx + 1 - rg.x);
+            nm = 0u;
             if (idx + 32 < hi) {
                 nid = ids[idx + 32];
                 nm = lm[idx + 32];
-            } else {
-                nm = 0u;
             }
-            const uint32_t bal = __ballot_sync(0xffffffffu, m != 0u);
-            if (bal == 0u) continue;
-            __syncwarp();
-            if (m) {
-                const int pos = __popc(bal & ((1u << lane) - 1u));
-                lidar_entry(rec[g], poses, it.col0, it.ncols, dh, dl, s, pos);
-                s_lanes[wib][pos] = m;
-                s_pos[wib][pos] = idx + 1 - rg.x;
-                s_gid[wib][pos] = g;
-            }
-            __syncwarp();
-            const int cnt = __popc(bal);
-            for (int j = 0; j < cnt; ++j) {
-                PairEval pe;
-                bool ok = lidar_pair_in(s, j, sb, (s_lanes[wib][j] >> lane) & 1u, dd, d,
-                                        P.alpha_min, P.alpha_max, pe);
-                ok = ok && s_pos[wib][j] <= last;
-                if (!__any_sync(0xffffffffu, ok)) continue;
-                float g[kG];
-#pragma unroll
-                for (int k = 0; k < kG; ++k) g[k] = 0.f;
-                if (ok) {
-                    const float4 m0 = s[0][j], m1 = s[1][j], m2 = s[2][j];
-                    const float Mr[9] = {m0.x, m0.y, m0.z, m1.x, m1.y, m1.z, m2.x, m2.y, m2.z};
-                    const float q[3] = {m1.w, m2.w, lid_u(s, j, sb).w};
-                    composite_grads(pe, m0.w, q, gQ, T, U, Ut, Mr, d, g);
+            const uint32_t least = base + 32 < hi ? (uint32_t)kBwBatch : 1u;
+            while (tail - head >= least) {
+                const int nb = (int)min((uint32_t)kBwBatch, tail - head);
+                posed_stage(rec, S, head, nb, poses, it.col0, it.ncols, dh, dl);
+                head += nb;
+                // the staged entries that reach a ray of this lane's column
+                const uint32_t lj = lane < nb ? S.lanes[lane] : 0u;
+                uint32_t G = 0u;
+                for (uint32_t rest = 0xffffffffu; rest;) {
+                    const uint32_t gm_g = __shfl_sync(0xffffffffu, gm, __ffs(rest) - 1);
+                    const uint32_t Gg = __ballot_sync(0xffffffffu, (lj & gm_g) != 0u);
+                    G = gm == gm_g ? Gg : G;
+                    rest &= ~gm_g;
                 }
-                warp_reduce_add16(g, gacc + (int64_t)s_gid[wib][j] * kG);
+                uint32_t used = 0u;      // entries this lane's ray composites
+                while (__any_sync(0xffffffffu, G != 0u)) {
+                    const bool has = G != 0u;
+                    const int j = has ? __ffs(G) - 1 : 0;
+                    G &= G - 1u;
+                    const bool in = has && ((S.lanes[j] >> lane) & 1u);
+                    PairEval pe;
+                    bool ok = lidar_pair_in(S.s, j, sb, in, dd, d, P.alpha_min, P.alpha_max, pe);
+                    ok = ok && S.pos[j] <= last;
+                    float2 wx = make_float2(0.f, 0.f);
+                    if (ok) {
+                        const float q[3] = {S.s[1][j].w, S.s[2][j].w, lid_u(S.s, j, sb).w};
+                        wx = ray_step(r, pe, q);
+                        used |= 1u << j;
+                    }
+                    if (in) S.wx[j][lane] = wx;
+                }
+                used = __reduce_or_sync(0xffffffffu, used);
+                __syncwarp();
+                if (used == 0u) continue;
+                const int j = lane & 15, r0 = lane & 16;
+                const bool use = (used >> j) & 1u;
+                const int jl = use ? j : 0;
+                const float4 m[3] = {S.s[0][jl], S.s[1][jl], S.s[2][jl]};
+                uint32_t rays = use ? (S.lanes[jl] >> r0) & 0xffffu : 0u;
+                GaussSums g;
+                clear(g);
+                while (rays) {
+                    const int k = r0 + __ffs(rays) - 1;
+                    rays &= rays - 1u;
+                    posed_pair(g, S, jl, k, m, S.wx[jl][k]);
+                }
+                __syncwarp();
+                add_sums(g, m[0].w, use, gacc + (int64_t)S.gid[jl] * kG);
             }
         }
     }
 }
 
 // ------------------------------------------------------------------ parameters
-__device__ __forceinline__ void sh_basis_grad(int deg, float x, float y, float z, float Y[16],
-                                              float dY[16][3])
+// Y_k(d) and its gradient w.r.t. d (as a polynomial in d), k = 0 .. (kDeg + 1)^2 - 1.
+template <int kDeg>
+__device__ __forceinline__ void sh_basis(float x, float y, float z, float Y[(kDeg + 1) * (kDeg + 1)])
 {
     const float xx = x * x, yy = y * y, zz = z * z;
-    for (int k = 0; k < 16; ++k) { Y[k] = 0.f; dY[k][0] = dY[k][1] = dY[k][2] = 0.f; }
     Y[0] = 0.28209479177387814f;
-    if (deg >= 1) {
+    if constexpr (kDeg >= 1) {
         const float c = 0.48860251190291992f;
-        Y[1] = -c * y; dY[1][1] = -c;
-        Y[2] = c * z;  dY[2][2] = c;
-        Y[3] = -c * x; dY[3][0] = -c;
+        Y[1] = -c * y;
+        Y[2] = c * z;
+        Y[3] = -c * x;
     }
-    if (deg >= 2) {
+    if constexpr (kDeg >= 2) {
         const float a = 1.0925484305920792f, b = 0.31539156525252005f, h = 0.54627421529603959f;
-        Y[4] = a * x * y;  dY[4][0] = a * y; dY[4][1] = a * x;
-        Y[5] = -a * y * z; dY[5][1] = -a * z; dY[5][2] = -a * y;
+        Y[4] = a * x * y;
+        Y[5] = -a * y * z;
         Y[6] = b * (2.f * zz - xx - yy);
-        dY[6][0] = -2.f * b * x; dY[6][1] = -2.f * b * y; dY[6][2] = 4.f * b * z;
-        Y[7] = -a * x * z; dY[7][0] = -a * z; dY[7][2] = -a * x;
-        Y[8] = h * (xx - yy); dY[8][0] = 2.f * h * x; dY[8][1] = -2.f * h * y;
+        Y[7] = -a * x * z;
+        Y[8] = h * (xx - yy);
     }
-    if (deg >= 3) {
+    if constexpr (kDeg >= 3) {
         const float c0 = 0.59004358992664352f, c1 = 2.8906114426405538f;
         const float c2 = 0.45704579946446572f, c3 = 0.37317633259011540f;
         const float c5 = 1.4453057213202769f;
         Y[9] = -c0 * y * (3.f * xx - yy);
-        dY[9][0] = -6.f * c0 * x * y; dY[9][1] = -c0 * (3.f * xx - 3.f * yy);
         Y[10] = c1 * x * y * z;
-        dY[10][0] = c1 * y * z; dY[10][1] = c1 * x * z; dY[10][2] = c1 * x * y;
         Y[11] = -c2 * y * (4.f * zz - xx - yy);
-        dY[11][0] = 2.f * c2 * x * y; dY[11][1] = -c2 * (4.f * zz - xx - 3.f * yy);
-        dY[11][2] = -8.f * c2 * y * z;
         Y[12] = c3 * z * (2.f * zz - 3.f * xx - 3.f * yy);
-        dY[12][0] = -6.f * c3 * x * z; dY[12][1] = -6.f * c3 * y * z;
-        dY[12][2] = c3 * (6.f * zz - 3.f * xx - 3.f * yy);
         Y[13] = -c2 * x * (4.f * zz - xx - yy);
-        dY[13][0] = -c2 * (4.f * zz - 3.f * xx - yy); dY[13][1] = 2.f * c2 * x * y;
-        dY[13][2] = -8.f * c2 * x * z;
         Y[14] = c5 * z * (xx - yy);
-        dY[14][0] = 2.f * c5 * x * z; dY[14][1] = -2.f * c5 * y * z; dY[14][2] = c5 * (xx - yy);
         Y[15] = -c0 * x * (xx - 3.f * yy);
-        dY[15][0] = -c0 * (3.f * xx - 3.f * yy); dY[15][1] = 6.f * c0 * x * y;
     }
 }
 
-// SH origin: (ox, oy, oz) for cameras; for LiDAR SH^l features, the origin
-// of the column pose that saw the mean, whose index the projection left in
-// the record's feat.w.
-__global__ void k_param_grads(const float *__restrict__ planes, int64_t pitch, int64_t n,
-                              int feature_kind, int sh_degree, int F, float ox, float oy,
-                              float oz, const GRec *__restrict__ rec,
-                              const float *__restrict__ poses, ActorParams A, float beam,
-                              int posed_origin,
-                              const float *__restrict__ gacc, float *__restrict__ gm,
-                              float *__restrict__ gls, float *__restrict__ gq,
-                              float *__restrict__ gop, float *__restrict__ gf)
+// sum_k h_k grad Y_k(d).
+template <int kDeg>
+__device__ __forceinline__ void sh_basis_grad(float x, float y, float z,
+                                              const float h[(kDeg + 1) * (kDeg + 1)], float g[3])
 {
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n) return;
-    float G[kG];
-    bool any = false;
+    const float xx = x * x, yy = y * y, zz = z * z;
+    g[0] = g[1] = g[2] = 0.f;
+    if constexpr (kDeg >= 1) {
+        const float c = 0.48860251190291992f;
+        g[0] -= c * h[3];
+        g[1] -= c * h[1];
+        g[2] += c * h[2];
+    }
+    if constexpr (kDeg >= 2) {
+        const float a = 1.0925484305920792f, b = 0.31539156525252005f, c = 0.54627421529603959f;
+        g[0] += a * y * h[4] - 2.f * b * x * h[6] - a * z * h[7] + 2.f * c * x * h[8];
+        g[1] += a * x * h[4] - a * z * h[5] - 2.f * b * y * h[6] - 2.f * c * y * h[8];
+        g[2] += -a * y * h[5] + 4.f * b * z * h[6] - a * x * h[7];
+    }
+    if constexpr (kDeg >= 3) {
+        const float c0 = 0.59004358992664352f, c1 = 2.8906114426405538f;
+        const float c2 = 0.45704579946446572f, c3 = 0.37317633259011540f;
+        const float c5 = 1.4453057213202769f;
+        g[0] += -6.f * c0 * x * y * h[9] + c1 * y * z * h[10] + 2.f * c2 * x * y * h[11] -
+                6.f * c3 * x * z * h[12] - c2 * (4.f * zz - 3.f * xx - yy) * h[13] +
+                2.f * c5 * x * z * h[14] - c0 * (3.f * xx - 3.f * yy) * h[15];
+        g[1] += -c0 * (3.f * xx - 3.f * yy) * h[9] + c1 * x * z * h[10] -
+                c2 * (4.f * zz - xx - 3.f * yy) * h[11] - 6.f * c3 * y * z * h[12] +
+                2.f * c2 * x * y * h[13] - 2.f * c5 * y * z * h[14] + 6.f * c0 * x * y * h[15];
+        g[2] += c1 * x * y * h[10] - 8.f * c2 * y * z * h[11] +
+                c3 * (6.f * zz - 3.f * xx - 3.f * yy) * h[12] - 8.f * c2 * x * z * h[13] +
+                c5 * (xx - yy) * h[14];
+    }
+}
+
+constexpr int kPgThreads = 128;     // Gaussians per block of k_param_grads
+
+// Add the block's rows of C floats, staged at s + row * stride, to out (rows
+// g0 .. g0 + ng - 1 of [n, C]); a group of four floats is skipped if no row in
+// it has a gradient (any: a bit a row).
+template <int C>
+__device__ __forceinline__ void add_rows(float *__restrict__ out, int64_t g0, int ng,
+                                         const float *s, int stride, const uint32_t *any)
+{
+    if (!out) return;
+    float *p = out + g0 * C;
+    const int tot = ng * C;
+    const int v4 = ((uintptr_t)out & 15u) == 0 ? tot / 4 : 0;   // then p is aligned, too
+    auto has = [&](int row) { return (any[row >> 5] >> (row & 31)) & 1u; };
+#pragma unroll 2
+    for (int j = threadIdx.x; j < v4; j += kPgThreads) {
+        int r[4];
+        bool some = false;
 #pragma unroll
-    for (int k = 0; k < kG; ++k) {
-        G[k] = gacc[g * kG + k];
-        any = any || G[k] != 0.f;
+        for (int k = 0; k < 4; ++k) {
+            r[k] = (4 * j + k) / C;
+            some = some || has(r[k]);
+        }
+        if (!some) continue;
+        float4 v = reinterpret_cast<float4 *>(p)[j];
+        v.x += s[r[0] * stride + 4 * j - r[0] * C];
+        v.y += s[r[1] * stride + 4 * j + 1 - r[1] * C];
+        v.z += s[r[2] * stride + 4 * j + 2 - r[2] * C];
+        v.w += s[r[3] * stride + 4 * j + 3 - r[3] * C];
+        reinterpret_cast<float4 *>(p)[j] = v;
     }
-    if (!any) return;
-    // an actor's Gaussian: the accumulated gradients are in world
-    // coordinates (M_w = S^-1 (Ra R)^T, mu_w = Ra mu + t); in its own frame
-    // dL/dM_k becomes Ra^T dL/dM_k and dL/dmu becomes Ra^T dL/dmu
-    float Ra[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f}, ta[3] = {0.f, 0.f, 0.f};
-    const int ak = A.of ? A.of[g] : -1;
-    const bool actor = ak >= 0 && ak < A.n;
-    if (actor) {
-        const float *P = A.poses + 12 * ak;
-        for (int i = 0; i < 3; ++i) {
-            for (int j = 0; j < 3; ++j) Ra[3 * i + j] = P[4 * i + j];
-            ta[i] = P[4 * i + 3];
-        }
+    for (int j = 4 * v4 + threadIdx.x; j < tot; j += kPgThreads)
+        if (has(j / C)) p[j] += s[(j / C) * stride + j % C];
+}
+
+// The 13 sums of each Gaussian (add_sums) to the raw parameters; the rows read
+// are cleared for the next backward.  kDeg: degree of the SH features, or -1
+// for three features used as they are.  SH origin: (ox, oy, oz) for cameras;
+// for LiDAR SH^l features and rolling shutters, the origin of the pose that
+// saw the mean, whose index the projection left in the record's feat.w.
+//
+// Bound by HBM: 64 bytes of sums, 236 of parameters and, read and written,
+// 236 of gradients for a Gaussian with one (degree 3).  The gradients are AoS
+// rows, staged in shared memory and added with 16-byte accesses: one thread
+// adding its own 192-byte row 4 bytes at a time, with the SH planes read twice
+// and the basis in local memory, took 365 us for 1M Gaussians, now 182 (LiDAR
+// features, 2M: 136 -> 96).
+template <int kDeg>
+__global__ void __launch_bounds__(kPgThreads)
+k_param_grads(const float *__restrict__ planes, int64_t pitch, int64_t n, int lidar, float ox,
+              float oy, float oz, const GRec *__restrict__ rec, const float *__restrict__ poses,
+              ActorParams A, float beam, int posed_origin, float *__restrict__ gacc,
+              float *__restrict__ gm, float *__restrict__ gls, float *__restrict__ gq,
+              float *__restrict__ gop, float *__restrict__ gf)
+{
+    constexpr int nc = kDeg < 0 ? 1 : (kDeg + 1) * (kDeg + 1), F = 3 * nc;
+    constexpr int fs = F | 1;            // odd: a thread's row in banks of its own
+    __shared__ float s_f[kPgThreads * fs], s_p[kPgThreads * 11];
+    __shared__ uint32_t s_any[kPgThreads / 32];
+    const int t = threadIdx.x;
+    const int64_t g0 = (int64_t)blockIdx.x * kPgThreads, g = g0 + t;
+    const int ng = n - g0 < kPgThreads ? (int)(n - g0) : kPgThreads;
+    float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0, a2 = a0;
+    float a3 = 0.f;
+    if (t < ng) {
+        const float4 *row = reinterpret_cast<const float4 *>(gacc + g * kG);
+        a0 = row[0];
+        a1 = row[1];
+        a2 = row[2];
+        a3 = row[3].x;
     }
-    // Beam divergence (Eq. 6): the record holds M of the smoothed covariance
-    // (rows m_k orthogonal), and the loss depends on M only through
-    // A = M^T M = Sigma_hat^-1, so dL/dM = 2 M S with S = sym(dL/dA):
-    // S = M^-1 dL/dM / 2, M^-1 = [m_k / |m_k|^2].  Then dL/dSigma_hat =
-    // H = -A S A, and Sigma_hat = Sigma + beam^2 (|v|^2 I - v v^T), v = mu - o,
-    // adds beam^2 (2 v tr(H) - 2 H v) to dL/dmu.
-    float H[9];
-    if (beam > 0.f) {
-        const GRec &rc = rec[g];
-        const float m[9] = {rc.m0.x, rc.m0.y, rc.m0.z, rc.m1.x, rc.m1.y, rc.m1.z,
-                            rc.m2.x, rc.m2.y, rc.m2.z};
-        float S[9], T[9], Am[9];
-        for (int i = 0; i < 9; ++i) S[i] = 0.f;
-        for (int k = 0; k < 3; ++k) {
-            const float mk2 = m[3 * k] * m[3 * k] + m[3 * k + 1] * m[3 * k + 1] +
-                              m[3 * k + 2] * m[3 * k + 2];
-            for (int i = 0; i < 3; ++i)
-                for (int j = 0; j < 3; ++j) S[3 * i + j] += 0.5f * m[3 * k + i] / mk2 * G[3 * k + j];
-        }
-        for (int i = 0; i < 3; ++i)
-            for (int j = i + 1; j < 3; ++j) {
-                const float a = 0.5f * (S[3 * i + j] + S[3 * j + i]);
-                S[3 * i + j] = S[3 * j + i] = a;
-            }
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j)
-                Am[3 * i + j] = m[i] * m[j] + m[3 + i] * m[3 + j] + m[6 + i] * m[6 + j];
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j)
-                T[3 * i + j] = S[3 * i] * Am[j] + S[3 * i + 1] * Am[3 + j] + S[3 * i + 2] * Am[6 + j];
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j)
-                H[3 * i + j] = -(Am[3 * i] * T[j] + Am[3 * i + 1] * T[3 + j] + Am[3 * i + 2] * T[6 + j]);
-        const float *P = poses + 12 * __float_as_uint(rc.feat.w);
-        float v[3];
-        for (int i = 0; i < 3; ++i) {
-            const float mw = Ra[3 * i] * planes[(Scene::kMean + 0) * pitch + g] +
-                             Ra[3 * i + 1] * planes[(Scene::kMean + 1) * pitch + g] +
-                             Ra[3 * i + 2] * planes[(Scene::kMean + 2) * pitch + g] + ta[i];
-            v[i] = mw - P[4 * i + 3];
-        }
-        const float tr = H[0] + H[4] + H[8], b2 = beam * beam;
-        for (int i = 0; i < 3; ++i)
-            G[9 + i] += b2 * (2.f * v[i] * tr -
-                              2.f * (H[3 * i] * v[0] + H[3 * i + 1] * v[1] + H[3 * i + 2] * v[2]));
-        if (actor) {    // H in the Gaussian's own frame: Ra^T H Ra
-            for (int i = 0; i < 3; ++i)
-                for (int j = 0; j < 3; ++j)
-                    T[3 * i + j] = H[3 * i] * Ra[j] + H[3 * i + 1] * Ra[3 + j] + H[3 * i + 2] * Ra[6 + j];
-            for (int i = 0; i < 3; ++i)
-                for (int j = 0; j < 3; ++j)
-                    H[3 * i + j] = Ra[i] * T[j] + Ra[3 + i] * T[3 + j] + Ra[6 + i] * T[6 + j];
-        }
-    }
-    if (actor) {
-        for (int k = beam > 0.f ? 3 : 0; k < 4; ++k) {   // the rows of dL/dM, then dL/dmu
-            const float x = G[3 * k], y = G[3 * k + 1], z = G[3 * k + 2];
-            G[3 * k] = Ra[0] * x + Ra[3] * y + Ra[6] * z;
-            G[3 * k + 1] = Ra[1] * x + Ra[4] * y + Ra[7] * z;
-            G[3 * k + 2] = Ra[2] * x + Ra[5] * y + Ra[8] * z;
-        }
-    }
-    float q[4];
-    for (int k = 0; k < 4; ++k) q[k] = planes[(Scene::kQuat + k) * pitch + g];
-    const float qn = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-    const float w = q[0] / qn, x = q[1] / qn, y = q[2] / qn, z = q[3] / qn;
-    const float R[9] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y),
-                        2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x),
-                        2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)};
-    float gR[9];
-    if (beam > 0.f) {
-        // Sigma = sum_k s_k^2 r_k r_k^T: dL/dls_k = 2 s_k^2 r_k^T H r_k,
-        // dL/dr_k = 2 s_k^2 H r_k
-        for (int k = 0; k < 3; ++k) {
-            const float s = expf(planes[(Scene::kLogScale + k) * pitch + g]), s2 = s * s;
-            const float rk[3] = {R[k], R[3 + k], R[6 + k]};
-            float Hr[3];
-            for (int i = 0; i < 3; ++i) Hr[i] = H[3 * i] * rk[0] + H[3 * i + 1] * rk[1] + H[3 * i + 2] * rk[2];
-            if (gls) gls[3 * g + k] += 2.f * s2 * (rk[0] * Hr[0] + rk[1] * Hr[1] + rk[2] * Hr[2]);
-            for (int i = 0; i < 3; ++i) gR[3 * i + k] = 2.f * s2 * Hr[i];
-        }
+    const bool any = a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f || a1.x != 0.f ||
+                     a1.y != 0.f || a1.z != 0.f || a1.w != 0.f || a2.x != 0.f || a2.y != 0.f ||
+                     a2.z != 0.f || a2.w != 0.f || a3 != 0.f;
+    const uint32_t bits = __ballot_sync(0xffffffffu, any);
+    if ((t & 31) == 0) s_any[t >> 5] = bits;
+    if (!__syncthreads_or(any)) return;
+    float *fo = s_f + t * fs, *po = s_p + t * 11;     // means 3, log-scales 3, quaternion 4, opacity
+    if (!any) {
+#pragma unroll
+        for (int k = 0; k < F; ++k) fo[k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 11; ++k) po[k] = 0.f;
     } else {
-        // M_k = r_k / s_k (r_k = column k of R): dL/dls_k = -G_k . M_k,
-        // dL/dr_k = G_k / s_k
-        for (int k = 0; k < 3; ++k) {
-            const float s = expf(planes[(Scene::kLogScale + k) * pitch + g]);
-            const float rk[3] = {R[k], R[3 + k], R[6 + k]};
-            const float Gk[3] = {G[3 * k], G[3 * k + 1], G[3 * k + 2]};
-            if (gls) gls[3 * g + k] += -(Gk[0] * rk[0] + Gk[1] * rk[1] + Gk[2] * rk[2]) / s;
-            for (int i = 0; i < 3; ++i) gR[3 * i + k] = Gk[i] / s;
-        }
-    }
-    if (gq) {
-        // partial derivatives of R(w,x,y,z) (entries row-major), times 2
-        const float dRw[9] = {0, -z, y, z, 0, -x, -y, x, 0};
-        const float dRx[9] = {0, y, z, y, -2 * x, -w, z, w, -2 * x};
-        const float dRy[9] = {-2 * y, x, w, x, 0, z, -w, z, -2 * y};
-        const float dRz[9] = {-2 * z, -w, x, w, -2 * z, y, x, y, 0};
-        float gqh[4] = {0, 0, 0, 0};
-        for (int i = 0; i < 9; ++i) {
-            gqh[0] += 2.f * dRw[i] * gR[i];
-            gqh[1] += 2.f * dRx[i] * gR[i];
-            gqh[2] += 2.f * dRy[i] * gR[i];
-            gqh[3] += 2.f * dRz[i] * gR[i];
-        }
-        const float dot = gqh[0] * w + gqh[1] * x + gqh[2] * y + gqh[3] * z;
-        const float qh[4] = {w, x, y, z};
-        for (int i = 0; i < 4; ++i) gq[4 * g + i] += (gqh[i] - qh[i] * dot) / qn;
-    }
-    if (gop) gop[g] += G[12];
-    float gmu[3] = {G[9], G[10], G[11]};
-    const float gc[3] = {G[13], G[14], G[15]};
-    if (sh_features(feature_kind)) {
-        // the SH origin: for LiDAR and rolling-shutter cameras, the origin of
-        // the pose (column, row) that saw the mean, whose index the projection
-        // left in the record's feat.w
-        const bool lidar = feature_kind == SG_FEATURES_LIDAR_SH;
-        if (lidar || posed_origin) {
-            const float *P = poses + 12 * __float_as_uint(rec[g].feat.w);
-            ox = P[3];
-            oy = P[7];
-            oz = P[11];
-        }
-        // the view direction, in the Gaussian's own frame (Ra^T (mu_w - o))
-        const float lx = planes[(Scene::kMean + 0) * pitch + g];
-        const float ly = planes[(Scene::kMean + 1) * pitch + g];
-        const float lz = planes[(Scene::kMean + 2) * pitch + g];
-        const float wx = Ra[0] * lx + Ra[1] * ly + Ra[2] * lz + ta[0] - ox;
-        const float wy = Ra[3] * lx + Ra[4] * ly + Ra[5] * lz + ta[1] - oy;
-        const float wz = Ra[6] * lx + Ra[7] * ly + Ra[8] * lz + ta[2] - oz;
-        const float mx = actor ? Ra[0] * wx + Ra[3] * wy + Ra[6] * wz : wx;
-        const float my = actor ? Ra[1] * wx + Ra[4] * wy + Ra[7] * wz : wy;
-        const float mz = actor ? Ra[2] * wx + Ra[5] * wy + Ra[8] * wz : wz;
-        const float dist = sqrtf(mx * mx + my * my + mz * mz);
-        const float inv = 1.f / dist;
-        const float dx = mx * inv, dy = my * inv, dz = mz * inv;
-        float Y[16], dY[16][3];
-        sh_basis_grad(sh_degree, dx, dy, dz, Y, dY);
-        const int nc = (sh_degree + 1) * (sh_degree + 1);
-        float gdir[3] = {0.f, 0.f, 0.f};
-        for (int ch = 0; ch < 3; ++ch) {
-            float acc = 0.f;
-            for (int k = 0; k < nc; ++k) acc += Y[k] * planes[(Scene::kFeat + 3 * k + ch) * pitch + g];
-            if (!lidar && acc + 0.5f < 0.f) continue;   // clamped colour channel
-            for (int k = 0; k < nc; ++k) {
-                if (gf) gf[g * F + 3 * k + ch] += Y[k] * gc[ch];
-                const float f = planes[(Scene::kFeat + 3 * k + ch) * pitch + g];
-                gdir[0] += gc[ch] * f * dY[k][0];
-                gdir[1] += gc[ch] * f * dY[k][1];
-                gdir[2] += gc[ch] * f * dY[k][2];
+        float4 *row = reinterpret_cast<float4 *>(gacc + g * kG);
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        row[0] = zero;
+        row[1] = zero;
+        row[2] = zero;
+        row[3] = zero;
+        const float S[9] = {a0.x, a0.y, a0.z, a0.y, a0.w, a1.x, a0.z, a1.x, a1.y};
+        const float u[3] = {a1.z, a1.w, a2.x};
+        const float gc[3] = {a2.z, a2.w, a3};
+        // an actor's Gaussian (M_w = S^-1 (Ra R)^T, mu_w = Ra mu + t): in its own
+        // frame dL/dM_k becomes Ra^T dL/dM_k and dL/dmu becomes Ra^T dL/dmu
+        float Ra[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f}, ta[3] = {0.f, 0.f, 0.f};
+        const int ak = A.of ? A.of[g] : -1;
+        const bool actor = ak >= 0 && ak < A.n;
+        if (actor) {
+            const float *P = A.poses + 12 * ak;
+            for (int i = 0; i < 3; ++i) {
+                for (int j = 0; j < 3; ++j) Ra[3 * i + j] = P[4 * i + j];
+                ta[i] = P[4 * i + 3];
             }
         }
-        const float dd = gdir[0] * dx + gdir[1] * dy + gdir[2] * dz;
-        gmu[0] += (gdir[0] - dx * dd) * inv;
-        gmu[1] += (gdir[1] - dy * dd) * inv;
-        gmu[2] += (gdir[2] - dz * dd) * inv;
-    } else if (gf) {
-        for (int ch = 0; ch < 3; ++ch) gf[g * F + ch] += gc[ch];
+        float mu[3], sc[3], q[4];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            mu[k] = planes[(Scene::kMean + k) * pitch + g];
+            sc[k] = expf(planes[(Scene::kLogScale + k) * pitch + g]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q[k] = planes[(Scene::kQuat + k) * pitch + g];
+        const float qn = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
+        const float w = q[0] / qn, x = q[1] / qn, y = q[2] / qn, z = q[3] / qn;
+        const float R[9] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z),
+                            2.f * (x * z + w * y), 2.f * (x * y + w * z),
+                            1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x),
+                            2.f * (x * z - w * y), 2.f * (y * z + w * x),
+                            1.f - 2.f * (x * x + y * y)};
+        // mu in the world, for the origins of beam divergence and SH
+        const float mw[3] = {Ra[0] * mu[0] + Ra[1] * mu[1] + Ra[2] * mu[2] + ta[0],
+                             Ra[3] * mu[0] + Ra[4] * mu[1] + Ra[5] * mu[2] + ta[1],
+                             Ra[6] * mu[0] + Ra[7] * mu[1] + Ra[8] * mu[2] + ta[2]};
+        float gmu[3], gs[3], gR[9];
+        if (beam > 0.f) {
+            // Beam divergence (Eq. 6): the record holds M of the smoothed
+            // covariance, on which the loss depends through A = M^T M =
+            // Sigma_hat^-1: dL/dSigma_hat = H = -M^T S M / 2.  Sigma_hat =
+            // Sigma + beam^2 (|v|^2 I - v v^T), v = mu - o, adds beam^2 (2 v
+            // tr(H) - 2 H v) to dL/dmu.
+            const GRec &rc = rec[g];
+            const float m[9] = {rc.m0.x, rc.m0.y, rc.m0.z, rc.m1.x, rc.m1.y, rc.m1.z,
+                                rc.m2.x, rc.m2.y, rc.m2.z};
+            float H[9], T[9], gw[3];
+            for (int k = 0; k < 3; ++k)
+                for (int j = 0; j < 3; ++j)
+                    T[3 * k + j] = S[3 * k] * m[j] + S[3 * k + 1] * m[3 + j] + S[3 * k + 2] * m[6 + j];
+            for (int i = 0; i < 3; ++i)
+                for (int j = 0; j < 3; ++j)
+                    H[3 * i + j] = -0.5f * (m[i] * T[j] + m[3 + i] * T[3 + j] + m[6 + i] * T[6 + j]);
+            const float *P = poses + 12 * __float_as_uint(rc.feat.w);
+            const float v[3] = {mw[0] - P[3], mw[1] - P[7], mw[2] - P[11]};
+            const float tr = H[0] + H[4] + H[8], b2 = beam * beam;
+            for (int i = 0; i < 3; ++i)
+                gw[i] = -(m[i] * u[0] + m[3 + i] * u[1] + m[6 + i] * u[2]) +
+                        b2 * (2.f * v[i] * tr -
+                              2.f * (H[3 * i] * v[0] + H[3 * i + 1] * v[1] + H[3 * i + 2] * v[2]));
+            // in the Gaussian's own frame: Ra^T gw, Ra^T H Ra
+            for (int i = 0; i < 3; ++i) gmu[i] = Ra[i] * gw[0] + Ra[3 + i] * gw[1] + Ra[6 + i] * gw[2];
+            if (actor) {
+                for (int i = 0; i < 3; ++i)
+                    for (int j = 0; j < 3; ++j)
+                        T[3 * i + j] = H[3 * i] * Ra[j] + H[3 * i + 1] * Ra[3 + j] + H[3 * i + 2] * Ra[6 + j];
+                for (int i = 0; i < 3; ++i)
+                    for (int j = 0; j < 3; ++j)
+                        H[3 * i + j] = Ra[i] * T[j] + Ra[3 + i] * T[3 + j] + Ra[6 + i] * T[6 + j];
+            }
+            // Sigma = sum_k s_k^2 r_k r_k^T: dL/dls_k = 2 s_k^2 r_k^T H r_k,
+            // dL/dr_k = 2 s_k^2 H r_k
+            for (int k = 0; k < 3; ++k) {
+                const float s2 = sc[k] * sc[k], rk[3] = {R[k], R[3 + k], R[6 + k]};
+                float Hr[3];
+                for (int i = 0; i < 3; ++i)
+                    Hr[i] = H[3 * i] * rk[0] + H[3 * i + 1] * rk[1] + H[3 * i + 2] * rk[2];
+                gs[k] = 2.f * s2 * (rk[0] * Hr[0] + rk[1] * Hr[1] + rk[2] * Hr[2]);
+                for (int i = 0; i < 3; ++i) gR[3 * i + k] = 2.f * s2 * Hr[i];
+            }
+        } else {
+            // M_k = r_k / s_k (r_k = column k of R, orthonormal), dL/dM_k = sum_j
+            // S_kj s_j r_j: dL/dls_k = -dL/dM_k . M_k = -S_kk, dL/dr_k = dL/dM_k /
+            // s_k, dL/dmu = -sum_k u_k r_k / s_k
+            const float is[3] = {1.f / sc[0], 1.f / sc[1], 1.f / sc[2]};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                gs[k] = -S[3 * k + k];
+                const float c0 = S[3 * k] * sc[0] * is[k], c1 = S[3 * k + 1] * sc[1] * is[k];
+                const float c2 = S[3 * k + 2] * sc[2] * is[k];
+                gmu[k] = -(u[0] * is[0] * R[3 * k] + u[1] * is[1] * R[3 * k + 1] +
+                           u[2] * is[2] * R[3 * k + 2]);
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    gR[3 * i + k] = c0 * R[3 * i] + c1 * R[3 * i + 1] + c2 * R[3 * i + 2];
+            }
+        }
+        // partial derivatives of R(w,x,y,z) (entries row-major), times 2
+        const float gw_ = 2.f * (-z * gR[1] + y * gR[2] + z * gR[3] - x * gR[5] - y * gR[6] + x * gR[7]);
+        const float gx_ = 2.f * (y * gR[1] + z * gR[2] + y * gR[3] - 2.f * x * gR[4] - w * gR[5] +
+                                 z * gR[6] + w * gR[7] - 2.f * x * gR[8]);
+        const float gy_ = 2.f * (-2.f * y * gR[0] + x * gR[1] + w * gR[2] + x * gR[3] + z * gR[5] -
+                                 w * gR[6] + z * gR[7] - 2.f * y * gR[8]);
+        const float gz_ = 2.f * (-2.f * z * gR[0] - w * gR[1] + x * gR[2] + w * gR[3] -
+                                 2.f * z * gR[4] + y * gR[5] + x * gR[6] + y * gR[7]);
+        const float dot = gw_ * w + gx_ * x + gy_ * y + gz_ * z, iq = 1.f / qn;
+        po[3] = gs[0]; po[4] = gs[1]; po[5] = gs[2];
+        po[6] = (gw_ - w * dot) * iq;
+        po[7] = (gx_ - x * dot) * iq;
+        po[8] = (gy_ - y * dot) * iq;
+        po[9] = (gz_ - z * dot) * iq;
+        po[10] = a2.y;
+        if constexpr (kDeg < 0) {
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) fo[ch] = gc[ch];
+        } else {
+            if (lidar || posed_origin) {
+                const float *P = poses + 12 * __float_as_uint(rec[g].feat.w);
+                ox = P[3];
+                oy = P[7];
+                oz = P[11];
+            }
+            // the view direction, in the Gaussian's own frame (Ra^T (mu_w - o))
+            const float wx = mw[0] - ox, wy = mw[1] - oy, wz = mw[2] - oz;
+            const float mx = actor ? Ra[0] * wx + Ra[3] * wy + Ra[6] * wz : wx;
+            const float my = actor ? Ra[1] * wx + Ra[4] * wy + Ra[7] * wz : wy;
+            const float mz = actor ? Ra[2] * wx + Ra[5] * wy + Ra[8] * wz : wz;
+            const float inv = 1.f / sqrtf(mx * mx + my * my + mz * mz);
+            const float dx = mx * inv, dy = my * inv, dz = mz * inv;
+            float Y[nc], h[nc], gdir[3];
+            sh_basis<(kDeg < 0 ? 0 : kDeg)>(dx, dy, dz, Y);
+#pragma unroll
+            for (int k = 0; k < nc; ++k) h[k] = 0.f;
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) {
+                float f[nc], acc = 0.f;
+#pragma unroll
+                for (int k = 0; k < nc; ++k) f[k] = planes[(Scene::kFeat + 3 * k + ch) * pitch + g];
+#pragma unroll
+                for (int k = 0; k < nc; ++k) acc += Y[k] * f[k];
+                const float gch = !lidar && acc + 0.5f < 0.f ? 0.f : gc[ch];   // clamped channel
+#pragma unroll
+                for (int k = 0; k < nc; ++k) {
+                    fo[3 * k + ch] = Y[k] * gch;
+                    h[k] += gch * f[k];
+                }
+            }
+            sh_basis_grad<(kDeg < 0 ? 0 : kDeg)>(dx, dy, dz, h, gdir);
+            const float dd = gdir[0] * dx + gdir[1] * dy + gdir[2] * dz;
+            gmu[0] += (gdir[0] - dx * dd) * inv;
+            gmu[1] += (gdir[1] - dy * dd) * inv;
+            gmu[2] += (gdir[2] - dz * dd) * inv;
+        }
+        po[0] = gmu[0]; po[1] = gmu[1]; po[2] = gmu[2];
     }
-    if (gm)
-        for (int k = 0; k < 3; ++k) gm[3 * g + k] += gmu[k];
+    __syncthreads();
+    add_rows<F>(gf, g0, ng, s_f, fs, s_any);
+    add_rows<3>(gm, g0, ng, s_p, 11, s_any);
+    add_rows<3>(gls, g0, ng, s_p + 3, 11, s_any);
+    add_rows<4>(gq, g0, ng, s_p + 6, 11, s_any);
+    add_rows<1>(gop, g0, ng, s_p + 10, 11, s_any);
 }
 
 static sg_status finish(const Scene &sc, Frame &fr, const float o[3], float beam,
                         const sg_grads &g, cudaStream_t st)
 {
     if (sc.n == 0) return SG_OK;
-    k_param_grads<<<(unsigned)((sc.n + 127) / 128), 128, 0, st>>>(
-        sc.d_planes, sc.pitch, sc.n, sc.feature_kind, sc.sh_degree, sc.F, o[0], o[1], o[2],
-        (const GRec *)fr.rec.p, fr.d_lidar_poses, actor_params(sc), beam, fr.kind == 2 ? 1 : 0,
-        (const float *)fr.gacc.p, g.d_g_means, g.d_g_log_scales, g.d_g_quats, g.d_g_opacity,
-        g.d_g_features);
+    auto kern = k_param_grads<-1>;
+    if (sh_features(sc.feature_kind))
+        kern = sc.sh_degree == 0 ? k_param_grads<0> : sc.sh_degree == 1 ? k_param_grads<1>
+               : sc.sh_degree == 2 ? k_param_grads<2> : k_param_grads<3>;
+    kern<<<(unsigned)((sc.n + kPgThreads - 1) / kPgThreads), kPgThreads, 0, st>>>(
+        sc.d_planes, sc.pitch, sc.n, sc.feature_kind == SG_FEATURES_LIDAR_SH ? 1 : 0, o[0], o[1],
+        o[2], (const GRec *)fr.rec.p, fr.d_lidar_poses, actor_params(sc), beam,
+        fr.kind == 2 ? 1 : 0, (float *)fr.gacc.p, g.d_g_means, g.d_g_log_scales, g.d_g_quats,
+        g.d_g_opacity, g.d_g_features);
     SG_LAUNCHED();
+    fr.gacc_clear = true;
+    return SG_OK;
+}
+
+// The accumulator, all zero: k_param_grads clears the rows it reads, so only
+// a new buffer, or one whose last backward did not get that far, is cleared here.
+static sg_status clear_sums(Frame &fr, int64_t n, cudaStream_t st)
+{
+    const void *had = fr.gacc.p;
+    const size_t bytes = fr.gacc.bytes;
+    sg_status s = ensure(fr.gacc, sizeof(float) * kG * (n > 0 ? n : 1));
+    if (s != SG_OK) return s;
+    if (fr.gacc.p != had || fr.gacc.bytes != bytes || !fr.gacc_clear)
+        SG_CUDA(cudaMemsetAsync(fr.gacc.p, 0, fr.gacc.bytes, st));
+    fr.gacc_clear = false;
     return SG_OK;
 }
 
@@ -782,13 +1026,13 @@ static int blocks_per_sm(const void *kern, int threads)
     return nb;
 }
 
-static sg_status persistent_grid(const void *kern, int64_t max_items, int64_t &grid)
+static sg_status persistent_grid(const void *kern, int warps, int64_t max_items, int64_t &grid)
 {
     int dev = 0, sms = 0;
     SG_CUDA(cudaGetDevice(&dev));
     SG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t cap = (max_items + kBwWarps - 1) / kBwWarps;
-    grid = (int64_t)sms * blocks_per_sm(kern, 32 * kBwWarps);
+    const int64_t cap = (max_items + warps - 1) / warps;
+    grid = (int64_t)sms * blocks_per_sm(kern, 32 * warps);
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
     return SG_OK;
@@ -802,9 +1046,8 @@ sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const f
         set_error("sg_backward_camera: the frame's render used another list segment length");
         return SG_ERR_INVALID;
     }
-    sg_status s = ensure(fr.gacc, sizeof(float) * kG * (sc.n > 0 ? sc.n : 1));
+    sg_status s = clear_sums(fr, sc.n, st);
     if (s != SG_OK) return s;
-    SG_CUDA(cudaMemsetAsync(fr.gacc.p, 0, sizeof(float) * kG * sc.n, st));
     const CamRender P = cam_render_params(cam, fr.opts);
     const int nt = cam.ntx * cam.nty;
     const WorkSize ws = work_size(nt, fr.n_pairs, kSegLen, 8);
@@ -813,9 +1056,10 @@ sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const f
     SG_CUDA(cudaMemsetAsync(counter, 0, sizeof(uint32_t), st));
     int64_t grid = 0;
     if (fr.kind == 2) {     // rolling shutter: poses per pixel row
-        if ((s = persistent_grid((const void *)k_backward_camera_rs, ws.max_items, grid)) != SG_OK)
+        if ((s = persistent_grid((const void *)k_backward_camera_rs, kBwWarpsPosed, ws.max_items,
+                                 grid)) != SG_OK)
             return s;
-        k_backward_camera_rs<<<(unsigned)grid, 32 * kBwWarps, 0, st>>>(
+        k_backward_camera_rs<<<(unsigned)grid, 32 * kBwWarpsPosed, 0, st>>>(
             P, (const GRec *)fr.rec.p, (const uint32_t *)fr.pvals[fr.pair_buf].p,
             (const uint2 *)fr.ranges.p, (const uint2 *)(cw + ws.info_bytes + ws.off_bytes),
             (const uint2 *)cw, (const uint32_t *)fr.scalars.p + 4, (const uint32_t *)fr.submask.p,
@@ -826,7 +1070,7 @@ sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const f
         const float o[3] = {0.f, 0.f, 0.f};
         return finish(sc, fr, o, 0.f, g, st);
     }
-    if ((s = persistent_grid((const void *)k_backward_camera, ws.max_items, grid)) != SG_OK)
+    if ((s = persistent_grid((const void *)k_backward_camera, kBwWarps, ws.max_items, grid)) != SG_OK)
         return s;
     k_backward_camera<<<(unsigned)grid, 32 * kBwWarps, 0, st>>>(
         P, (const GRec *)fr.rec.p, (const uint32_t *)fr.pvals[fr.pair_buf].p,
@@ -845,9 +1089,8 @@ sg_status backward_lidar(const Scene &sc, const Lidar &L, Frame &fr, const float
                          const float *g_int, const float *g_drop, const float *g_alpha,
                          const sg_grads &g, cudaStream_t st)
 {
-    sg_status s = ensure(fr.gacc, sizeof(float) * kG * (sc.n > 0 ? sc.n : 1));
+    sg_status s = clear_sums(fr, sc.n, st);
     if (s != SG_OK) return s;
-    SG_CUDA(cudaMemsetAsync(fr.gacc.p, 0, sizeof(float) * kG * sc.n, st));
     const LidRender P = lidar_render_params(L, fr.opts);
     if (L.n_items > 0) {
         const WorkSize ws = work_size(L.n_items, fr.n_pairs * L.max_items_per_tile, kSegLen, 1);
@@ -855,9 +1098,10 @@ sg_status backward_lidar(const Scene &sc, const Lidar &L, Frame &fr, const float
         uint32_t *counter = (uint32_t *)fr.scalars.p + 6;
         SG_CUDA(cudaMemsetAsync(counter, 0, sizeof(uint32_t), st));
         int64_t grid = 0;
-        if ((s = persistent_grid((const void *)k_backward_lidar, ws.max_items, grid)) != SG_OK)
+        if ((s = persistent_grid((const void *)k_backward_lidar, kBwWarpsPosed, ws.max_items, grid)) !=
+            SG_OK)
             return s;
-        k_backward_lidar<<<(unsigned)grid, 32 * kBwWarps, 0, st>>>(
+        k_backward_lidar<<<(unsigned)grid, 32 * kBwWarpsPosed, 0, st>>>(
             P, L.d_items, L.d_item_rays, L.d_ray_e, L.d_tile_u, fr.d_lidar_poses,
             L.d_tile_items, (const uint32_t *)fr.lmask.p, fr.lmask_stride,
             (const GRec *)fr.rec.p, (const uint32_t *)fr.pvals[fr.pair_buf].p,

@@ -218,9 +218,10 @@ struct Frame {
     // per-ray saved state: (T_final, omega, Z, LiDAR drop) and contributor count
     Buf ray_state, n_contrib;
     Buf ray_feat;     // per ray: the final feature sums (F0, F1, F2, 0), for the backward
-    // backward accumulators: per Gaussian dL/dM (9), dL/dmu (3), dL/dsigma,
-    // dL/dfeature (3)
+    // backward accumulators, 16 floats per Gaussian (backward.cu: add_sums);
+    // gacc_clear: every one is zero (what is queued included)
     Buf gacc;
+    bool gacc_clear = false;
     Buf scalars;      // device scalars: [0] valid Gaussians [1] pairs [2] work-item
                       // counter [3] pairs dropped over capacity [4..5] work-item counts
                       // [6] backward work counter [7] deferred re-walks

@@ -156,18 +156,21 @@ __device__ __forceinline__ float4 lid_u(float4 (*s)[32], int j, int sb)
     return lid_col(s, j, 3, (sb - 3) >> 2);
 }
 
-__device__ __forceinline__ void lidar_entry(const GRec &r, const float *poses, int col0,
-                                            int ncols, const float dh[3], const float dl[3],
-                                            float4 (*s)[32], int pos)
+// Column slots [sl0, sl1) of entry pos, and its planes if slot 0 is among them.
+__device__ __forceinline__ void lidar_entry_slots(const GRec &r, const float *poses, int col0,
+                                                  int sl0, int sl1, const float dh[3],
+                                                  const float dl[3], float4 (*s)[32], int pos)
 {
     const float mu[3] = {r.mu_sigma.x, r.mu_sigma.y, r.mu_sigma.z};
     const float M0[3] = {r.m0.x, r.m0.y, r.m0.z}, M1[3] = {r.m1.x, r.m1.y, r.m1.z},
                 M2[3] = {r.m2.x, r.m2.y, r.m2.z};
     const float f0 = r.m0.w, f1 = r.m1.w, f2 = r.m2.w;
-    s[0][pos] = make_float4(M0[0], M0[1], M0[2], r.mu_sigma.w);
-    s[1][pos] = make_float4(M1[0], M1[1], M1[2], r.feat.x);
-    s[2][pos] = make_float4(M2[0], M2[1], M2[2], r.feat.y);
-    for (int sl = 0; sl < ncols; ++sl) {
+    if (sl0 == 0) {
+        s[0][pos] = make_float4(M0[0], M0[1], M0[2], r.mu_sigma.w);
+        s[1][pos] = make_float4(M1[0], M1[1], M1[2], r.feat.x);
+        s[2][pos] = make_float4(M2[0], M2[1], M2[2], r.feat.y);
+    }
+    for (int sl = sl0; sl < sl1; ++sl) {
         const float *Po = poses + 12 * (col0 + sl);
         const float o[3] = {Po[3], Po[7], Po[11]};
         float w[3], vh[3];
@@ -183,6 +186,13 @@ __device__ __forceinline__ void lidar_entry(const GRec &r, const float *poses, i
                                              f2 * (M2[0] * vh[1] - M2[1] * vh[0]), f2 * dot3(M2, w));
         lid_col(s, pos, 3, sl) = make_float4(dot3(M0, vh), dot3(M1, vh), dot3(M2, vh), r.feat.z);
     }
+}
+
+__device__ __forceinline__ void lidar_entry(const GRec &r, const float *poses, int col0,
+                                            int ncols, const float dh[3], const float dl[3],
+                                            float4 (*s)[32], int pos)
+{
+    lidar_entry_slots(r, poses, col0, 0, ncols, dh, dl, s, pos);
 }
 
 // Evaluate one LiDAR pair (entry j of the warp's block, planes of its
