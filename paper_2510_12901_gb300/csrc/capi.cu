@@ -251,6 +251,7 @@ static sg_status frame_prepare(Frame &fr, int64_t n, int64_t nrays, int64_t ntil
     }
     SG_ENS(fr.offsets, sizeof(uint32_t) * (n > 0 ? n : 1));
     SG_ENS(fr.owner, sizeof(uint32_t) * bin_owner_words(n));
+    SG_ENS(fr.hist, sizeof(uint32_t) * depth_stage_words(n));
     SG_ENS(fr.ranges, sizeof(uint2) * (ntiles > 0 ? ntiles : 1));
     SG_ENS(fr.ray_state, sizeof(float4) * (nrays > 0 ? nrays : 1));
     SG_ENS(fr.ray_feat, sizeof(float4) * (nrays > 0 ? nrays : 1));
@@ -361,13 +362,14 @@ static sg_status bin_and_sort(Frame &fr, int64_t n, int ntx, int64_t ntiles, int
     while (((int64_t)1 << bits) < ntiles) ++bits;
     // binning counts the tile sort's digits as it writes the pairs
     uint32_t *hist = nullptr;
-    if (K > 0 && (s = radix_prepare(K, (bits + 7) / 8, fr, st, &hist, 0)) != SG_OK) return s;
-    const uint32_t *err = sc + kScalStatus;
+    if (K > 0 && (s = tile_scratch(K, (bits + 7) / 8, fr, st, &hist)) != SG_OK) return s;
+    uint32_t *err = sc + kScalStatus;
     s = bin_pairs((const uint32_t *)fr.dvals[fr.depth_buf].p, (const uint32_t *)fr.offsets.p, sc,
-                  (const int4 *)fr.tiles.p, ntx, wrap, K, pk[0], pv[0], st, err, fr.owner, hist, bits);
+                  (const int4 *)fr.tiles.p, ntx, wrap, K, pk[0], pv[0], st, err, fr.owner,
+                  (uint2 *)fr.ranges.p, ntiles, hist, bits);
     if (s != SG_OK) return s;
     int pb = 0;
-    s = radix_sort_pairs(pk, pv, K, sc + 1, 0, bits, fr, st, &pb, SG_LOOKBACK_TILE_SORT);
+    s = radix_sort_pairs(pk, pv, K, sc + 1, 0, bits, hist, err, st, &pb, SG_LOOKBACK_TILE_SORT);
     if (s != SG_OK) return s;
     fr.pair_buf = pb;
     if (fr.kind == 1) {   // LiDAR lists also get their per-item ray masks
@@ -377,11 +379,11 @@ static sg_status bin_and_sort(Frame &fr, int64_t n, int ntx, int64_t ntiles, int
         const size_t by =
             sizeof(uint32_t) * (size_t)(K > 0 ? fr.lmask_stride : 1) * L.max_items_per_tile;
         if ((s = ensure(fr.lmask, by)) != SG_OK) return s;
-        s = lidar_tile_ranges(pk[pb], sc + 1, K, (uint2 *)fr.ranges.p, ntiles, st, err, pv[pb],
+        s = lidar_tile_ranges(pk[pb], sc + 1, K, (uint2 *)fr.ranges.p, st, err, pv[pb],
                               (const float4 *)fr.rect.p, L, (uint32_t *)fr.lmask.p, fr.lmask_stride);
     } else {   // camera lists also get their column/row words
         if ((s = ensure(fr.submask, 4 * (size_t)(K > 0 ? K : 1))) != SG_OK) return s;
-        s = tile_ranges(pk[pb], sc + 1, K, (uint2 *)fr.ranges.p, ntiles, st, err, pv[pb],
+        s = tile_ranges(pk[pb], sc + 1, K, (uint2 *)fr.ranges.p, st, err, pv[pb],
                         (const float4 *)fr.rect.p, ntx, (uint32_t *)fr.submask.p);
     }
     if (s != SG_OK) return s;
@@ -1088,9 +1090,8 @@ sg_status sg_workspace_bytes(sg_scene scene, int sensor_kind, int64_t n_rays, si
     b += grown(8 * (size_t)units) + grown(4 * (size_t)units);
     // pairs: keys and ids (x2), camera column/row masks or LiDAR ray masks
     b += 4 * grown(4 * (size_t)K) + grown(4 * (size_t)K * per_tile);
-    // sort scratch: the larger of the depth stage's and the tile sort's
-    const int64_t hd = depth_stage_words(n), ht = radix_scratch_words(K, 3);
-    b += grown(4 * (size_t)(hd > ht ? hd : ht));
+    // sort scratch: the depth stage's and the tile sort's
+    b += grown(4 * (size_t)depth_stage_words(n)) + grown(4 * (size_t)radix_scratch_words(K, 3));
     const WorkSize ws = work_size(units, K * per_tile, kSegLen, cam ? 8 : 1);
     b += grown(ws.work_bytes) + grown(ws.partial_bytes);
     b += grown(64) + grown(sizeof(RenderDesc));   // scalars, descriptor

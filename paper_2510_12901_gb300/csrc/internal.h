@@ -208,6 +208,8 @@ struct Frame {
     // depth sort / offsets
     Buf dkeys[2], dvals[2], offsets, hist;
     Buf owner;        // owner of the first pair of each binning block
+    Buf tscratch;     // tile sort's scratch; the compaction zeroed its first tscratch_zeroed bytes
+    size_t tscratch_zeroed = 0;
     // pairs; LiDAR: per (work item of the pair's tile, pair) the 32-bit mask
     // of the item's rays inside the Gaussian's box, planes of lmask_stride
     Buf pkeys[2], pvals[2], ranges, order, submask, lmask;
@@ -346,41 +348,45 @@ constexpr int64_t radix_scratch_words(int64_t n_max, int passes)
 constexpr int kChainTile = 2048;
 constexpr int64_t depth_stage_words(int64_t n)
 {
-    return radix_scratch_words(n, 4) + 2 * (2 + 2 * ((n + kChainTile - 1) / kChainTile));
+    const int64_t w = radix_scratch_words(n, 4) + 2 * (2 + 2 * ((n + kChainTile - 1) / kChainTile));
+    return (w + 3) / 4 * 4;      // zeroed 16 bytes at a time
 }
 // Pairs per binning block, and the entries of the table of their first
 // pairs' owners (blocks beyond it search the offsets): 32 pairs a Gaussian
 // and two million more.
 constexpr int kBinChunk = 2048;
 constexpr int64_t bin_owner_words(int64_t n) { return n / 64 + 1024; }
-sg_status radix_prepare(int64_t n_max, int passes, Frame &fr, cudaStream_t st, uint32_t **hist,
-                        int64_t extra);
+// The tile sort's scratch for up to n_max pairs in `passes` passes, all zero
+// (the compaction of this render zeroed it if it was large enough then).
+sg_status tile_scratch(int64_t n_max, int passes, Frame &fr, cudaStream_t st, uint32_t **hist);
 // Stable sort of up to n pairs (*d_n of them) by key bits [begin_bit,
-// end_bit); the digit counts are in the scratch that radix_prepare returned.
-// site: SG_LOOKBACK_DEPTH_SORT or SG_LOOKBACK_TILE_SORT (the test hook's site).
-// keep_keys = false: only the values are needed (keys[*result_buf] is stale).
-sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n,
-                           const uint32_t *d_n, int begin_bit, int end_bit, Frame &fr,
+// end_bit); scratch: radix_scratch_words(n, passes) words, zero but for the
+// digit counts at its start.  site: SG_LOOKBACK_DEPTH_SORT or
+// SG_LOOKBACK_TILE_SORT (the test hook's site).  keep_keys = false: only the
+// values are needed (keys[*result_buf] is stale).
+sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n, const uint32_t *d_n,
+                           int begin_bit, int end_bit, uint32_t *scratch, uint32_t *d_err,
                            cudaStream_t st, int *result_buf, int site, bool keep_keys = true);
 // The depth stage: the Gaussians with a non-zero tile count sorted by depth
 // (keys/vals[*result_buf]: depth bits, ids), d_scal[0] = their number,
 // d_offsets = exclusive scan of their tile counts in that order, d_scal[1]
-// = the pair total.
+// = the pair total.  Its scratch (fr.hist) was zeroed by the projection.
 sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, uint32_t *keys[2],
                       uint32_t *vals[2], uint32_t *d_scal, uint32_t *d_offsets, Frame &fr,
                       cudaStream_t st, int *result_buf);
-// With d_hist (zeroed by radix_prepare), k_bin also counts the digits of
-// the tile sort over end_bit bits, for radix_sort_pairs.  d_err: the frame's
-// status word (nothing is written once it is set).
+// With d_hist (in the tile sort's zeroed scratch), k_bin also counts the
+// digits of the tile sort over end_bit bits, for radix_sort_pairs.  d_err: the
+// frame's status word (no pair is written once it is set).  It also empties
+// the ntiles ranges that the tile ranges are written to.
 sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint32_t *d_nvalid,
                     const int4 *d_tiles, int ntx, int wrap_x, int64_t cap, uint32_t *d_keys,
                     uint32_t *d_vals, cudaStream_t st, const uint32_t *d_err, const Buf &owner,
-                    uint32_t *d_hist = nullptr, int end_bit = 0);
+                    uint2 *d_ranges, int64_t ntiles, uint32_t *d_hist = nullptr, int end_bit = 0);
 // Per-tile ranges of the sorted pairs; with d_mask (camera lists), also the
 // per-pair sub-block masks (d_ids, d_rects, ntx: the pairs' Gaussians, the
 // per-Gaussian extent boxes, tiles per row).
 sg_status tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max, uint2 *d_ranges,
-                      int64_t ntiles, cudaStream_t st, const uint32_t *d_err,
+                      cudaStream_t st, const uint32_t *d_err,
                       const uint32_t *d_ids = nullptr, const float4 *d_rects = nullptr,
                       int ntx = 0, uint32_t *d_words = nullptr);
 // LiDAR lists: ranges, and for every pair and every work item of its tile
@@ -388,9 +394,9 @@ sg_status tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max
 // for the k-th item of the tile, by the compositing's own float test; stride
 // a multiple of 4).
 sg_status lidar_tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max,
-                            uint2 *d_ranges, int64_t ntiles, cudaStream_t st,
-                            const uint32_t *d_err, const uint32_t *d_ids,
-                            const float4 *d_rects, const Lidar &L, uint32_t *d_lmask,
+                            uint2 *d_ranges, cudaStream_t st, const uint32_t *d_err,
+                            const uint32_t *d_ids, const float4 *d_rects, const Lidar &L,
+                            uint32_t *d_lmask,
                             int64_t lmask_stride);
 sg_status clamp_pairs(uint32_t *d_K, int64_t cap, uint32_t *d_dropped, cudaStream_t st);
 
@@ -410,10 +416,10 @@ sg_status render_camera(const Camera &cam, const sg_render_opts &o, Frame &fr, c
 bool camera_forward_only(const Camera &cam, const Frame &fr);
 sg_status render_camera_fwd(const Camera &cam, const sg_render_opts &o, Frame &fr,
                             cudaStream_t st);
-// render.cu: the compositing's work items (k_work_count, k_work_emit) of
-// n_units units with `subs` sub-units each, in the camwork layout of ws.
-
-sg_status launch_work_items(Frame &fr, const WorkSize &ws, const LidarItem *unit_tile,
+// render.cu: the compositing's work items in the camwork layout of ws, for
+// the n_units units of n_tiles tiles (lidar: its work items; NULL: a camera,
+// whose units are its tiles) with `subs` sub-units each.
+sg_status launch_work_items(Frame &fr, const WorkSize &ws, const Lidar *lidar, int n_tiles,
                             int n_units, int subs, uint32_t seg_len, cudaStream_t st);
 // rolling shutter: the RenderDesc's poses are per pixel row
 sg_status render_camera_rs(const Camera &cam, const sg_render_opts &o, Frame &fr,
@@ -447,7 +453,7 @@ namespace sg {
 template <class Fn> inline void for_each_buf(Frame &f, Fn fn)
 {
     Buf *bufs[] = {&f.rec, &f.rect, &f.tiles, &f.depth, &f.count, &f.mean2d, &f.cov2d,
-                   &f.dkeys[0], &f.dkeys[1], &f.dvals[0], &f.dvals[1], &f.offsets, &f.hist, &f.owner,
+                   &f.dkeys[0], &f.dkeys[1], &f.dvals[0], &f.dvals[1], &f.offsets, &f.hist, &f.owner, &f.tscratch,
                    &f.pkeys[0], &f.pkeys[1], &f.pvals[0], &f.pvals[1], &f.ranges, &f.order, &f.submask,
                    &f.lmask, &f.camwork,
                    &f.partials, &f.ray_state, &f.n_contrib, &f.ray_feat, &f.gacc, &f.scalars,

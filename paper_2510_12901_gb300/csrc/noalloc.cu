@@ -27,9 +27,8 @@ constexpr size_t kStG16 = al(16 * kStMaxGauss);       // float4 / int4 per Gauss
 constexpr size_t kStG8 = al(8 * kStMaxGauss);
 constexpr size_t kStG4 = al(4 * kStMaxGauss);
 constexpr size_t kStP4 = al(4 * kStMaxPairs);
-constexpr size_t kStHist = al(4 * (radix_scratch_words(kStMaxPairs, 4) > depth_stage_words(kStMaxGauss)
-                                       ? radix_scratch_words(kStMaxPairs, 4)
-                                       : depth_stage_words(kStMaxGauss)));
+constexpr size_t kStHist = al(4 * depth_stage_words(kStMaxGauss));
+constexpr size_t kStTile = al(4 * radix_scratch_words(kStMaxPairs, 4));
 constexpr WorkSize kStWork = work_size(kStMaxTiles, kStMaxPairs, kSegLenStatic, 8);
 constexpr size_t kStBytes = kStRec + 3 * kStG16 + kStG8 +       // rec, rect, tiles, cov2d, mean2d
                             2 * kStG4 +                          // depth, count
@@ -37,7 +36,7 @@ constexpr size_t kStBytes = kStRec + 3 * kStG16 + kStG8 +       // rec, rect, ti
                             kStG4 +                              // offsets
                             al(4 * bin_owner_words(kStMaxGauss)) + // binning blocks' owners
                             4 * kStP4 +                          // pair keys/values x2
-                            kStHist +
+                            kStHist + kStTile +                  // sort scratch
                             al(8 * kStMaxTiles) + al(4 * kStMaxTiles) +  // ranges, order
                             2 * al(16 * kStMaxRays) + al(4 * kStMaxRays) + // ray state, features,
                                                                          // contributors
@@ -142,6 +141,7 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
         carve(fr.pvals[i], cur, kStP4);
     }
     carve(fr.hist, cur, kStHist);
+    carve(fr.tscratch, cur, kStTile);
     carve(fr.ranges, cur, al(8 * kStMaxTiles));
     carve(fr.order, cur, al(4 * kStMaxTiles));
     carve(fr.ray_state, cur, al(16 * kStMaxRays));
@@ -201,18 +201,18 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
     int bits = 1;
     while (((int64_t)1 << bits) < nt) ++bits;
     uint32_t *hist = nullptr;
-    if (K > 0 && (s = radix_prepare(K, (bits + 7) / 8, fr, st, &hist, 0)) != SG_OK) return s;
-    const uint32_t *err = scal + kScalStatus;
+    if (K > 0 && (s = tile_scratch(K, (bits + 7) / 8, fr, st, &hist)) != SG_OK) return s;
+    uint32_t *err = scal + kScalStatus;
     if ((s = bin_pairs(dv[rb], (const uint32_t *)fr.offsets.p, scal, (const int4 *)fr.tiles.p,
-                       c.ntx, 0, K, pk[0], pv[0], st, err, fr.owner, hist, bits)) !=
-        SG_OK)
+                       c.ntx, 0, K, pk[0], pv[0], st, err, fr.owner, (uint2 *)fr.ranges.p, nt, hist,
+                       bits)) != SG_OK)
         return s;
     int pb = 0;
-    if ((s = radix_sort_pairs(pk, pv, K, scal + 1, 0, bits, fr, st, &pb,
+    if ((s = radix_sort_pairs(pk, pv, K, scal + 1, 0, bits, hist, err, st, &pb,
                               SG_LOOKBACK_TILE_SORT)) != SG_OK)
         return s;
     fr.pair_buf = pb;
-    if ((s = tile_ranges(pk[pb], scal + 1, K, (uint2 *)fr.ranges.p, nt, st, err, pv[pb],
+    if ((s = tile_ranges(pk[pb], scal + 1, K, (uint2 *)fr.ranges.p, st, err, pv[pb],
                          (const float4 *)fr.rect.p, c.ntx, (uint32_t *)fr.submask.p)) != SG_OK)
         return s;
     return render_camera(c, *opts, fr, st);

@@ -40,6 +40,15 @@ static UTParams ut_params(const sg_render_opts &o)
     return u;
 }
 
+// Zero the depth stage's scratch, which the kernels after the projection fill
+// (a launch of its own for these few bytes costs as much as a small sort pass).
+__device__ __forceinline__ void zero_scratch(uint4 *__restrict__ z, int64_t n)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        z[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 struct Activated {
     float mu[3], R[9], s[3], sigma;
 };
@@ -257,8 +266,9 @@ k_project_camera(const float *__restrict__ planes, int64_t pitch, int64_t n, int
                  float4 *__restrict__ rect_out, int4 *__restrict__ tiles_out,
                  float *__restrict__ depth_out, uint32_t *__restrict__ count_out,
                  float2 *__restrict__ mean_out, float4 *__restrict__ cov_out,
-                 uint32_t *__restrict__ status)
+                 uint32_t *__restrict__ status, uint4 *__restrict__ zero, int64_t nzero)
 {
+    zero_scratch(zero, nzero);
     __shared__ float s_c2w[12];   // the pose, from the render's descriptor
     // SH features: the block's run of every coefficient plane, [plane][thread],
     // brought in by bulk copies (TMA) while the sigma points are projected
@@ -402,7 +412,8 @@ sg_status project_camera(const Scene &sc, const Camera &cam, const sg_render_opt
         sc.d_planes, sc.pitch, sc.n, sc.feature_kind, sc.sh_degree, actor_params(sc), C,
         (const RenderDesc *)fr.desc.p, U, (GRec *)fr.rec.p,
         (float4 *)fr.rect.p, (int4 *)fr.tiles.p, (float *)fr.depth.p, (uint32_t *)fr.count.p,
-        (float2 *)fr.mean2d.p, (float4 *)fr.cov2d.p, (uint32_t *)fr.scalars.p + kScalStatus);
+        (float2 *)fr.mean2d.p, (float4 *)fr.cov2d.p, (uint32_t *)fr.scalars.p + kScalStatus,
+        (uint4 *)fr.hist.p, depth_stage_words(sc.n) / 4);
     SG_LAUNCHED();
     return SG_OK;
 }
@@ -590,8 +601,10 @@ k_project_lidar(const float *__restrict__ planes, int64_t pitch, int64_t n, int 
                 int cull, GRec *__restrict__ rec, float4 *__restrict__ rect_out,
                 int4 *__restrict__ tiles_out, float *__restrict__ depth_out,
                 uint32_t *__restrict__ count_out, float2 *__restrict__ mean_out,
-                float4 *__restrict__ cov_out, uint32_t *__restrict__ status)
+                float4 *__restrict__ cov_out, uint32_t *__restrict__ status,
+                uint4 *__restrict__ zero, int64_t nzero)
 {
+    zero_scratch(zero, nzero);
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g == 0) *status = 0u;     // a new render: no look-back wait has given up
     if (g >= n) return;
@@ -752,7 +765,8 @@ sg_status project_lidar(const Scene &sc, const Lidar &Ld, const sg_render_opts &
         (const RenderDesc *)fr.desc.p, U, o.cull,
         (GRec *)fr.rec.p, (float4 *)fr.rect.p,
         (int4 *)fr.tiles.p, (float *)fr.depth.p, (uint32_t *)fr.count.p, (float2 *)fr.mean2d.p,
-        (float4 *)fr.cov2d.p, (uint32_t *)fr.scalars.p + kScalStatus);
+        (float4 *)fr.cov2d.p, (uint32_t *)fr.scalars.p + kScalStatus, (uint4 *)fr.hist.p,
+        depth_stage_words(sc.n) / 4);
     SG_LAUNCHED();
     return SG_OK;
 }

@@ -167,9 +167,121 @@ k_work_emit(const uint2 *__restrict__ ranges, const LidarItem *__restrict__ unit
     if (nseg > 1 && lane < subs) arrive[pb * subs + lane] = 0u;
 }
 
-// Launch both: the work items of `n_units` units into the frame's camwork
-// buffer laid out by ws (its unit-offset region holds the scratch words).
-sg_status launch_work_items(Frame &fr, const WorkSize &ws, const LidarItem *unit_tile,
+// The same in one launch, for up to kWorkOneTiles tiles: a block takes
+// kWorkShare tiles, reads every tile's list length itself (80 KB from L2 at
+// 10000 tiles), sums the items of all buckets and of its predecessors' shares,
+// and so knows the first item of its share of each bucket and its first
+// partial slot without waiting for another block.  Shares are small so that
+// writing the items, about 60 instructions a tile, is spread over the chip.
+// One launch for a memset and two kernels: at 9600 tiles 15 us for 17 and two
+// launches more, at 16 tiles 6 us for 8 (shares of 1024 tiles: 23 and 10).
+// Beyond kWorkOneTiles the lengths no longer fit a block's registers, and the
+// two grid-wide kernels take over.
+constexpr int kWorkThreads = 1024, kWorkChunks = 12;
+constexpr int kWorkOneTiles = kWorkThreads * kWorkChunks;
+constexpr int kWorkShare = 256, kWorkPerWarp = kWorkShare / (kWorkThreads / 32);
+
+__global__ void __launch_bounds__(kWorkThreads)
+k_work_items(const uint2 *__restrict__ ranges, const uint2 *__restrict__ tile_items, int n_tiles,
+             int subs, uint32_t seg_len, uint32_t *__restrict__ counts,
+             uint32_t *__restrict__ counter, uint2 *__restrict__ unit_info,
+             uint2 *__restrict__ items, uint32_t *__restrict__ arrive)
+{
+    // items per bucket: of all tiles, of the earlier blocks' tiles, handed out
+    // by this block; the buckets' first items; partial slots likewise
+    __shared__ uint32_t s_tot[34], s_pre[34], s_cur[34], s_base[34];
+    constexpr int kSlots = 33;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t < 34) s_tot[t] = s_pre[t] = s_cur[t] = 0u;
+    uint32_t len[kWorkChunks], mult[kWorkChunks];
+#pragma unroll
+    for (int c = 0; c < kWorkChunks; ++c) {
+        const int i = c * kWorkThreads + t;
+        const uint2 r = i < n_tiles ? ranges[i] : make_uint2(0u, 0u);
+        len[c] = r.y - r.x;
+        mult[c] = i < n_tiles ? (tile_items ? tile_items[i].y : 1u) : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kWorkChunks; ++c) {
+        if (c * kWorkThreads >= n_tiles) break;
+        const uint32_t nseg = unit_segments(len[c], seg_len), n = mult[c] * (uint32_t)subs * nseg;
+        const uint32_t b = len_bucket(len[c]);
+        const uint32_t slots = nseg > 1 ? mult[c] * nseg : 0u;
+        const uint32_t peers = __match_any_sync(0xffffffffu, b);
+        const uint32_t sum = __reduce_add_sync(peers, n);
+        const uint32_t ssum = __reduce_add_sync(0xffffffffu, slots);
+        const bool mine = c * kWorkThreads + 32 * warp < (int)blockIdx.x * kWorkShare;
+        if (lane == __ffs(peers) - 1 && sum) {
+            atomicAdd(&s_tot[b], sum);
+            if (mine) atomicAdd(&s_pre[b], sum);
+        }
+        if (lane == 0 && ssum) {
+            atomicAdd(&s_tot[kSlots], ssum);
+            if (mine) atomicAdd(&s_pre[kSlots], ssum);
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {        // the buckets' first items: longest lists first
+        uint32_t inc = s_tot[lane];
+        const uint32_t v = inc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += x;
+        }
+        s_base[lane] = inc - v;
+        if (lane == 31) {
+            s_base[32] = inc;
+            if (blockIdx.x == 0) {
+                counts[0] = inc + s_tot[32];
+                counts[1] = s_tot[kSlots];
+                counts[3] = 0u;      // deferred re-walks
+                *counter = 0u;
+            }
+        }
+    }
+    __syncthreads();
+    // this block's tiles: kWorkPerWarp lanes a warp take their tiles' runs, the
+    // warp writes them
+    const int tile = (int)blockIdx.x * kWorkShare + warp * kWorkPerWarp + lane;
+    uint32_t mylen = 0u, mymult = 0u, first = (uint32_t)tile;
+    if (lane < kWorkPerWarp && tile < n_tiles) {
+        const uint2 r = ranges[tile];
+        mylen = r.y - r.x;
+        mymult = 1u;
+        if (tile_items) {
+            const uint2 ti = tile_items[tile];
+            first = ti.x;
+            mymult = ti.y;
+        }
+    }
+    const uint32_t nseg = unit_segments(mylen, seg_len), per = (uint32_t)subs * nseg;
+    uint32_t ib = 0u, pb = 0u;
+    if (mymult) {
+        const uint32_t b = len_bucket(mylen);
+        ib = s_base[b] + s_pre[b] + atomicAdd(&s_cur[b], mymult * per);
+        if (nseg > 1) pb = s_pre[kSlots] + atomicAdd(&s_cur[kSlots], mymult * nseg);
+        for (uint32_t k = 0; k < mymult; ++k) unit_info[first + k] = make_uint2(nseg, pb + k * nseg);
+    }
+    for (uint32_t rest = __ballot_sync(0xffffffffu, mymult != 0u); rest; rest &= rest - 1u) {
+        const int l = __ffs(rest) - 1;
+        const uint32_t lm = __shfl_sync(0xffffffffu, mymult, l), lp = __shfl_sync(0xffffffffu, per, l);
+        const uint32_t li = __shfl_sync(0xffffffffu, ib, l), lf = __shfl_sync(0xffffffffu, first, l);
+        const uint32_t ls = __shfl_sync(0xffffffffu, nseg, l), lb = __shfl_sync(0xffffffffu, pb, l);
+        for (uint32_t i = lane; i < lm * lp; i += 32) {
+            const uint32_t k = lm == 1u ? 0u : i / lp;
+            items[li + i] = make_uint2(lf + k, i - k * lp);
+        }
+        if (ls > 1)
+            for (uint32_t i = lane; i < lm * (uint32_t)subs; i += 32)
+                arrive[(lb + (i / subs) * ls) * subs + i % subs] = 0u;
+    }
+}
+
+// The work items into the frame's camwork buffer laid out by ws (its
+// unit-offset region holds the two-kernel form's scratch words).
+sg_status launch_work_items(Frame &fr, const WorkSize &ws, const Lidar *lidar, int n_tiles,
                             int n_units, int subs, uint32_t seg_len, cudaStream_t st)
 {
     unsigned char *cw = (unsigned char *)fr.camwork.p;
@@ -177,21 +289,29 @@ sg_status launch_work_items(Frame &fr, const WorkSize &ws, const LidarItem *unit
     uint32_t *scratch = (uint32_t *)(cw + ws.info_bytes);
     uint2 *items = (uint2 *)(cw + ws.info_bytes + ws.off_bytes);
     uint32_t *arrive = (uint32_t *)(cw + ws.info_bytes + ws.off_bytes + ws.items_bytes);
+    uint32_t *counts = (uint32_t *)fr.scalars.p + 4, *counter = (uint32_t *)fr.scalars.p + 2;
+    const uint2 *ranges = (const uint2 *)fr.ranges.p;
+    if (n_tiles <= kWorkOneTiles) {
+        const unsigned g = (unsigned)((n_tiles + kWorkShare - 1) / kWorkShare);
+        k_work_items<<<g > 0 ? g : 1, kWorkThreads, 0, st>>>(
+            ranges, lidar ? lidar->d_tile_items : nullptr, n_tiles, subs, seg_len, counts, counter,
+            unit_info, items, arrive);
+        SG_LAUNCHED();
+        return SG_OK;
+    }
+    const LidarItem *unit_tile = lidar ? lidar->d_items : nullptr;
     if (ws.off_bytes < sizeof(uint32_t) * kWsWords) {
         set_error("internal: work-item scratch too small");
         return SG_ERR_INVALID;
     }
     SG_CUDA(cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * kWsWords, st));
     const unsigned g1 = (unsigned)((n_units + 255) / 256);
-    k_work_count<<<g1 > 0 ? g1 : 1, 256, 0, st>>>((const uint2 *)fr.ranges.p, unit_tile, n_units,
-                                                  subs, seg_len, scratch,
-                                                  (uint32_t *)fr.scalars.p + 4,
-                                                  (uint32_t *)fr.scalars.p + 2);
+    k_work_count<<<g1 > 0 ? g1 : 1, 256, 0, st>>>(ranges, unit_tile, n_units, subs, seg_len, scratch,
+                                                  counts, counter);
     SG_LAUNCHED();
     if (n_units > 0) {
         k_work_emit<<<(unsigned)((n_units + 7) / 8), 256, 0, st>>>(
-            (const uint2 *)fr.ranges.p, unit_tile, n_units, subs, seg_len, scratch, unit_info,
-            items, arrive);
+            ranges, unit_tile, n_units, subs, seg_len, scratch, unit_info, items, arrive);
         SG_LAUNCHED();
     }
     return SG_OK;
@@ -478,7 +598,7 @@ sg_status render_camera(const Camera &cam, const sg_render_opts &o, Frame &fr, c
     uint32_t *arrive = (uint32_t *)(cw + ws.info_bytes + ws.off_bytes + ws.items_bytes);
     const uint32_t *counts = (const uint32_t *)fr.scalars.p + 4;    // [0] items [1] slots
     uint32_t *counter = (uint32_t *)fr.scalars.p + 2;
-    if ((s = launch_work_items(fr, ws, nullptr, nt, 8, fr.seg_len, st)) != SG_OK) return s;
+    if ((s = launch_work_items(fr, ws, nullptr, nt, nt, 8, fr.seg_len, st)) != SG_OK) return s;
     const uint32_t *ids = (const uint32_t *)fr.pvals[fr.pair_buf].p;
     int dev = 0, sms = 0;
     SG_CUDA(cudaGetDevice(&dev));
@@ -716,7 +836,7 @@ sg_status render_camera_rs(const Camera &cam, const sg_render_opts &o, Frame &fr
     uint32_t *arrive = (uint32_t *)(cw + ws.info_bytes + ws.off_bytes + ws.items_bytes);
     const uint32_t *counts = (const uint32_t *)fr.scalars.p + 4;
     uint32_t *counter = (uint32_t *)fr.scalars.p + 2;
-    if ((s = launch_work_items(fr, ws, nullptr, nt, 8, fr.seg_len, st)) != SG_OK) return s;
+    if ((s = launch_work_items(fr, ws, nullptr, nt, nt, 8, fr.seg_len, st)) != SG_OK) return s;
     const uint32_t *ids = (const uint32_t *)fr.pvals[fr.pair_buf].p;
     int dev = 0, sms = 0, nb = 0;
     SG_CUDA(cudaGetDevice(&dev));
@@ -1005,7 +1125,7 @@ sg_status render_lidar(const Lidar &L, const sg_render_opts &o, Frame &fr, cudaS
     if (s == SG_OK) s = ensure(fr.camwork, ws.work_bytes);
     if (s == SG_OK) s = ensure(fr.partials, ws.partial_bytes);
     if (s != SG_OK) return s;
-    if ((s = launch_work_items(fr, ws, L.d_items, L.n_items, 1, kSegLen, st)) != SG_OK) return s;
+    if ((s = launch_work_items(fr, ws, &L, L.n_theta * L.nphi, L.n_items, 1, kSegLen, st)) != SG_OK) return s;
     unsigned char *cw = (unsigned char *)fr.camwork.p;
     const uint2 *unit_info = (const uint2 *)cw;
     const uint2 *work = (const uint2 *)(cw + ws.info_bytes + ws.off_bytes);

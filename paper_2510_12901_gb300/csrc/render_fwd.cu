@@ -516,7 +516,7 @@ sg_status render_camera_fwd(const Camera &cam, const sg_render_opts &o, Frame &f
     uint32_t *arrive = (uint32_t *)(cw + ws.info_bytes + ws.off_bytes + ws.items_bytes);
     const uint32_t *counts = (const uint32_t *)fr.scalars.p + 4;    // [0] items [1] slots
     uint32_t *counter = (uint32_t *)fr.scalars.p + 2;
-    if ((s = launch_work_items(fr, ws, nullptr, nt, 8, kFwdSeg, st)) != SG_OK) return s;
+    if ((s = launch_work_items(fr, ws, nullptr, nt, nt, 8, kFwdSeg, st)) != SG_OK) return s;
     const uint32_t *ids = (const uint32_t *)fr.pvals[fr.pair_buf].p;
     int dev = 0, sms = 0;
     SG_CUDA(cudaGetDevice(&dev));

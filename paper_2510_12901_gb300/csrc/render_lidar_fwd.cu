@@ -406,7 +406,8 @@ sg_status render_lidar_fwd(const Lidar &L, const sg_render_opts &o, Frame &fr, c
     if (s == SG_OK) s = ensure(fr.camwork, ws.work_bytes);
     if (s == SG_OK) s = ensure(fr.partials, ws.partial_bytes);
     if (s != SG_OK) return s;
-    if ((s = launch_work_items(fr, ws, L.d_items, L.n_items, 1, kLfSeg, st)) != SG_OK) return s;
+    if ((s = launch_work_items(fr, ws, &L, L.n_theta * L.nphi, L.n_items, 1, kLfSeg, st)) != SG_OK)
+        return s;
     unsigned char *cw = (unsigned char *)fr.camwork.p;
     const uint2 *unit_info = (const uint2 *)cw;
     const uint2 *work = (const uint2 *)(cw + ws.info_bytes + ws.off_bytes);

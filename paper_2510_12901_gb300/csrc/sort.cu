@@ -49,7 +49,7 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid)
 // Stable LSD radix sort of (key, value) pairs, digits of at most 8 bits, one
 // kernel per digit pass with decoupled look-back (the "onesweep" scheme):
 //   1. the kernel that writes the keys counts the digits of every pass
-//      (k_compact_depth, k_bin) into scratch that radix_prepare zeroed;
+//      (k_compact_depth, k_bin) into scratch zeroed before;
 //   2. per pass, the exclusive scan of its digit counts gives the first
 //      output position of each digit (every block of the pass scans them);
 //   3. k_onesweep, per pass: a block takes the next tile of kRadixTile pairs
@@ -302,24 +302,23 @@ k_onesweep(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ va
     }
 }
 
-// Zero the radix scratch (histograms, tickets, look-back words) for a sort
-// of up to n_max pairs in `passes` passes; *hist gets the histograms, which
-// the kernel that writes the keys fills before radix_sort_pairs runs.
-// `extra` more zeroed words follow the scratch (at hist + radix_scratch_words).
-sg_status radix_prepare(int64_t n_max, int passes, Frame &fr, cudaStream_t st, uint32_t **hist,
-                        int64_t extra)
+sg_status tile_scratch(int64_t n_max, int passes, Frame &fr, cudaStream_t st, uint32_t **hist)
 {
-    const int64_t words = radix_scratch_words(n_max, passes) + extra;
-    sg_status s = ensure(fr.hist, sizeof(uint32_t) * words);
+    const void *had = fr.tscratch.p;
+    const size_t bytes = sizeof(uint32_t) * (size_t)radix_scratch_words(n_max, passes);
+    sg_status s = ensure(fr.tscratch, bytes);
     if (s != SG_OK) return s;
-    SG_CUDA(cudaMemsetAsync(fr.hist.p, 0, sizeof(uint32_t) * words, st));
-    *hist = (uint32_t *)fr.hist.p;
+    if (fr.tscratch.p != had || bytes > fr.tscratch_zeroed)
+        SG_CUDA(cudaMemsetAsync(fr.tscratch.p, 0, bytes, st));
+    fr.tscratch_zeroed = 0;      // in use from here on
+    *hist = (uint32_t *)fr.tscratch.p;
     return SG_OK;
 }
 
 sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
-                           const uint32_t *d_n, int begin_bit, int end_bit, Frame &fr,
-                           cudaStream_t st, int *result_buf, int site, bool keep_keys)
+                           const uint32_t *d_n, int begin_bit, int end_bit, uint32_t *scratch,
+                           uint32_t *d_err, cudaStream_t st, int *result_buf, int site,
+                           bool keep_keys)
 {
     *result_buf = 0;
     if (n_max <= 0 || end_bit <= begin_bit) return SG_OK;
@@ -329,10 +328,9 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
     }
     const int passes = (end_bit - begin_bit + 7) / 8;
     const int64_t tiles = (n_max + kRadixTile - 1) / kRadixTile;
-    uint32_t *hist = (uint32_t *)fr.hist.p;
+    uint32_t *hist = scratch;
     uint32_t *tickets = hist + 2 * 256 * passes;            // [passes], padded to 16
     uint32_t *lookback = tickets + 16;
-    uint32_t *err = (uint32_t *)fr.scalars.p + kScalStatus;
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
         const int b = radix_bit(begin_bit, end_bit, p);
@@ -340,7 +338,7 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
         uint32_t *keys_out = p == passes - 1 && !keep_keys ? nullptr : keys[cur ^ 1];
         k_onesweep<<<(unsigned)tiles, kRadixThreads, 0, st>>>(
             keys[cur], vals[cur], keys_out, vals[cur ^ 1], d_n, b, (1u << bits) - 1u,
-            hist + 256 * p, lookback + (int64_t)p * tiles * 256, tickets + p, err, site);
+            hist + 256 * p, lookback + (int64_t)p * tiles * 256, tickets + p, d_err, site);
         SG_LAUNCHED();
         cur ^= 1;
     }
@@ -455,10 +453,14 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
                 int64_t ntiles, uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
                 uint32_t *__restrict__ d_nvalid, uint32_t *__restrict__ hist,
                 unsigned long long *__restrict__ lb, uint32_t *__restrict__ ticket,
-                uint32_t *__restrict__ err)
+                uint32_t *__restrict__ err, uint4 *__restrict__ zero, int64_t nzero)
 {
     __shared__ uint32_t s_h[4][256];
     __shared__ ChainShared S;
+    // the tile sort's scratch, zeroed here rather than by a launch of its own
+    for (int64_t i = (int64_t)blockIdx.x * kChainThreads + threadIdx.x; i < nzero;
+         i += (int64_t)gridDim.x * kChainThreads)
+        zero[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int i = threadIdx.x; i < 4 * 256; i += kChainThreads) (&s_h[0][0])[i] = 0;
     if (threadIdx.x == 0) S.tile = atomicAdd(ticket, 1u);
     __syncthreads();
@@ -598,6 +600,7 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
                       cudaStream_t st, int *result_buf)
 {
     *result_buf = 0;
+    fr.tscratch_zeroed = 0;
     if (n <= 0) {   // no projection kernel ran: clear the status word too
         SG_CUDA(cudaMemsetAsync(d_scal, 0, 4 * (kScalStatus + 1), st));
         return SG_OK;
@@ -609,19 +612,23 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     // after the radix scratch, zeroed with it: two tickets, then one 64-bit
     // word per tile for each of the two chained scans
     const int64_t ntiles = (n + kChainTile - 1) / kChainTile;
-    uint32_t *hist = nullptr;
-    sg_status s =
-        radix_prepare(n, 4, fr, st, &hist, depth_stage_words(n) - radix_scratch_words(n, 4));
-    if (s != SG_OK) return s;
+    if (fr.hist.bytes < sizeof(uint32_t) * (size_t)depth_stage_words(n)) {
+        set_error("internal: depth stage scratch missing");
+        return SG_ERR_INVALID;
+    }
+    uint32_t *hist = (uint32_t *)fr.hist.p;
+    sg_status s;
     static_assert(radix_scratch_words(1, 4) % 2 == 0, "64-bit chain words stay aligned");
     unsigned long long *chain = (unsigned long long *)(hist + radix_scratch_words(n, 4));
     uint32_t *tickets = (uint32_t *)chain;                 // [0] compaction, [1] offsets
     uint32_t *err = (uint32_t *)fr.scalars.p + kScalStatus;
     k_compact_depth<<<(unsigned)ntiles, kChainThreads, 0, st>>>(
-        d_count, d_depth, n, ntiles, keys[0], vals[0], d_scal, hist, chain + 2, tickets, err);
+        d_count, d_depth, n, ntiles, keys[0], vals[0], d_scal, hist, chain + 2, tickets, err,
+        (uint4 *)fr.tscratch.p, (int64_t)(fr.tscratch.bytes / 16));
     SG_LAUNCHED();
+    fr.tscratch_zeroed = fr.tscratch.bytes / 16 * 16;
     // (only the ids of the sorted order are read again)
-    if ((s = radix_sort_pairs(keys, vals, n, d_scal, 0, 32, fr, st, result_buf,
+    if ((s = radix_sort_pairs(keys, vals, n, d_scal, 0, 32, hist, err, st, result_buf,
                               SG_LOOKBACK_DEPTH_SORT, false)) != SG_OK)
         return s;
     const bool small = n <= kOffSmallN;
@@ -668,8 +675,12 @@ k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
       const uint32_t *__restrict__ d_scal, const int4 *__restrict__ tiles, int ntx, int wrap_x,
       uint32_t cap, uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
       uint32_t *__restrict__ hist, int end_bit, const uint32_t *__restrict__ err,
-      const uint32_t *__restrict__ owner, int64_t owner_cap)
+      const uint32_t *__restrict__ owner, int64_t owner_cap, uint2 *__restrict__ ranges,
+      int64_t ntiles)
 {
+    for (int64_t i = (int64_t)blockIdx.x * kBinThreads + threadIdx.x; i < ntiles;
+         i += (int64_t)gridDim.x * kBinThreads)
+        ranges[i] = make_uint2(0u, 0u);     // every tile's list empty, for the tile ranges
     // per Gaussian of the block: first pair, id, tile columns (first, count),
     // tile rows (first, last); per pair: its owner, where it is the first
     __shared__ uint32_t s_off[kBinChunk + 1], s_id[kBinChunk + 1];
@@ -786,16 +797,19 @@ k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
 sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint32_t *d_nvalid,
                     const int4 *d_tiles, int ntx, int wrap_x, int64_t cap, uint32_t *d_keys,
                     uint32_t *d_vals, cudaStream_t st, const uint32_t *d_err, const Buf &owner,
-                    uint32_t *d_hist, int end_bit)
+                    uint2 *d_ranges, int64_t ntiles, uint32_t *d_hist, int end_bit)
 {
-    if (cap <= 0) return SG_OK;
+    if (cap <= 0) {
+        SG_CUDA(cudaMemsetAsync(d_ranges, 0, sizeof(uint2) * ntiles, st));
+        return SG_OK;
+    }
     if (d_hist && (end_bit < 1 || end_bit > 8 * kBinPasses)) {
         set_error("internal: %d-bit tile ids", end_bit);
         return SG_ERR_INVALID;
     }
     k_bin<<<(unsigned)((cap + kBinChunk - 1) / kBinChunk), kBinThreads, 0, st>>>(
         d_ids, d_offsets, d_nvalid, d_tiles, ntx, wrap_x, (uint32_t)cap, d_keys, d_vals, d_hist,
-        end_bit, d_err, (const uint32_t *)owner.p, (int64_t)(owner.bytes / 4));
+        end_bit, d_err, (const uint32_t *)owner.p, (int64_t)(owner.bytes / 4), d_ranges, ntiles);
     SG_LAUNCHED();
     return SG_OK;
 }
@@ -808,7 +822,7 @@ sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint
 // sub-block and which of its lanes the box holds, so it never stages an
 // entry that no live ray of its sub-block can see and loads no box.  After a
 // look-back wait gave up (*err) the pairs may hold stale tile ids: every
-// range stays empty (zeroed before the launch).
+// range stays empty (zeroed by the binning).
 // Each thread takes kRangePer consecutive pairs (16-byte loads of keys and
 // ids; the lists' buffers are 256-byte aligned), the boxes' loads issued
 // together.  The columns whose centre c + 1/2 is in [lo, hi] are the run from
@@ -907,10 +921,9 @@ k_ranges(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K,
 }
 
 sg_status tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max, uint2 *d_ranges,
-                      int64_t ntiles, cudaStream_t st, const uint32_t *d_err,
+                      cudaStream_t st, const uint32_t *d_err,
                       const uint32_t *d_ids, const float4 *d_rects, int ntx, uint32_t *d_words)
 {
-    SG_CUDA(cudaMemsetAsync(d_ranges, 0, sizeof(uint2) * ntiles, st));
     if (K_max == 0) return SG_OK;
     const unsigned grid = (unsigned)((K_max + 256 * kRangePer - 1) / (256 * kRangePer));
     if (d_words)
@@ -1006,12 +1019,11 @@ k_ranges_lidar(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d
 }
 
 sg_status lidar_tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max,
-                            uint2 *d_ranges, int64_t ntiles, cudaStream_t st,
-                            const uint32_t *d_err, const uint32_t *d_ids,
-                            const float4 *d_rects, const Lidar &L, uint32_t *d_lmask,
+                            uint2 *d_ranges, cudaStream_t st, const uint32_t *d_err,
+                            const uint32_t *d_ids, const float4 *d_rects, const Lidar &L,
+                            uint32_t *d_lmask,
                             int64_t lmask_stride)
 {
-    SG_CUDA(cudaMemsetAsync(d_ranges, 0, sizeof(uint2) * ntiles, st));
     if (K_max == 0) return SG_OK;
     const unsigned grid = (unsigned)((K_max + 256 * kRangePer - 1) / (256 * kRangePer));
     k_ranges_lidar<<<grid, 256, 0, st>>>(
