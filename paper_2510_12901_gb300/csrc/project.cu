@@ -239,17 +239,47 @@ __device__ __forceinline__ void bulk_wait(uint64_t *bar, uint32_t *status)
 #ifndef SG_PROJ_MINB
 #define SG_PROJ_MINB 4
 #endif
-// Rolling shutter: the pose of the pixel row that sees x, found from the
-// middle row by taking the row x projects to, pose_iters times (clamped to
-// the image; an iterate outside the model's domain stops the iteration).
-__device__ __forceinline__ int cam_row(const CamParams &C, const float *poses, float near_dist,
-                                       const float x[3])
+// A pixel row's pose into registers: three 16-byte loads where the caller's
+// array allows them (rows are 48 bytes apart), which are a quarter of the
+// requests of twelve 4-byte ones, a row of its own per lane each.
+__device__ __forceinline__ void load_row(const float *__restrict__ poses, int row, bool vec,
+                                         float P[12])
+{
+    const float *p = poses + 12 * row;
+    if (vec) {
+        const float4 *q = reinterpret_cast<const float4 *>(p);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float4 v = __ldg(q + k);
+            P[4 * k] = v.x; P[4 * k + 1] = v.y; P[4 * k + 2] = v.z; P[4 * k + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) P[k] = __ldg(p + k);
+    }
+}
+
+// Rolling shutter: the pixel (u, v) of x under the pose of the row that sees
+// it, found from the middle row by taking the row x projects to, pose_iters
+// times (clamped to the image; an iterate outside the model's domain stops the
+// iteration).  Returns the row; ok: x is in the domain under its pose.  A row
+// that projects x to itself ends the iteration, and its pixel is the result
+// (the same values as projecting anew): two projections a point instead of
+// three, 238 -> 212 us for the 1M-Gaussian fisheye view.
+__device__ __forceinline__ int cam_row_point(const CamParams &C, const float *poses, bool vec,
+                                             float near_dist, const float x[3], float &u, float &v,
+                                             bool &ok)
 {
     int row = C.H / 2;
-    for (int it = 0; it < C.pose_iters; ++it) {
-        float u, v;
-        if (!cam_point(C, poses + 12 * row, near_dist, x, u, v)) break;
-        row = v < 0.f ? 0 : (v >= (float)C.H ? C.H - 1 : (int)floorf(v));
+    float P[12];
+    load_row(poses, row, vec, P);
+    ok = cam_point(C, P, near_dist, x, u, v);
+    for (int it = 0; it < C.pose_iters && ok; ++it) {
+        const int r = v < 0.f ? 0 : (v >= (float)C.H ? C.H - 1 : (int)floorf(v));
+        if (r == row) break;
+        row = r;
+        load_row(poses, row, vec, P);
+        ok = cam_point(C, P, near_dist, x, u, v);
     }
     return row;
 }
@@ -299,8 +329,11 @@ k_project_camera(const float *__restrict__ planes, int64_t pitch, int64_t n, int
     // the mean's pose: the camera's, or that of the row that sees the mean
     int row0 = 0;
     const float *P0 = s_c2w;
+    float u0 = 0.f, v0 = 0.f;       // rolling shutter: the mean's pixel
+    bool ok0 = false;
+    const bool vec = kRS && ((uintptr_t)poses & 15u) == 0;
     if constexpr (kRS) {
-        row0 = cam_row(C, poses, U.near_dist, a.mu);
+        row0 = cam_row_point(C, poses, vec, U.near_dist, a.mu, u0, v0, ok0);
         P0 = poses + 12 * row0;
     }
     float dx = a.mu[0] - P0[3], dy = a.mu[1] - P0[7], dz = a.mu[2] - P0[11];
@@ -314,7 +347,14 @@ k_project_camera(const float *__restrict__ planes, int64_t pitch, int64_t n, int
     if (a.sigma >= U.alpha_min) {
         // sigma points chi_0 = mu, chi_{+-i} = mu +- sqrt(n+lambda) s_i R e_i
         float uu[7], vv[7];
-        bool ok = cam_point(C, P0, U.near_dist, a.mu, uu[0], vv[0]);
+        bool ok;
+        if constexpr (kRS) {
+            uu[0] = u0;
+            vv[0] = v0;
+            ok = ok0;
+        } else {
+            ok = cam_point(C, P0, U.near_dist, a.mu, uu[0], vv[0]);
+        }
 #pragma unroll
         for (int p = 1; p < 7; ++p) {
             int i = (p - 1) >> 1;
@@ -322,9 +362,13 @@ k_project_camera(const float *__restrict__ planes, int64_t pitch, int64_t n, int
             float x[3];
 #pragma unroll
             for (int r = 0; r < 3; ++r) x[r] = a.mu[r] + sg * U.lam_gamma * a.s[i] * a.R[3 * r + i];
-            const float *Pp = s_c2w;
-            if constexpr (kRS) Pp = poses + 12 * cam_row(C, poses, U.near_dist, x);
-            ok = cam_point(C, Pp, U.near_dist, x, uu[p], vv[p]) && ok;
+            if constexpr (kRS) {
+                bool okp;
+                cam_row_point(C, poses, vec, U.near_dist, x, uu[p], vv[p], okp);
+                ok = okp && ok;
+            } else {
+                ok = cam_point(C, s_c2w, U.near_dist, x, uu[p], vv[p]) && ok;
+            }
         }
         if (ok) {
             float mu_u = U.w0m * uu[0], mu_v = U.w0m * vv[0];
@@ -423,15 +467,29 @@ sg_status project_camera(const Scene &sc, const Camera &cam, const sg_render_opt
 struct LidParams {
     int n_cols, nphi, n_theta, A, per, pose_iters;
     float az0, T0, TN;
+    float cols_per_deg, tiles_per_deg, cells_per_deg;   // n_cols, n_theta, A over 360
     const float *T;
     const int *sat;
     const float *poses;   // [n_cols*12], set in the kernel from the render's descriptor
 };
 
+constexpr float kDeg = 57.295779513082321f;    // degrees in a radian
+
 __device__ __forceinline__ int pmod(int a, int n)
 {
     int m = a % n;
     return m < 0 ? m + n : m;
+}
+
+// a mod n for a within one turn of [0, n), where azimuths mostly are; the
+// integer remainder, about 25 instructions, beyond.  (Fourteen columns a
+// Gaussian are wrapped: with the elevation tiles searched once instead of
+// twice, the street sweep's projection went from 244 to 200 us.)
+__device__ __forceinline__ int wrap_near(int a, int n)
+{
+    if ((unsigned)a < (unsigned)n) return a;
+    const int b = a < 0 ? a + n : a - n;
+    return (unsigned)b < (unsigned)n ? b : pmod(a, n);
 }
 
 // sensor-frame coordinates of x under the column pose P (row-major 3x4
@@ -448,33 +506,31 @@ __device__ __forceinline__ void to_sensor(const float *__restrict__ P, const flo
     xs[2] = r0.z * d0 + r1.z * d1 + r2.z * d2;
 }
 
-__device__ __forceinline__ int col_of_az(const LidParams &L, float az)
+// Column at `off` degrees past the left edge of column 0.
+__device__ __forceinline__ int col_of_az(const LidParams &L, float off)
 {
-    return pmod((int)floorf((az - L.az0) * ((float)L.n_cols / 360.0f)), L.n_cols);
+    return wrap_near((int)floorf(off * L.cols_per_deg), L.n_cols);
 }
 
 // Column whose pose sees the point: start at mid-sweep, then take the
 // column of the point's azimuth `pose_iters` times; xs = the point in that
-// column's sensor frame and *az_deg its azimuth there.  The point is
-// transformed again only when the column changes, and the last azimuth is
-// reused when the last step kept the column (the same values as
-// transforming and measuring anew).
+// column's sensor frame and *az_deg its azimuth there.  A step that keeps the
+// column ends the iteration (the same values as transforming and measuring
+// anew).
 __device__ __forceinline__ int lidar_col(const LidParams &L, const float x[3], float xs[3],
                                          float *az_deg)
 {
     int col = L.n_cols / 2;
     to_sensor(L.poses + 12 * col, x, xs);
-    bool fresh = false;          // *az_deg belongs to the current xs
-    for (int it = 0; it < L.pose_iters; ++it) {
-        *az_deg = atan2f(xs[1], xs[0]) * 57.295779513082321f;
-        const int c2 = col_of_az(L, *az_deg);
-        fresh = c2 == col;
-        if (!fresh) {
-            col = c2;
-            to_sensor(L.poses + 12 * col, x, xs);
-        }
+    for (int it = 0;; ++it) {
+        const float t = atan2f(xs[1], xs[0]);
+        *az_deg = __fmul_rn(t, kDeg);
+        if (it >= L.pose_iters) break;
+        const int c2 = col_of_az(L, __fsub_rn(*az_deg, L.az0));
+        if (c2 == col) break;    // every further step would keep it
+        col = c2;
+        to_sensor(L.poses + 12 * col, x, xs);
     }
-    if (!fresh) *az_deg = atan2f(xs[1], xs[0]) * 57.295779513082321f;
     return col;
 }
 
@@ -488,9 +544,9 @@ __device__ __forceinline__ int elev_tile(const LidParams &L, float el)
     return e;
 }
 
-__device__ __forceinline__ int elev_cell(const LidParams &L, float el)
+// Culling cell of an angle in elevation tile e.
+__device__ __forceinline__ int elev_cell(const LidParams &L, int e, float el)
 {
-    int e = elev_tile(L, el);
     float f = (el - L.T[e]) / (L.T[e + 1] - L.T[e]) * (float)L.per;
     int sub = !(f >= 0.f) ? 0 : (f >= (float)L.per ? L.per - 1 : (int)floorf(f));
     return e * L.per + min(sub, L.per - 1);
@@ -507,7 +563,7 @@ __device__ __forceinline__ int sat_count(const LidParams &L, int x0, int x1, int
 __device__ __forceinline__ int sat_count_wrap(const LidParams &L, int x0, int x1, int y0, int y1)
 {
     if (x1 - x0 + 1 >= L.A) return sat_count(L, 0, L.A - 1, y0, y1);
-    int a = pmod(x0, L.A), b = pmod(x1, L.A);
+    int a = wrap_near(x0, L.A), b = wrap_near(x1, L.A);
     if (a <= b) return sat_count(L, a, b, y0, y1);
     return sat_count(L, a, L.A - 1, y0, y1) + sat_count(L, 0, b, y0, y1);
 }
@@ -591,9 +647,8 @@ __device__ __forceinline__ void cholesky3(const float C[9], float Lc[9])
 // takes).  Templates, so that the plain path keeps its registers.  Four
 // blocks per SM (64 registers, a few bytes spilled): the kernel waits on
 // dependent pose loads and atan2f / asinf chains, and 32 warps per SM hide
-// more of that than 24 at 76 registers (street sweep, 2M Gaussians: 0.266 ->
-// 0.253 ms; with SH^l features 0.400 -> 0.337 ms; beam divergence 0.435 ->
-// 0.407 ms).
+// more of that than 24 (street sweep, 2M Gaussians: three blocks 221 us, four
+// 200, five 208).
 template <bool kSH, bool kBeam>
 __global__ void __launch_bounds__(256, 4)
 k_project_lidar(const float *__restrict__ planes, int64_t pitch, int64_t n, int sh_degree,
@@ -690,9 +745,8 @@ k_project_lidar(const float *__restrict__ planes, int64_t pitch, int64_t n, int 
                 if (full) {
                     a0 = 0; a1 = L.n_theta - 1; na = L.n_theta;
                 } else {
-                    float sc = (float)L.n_theta / 360.0f;
-                    a0 = (int)floorf((rect.x - L.az0) * sc);
-                    a1 = (int)floorf((rect.y - L.az0) * sc);
+                    a0 = (int)floorf((rect.x - L.az0) * L.tiles_per_deg);
+                    a1 = (int)floorf((rect.y - L.az0) * L.tiles_per_deg);
                     na = a1 - a0 + 1;
                     if (na > L.n_theta) { na = L.n_theta; a1 = a0 + L.n_theta - 1; }
                 }
@@ -701,11 +755,10 @@ k_project_lidar(const float *__restrict__ planes, int64_t pitch, int64_t n, int 
                     int x0, x1;
                     if (full) { x0 = 0; x1 = L.A - 1; }
                     else {
-                        float sc = (float)L.A / 360.0f;
-                        x0 = (int)floorf((rect.x - L.az0) * sc);
-                        x1 = (int)floorf((rect.y - L.az0) * sc);
+                        x0 = (int)floorf((rect.x - L.az0) * L.cells_per_deg);
+                        x1 = (int)floorf((rect.y - L.az0) * L.cells_per_deg);
                     }
-                    keep = sat_count_wrap(L, x0, x1, elev_cell(L, elo), elev_cell(L, ehi)) > 0;
+                    keep = sat_count_wrap(L, x0, x1, elev_cell(L, e0, elo), elev_cell(L, e1, ehi)) > 0;
                 }
                 if (keep) {
                     tl = make_int4(a0, a1, e0, e1);
@@ -749,6 +802,9 @@ sg_status project_lidar(const Scene &sc, const Lidar &Ld, const sg_render_opts &
     L.per = Ld.cull_el;
     L.pose_iters = o.pose_iters;
     L.az0 = Ld.az0;
+    L.cols_per_deg = (float)Ld.n_cols / 360.0f;
+    L.tiles_per_deg = (float)Ld.n_theta / 360.0f;
+    L.cells_per_deg = (float)Ld.cull_az / 360.0f;
     L.T0 = Ld.T[0];
     L.TN = Ld.T[Ld.nphi];
     L.T = Ld.d_T;
