@@ -516,7 +516,9 @@ __device__ __forceinline__ int col_of_az(const LidParams &L, float off)
 // column of the point's azimuth `pose_iters` times; xs = the point in that
 // column's sensor frame and *az_deg its azimuth there.  A step that keeps the
 // column ends the iteration (the same values as transforming and measuring
-// anew).
+// anew).  The offset from column 0's edge is rounded once in the first step
+// and twice in the later ones, spelled out so that a point within rounding of
+// a column's edge takes the same column however the loop is compiled.
 __device__ __forceinline__ int lidar_col(const LidParams &L, const float x[3], float xs[3],
                                          float *az_deg)
 {
@@ -526,7 +528,8 @@ __device__ __forceinline__ int lidar_col(const LidParams &L, const float x[3], f
         const float t = atan2f(xs[1], xs[0]);
         *az_deg = __fmul_rn(t, kDeg);
         if (it >= L.pose_iters) break;
-        const int c2 = col_of_az(L, __fsub_rn(*az_deg, L.az0));
+        const float off = it == 0 ? __fmaf_rn(t, kDeg, -L.az0) : __fsub_rn(*az_deg, L.az0);
+        const int c2 = col_of_az(L, off);
         if (c2 == col) break;    // every further step would keep it
         col = c2;
         to_sensor(L.poses + 12 * col, x, xs);
