@@ -176,27 +176,12 @@ __device__ __forceinline__ void start_ray(RayGrad &r, const float4 *slot, const 
     r.U = gQ[0] * Q[0] + gQ[1] * Q[1] + gQ[2] * Q[2] + gQ[3] * Q[3] + gQ[4] * Q[4];
 }
 
-// Push the window's entries that reach a lane of `act` to the warp's queue.
-__device__ __forceinline__ void push(uint2 *cand, uint32_t *cpos, uint32_t &tail, uint32_t gid,
-                                     uint32_t lanes, uint32_t pos)
-{
-    const uint32_t bal = __ballot_sync(0xffffffffu, lanes != 0u);
-    if (lanes) {
-        const uint32_t at =
-            (tail + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))) % kBwQueue;
-        cand[at] = make_uint2(gid, lanes);
-        cpos[at] = pos;
-    }
-    tail += __popc(bal);
-}
-
 // ------------------------------------------------------------------ camera
 struct BwCam {                     // a warp's shared memory
     float4 e[8][32];               // staged entries (cam_entry's planes 0..7)
     float2 wx[kBwBatch][33];       // (w, x) per (entry, ray); rows an odd number of banks apart
     float4 ray[2][32];             // (dd, gZ), (gF, 0)
-    uint2 cand[kBwQueue];          // waiting: (Gaussian, lane mask)
-    uint32_t cpos[kBwQueue];       // and list position
+    EntryQueue<kBwQueue> q;
     uint32_t pos[32], lanes[32], gid[32];
     float ref[6];
 };
@@ -211,13 +196,13 @@ __device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose
     const int lane = threadIdx.x & 31;
     __syncwarp();
     if (lane < n) {
-        const uint2 c = S.cand[(head + lane) % kBwQueue];
+        const uint2 c = S.q.cand[(head + lane) % kBwQueue];
         float4 ent[9];
         cam_entry(rec[c.x], pose.t, dh, dl, ent, kResponseScale);
 #pragma unroll
         for (int k = 0; k < 8; ++k) S.e[k][lane] = ent[k];
         S.lanes[lane] = c.y;
-        S.pos[lane] = S.cpos[(head + lane) % kBwQueue];
+        S.pos[lane] = S.q.pos[(head + lane) % kBwQueue];
         S.gid[lane] = c.x;
     }
     __syncwarp();
@@ -341,7 +326,7 @@ k_backward_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__r
             // reaches none of them contributes to no ray and is not staged
             const uint32_t act = __ballot_sync(0xffffffffu, rg.x + last > base);
             const uint32_t idx = base + lane;
-            push(S.cand, S.cpos, tail, nid, word_lanes(ncr, sub) & act, idx + 1 - rg.x);
+            push(S.q, tail, nid, word_lanes(ncr, sub) & act, idx + 1 - rg.x);
             ncr = 0u;
             if (idx + 32 < hi) {
                 ncr = crw[idx + 32];
@@ -367,8 +352,7 @@ struct BwPosed {                   // a warp's shared memory
     float4 s[(3 * 32 + kBwBatch * kLidEntryStride + 31) / 32][32];
     float2 wx[kBwBatch][33];
     float4 ray[3][32];             // (dd, gZ), (d, slot), (gF, 0)
-    uint2 cand[kBwQueue];
-    uint32_t cpos[kBwQueue];
+    EntryQueue<kBwQueue> q;
     uint32_t pos[kBwBatch], lanes[kBwBatch], gid[kBwBatch];
 };
 
@@ -379,11 +363,11 @@ __device__ __forceinline__ void posed_stage(const GRec *__restrict__ rec, BwPose
     const int lane = threadIdx.x & 31, j = lane & 15, half = lane >> 4;
     __syncwarp();
     if (j < n) {
-        const uint2 c = S.cand[(head + j) % kBwQueue];
+        const uint2 c = S.q.cand[(head + j) % kBwQueue];
         lidar_entry_slots(rec[c.x], poses, first, 2 * half, min(slots, 2 * half + 2), dh, dl, S.s, j);
         if (half == 0) {
             S.lanes[j] = c.y;
-            S.pos[j] = S.cpos[(head + j) % kBwQueue];
+            S.pos[j] = S.q.pos[(head + j) % kBwQueue];
             S.gid[j] = c.x;
         }
     }
@@ -478,7 +462,7 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
         for (uint32_t base = lo; base < hi; base += 32) {
             const uint32_t act = __ballot_sync(0xffffffffu, rg.x + last > base);
             const uint32_t idx = base + lane;
-            push(S.cand, S.cpos, tail, nid, word_lanes(ncr, sub) & act, idx + 1 - rg.x);
+            push(S.q, tail, nid, word_lanes(ncr, sub) & act, idx + 1 - rg.x);
             ncr = 0u;
             if (idx + 32 < hi) {
                 ncr = crw[idx + 32];
@@ -605,7 +589,7 @@ k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
         for (uint32_t base = lo; base < hi; base += 32) {
             const uint32_t act = __ballot_sync(0xffffffffu, rg.x + last > base);
             const uint32_t idx = base + lane;
-            push(S.cand, S.cpos, tail, nid, nm & act, idx + 1 - rg.x);
+            push(S.q, tail, nid, nm & act, idx + 1 - rg.x);
             nm = 0u;
             if (idx + 32 < hi) {
                 nid = ids[idx + 32];

@@ -627,22 +627,29 @@ sg_status render_camera(const Camera &cam, const sg_render_opts &o, Frame &fr, c
 // and a ray's direction is its tile reference ray under the sub-block's
 // first row's pose plus its offset under its own row's pose (sensor_ray).
 
-// Composite entries [lo, hi) that reach sub-block `sub` (first pixel sbx,
-// sby; rows r0 .. r0 + nrows - 1) into the lane's accumulator; sb: the
-// lane's row slot.  As cam_walk.
+constexpr int kWalkQueue = 64;     // a window of 32, after at most 31 left over
+
+// Composite entries [lo, hi) that reach sub-block `sub` (first pixel row sby;
+// rows sby .. sby + nrows - 1) into the lane's accumulator; sb: the lane's row
+// slot.  As cam_walk, over windows of 32.  Staging an entry for four rows takes
+// about 500 instructions a pass, a third of a window's entries reach a
+// sub-block: staged 32 at a time from the queue instead of per window, the
+// 1M-Gaussian fisheye view went from 500 to 427 us.  The queue's head holds the
+// staged entries' masks and positions (copies of them would cost a block an SM).
+// The one-pose camera stages each window by itself: its staging is short, and
+// the queue only lengthens a small image's chain (251 x 243: 264 -> 272 us).
 __device__ __forceinline__ bool cam_walk_rs(const CamRender &P, const GRec *__restrict__ rec,
                                             const uint32_t *__restrict__ ids,
-                                            const uint32_t *__restrict__ crw, int sub,
-                                            int sbx, int sby, uint32_t lo, uint32_t hi,
-                                            uint32_t begin, const float *__restrict__ poses,
-                                            int nrows, int sb, const float dh[3],
-                                            const float dl[3], const float dd[3],
-                                            const float d[3], float4 (*s)[32], uint32_t *s_pos,
-                                            uint32_t *s_lanes, CamAcc &a, bool done)
+                                            const uint32_t *__restrict__ crw, int sub, int sby,
+                                            uint32_t lo, uint32_t hi, uint32_t begin,
+                                            const float *__restrict__ poses, int nrows, int sb,
+                                            const float dh[3], const float dl[3],
+                                            const float dd[3], const float d[3], float4 (*s)[32],
+                                            EntryQueue<kWalkQueue> &Q, CamAcc &a, bool done)
 {
     const int lane = threadIdx.x & 31;
     const bool done0 = done;
-    uint32_t ncr = 0u, nid = 0u;    // the next batch's, as in cam_walk
+    uint32_t ncr = 0u, nid = 0u, head = 0u, tail = 0u;    // the next window's, as in cam_walk
     if (lo + lane < hi) {
         ncr = crw[lo + lane];
         nid = ids[lo + lane];
@@ -651,42 +658,40 @@ __device__ __forceinline__ bool cam_walk_rs(const CamRender &P, const GRec *__re
         const uint32_t act = __ballot_sync(0xffffffffu, !done);
         if (act == 0u) break;
         const uint32_t idx = base + lane;
-        const uint32_t g = nid;
-        const uint32_t lm = word_lanes(ncr, sub) & act;
+        push(Q, tail, nid, word_lanes(ncr, sub) & act, idx + 1 - begin);
+        ncr = 0u;
         if (idx + 32 < hi) {
             ncr = crw[idx + 32];
             nid = ids[idx + 32];
-        } else {
-            ncr = 0u;
         }
-        const uint32_t bal = __ballot_sync(0xffffffffu, lm != 0u);
-        if (bal == 0u) continue;
-        __syncwarp();
-        if (lm) {
-            const int pos = __popc(bal & ((1u << lane) - 1u));
-            lidar_entry(rec[g], poses, sby, nrows, dh, dl, s, pos);
-            s_lanes[pos] = lm;
-            s_pos[pos] = idx + 1 - begin;
-        }
-        __syncwarp();
-        const int n = __popc(bal);
-        for (int j = 0; j < n; ++j) {
-            PairEval pe;
-            bool ok = lidar_pair_in(s, j, sb, (s_lanes[j] >> lane) & 1u, dd, d, P.alpha_min,
-                                    P.alpha_max, pe);
-            ok = ok && !done;
-            const float Tn = a.T * (1.f - pe.alpha);
-            const bool stop = ok && Tn < P.t_min;
-            done = done || stop;
-            ok = ok && !stop;
-            const float wgt = ok ? pe.alpha * a.T : 0.f;
-            a.c0 += wgt * s[1][j].w;
-            a.c1 += wgt * s[2][j].w;
-            a.c2 += wgt * lid_u(s, j, sb).w;
-            a.Z += wgt * pe.tau;
-            a.W += wgt;
-            a.T = ok ? Tn : a.T;
-            a.last = ok ? s_pos[j] : a.last;
+        const uint32_t least = base + 32 < hi ? 32u : 1u;
+        while (tail - head >= least) {
+            const int n = (int)min(32u, tail - head);
+            __syncwarp();
+            if (lane < n)
+                lidar_entry(rec[Q.cand[(head + lane) % kWalkQueue].x], poses, sby, nrows, dh, dl, s,
+                            lane);
+            __syncwarp();
+            for (int j = 0; j < n; ++j) {
+                const uint32_t at = (head + j) % kWalkQueue;
+                PairEval pe;
+                bool ok = lidar_pair_in(s, j, sb, (Q.cand[at].y >> lane) & 1u, dd, d, P.alpha_min,
+                                        P.alpha_max, pe);
+                ok = ok && !done;
+                const float Tn = a.T * (1.f - pe.alpha);
+                const bool stop = ok && Tn < P.t_min;
+                done = done || stop;
+                ok = ok && !stop;
+                const float wgt = ok ? pe.alpha * a.T : 0.f;
+                a.c0 += wgt * s[1][j].w;
+                a.c1 += wgt * s[2][j].w;
+                a.c2 += wgt * lid_u(s, j, sb).w;
+                a.Z += wgt * pe.tau;
+                a.W += wgt;
+                a.T = ok ? Tn : a.T;
+                a.last = ok ? Q.pos[at] : a.last;
+            }
+            head += n;
         }
     }
     return done && !done0;
@@ -706,8 +711,9 @@ __device__ __forceinline__ void cam_rs_ray(const float *__restrict__ poses,
     sensor_ray(poses + 12 * sby, u[0], u[1], u[2], poses + 12 * row, e, dh, dl, dd, d);
 }
 
+constexpr int kRsWarps = 4;        // warps per block
 template <uint32_t kSeg>
-__global__ void __launch_bounds__(32 * kCamWarps)
+__global__ void __launch_bounds__(32 * kRsWarps)
 k_render_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
                    const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
                    const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
@@ -717,9 +723,8 @@ k_render_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__
                    const RenderDesc *__restrict__ D, float4 *__restrict__ ray_state,
                    float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
-    __shared__ float4 s_all[kCamWarps][kLidPlanes][32];
-    __shared__ uint32_t s_pos[kCamWarps][32];
-    __shared__ uint32_t s_lanes[kCamWarps][32];
+    __shared__ float4 s_all[kRsWarps][kLidPlanes][32];
+    __shared__ EntryQueue<kWalkQueue> s_q[kRsWarps];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     float4(*s_e)[32] = s_all[wib];
     const float *__restrict__ poses = D->poses;
@@ -746,9 +751,8 @@ k_render_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__
         const uint32_t lo = rg.x + (uint32_t)seg * kSeg;
         const uint32_t hi = min(rg.y, lo + kSeg);
         CamAcc a = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u};
-        const bool stopped = cam_walk_rs(P, rec, ids, crw, sub, sbx, sby, lo, hi, rg.x, poses,
-                                         nrows, sb, dh, dl, dd, d, s_e, s_pos[wib], s_lanes[wib],
-                                         a, no_ray);
+        const bool stopped = cam_walk_rs(P, rec, ids, crw, sub, sby, lo, hi, rg.x, poses, nrows,
+                                         sb, dh, dl, dd, d, s_e, s_q[wib], a, no_ray);
         if (ti.x > 1) {
             put_state(partials + ((size_t)(ti.y + seg) * 256 + sub * 32 + lane) * 2, a, stopped);
             __threadfence();
@@ -784,9 +788,8 @@ k_render_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__
                 }
                 if (__any_sync(0xffffffffu, redo)) {
                     const uint32_t l0 = rg.x + sgi * kSeg;
-                    cam_walk_rs(P, rec, ids, crw, sub, sbx, sby, l0, min(rg.y, l0 + kSeg),
-                                rg.x, poses, nrows, sb, dh, dl, dd, d, s_e, s_pos[wib],
-                                s_lanes[wib], a, !redo);
+                    cam_walk_rs(P, rec, ids, crw, sub, sby, l0, min(rg.y, l0 + kSeg), rg.x, poses,
+                                nrows, sb, dh, dl, dd, d, s_e, s_q[wib], a, !redo);
                 }
                 fin = fin || redo;
             }
@@ -842,13 +845,13 @@ sg_status render_camera_rs(const Camera &cam, const sg_render_opts &o, Frame &fr
     SG_CUDA(cudaGetDevice(&dev));
     SG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_render_camera_rs<kSegLen>,
-                                                      32 * kCamWarps, 0) != cudaSuccess || nb < 1)
+                                                      32 * kRsWarps, 0) != cudaSuccess || nb < 1)
         nb = 4;
-    const int64_t cap = (ws.max_items + kCamWarps - 1) / kCamWarps;
+    const int64_t cap = (ws.max_items + kRsWarps - 1) / kRsWarps;
     int64_t grid = (int64_t)sms * nb;
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
-    k_render_camera_rs<kSegLen><<<(unsigned)grid, 32 * kCamWarps, 0, st>>>(
+    k_render_camera_rs<kSegLen><<<(unsigned)grid, 32 * kRsWarps, 0, st>>>(
         P, (const GRec *)fr.rec.p, ids, (const uint2 *)fr.ranges.p, items, tile_info, counts,
         (const uint32_t *)fr.submask.p, counter, arrive, (float4 *)fr.partials.p, cam.d_pix,
         cam.d_tile_dir, (const RenderDesc *)fr.desc.p, saved_state(fr),
@@ -865,20 +868,21 @@ sg_status render_camera_rs(const Camera &cam, const sg_render_opts &o, Frame &fr
 // Batches of 32 list entries are staged through the warp's shared-memory
 // slice with their per-column moments.
 
-// Per-warp shared state of a LiDAR work item: staged entries, their ray
-// masks and list positions.
+// Per-warp shared state of a LiDAR work item: staged entries, and the queue,
+// whose head holds their ray masks and list positions while they are staged.
 struct LidStage {
     float4 (*s)[32];
-    uint32_t *lanes, *pos;
+    EntryQueue<kWalkQueue> *q;
 };
 
 // Composite entries [lo, hi) of the item's list (first entry `begin`): the
 // item's ray masks of a window of 32 entries (written with the tile ranges,
 // lmask[i] for list entry i) select the entries that reach a ray still
-// compositing; only those are staged.  The lanes of one column (a group)
-// then evaluate, in list order, the staged entries whose box holds a ray of
-// that column, while the other groups evaluate theirs.  Returns whether the
-// lane's ray stopped at T_min.
+// compositing; those are queued and staged 32 at a time (street sweep of 2M:
+// 366 -> 356 us with the deferred re-walks).  The lanes of one column (a
+// group) then evaluate, in list order, the staged entries whose box
+// holds a ray of that column, while the other groups evaluate theirs.
+// Returns whether the lane's ray stopped at T_min.
 __device__ __forceinline__ bool lidar_walk(const LidRender &P, const GRec *__restrict__ rec,
                                            const uint32_t *__restrict__ ids,
                                            const uint32_t *__restrict__ lmask,
@@ -891,8 +895,8 @@ __device__ __forceinline__ bool lidar_walk(const LidRender &P, const GRec *__res
     const int lane = threadIdx.x & 31;
     const bool done0 = done;
     const uint32_t gm = __match_any_sync(0xffffffffu, sb);   // lanes of this lane's column
-    // the next batch's ray masks and ids, loaded one batch ahead
-    uint32_t nm = 0u, nid = 0u;
+    // the next window's ray masks and ids, loaded one ahead
+    uint32_t nm = 0u, nid = 0u, head = 0u, tail = 0u;
     if (lo + lane < hi) {
         nm = lmask[lo + lane];
         nid = ids[lo + lane];
@@ -902,57 +906,54 @@ __device__ __forceinline__ bool lidar_walk(const LidRender &P, const GRec *__res
         const uint32_t act = __ballot_sync(0xffffffffu, !done);
         if (act == 0u) break;
         const uint32_t idx = base + lane;
-        const uint32_t g = nid;
-        const uint32_t m = nm & act;
+        push(*L.q, tail, nid, nm & act, idx + 1 - begin);
+        nm = 0u;
         if (idx + 32 < hi) {
             nm = lmask[idx + 32];
             nid = ids[idx + 32];
-        } else {
-            nm = 0u;
         }
-        const uint32_t bal = __ballot_sync(0xffffffffu, m != 0u);
-        if (bal == 0u) continue;
-        __syncwarp();
-        if (m) {
-            const int pos = __popc(bal & ((1u << lane) - 1u));
-            lidar_entry(rec[g], poses, it.col0, it.ncols, dh, dl, L.s, pos);
-            L.lanes[pos] = m;
-            L.pos[pos] = idx + 1 - begin;
-        }
-        __syncwarp();
-        // the staged entries that reach a ray of this lane's column group:
-        // the groups (lanes of one column) walk their own entries side by
-        // side, so an entry whose box holds rays of one column takes one
-        // step of that group only
-        const int n = __popc(bal);
-        const uint32_t lj = lane < n ? L.lanes[lane] : 0u;
-        uint32_t G = 0u;
-        for (uint32_t rest = 0xffffffffu; rest;) {
-            const uint32_t gm_g = __shfl_sync(0xffffffffu, gm, __ffs(rest) - 1);
-            const uint32_t Gg = __ballot_sync(0xffffffffu, (lj & gm_g) != 0u);
-            G = gm == gm_g ? Gg : G;
-            rest &= ~gm_g;
-        }
-        while (__any_sync(0xffffffffu, G != 0u)) {
-            const bool has = G != 0u;
-            const int j = has ? __ffs(G) - 1 : 0;
-            G &= G - 1u;
-            PairEval pe;
-            bool ok = lidar_pair_in(L.s, j, sb, has && ((L.lanes[j] >> lane) & 1u), dd, d,
-                                    P.alpha_min, P.alpha_max, pe);
-            ok = ok && !done;
-            const float Tn = a.T * (1.f - pe.alpha);
-            const bool stop = ok && Tn < P.t_min;
-            done = done || stop;
-            ok = ok && !stop;
-            const float wgt = ok ? pe.alpha * a.T : 0.f;
-            a.c0 += wgt * L.s[1][j].w;
-            a.c1 += wgt * L.s[2][j].w;
-            a.c2 += wgt * lid_u(L.s, j, sb).w;
-            a.Z += wgt * pe.tau;
-            a.W += wgt;
-            a.T = ok ? Tn : a.T;
-            a.last = ok ? L.pos[j] : a.last;
+        const uint32_t least = base + 32 < hi ? 32u : 1u;     // at the end, what is left
+        while (tail - head >= least) {
+            const int n = (int)min(32u, tail - head);
+            __syncwarp();
+            const uint2 c = lane < n ? L.q->cand[(head + lane) % kWalkQueue] : make_uint2(0u, 0u);
+            if (lane < n) lidar_entry(rec[c.x], poses, it.col0, it.ncols, dh, dl, L.s, lane);
+            __syncwarp();
+            // the staged entries that reach a ray of this lane's column group:
+            // the groups (lanes of one column) walk their own entries side by
+            // side, so an entry whose box holds rays of one column takes one
+            // step of that group only
+            const uint32_t lj = c.y;
+            uint32_t G = 0u;
+            for (uint32_t rest = 0xffffffffu; rest;) {
+                const uint32_t gm_g = __shfl_sync(0xffffffffu, gm, __ffs(rest) - 1);
+                const uint32_t Gg = __ballot_sync(0xffffffffu, (lj & gm_g) != 0u);
+                G = gm == gm_g ? Gg : G;
+                rest &= ~gm_g;
+            }
+            while (__any_sync(0xffffffffu, G != 0u)) {
+                const bool has = G != 0u;
+                const int j = has ? __ffs(G) - 1 : 0;
+                G &= G - 1u;
+                const uint32_t at = (head + j) % kWalkQueue;
+                PairEval pe;
+                bool ok = lidar_pair_in(L.s, j, sb, has && ((L.q->cand[at].y >> lane) & 1u), dd, d,
+                                        P.alpha_min, P.alpha_max, pe);
+                ok = ok && !done;
+                const float Tn = a.T * (1.f - pe.alpha);
+                const bool stop = ok && Tn < P.t_min;
+                done = done || stop;
+                ok = ok && !stop;
+                const float wgt = ok ? pe.alpha * a.T : 0.f;
+                a.c0 += wgt * L.s[1][j].w;
+                a.c1 += wgt * L.s[2][j].w;
+                a.c2 += wgt * lid_u(L.s, j, sb).w;
+                a.Z += wgt * pe.tau;
+                a.W += wgt;
+                a.T = ok ? Tn : a.T;
+                a.last = ok ? L.q->pos[at] : a.last;
+            }
+            head += n;
         }
     }
     return done && !done0;
@@ -982,9 +983,9 @@ k_render_lidar(LidRender P, const LidarItem *__restrict__ items,
                float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
     __shared__ float4 s_all[kLidarWarps][kLidPlanes][32];
-    __shared__ uint32_t s_lanes[kLidarWarps][32], s_pos[kLidarWarps][32];
+    __shared__ EntryQueue<kWalkQueue> s_q[kLidarWarps];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const LidStage stg = {s_all[wib], s_lanes[wib], s_pos[wib]};
+    const LidStage stg = {s_all[wib], &s_q[wib]};
     const float *__restrict__ poses = D->poses;
     const uint32_t n_work = kFix ? *F.n_fix : counts[0];
     uint32_t fix_next = blockIdx.x * kLidarWarps + wib;

@@ -84,6 +84,30 @@ __device__ __forceinline__ void cam_ray_offset(const CamPose &P, const float4 e,
     for (int i = 0; i < 3; ++i) dd[i] = P.R[3 * i] * e.x + P.R[3 * i + 1] * e.y + P.R[3 * i + 2] * e.z;
 }
 
+// A warp's queue of list entries to stage, a ring of kN: (Gaussian, lane mask)
+// and list position.  A walk pushes the entries of its windows that reach a
+// live ray and stages them 32 (or 16) at a time, so that every lane of a
+// staging pass has an entry whatever share of a window reaches the rays.
+template <int kN>
+struct EntryQueue {
+    uint2 cand[kN];
+    uint32_t pos[kN];
+};
+
+// Push this lane's entry of a window if it reaches a lane in `lanes`.
+template <int kN>
+__device__ __forceinline__ void push(EntryQueue<kN> &Q, uint32_t &tail, uint32_t gid, uint32_t lanes,
+                                     uint32_t pos)
+{
+    const uint32_t bal = __ballot_sync(0xffffffffu, lanes != 0u);
+    if (lanes) {
+        const uint32_t at = (tail + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))) % kN;
+        Q.cand[at] = make_uint2(gid, lanes);
+        Q.pos[at] = pos;
+    }
+    tail += __popc(bal);
+}
+
 // Deferred re-walks of the compositing (scalars[7] of them): (unit, work
 // code, lane mask, 0), the work code as in the work items.
 struct FixList {
