@@ -92,6 +92,11 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
+
 __device__ __forceinline__ bool cam_pair_scaled(const float4 q0, const float4 q1, const float4 q2,
                                                 const float4 m0, const float4 m1, const float4 m2,
                                                 const float4 mv, bool in_box, const float dd[3],

@@ -29,19 +29,17 @@
 namespace sg {
 
 constexpr int kFwdWarps = 4;        // warps per block of the persistent grid
-// blocks per SM the register budget is set for (72 registers; a few bytes of
-// the merge spill).  Measured (1920x1080 pinhole, 2M Gaussians): 6 blocks 744,
-// 7 blocks 736, 8 blocks 761 us.
-constexpr int kFwdBlocks = 7;
+// blocks per SM the register budget is set for (64 registers; a few bytes of
+// the merge spill).  Measured (1920x1080 pinhole of 2M Gaussians / 641x479
+// fisheye of 100k): 6 blocks 651 / 43, 7 blocks 643 / 46, 8 blocks 624 / 48, 9
+// blocks 656 / 54 us.
+constexpr int kFwdBlocks = 8;
 // List entries a warp scans at a time: kFwdPer per lane.  Those that reach a
 // live ray of the sub-block (about a third on the street views) go to a queue
 // and are staged 32 at a time, so that the staging pass, one entry per lane,
 // runs with all its lanes busy whatever the window.  Measured (1920x1080
-// pinhole, 2M Gaussians): 32 entries 716, 64 711, 96 736 us.
-#ifndef SG_FWD_PER_LANE
-#define SG_FWD_PER_LANE 2
-#endif
-constexpr int kFwdPer = SG_FWD_PER_LANE;
+// pinhole, 2M Gaussians): 32 entries 636, 64 624, 96 628 us.
+constexpr int kFwdPer = 2;
 constexpr int kFwdWin = 32 * kFwdPer;
 constexpr int kFwdStage = 32;         // staged entries held in shared memory at once
 // the queue of entries to stage: a window's, after at most 31 left over
@@ -168,18 +166,22 @@ __device__ __forceinline__ bool fwd_unseen(const float a[3], const float p1[3], 
 }
 
 // A staged entry, 7 float4 (one per shared-memory plane):
-//   0 (a0, p01, p02, a1)   1 (p11, p12, a2, p21)   2 (p22, b0, m01, m02)
-//   3 (b1, m11, m12, b2)   4 (m21, m22, t0, t1)    5 (t2, sigma, c0, c1)
-//   6 (c2, lane mask, 0, 0)
+//   k = 0..2 (a_k, b_k, p_k1, m_k1)   3 (p02, m02, p12, m12)   4 (p22, m22, t0, t1)
+//   5 (t2, sigma, lane mask, c2)      6 (c0, c1, 0, 0)
 // with p_kj = f_k M_k . (v x e_j) and m_kj = M_k . e_j.  The P terms (a, p)
 // carry the response scale sqrt(log2(e) / 2), as in cam_pair_scaled, so that
 // |num|^2 / |den|^2 is the exponent of 2.  ref: the tile's reference frame
 // (dh, dl, e_1, e_2), in the warp's shared memory.
-// The entry goes to slot `t` of the warp's planes s, with its lane mask.
-// Returns whether some ray of the sub-block (s_reg) may composite it.
-__device__ __forceinline__ bool fwd_entry(const GRec &r, const float o[3], const float *ref,
+// Every lane calls it with an entry (live: one that counts).  The entries that
+// some ray of the sub-block (s_reg) may composite go to the warp's planes s, in
+// lane order, each with its lane mask; returns their number.  The test comes
+// before the stores, so that nothing has to be moved up past the entries left
+// out (moving them through shared memory took a tenth of the kernel's
+// instructions: 671 -> 643 us); the features, which it does not need, are read
+// after it.
+__device__ __forceinline__ int fwd_entry(const GRec &r, const float4 *pfeat, bool live, const float o[3], const float *ref,
                                           const float *s_reg, float alpha_min, uint32_t lanes,
-                                          float4 (*s)[kFwdStage], int t)
+                                          float4 (*s)[kFwdStage])
 {
     const float mu[3] = {r.mu_sigma.x, r.mu_sigma.y, r.mu_sigma.z}, sigma = r.mu_sigma.w;
     const float M[3][3] = {{r.m0.x, r.m0.y, r.m0.z}, {r.m1.x, r.m1.y, r.m1.z},
@@ -203,88 +205,89 @@ __device__ __forceinline__ bool fwd_entry(const GRec &r, const float o[3], const
         m2[k] = dot3(M[k], e2);
         mv[k] = dot3(M[k], vh);
     }
-    s[0][t] = make_float4(a[0], p1[0], p2[0], a[1]);
-    s[1][t] = make_float4(p1[1], p2[1], a[2], p1[2]);
-    s[2][t] = make_float4(p2[2], b[0], m1[0], m2[0]);
-    s[3][t] = make_float4(b[1], m1[1], m2[1], b[2]);
-    s[4][t] = make_float4(m1[2], m2[2], dot3(mv, b), dot3(mv, m1));
-    s[5][t] = make_float4(dot3(mv, m2), sigma, r.feat.x, r.feat.y);
-    s[6][t] = make_float4(r.feat.z, __uint_as_float(lanes), 0.f, 0.f);
-    return s_reg[7] == 0.f || !fwd_unseen(a, p1, p2, b, m1, m2, sigma, alpha_min, s_reg);
+    const float t0 = dot3(mv, b), t1 = dot3(mv, m1), t2 = dot3(mv, m2);
+    const bool keep = live && (s_reg[7] == 0.f ||
+                               !fwd_unseen(a, p1, p2, b, m1, m2, sigma, alpha_min, s_reg));
+    const uint32_t kb = __ballot_sync(0xffffffffu, keep);
+    if (keep) {
+        const int t = __popc(kb & ((1u << (threadIdx.x & 31)) - 1u));
+        const float4 feat = *pfeat;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s[k][t] = make_float4(a[k], b[k], p1[k], m1[k]);
+        s[3][t] = make_float4(p2[0], m2[0], p2[1], m2[1]);
+        s[4][t] = make_float4(p2[2], m2[2], t0, t1);
+        s[5][t] = make_float4(t2, sigma, __uint_as_float(lanes), feat.z);
+        s[6][t] = make_float4(feat.x, feat.y, 0.f, 0.f);
+    }
+    return __popc(kb);
 }
 
 struct FwdAcc {
     float T, W, Z, c0, c1, c2;
 };
 
+// A ray that has stopped (or a lane without one) has T = -1: whatever alpha,
+// T (1 - alpha) is then below t_min and nothing is added, so that the loop
+// needs no flag of its own.
+constexpr float kFwdStopped = -1.f;
+
 // Composite the n staged entries into the lane's accumulator (ray with
-// tangent-plane coordinates (x, y)); done: the ray has stopped (or has none).
+// tangent-plane coordinates (x, y)).  At alpha = 0 the step changes nothing.
+// The warps issue instructions in 70% of the cycles and shared memory returns
+// data in 85%, so what counts is instructions an entry: numerator and
+// denominator of a component go side by side through packed FMAs (1920x1080
+// pinhole of 2M: 711 -> 698 us), the flag went into T, and two entries a pass
+// share the loop (-> 671).
 __device__ __forceinline__ void fwd_composite(const CamRender &P, float4 (*s)[kFwdStage], int n,
-                                              float x, float y, FwdAcc &a, bool &done)
+                                              float x, float y, FwdAcc &a)
 {
     const uint32_t bit = 1u << (threadIdx.x & 31);
+    const float2 xx = make_float2(x, x), yy = make_float2(y, y);
+    float2 c01 = make_float2(a.c0, a.c1);
+#pragma unroll 2
     for (int j = 0; j < n; ++j) {
         const float4 A = s[0][j], B = s[1][j], C = s[2][j], D = s[3][j], E = s[4][j];
         const float4 F = s[5][j], G = s[6][j];
-        const float n0 = fmaf(A.z, y, fmaf(A.y, x, A.x));
-        const float n1 = fmaf(B.y, y, fmaf(B.x, x, A.w));
-        const float n2 = fmaf(C.x, y, fmaf(B.w, x, B.z));
-        const float d0 = fmaf(C.w, y, fmaf(C.z, x, C.y));
-        const float d1 = fmaf(D.z, y, fmaf(D.y, x, D.x));
-        const float d2 = fmaf(E.y, y, fmaf(E.x, x, D.w));
+        // (num_k, den_k) side by side
+        const float2 q0 = fma2(lo2(D), yy, fma2(hi2(A), xx, lo2(A)));
+        const float2 q1 = fma2(hi2(D), yy, fma2(hi2(B), xx, lo2(B)));
+        const float2 q2 = fma2(lo2(E), yy, fma2(hi2(C), xx, lo2(C)));
         const float tn = fmaf(F.x, y, fmaf(E.w, x, E.z));
-        const float inv = __fdividef(1.f, d0 * d0 + d1 * d1 + d2 * d2);
-        const float rho = ex2_approx(-((n0 * n0 + n1 * n1 + n2 * n2) * inv));
-        const float alpha = fminf(F.y * rho, P.alpha_max);
-        const bool in = (__float_as_uint(G.y) & bit) != 0u;
-        const bool ok = in && tn > 0.f && alpha >= P.alpha_min && !done;
+        const float2 q = fma2(q2, q2, fma2(q0, q0, mul2(q1, q1)));
+        const float inv = __fdividef(1.f, q.y);
+        const float rho = ex2_approx(-(q.x * inv));
+        const float al = fminf(F.y * rho, P.alpha_max);
+        const bool in = (__float_as_uint(F.z) & bit) != 0u;
+        const float alpha = in && tn > 0.f && al >= P.alpha_min ? al : 0.f;
         const float w = alpha * a.T;
-        const float Tn = a.T - w;
-        const bool stop = ok && Tn < P.t_min;
-        done = done || stop;
-        const bool take = ok && !stop;
-        const float wgt = take ? w : 0.f;
-        a.c0 += wgt * F.z;
-        a.c1 += wgt * F.w;
-        a.c2 += wgt * G.x;
+        const float Tn = __fsub_rn(a.T, w);
+        const bool go = Tn >= P.t_min;
+        const float wgt = go ? w : 0.f;
+        a.T = go ? Tn : kFwdStopped;
+        c01 = fma2(make_float2(wgt, wgt), lo2(G), c01);
+        a.c2 += wgt * F.w;
         a.Z += wgt * (tn * inv);
         a.W += wgt;
-        a.T = take ? Tn : a.T;
     }
+    a.c0 = c01.x;
+    a.c1 = c01.y;
 }
 
 // Stage the n <= 32 entries waiting at the head of the warp's queue and
-// composite the ones a ray of the sub-block may composite.  Each lane stages
-// one entry at its own slot, tests it, and moves it to its place among the
-// kept ones (through shared memory, a plane at a time: the 28 registers of an
-// entry do not fit beside the test's).
+// composite the ones a ray of the sub-block may composite.
 __device__ __forceinline__ void fwd_batch(const CamRender &P, const CamPose &pose,
                                           const GRec *__restrict__ rec, const float *ref,
                                           const uint2 *cand, uint32_t head, int n, float x, float y,
-                                          float4 (*s)[kFwdStage], FwdAcc &a, bool &done)
+                                          float4 (*s)[kFwdStage], FwdAcc &a)
 {
     const int lane = threadIdx.x & 31;
-    bool keep = false;
     __syncwarp();
-    if (lane < n) {
-        const uint2 c = cand[(head + lane) % kFwdQueue];
-        keep = fwd_entry(rec[c.x], pose.t, ref, ref + 12, P.alpha_min, c.y, s, lane);
-    }
-    const uint32_t kb = __ballot_sync(0xffffffffu, keep);
-    const int m = __popc(kb);
+    // lanes without an entry take the first one's record and drop it
+    const bool live = lane < n;
+    const uint2 c = cand[(head + (live ? lane : 0)) % kFwdQueue];
+    const int m = fwd_entry(rec[c.x], &rec[c.x].feat, live, pose.t, ref, ref + 12, P.alpha_min, c.y, s);
     __syncwarp();
-    if (m != n) {
-        const int t = __popc(kb & ((1u << lane) - 1u));
-#pragma unroll
-        for (int k = 0; k < 7; ++k) {
-            float4 e;
-            if (keep) e = s[k][lane];
-            __syncwarp();
-            if (keep) s[k][t] = e;
-        }
-        __syncwarp();
-    }
-    fwd_composite(P, s, m, x, y, a, done);
+    fwd_composite(P, s, m, x, y, a);
 }
 
 // Composite list entries [lo, hi) of a tile that can reach sub-block `sub`
@@ -301,7 +304,7 @@ __device__ __forceinline__ void fwd_walk(const CamRender &P, const CamPose &pose
                                          const uint32_t *__restrict__ crw, int sub, uint32_t lo,
                                          uint32_t hi, const float *ref, float x, float y,
                                          float4 (*s)[kFwdStage], uint2 *cand, FwdAcc &a,
-                                         bool &done, float *region = nullptr)
+                                         float *region = nullptr)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
@@ -315,9 +318,9 @@ __device__ __forceinline__ void fwd_walk(const CamRender &P, const CamPose &pose
         ncr[w] = i < hi ? crw[i] : 0u;
         nid[w] = i < hi ? ids[i] : 0u;
     }
-    if (region) fwd_region(x, y, !done, region);    // while they arrive
+    if (region) fwd_region(x, y, a.T >= 0.f, region);    // while they arrive
     for (uint32_t base = lo; base < hi; base += kFwdWin) {
-        const uint32_t act = __ballot_sync(0xffffffffu, !done);
+        const uint32_t act = __ballot_sync(0xffffffffu, a.T >= 0.f);
         if (act == 0u) return;
 #pragma unroll
         for (int w = 0; w < kFwdPer; ++w) {
@@ -336,7 +339,7 @@ __device__ __forceinline__ void fwd_walk(const CamRender &P, const CamPose &pose
         const uint32_t least = base + kFwdWin < hi ? 32u : 1u;
         while (tail - head >= least) {
             const uint32_t n = min(32u, tail - head);
-            fwd_batch(P, pose, rec, ref, cand, head, (int)n, x, y, s, a, done);
+            fwd_batch(P, pose, rec, ref, cand, head, (int)n, x, y, s, a);
             head += n;
         }
     }
@@ -391,14 +394,13 @@ k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *_
         const uint2 rg = ranges[tile];
         const uint32_t lo = rg.x + (uint32_t)seg * kSeg;
         const uint32_t hi = min(rg.y, lo + kSeg);
-        FwdAcc a = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        bool done = no_ray;
-        fwd_walk(P, s_pose, rec, ids, crw, sub, lo, hi, s_ref, e.x, e.y, s_e, cand, a, done,
+        FwdAcc a = {no_ray ? kFwdStopped : 1.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        fwd_walk(P, s_pose, rec, ids, crw, sub, lo, hi, s_ref, e.x, e.y, s_e, cand, a,
                  s_ref + 12);
         if (ti.x > 1) {
             // long tile: publish this run, and combine if it is the last one
             fwd_put(partials + ((size_t)(ti.y + seg) * 256 + sub * 32 + lane) * 2, a,
-                    done && !no_ray);
+                    a.T < 0.f && !no_ray);
             __threadfence();
             __syncwarp();
             uint32_t prev = 0;
@@ -453,10 +455,12 @@ k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *_
                 const uint32_t r = __reduce_min_sync(0xffffffffu, pend ? stop_run : 0xffffffffu);
                 if (r == 0xffffffffu) break;
                 const bool mine = pend && stop_run == r;
-                bool dn = !mine;
+                const float T = a.T;
+                if (!mine) a.T = kFwdStopped;
                 const uint32_t l0 = rg.x + r * kSeg;
                 fwd_walk(P, s_pose, rec, ids, crw, sub, l0, min(rg.y, l0 + kSeg), s_ref, e.x, e.y,
-                         s_e, cand, a, dn);
+                         s_e, cand, a);
+                if (!mine) a.T = T;
                 pend = pend && !mine;
             }
         }
