@@ -233,19 +233,19 @@ __device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose
         GaussSums g;
         clear(g);
         const int il = use ? i : b0;
-        const float4 q0 = S.e[0][il], q1 = S.e[1][il], q2 = S.e[2][il];
-        const float4 m0 = S.e[3][il], m1 = S.e[4][il], m2 = S.e[5][il];
+        const float4 e0 = S.e[0][il], e1 = S.e[1][il], e2 = S.e[2][il];
+        const float4 e3 = S.e[3][il], e4 = S.e[4][il], e5 = S.e[5][il];
 #pragma unroll 4
         for (int k = 0; k < 16; ++k) {
             const float4 d = S.ray[0][r0 + k], f = S.ray[1][r0 + k];
             const float2 wx = use ? S.wx[j][r0 + k] : make_float2(0.f, 0.f);
             if (wx.x == 0.f) continue;      // not composited
-            const float num[3] = {q0.w + q0.x * d.x + q0.y * d.y + q0.z * d.z,
-                                  q1.w + q1.x * d.x + q1.y * d.y + q1.z * d.z,
-                                  q2.w + q2.x * d.x + q2.y * d.y + q2.z * d.z};
-            const float den[3] = {m0.w + m0.x * d.x + m0.y * d.y + m0.z * d.z,
-                                  m1.w + m1.x * d.x + m1.y * d.y + m1.z * d.z,
-                                  m2.w + m2.x * d.x + m2.y * d.y + m2.z * d.z};
+            const float2 xx = make_float2(d.x, d.x), yy = make_float2(d.y, d.y);
+            const float2 zz = make_float2(d.z, d.z);
+            const float2 v0 = fma2(hi2(e3), zz, fma2(lo2(e3), yy, fma2(hi2(e0), xx, lo2(e0))));
+            const float2 v1 = fma2(hi2(e4), zz, fma2(lo2(e4), yy, fma2(hi2(e1), xx, lo2(e1))));
+            const float2 v2 = fma2(hi2(e5), zz, fma2(lo2(e5), yy, fma2(hi2(e2), xx, lo2(e2))));
+            const float num[3] = {v0.x, v1.x, v2.x}, den[3] = {v0.y, v1.y, v2.y};
             const float gF[3] = {f.x, f.y, f.z};
             add_pair(g, num, den, 1.f / kResponseScale, wx, gF, d.w);
         }

@@ -37,10 +37,11 @@ __device__ __forceinline__ float dot3(const float a[3], const float b[3])
 }
 
 // Camera entry, 9 float4 (one per shared-memory plane):
-//   e[0..2] = (P row k, a_k)       e[3..5] = (M row k, M_k . d_T)
-//   e[6]    = (M v, sigma)         e[7] = features      e[8] = extent box
-// pscale multiplies the P rows and a (planes 0..2), so that |num|^2 comes
-// out scaled (the forward folds -1/2 log2(e) of the response into it).
+//   e[k] = (a_k, M_k . d_T, P_k0, M_k0)   e[3 + k] = (P_k1, M_k1, P_k2, M_k2)
+//   e[6] = (M v, sigma)                   e[7] = features   e[8] = extent box
+// numerator and denominator terms side by side, for packed FMAs.  pscale
+// multiplies the P rows and a, so that |num|^2 comes out scaled (the forward
+// folds -1/2 log2(e) of the response into it).
 __device__ __forceinline__ void cam_entry(const GRec &r, const float o[3], const float dh[3],
                                           const float dl[3], float4 e[9], float pscale = 1.f)
 {
@@ -51,15 +52,18 @@ __device__ __forceinline__ void cam_entry(const GRec &r, const float o[3], const
     precise_moment(mu, o, dh, dl, w, vh);
     // P rows: f_k (M_k x v), since M_k . (v x dd) = dd . (M_k x v)
     const float f0 = pscale * r.m0.w, f1 = pscale * r.m1.w, f2 = pscale * r.m2.w;
-    e[0] = make_float4(f0 * (M0[1] * vh[2] - M0[2] * vh[1]), f0 * (M0[2] * vh[0] - M0[0] * vh[2]),
-                       f0 * (M0[0] * vh[1] - M0[1] * vh[0]), f0 * dot3(M0, w));
-    e[1] = make_float4(f1 * (M1[1] * vh[2] - M1[2] * vh[1]), f1 * (M1[2] * vh[0] - M1[0] * vh[2]),
-                       f1 * (M1[0] * vh[1] - M1[1] * vh[0]), f1 * dot3(M1, w));
-    e[2] = make_float4(f2 * (M2[1] * vh[2] - M2[2] * vh[1]), f2 * (M2[2] * vh[0] - M2[0] * vh[2]),
-                       f2 * (M2[0] * vh[1] - M2[1] * vh[0]), f2 * dot3(M2, w));
-    e[3] = make_float4(M0[0], M0[1], M0[2], dot3(M0, dh));
-    e[4] = make_float4(M1[0], M1[1], M1[2], dot3(M1, dh));
-    e[5] = make_float4(M2[0], M2[1], M2[2], dot3(M2, dh));
+    const float P0[3] = {f0 * (M0[1] * vh[2] - M0[2] * vh[1]), f0 * (M0[2] * vh[0] - M0[0] * vh[2]),
+                         f0 * (M0[0] * vh[1] - M0[1] * vh[0])};
+    const float P1[3] = {f1 * (M1[1] * vh[2] - M1[2] * vh[1]), f1 * (M1[2] * vh[0] - M1[0] * vh[2]),
+                         f1 * (M1[0] * vh[1] - M1[1] * vh[0])};
+    const float P2[3] = {f2 * (M2[1] * vh[2] - M2[2] * vh[1]), f2 * (M2[2] * vh[0] - M2[0] * vh[2]),
+                         f2 * (M2[0] * vh[1] - M2[1] * vh[0])};
+    e[0] = make_float4(f0 * dot3(M0, w), dot3(M0, dh), P0[0], M0[0]);
+    e[1] = make_float4(f1 * dot3(M1, w), dot3(M1, dh), P1[0], M1[0]);
+    e[2] = make_float4(f2 * dot3(M2, w), dot3(M2, dh), P2[0], M2[0]);
+    e[3] = make_float4(P0[1], M0[1], P0[2], M0[2]);
+    e[4] = make_float4(P1[1], M1[1], P1[2], M1[2]);
+    e[5] = make_float4(P2[1], M2[1], P2[2], M2[2]);
     e[6] = make_float4(dot3(M0, vh), dot3(M1, vh), dot3(M2, vh), r.mu_sigma.w);
     e[7] = r.feat;
     e[8] = r.rect;
@@ -97,28 +101,31 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
-__device__ __forceinline__ bool cam_pair_scaled(const float4 q0, const float4 q1, const float4 q2,
-                                                const float4 m0, const float4 m1, const float4 m2,
+__device__ __forceinline__ bool cam_pair_scaled(const float4 e0, const float4 e1, const float4 e2,
+                                                const float4 e3, const float4 e4, const float4 e5,
                                                 const float4 mv, bool in_box, const float dd[3],
                                                 float alpha_min, float alpha_max, PairEval &pe)
 {
-    const float n0 = q0.w + q0.x * dd[0] + q0.y * dd[1] + q0.z * dd[2];
-    const float n1 = q1.w + q1.x * dd[0] + q1.y * dd[1] + q1.z * dd[2];
-    const float n2 = q2.w + q2.x * dd[0] + q2.y * dd[1] + q2.z * dd[2];
-    pe.e[0] = m0.w + m0.x * dd[0] + m0.y * dd[1] + m0.z * dd[2];
-    pe.e[1] = m1.w + m1.x * dd[0] + m1.y * dd[1] + m1.z * dd[2];
-    pe.e[2] = m2.w + m2.x * dd[0] + m2.y * dd[1] + m2.z * dd[2];
-    pe.inv = __fdividef(1.f, pe.e[0] * pe.e[0] + pe.e[1] * pe.e[1] + pe.e[2] * pe.e[2]);
+    const float2 xx = make_float2(dd[0], dd[0]), yy = make_float2(dd[1], dd[1]);
+    const float2 zz = make_float2(dd[2], dd[2]);
+    const float2 r0 = fma2(hi2(e3), zz, fma2(lo2(e3), yy, fma2(hi2(e0), xx, lo2(e0))));
+    const float2 r1 = fma2(hi2(e4), zz, fma2(lo2(e4), yy, fma2(hi2(e1), xx, lo2(e1))));
+    const float2 r2 = fma2(hi2(e5), zz, fma2(lo2(e5), yy, fma2(hi2(e2), xx, lo2(e2))));
+    const float2 sq = fma2(r2, r2, fma2(r0, r0, mul2(r1, r1)));     // |num|^2, |den|^2
+    pe.e[0] = r0.y;
+    pe.e[1] = r1.y;
+    pe.e[2] = r2.y;
+    pe.inv = __fdividef(1.f, sq.y);
     pe.tau = (mv.x * pe.e[0] + mv.y * pe.e[1] + mv.z * pe.e[2]) * pe.inv;
-    const float d2s = (n0 * n0 + n1 * n1 + n2 * n2) * pe.inv;
+    const float d2s = sq.x * pe.inv;
     pe.rho = ex2_approx(-d2s);
     const float a = mv.w * pe.rho;
     pe.clamped = a > alpha_max;
     pe.alpha = fminf(a, alpha_max);
     constexpr float kInv = 1.f / kResponseScale;
-    pe.n[0] = n0 * kInv;
-    pe.n[1] = n1 * kInv;
-    pe.n[2] = n2 * kInv;
+    pe.n[0] = r0.x * kInv;
+    pe.n[1] = r1.x * kInv;
+    pe.n[2] = r2.x * kInv;
     pe.D2 = d2s * (kInv * kInv);
     return in_box && pe.tau > 0.f && pe.alpha >= alpha_min;
 }

@@ -7,7 +7,7 @@
 namespace sg {
 
 struct CamRender {
-    int W, H, ntx;
+    int W, H, ntx, sms;
     float alpha_min, alpha_max, t_min;
 };
 
@@ -39,12 +39,35 @@ struct LidRender {
     float alpha_min, alpha_max, t_min;
 };
 
+inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        sms = 152;
+    return sms;
+}
+
+// The warps of a persistent grid take their first items as they start, all of
+// an SM's at once, so with fewer items than warps the first SMs get more of
+// them.  A warp takes part only if it is among the first n_items when the warps
+// are counted across the SMs (block b starts on SM b mod sms), which spreads
+// the items evenly.  A 251x243 view of 20011 Gaussians, some 2300 items of up
+// to 1024 entries: 144 -> 119 us of compositing; nothing with more items than
+// warps, and at 130 items (64x64) the same 19 us.
+__device__ __forceinline__ bool warp_takes_part(int sms, uint32_t n_items)
+{
+    const uint32_t row = (threadIdx.x >> 5) + (blockDim.x >> 5) * (blockIdx.x / (uint32_t)sms);
+    return blockIdx.x % (uint32_t)sms + (uint32_t)sms * row < n_items;
+}
+
 inline CamRender cam_render_params(const Camera &cam, const sg_render_opts &o)
 {
     CamRender P;
     P.W = cam.width;
     P.H = cam.height;
     P.ntx = cam.ntx;
+    P.sms = sm_count();
     P.alpha_min = o.alpha_min;
     P.alpha_max = o.alpha_max;
     P.t_min = o.t_min;
