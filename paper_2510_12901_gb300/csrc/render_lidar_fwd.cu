@@ -23,8 +23,8 @@
 // d_r = h_c + tan(el_r) z_c in double, split in two floats, so a_k keeps the
 // error-free moment of render.cu.  D^2 does not depend on the length of d',
 // and tau_max along d' is the range along the unit ray divided by |d'| =
-// 1 / cos(el).  A pair costs 7 FMAs for the affine parts (18 with the
-// 3-vector offsets of k_render_lidar) and 5 shared-memory loads (7).
+// 1 / cos(el).  A pair costs 4 packed FMAs for the affine parts (18 with the
+// 3-vector offsets of k_render_lidar) and 6 shared-memory loads (9).
 #include <math.h>
 
 #include "pairs.cuh"
@@ -33,18 +33,18 @@
 namespace sg {
 
 constexpr int kLfWarps = 4;     // warps per block of the persistent grid
-// blocks per SM: the staged entries take 8.5 KB of shared memory per warp
-constexpr int kLfBlocks = 6;
+// Blocks per SM.  The staged entries take 9 KB of shared memory a warp, and what
+// the blocks leave of an SM's 228 KB is L1 for the records they stage.  Street
+// sweep of 2M / 64 x 1024 of 0.5M with beam divergence: 6 blocks 258 / 165, 5
+// blocks 226 / 150, 4 blocks 220 / 141, 3 blocks 220 / 144 us.
+constexpr int kLfBlocks = 4;
 // List entries a warp scans per window: kLfPer per lane.  The entries of the
 // window that reach a live ray (about half of them on the street sweep) go to
 // a queue and are staged 32 at a time, so that the staging pass, one entry per
 // lane, runs with all its lanes busy.  Measured: street sweep of 2M 287 -> 280
 // us, 64 x 1024 of 0.5M with beam divergence 214 -> 196 us (one entry a lane
 // 284 and 202).
-#ifndef SG_LF_PER_LANE
-#define SG_LF_PER_LANE 2
-#endif
-constexpr int kLfPer = SG_LF_PER_LANE;
+constexpr int kLfPer = 2;
 constexpr int kLfWin = 32 * kLfPer;
 constexpr int kLfQueue = kLfPer == 1 ? 64 : 128;
 static_assert(kLfWin + 31 <= kLfQueue, "staging queue");
@@ -54,7 +54,7 @@ static_assert(kLfWin + 31 <= kLfQueue, "staging queue");
 // lanes of a beam group read them in one piece), and the lanes staging 32
 // entries at once write distinct banks.
 struct LfShared {
-    float4 q[3][32 * kLidarColsMax];   // (a0, p0, a1, p1) (a2, p2, b0, m0) (b1, m1, b2, m2)
+    float4 q[3][32 * kLidarColsMax];   // (a_k, b_k, p_k, m_k), for packed FMAs
     float2 t[32 * kLidarColsMax];      // (t0, t1)
     float4 e[32];                      // (sigma, f0, f1, f2)
     uint32_t lanes[32];                // staged entry's ray mask
@@ -93,12 +93,19 @@ __device__ __forceinline__ void lf_entry(const GRec &r, LfShared &S, int pos, in
             mv[k] = dot3(M[k], vh);
         }
         const int qi = lf_qi(pos, sl);
-        S.q[0][qi] = make_float4(a[0], p[0], a[1], p[1]);
-        S.q[1][qi] = make_float4(a[2], p[2], b[0], m[0]);
-        S.q[2][qi] = make_float4(b[1], m[1], b[2], m[2]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) S.q[k][qi] = make_float4(a[k], b[k], p[k], m[k]);
         S.t[lf_ti(pos, sl)] = make_float2(dot3(mv, b), dot3(mv, m));
     }
 }
+
+// Entries a loop pass evaluates before it adds them to the sums in turn.  The
+// walk waits for latencies (a group has a few entries a batch, each a chain of
+// about 20 dependent instructions), and independent evaluations overlap.  Street
+// sweep / 64 x 1024, 4 blocks an SM: 1 entry 280 / 196 (6 blocks), 2 entries 223
+// / 149, 3 entries 220 / 141, 4 entries 227 / 145 us; the deferred re-walks 44 /
+// 53 with 1, 33 / 34 with 3.
+constexpr int kLfPass = 3;
 
 // A ray's running sums.  T = 0 marks a ray that has stopped (or has none, or
 // sits out a re-walk): every later weight alpha T is then 0.  A live ray's
@@ -122,6 +129,7 @@ __device__ __forceinline__ void lf_walk(const LidRender &P, const GRec *__restri
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
     const uint32_t bit = 1u << lane;
+    const float2 xx = make_float2(x, x);
     uint32_t head = 0u, tail = 0u;
     // the next window's ray masks and ids (entries lane + 32 w of it), loaded
     // one window ahead
@@ -168,33 +176,41 @@ __device__ __forceinline__ void lf_walk(const LidRender &P, const GRec *__restri
                 rest &= ~gm_g;
             }
             while (__any_sync(0xffffffffu, G != 0u)) {
-                const bool has = G != 0u;
-                const int j = has ? __ffs(G) - 1 : 0;
-                G &= G - 1u;
-                const int qi = lf_qi(j, sl);
-                const float4 A = S.q[0][qi], B = S.q[1][qi], C = S.q[2][qi];
-                const float2 U = S.t[lf_ti(j, sl)];
-                const float4 E = S.e[j];
-                const bool in = has && (S.lanes[j] & bit) != 0u;
-                const float n0 = fmaf(A.y, x, A.x), n1 = fmaf(A.w, x, A.z);
-                const float n2 = fmaf(B.y, x, B.x);
-                const float d0 = fmaf(B.w, x, B.z), d1 = fmaf(C.y, x, C.x);
-                const float d2 = fmaf(C.w, x, C.z);
-                const float tn = fmaf(U.y, x, U.x);
-                const float inv = __fdividef(1.f, d0 * d0 + d1 * d1 + d2 * d2);
-                const float rho = ex2_approx(-((n0 * n0 + n1 * n1 + n2 * n2) * inv));
-                const float alpha = fminf(E.x * rho, P.alpha_max);
-                const bool ok = in && tn > 0.f && alpha >= P.alpha_min;
-                const float w = (ok ? alpha : 0.f) * a.T;
-                const float Tn = a.T - w;
-                const bool stop = Tn < P.t_min;
-                const float wgt = stop ? 0.f : w;
-                a.T = stop ? 0.f : Tn;
-                a.c0 += wgt * E.y;
-                a.c1 += wgt * E.z;
-                a.c2 += wgt * E.w;
-                a.W += wgt;
-                a.Z += wgt * (tn * inv);
+                float alpha[kLfPass], tau[kLfPass];
+                float4 E[kLfPass];
+#pragma unroll
+                for (int k = 0; k < kLfPass; ++k) {
+                    const bool has = G != 0u;
+                    const int j = has ? __ffs(G) - 1 : 0;
+                    G &= G - 1u;
+                    const int qi = lf_qi(j, sl);
+                    const float4 A = S.q[0][qi], B = S.q[1][qi], C = S.q[2][qi];
+                    const float2 U = S.t[lf_ti(j, sl)];
+                    E[k] = S.e[j];
+                    const bool in = has && (S.lanes[j] & bit) != 0u;
+                    const float2 q0 = fma2(hi2(A), xx, lo2(A)), q1 = fma2(hi2(B), xx, lo2(B));
+                    const float2 q2 = fma2(hi2(C), xx, lo2(C));
+                    const float tn = fmaf(U.y, x, U.x);
+                    const float2 q = fma2(q2, q2, fma2(q0, q0, mul2(q1, q1)));
+                    const float inv = __fdividef(1.f, q.y);
+                    const float rho = ex2_approx(-(q.x * inv));
+                    const float al = fminf(E[k].x * rho, P.alpha_max);
+                    alpha[k] = in && tn > 0.f && al >= P.alpha_min ? al : 0.f;
+                    tau[k] = tn * inv;
+                }
+#pragma unroll
+                for (int k = 0; k < kLfPass; ++k) {
+                    const float w = alpha[k] * a.T;
+                    const float Tn = __fsub_rn(a.T, w);
+                    const bool stop = Tn < P.t_min;
+                    const float wgt = stop ? 0.f : w;
+                    a.T = stop ? 0.f : Tn;
+                    a.c0 += wgt * E[k].y;
+                    a.c1 += wgt * E[k].z;
+                    a.c2 += wgt * E[k].w;
+                    a.W += wgt;
+                    a.Z += wgt * tau[k];
+                }
             }
         }
     }
