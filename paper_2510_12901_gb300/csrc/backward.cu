@@ -176,6 +176,8 @@ __device__ __forceinline__ void start_ray(RayGrad &r, const float4 *slot, const 
     r.U = gQ[0] * Q[0] + gQ[1] * Q[1] + gQ[2] * Q[2] + gQ[3] * Q[3] + gQ[4] * Q[4];
 }
 
+constexpr int kBwPass = 2;
+
 // ------------------------------------------------------------------ camera
 struct BwCam {                     // a warp's shared memory
     float4 e[8][32];               // staged entries (cam_entry's planes 0..7)
@@ -209,21 +211,29 @@ __device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose
     for (int b0 = 0; b0 < n; b0 += kBwBatch) {
         const int nb = min(kBwBatch, n - b0);
         uint32_t used = 0u;        // entries with a composited pair
-        for (int j = 0; j < nb; ++j) {
-            const int i = b0 + j;
-            PairEval pe;
-            bool ok = cam_pair_scaled(S.e[0][i], S.e[1][i], S.e[2][i], S.e[3][i], S.e[4][i],
-                                      S.e[5][i], S.e[6][i], (S.lanes[i] >> lane) & 1u, dd,
-                                      P.alpha_min, P.alpha_max, pe);
-            ok = ok && S.pos[i] <= last;
-            float2 wx = make_float2(0.f, 0.f);
-            if (ok) {
-                const float4 col = S.e[7][i];
-                const float q[3] = {col.x, col.y, col.z};
-                wx = ray_step(r, pe, q);
+        for (int j0 = 0; j0 < nb; j0 += kBwPass) {
+            PairEval pe[kBwPass];
+            bool ok[kBwPass];
+#pragma unroll
+            for (int k = 0; k < kBwPass; ++k) {
+                const int i = min(b0 + j0 + k, n - 1);
+                ok[k] = cam_pair_scaled(S.e[0][i], S.e[1][i], S.e[2][i], S.e[3][i], S.e[4][i],
+                                        S.e[5][i], S.e[6][i], (S.lanes[i] >> lane) & 1u, dd,
+                                        P.alpha_min, P.alpha_max, pe[k]);
+                ok[k] = ok[k] && S.pos[i] <= last && j0 + k < nb;
             }
-            S.wx[j][lane] = wx;
-            used |= (__any_sync(0xffffffffu, ok) ? 1u : 0u) << j;
+#pragma unroll
+            for (int k = 0; k < kBwPass; ++k) {
+                const int i = min(b0 + j0 + k, n - 1);
+                float2 wx = make_float2(0.f, 0.f);
+                if (ok[k]) {
+                    const float4 col = S.e[7][i];
+                    const float q[3] = {col.x, col.y, col.z};
+                    wx = ray_step(r, pe[k], q);
+                }
+                if (kBwPass == 1 || j0 + k < kBwBatch) S.wx[j0 + k][lane] = wx;
+                used |= (__any_sync(0xffffffffu, ok[k]) ? 1u : 0u) << (j0 + k);
+            }
         }
         __syncwarp();
         if (used == 0u) continue;
