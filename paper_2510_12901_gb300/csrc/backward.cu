@@ -276,6 +276,7 @@ k_backward_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__r
                   const float *__restrict__ g_alpha, const float *__restrict__ g_depth,
                   float *__restrict__ gacc)
 {
+    after_previous();
     __shared__ BwCam s_all[kBwWarps];
     __shared__ CamPose s_pose;
     load_cam_pose(D, s_pose);
@@ -416,6 +417,7 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
                      const float *__restrict__ g_alpha, const float *__restrict__ g_depth,
                      float *__restrict__ gacc)
 {
+    after_previous();
     __shared__ BwPosed s_all[kBwWarpsPosed];
     const int lane = threadIdx.x & 31;
     BwPosed &S = s_all[threadIdx.x >> 5];
@@ -535,6 +537,7 @@ k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
                  const float *__restrict__ g_int, const float *__restrict__ g_drop,
                  const float *__restrict__ g_alpha, float *__restrict__ gacc)
 {
+    after_previous();
     __shared__ BwPosed s_all[kBwWarpsPosed];
     const int lane = threadIdx.x & 31;
     BwPosed &S = s_all[threadIdx.x >> 5];
@@ -783,6 +786,7 @@ k_param_grads(const float *__restrict__ planes, int64_t pitch, int64_t n, int li
               float *__restrict__ gm, float *__restrict__ gls, float *__restrict__ gq,
               float *__restrict__ gop, float *__restrict__ gf)
 {
+    after_previous();
     constexpr int nc = kDeg < 0 ? 1 : (kDeg + 1) * (kDeg + 1), F = 3 * nc;
     constexpr int fs = F | 1;            // odd: a thread's row in banks of its own
     __shared__ float s_f[kPgThreads * fs], s_p[kPgThreads * 11];
@@ -987,7 +991,7 @@ static sg_status finish(const Scene &sc, Frame &fr, const float o[3], float beam
     if (sh_features(sc.feature_kind))
         kern = sc.sh_degree == 0 ? k_param_grads<0> : sc.sh_degree == 1 ? k_param_grads<1>
                : sc.sh_degree == 2 ? k_param_grads<2> : k_param_grads<3>;
-    kern<<<(unsigned)((sc.n + kPgThreads - 1) / kPgThreads), kPgThreads, 0, st>>>(
+    launch_after(kern, (unsigned)((sc.n + kPgThreads - 1) / kPgThreads), kPgThreads, 0, st,
         sc.d_planes, sc.pitch, sc.n, sc.feature_kind == SG_FEATURES_LIDAR_SH ? 1 : 0, o[0], o[1],
         o[2], (const GRec *)fr.rec.p, fr.d_lidar_poses, actor_params(sc), beam,
         fr.kind == 2 ? 1 : 0, (float *)fr.gacc.p, g.d_g_means, g.d_g_log_scales, g.d_g_quats,
@@ -1053,7 +1057,7 @@ sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const f
         if ((s = persistent_grid((const void *)k_backward_camera_rs, kBwWarpsPosed, ws.max_items,
                                  grid)) != SG_OK)
             return s;
-        k_backward_camera_rs<<<(unsigned)grid, 32 * kBwWarpsPosed, 0, st>>>(
+        launch_after(k_backward_camera_rs, (unsigned)grid, 32 * kBwWarpsPosed, 0, st,
             P, (const GRec *)fr.rec.p, (const uint32_t *)fr.pvals[fr.pair_buf].p,
             (const uint2 *)fr.ranges.p, (const uint2 *)(cw + ws.info_bytes + ws.off_bytes),
             (const uint2 *)cw, (const uint32_t *)fr.scalars.p + 4, (const uint32_t *)fr.submask.p,
@@ -1066,7 +1070,7 @@ sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const f
     }
     if ((s = persistent_grid((const void *)k_backward_camera, kBwWarps, ws.max_items, grid)) != SG_OK)
         return s;
-    k_backward_camera<<<(unsigned)grid, 32 * kBwWarps, 0, st>>>(
+    launch_after(k_backward_camera, (unsigned)grid, 32 * kBwWarps, 0, st,
         P, (const GRec *)fr.rec.p, (const uint32_t *)fr.pvals[fr.pair_buf].p,
         (const uint2 *)fr.ranges.p, (const uint2 *)(cw + ws.info_bytes + ws.off_bytes),
         (const uint2 *)cw, (const uint32_t *)fr.scalars.p + 4, (const uint32_t *)fr.submask.p,
@@ -1095,7 +1099,7 @@ sg_status backward_lidar(const Scene &sc, const Lidar &L, Frame &fr, const float
         if ((s = persistent_grid((const void *)k_backward_lidar, kBwWarpsPosed, ws.max_items, grid)) !=
             SG_OK)
             return s;
-        k_backward_lidar<<<(unsigned)grid, 32 * kBwWarpsPosed, 0, st>>>(
+        launch_after(k_backward_lidar, (unsigned)grid, 32 * kBwWarpsPosed, 0, st,
             P, L.d_items, L.d_item_rays, L.d_ray_e, L.d_tile_u, fr.d_lidar_poses,
             L.d_tile_items, (const uint32_t *)fr.lmask.p, fr.lmask_stride,
             (const GRec *)fr.rec.p, (const uint32_t *)fr.pvals[fr.pair_buf].p,

@@ -187,6 +187,7 @@ k_work_items(const uint2 *__restrict__ ranges, const uint2 *__restrict__ tile_it
              uint32_t *__restrict__ counter, uint2 *__restrict__ unit_info,
              uint2 *__restrict__ items, uint32_t *__restrict__ arrive)
 {
+    after_previous();
     // items per bucket: of all tiles, of the earlier blocks' tiles, handed out
     // by this block; the buckets' first items; partial slots likewise
     __shared__ uint32_t s_tot[34], s_pre[34], s_cur[34], s_base[34];
@@ -293,7 +294,7 @@ sg_status launch_work_items(Frame &fr, const WorkSize &ws, const Lidar *lidar, i
     const uint2 *ranges = (const uint2 *)fr.ranges.p;
     if (n_tiles <= kWorkOneTiles) {
         const unsigned g = (unsigned)((n_tiles + kWorkShare - 1) / kWorkShare);
-        k_work_items<<<g > 0 ? g : 1, kWorkThreads, 0, st>>>(
+        launch_after(k_work_items, g > 0 ? g : 1, kWorkThreads, 0, st,
             ranges, lidar ? lidar->d_tile_items : nullptr, n_tiles, subs, seg_len, counts, counter,
             unit_info, items, arrive);
         SG_LAUNCHED();
@@ -471,6 +472,7 @@ k_render_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__res
                 const RenderDesc *__restrict__ D, float4 *__restrict__ ray_state,
                 float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
+    after_previous();
     __shared__ float4 s_all[kCamWarps][8][32];
     __shared__ uint32_t s_pos[kCamWarps][32];
     __shared__ float s_refs[kCamWarps][6];
@@ -621,7 +623,7 @@ sg_status render_camera(const Camera &cam, const sg_render_opts &o, Frame &fr, c
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
     auto kern = dflt ? k_render_camera<kSegLen> : k_render_camera<kSegLenStatic>;
-    kern<<<(unsigned)grid, 32 * kCamWarps, 0, st>>>(
+    launch_after(kern, (unsigned)grid, 32 * kCamWarps, 0, st,
         P, (const GRec *)fr.rec.p, ids, (const uint2 *)fr.ranges.p, items, tile_info, counts,
         (const uint32_t *)fr.submask.p, counter, arrive, (float4 *)fr.partials.p, cam.d_pix,
         cam.d_tile_dir, (const RenderDesc *)fr.desc.p, saved_state(fr),
@@ -734,6 +736,7 @@ k_render_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__
                    const RenderDesc *__restrict__ D, float4 *__restrict__ ray_state,
                    float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
+    after_previous();
     __shared__ float4 s_all[kRsWarps][kLidPlanes][32];
     __shared__ EntryQueue<kWalkQueue> s_q[kRsWarps];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -862,7 +865,7 @@ sg_status render_camera_rs(const Camera &cam, const sg_render_opts &o, Frame &fr
     int64_t grid = (int64_t)sms * nb;
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
-    k_render_camera_rs<kSegLen><<<(unsigned)grid, 32 * kRsWarps, 0, st>>>(
+    launch_after(k_render_camera_rs<kSegLen>, (unsigned)grid, 32 * kRsWarps, 0, st,
         P, (const GRec *)fr.rec.p, ids, (const uint2 *)fr.ranges.p, items, tile_info, counts,
         (const uint32_t *)fr.submask.p, counter, arrive, (float4 *)fr.partials.p, cam.d_pix,
         cam.d_tile_dir, (const RenderDesc *)fr.desc.p, saved_state(fr),
@@ -1031,6 +1034,7 @@ k_render_lidar(LidRender P, const LidarItem *__restrict__ items,
                const RenderDesc *__restrict__ D, float4 *__restrict__ ray_state,
                float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
+    after_previous();
     __shared__ float4 s_all[kLidarWarps][kLidPlanes][32];
     __shared__ EntryQueue<kWalkQueue> s_q[kLidarWarps];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1189,7 +1193,7 @@ sg_status render_lidar(const Lidar &L, const sg_render_opts &o, Frame &fr, cudaS
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
     const FixList F = fix_list(fr, ws);
-    k_render_lidar<false><<<(unsigned)grid, 32 * kLidarWarps, 0, st>>>(
+    launch_after(k_render_lidar<false>, (unsigned)grid, 32 * kLidarWarps, 0, st,
         P, L.d_items, L.d_item_rays, L.d_ray_e, L.d_tile_u, L.d_tile_items,
         (const uint32_t *)fr.lmask.p, fr.lmask_stride,
         (const GRec *)fr.rec.p, ids, (const uint2 *)fr.ranges.p, work, unit_info,
@@ -1200,7 +1204,7 @@ sg_status render_lidar(const Lidar &L, const sg_render_opts &o, Frame &fr, cudaS
     if (ws.max_slots > 0) {       // some item may be split: the deferred re-walks
         const int64_t fcap = (ws.max_fixes + kLidarWarps - 1) / kLidarWarps;
         const int64_t fgrid = grid < fcap ? grid : fcap;
-        k_render_lidar<true><<<(unsigned)fgrid, 32 * kLidarWarps, 0, st>>>(
+        launch_after(k_render_lidar<true>, (unsigned)fgrid, 32 * kLidarWarps, 0, st,
             P, L.d_items, L.d_item_rays, L.d_ray_e, L.d_tile_u, L.d_tile_items,
             (const uint32_t *)fr.lmask.p, fr.lmask_stride,
             (const GRec *)fr.rec.p, ids, (const uint2 *)fr.ranges.p, work, unit_info,

@@ -363,6 +363,7 @@ k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *_
                     const float4 *__restrict__ pix2, const double *__restrict__ tile_dir,
                     const float *__restrict__ tile_basis, const RenderDesc *__restrict__ D)
 {
+    after_previous();
     __shared__ float4 s_all[kFwdWarps][7][kFwdStage];
     __shared__ uint2 s_cand[kFwdWarps][kFwdQueue];
     __shared__ __align__(16) float s_refs[kFwdWarps][12 + kRegion];
@@ -529,7 +530,7 @@ sg_status render_camera_fwd(const Camera &cam, const sg_render_opts &o, Frame &f
     int64_t grid = (int64_t)sms * fwd_blocks_per_sm();
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
-    k_render_camera_fwd<kFwdSeg><<<(unsigned)grid, 32 * kFwdWarps, 0, st>>>(
+    launch_after(k_render_camera_fwd<kFwdSeg>, (unsigned)grid, 32 * kFwdWarps, 0, st,
         P, (const GRec *)fr.rec.p, ids, (const uint2 *)fr.ranges.p, items, tile_info, counts,
         (const uint32_t *)fr.submask.p, counter, arrive, (float4 *)fr.partials.p, cam.d_pix2,
         cam.d_tile_dir, cam.d_tile_basis, (const RenderDesc *)fr.desc.p);

@@ -261,6 +261,7 @@ k_render_lidar_fwd(LidRender P, const LidarItem *__restrict__ items,
                    uint32_t *__restrict__ counter, uint32_t *__restrict__ arrive,
                    float4 *__restrict__ partials, FixList F, const RenderDesc *__restrict__ D)
 {
+    after_previous();
     __shared__ LfShared s_all[kLfWarps];
     const int lane = threadIdx.x & 31;
     LfShared &S = s_all[threadIdx.x >> 5];
@@ -430,7 +431,7 @@ sg_status render_lidar_fwd(const Lidar &L, const sg_render_opts &o, Frame &fr, c
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
     const FixList F = fix_list(fr, ws);
-    k_render_lidar_fwd<false><<<(unsigned)grid, 32 * kLfWarps, 0, st>>>(
+    launch_after(k_render_lidar_fwd<false>, (unsigned)grid, 32 * kLfWarps, 0, st,
         P, L.d_items, L.d_item_rays, L.d_ray_tau, L.d_item_ref, L.d_tile_items,
         (const uint32_t *)fr.lmask.p, fr.lmask_stride, (const GRec *)fr.rec.p, ids,
         (const uint2 *)fr.ranges.p, work, unit_info, (const uint32_t *)fr.scalars.p + 4,
@@ -440,7 +441,7 @@ sg_status render_lidar_fwd(const Lidar &L, const sg_render_opts &o, Frame &fr, c
     if (ws.max_slots > 0) {       // some item may be split: the deferred re-walks
         const int64_t fcap = (ws.max_fixes + kLfWarps - 1) / kLfWarps;
         const int64_t fgrid = grid < fcap ? grid : fcap;
-        k_render_lidar_fwd<true><<<(unsigned)fgrid, 32 * kLfWarps, 0, st>>>(
+        launch_after(k_render_lidar_fwd<true>, (unsigned)fgrid, 32 * kLfWarps, 0, st,
             P, L.d_items, L.d_item_rays, L.d_ray_tau, L.d_item_ref, L.d_tile_items,
             (const uint32_t *)fr.lmask.p, fr.lmask_stride, (const GRec *)fr.rec.p, ids,
             (const uint2 *)fr.ranges.p, work, unit_info, (const uint32_t *)fr.scalars.p + 4,

@@ -153,6 +153,7 @@ k_onesweep(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ va
            const uint32_t *__restrict__ hist, uint32_t *__restrict__ lookback,
            uint32_t *__restrict__ ticket, uint32_t *__restrict__ err, int site)
 {
+    after_previous();
     // the warps' digit counts, then the look-back groups' sums
     __shared__ __align__(16) union {
         uint16_t cnt[kRadixWarps][256];
@@ -336,7 +337,7 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
         const int b = radix_bit(begin_bit, end_bit, p);
         const int bits = radix_bit(begin_bit, end_bit, p + 1) - b;
         uint32_t *keys_out = p == passes - 1 && !keep_keys ? nullptr : keys[cur ^ 1];
-        k_onesweep<<<(unsigned)tiles, kRadixThreads, 0, st>>>(
+        launch_after(k_onesweep, (unsigned)tiles, kRadixThreads, 0, st,
             keys[cur], vals[cur], keys_out, vals[cur ^ 1], d_n, b, (1u << bits) - 1u,
             hist + 256 * p, lookback + (int64_t)p * tiles * 256, tickets + p, d_err, site);
         SG_LAUNCHED();
@@ -455,6 +456,7 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
                 unsigned long long *__restrict__ lb, uint32_t *__restrict__ ticket,
                 uint32_t *__restrict__ err, uint4 *__restrict__ zero, int64_t nzero)
 {
+    after_previous();
     __shared__ uint32_t s_h[4][256];
     __shared__ ChainShared S;
     // the tile sort's scratch, zeroed here rather than by a launch of its own
@@ -525,6 +527,7 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
                uint32_t *__restrict__ ticket, uint32_t *__restrict__ err,
                uint32_t *__restrict__ owner, int64_t owner_cap)
 {
+    after_previous();
     constexpr int kOffTile = kOffChunks * kChainThreads;
     __shared__ ChainShared S;
     if (threadIdx.x == 0) S.tile = atomicAdd(ticket, 1u);
@@ -622,7 +625,7 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     unsigned long long *chain = (unsigned long long *)(hist + radix_scratch_words(n, 4));
     uint32_t *tickets = (uint32_t *)chain;                 // [0] compaction, [1] offsets
     uint32_t *err = (uint32_t *)fr.scalars.p + kScalStatus;
-    k_compact_depth<<<(unsigned)ntiles, kChainThreads, 0, st>>>(
+    launch_after(k_compact_depth, (unsigned)ntiles, kChainThreads, 0, st,
         d_count, d_depth, n, ntiles, keys[0], vals[0], d_scal, hist, chain + 2, tickets, err,
         (uint4 *)fr.tscratch.p, (int64_t)(fr.tscratch.bytes / 16));
     SG_LAUNCHED();
@@ -634,7 +637,7 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     const bool small = n <= kOffSmallN;
     const int64_t off_tile = (int64_t)kChainThreads * (small ? kOffSmall : kOffLarge);
     auto k_off = small ? k_pair_offsets<kOffSmall> : k_pair_offsets<kOffLarge>;
-    k_off<<<(unsigned)((n + off_tile - 1) / off_tile), kChainThreads, 0, st>>>(
+    launch_after(k_off, (unsigned)((n + off_tile - 1) / off_tile), kChainThreads, 0, st,
         vals[*result_buf], d_count, n, d_scal, d_offsets, d_scal + 1, chain + 2 + ntiles,
         tickets + 1, err, (uint32_t *)fr.owner.p, (int64_t)(fr.owner.bytes / 4));
     SG_LAUNCHED();
@@ -678,6 +681,7 @@ k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
       const uint32_t *__restrict__ owner, int64_t owner_cap, uint2 *__restrict__ ranges,
       int64_t ntiles)
 {
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * kBinThreads + threadIdx.x; i < ntiles;
          i += (int64_t)gridDim.x * kBinThreads)
         ranges[i] = make_uint2(0u, 0u);     // every tile's list empty, for the tile ranges
@@ -807,7 +811,7 @@ sg_status bin_pairs(const uint32_t *d_ids, const uint32_t *d_offsets, const uint
         set_error("internal: %d-bit tile ids", end_bit);
         return SG_ERR_INVALID;
     }
-    k_bin<<<(unsigned)((cap + kBinChunk - 1) / kBinChunk), kBinThreads, 0, st>>>(
+    launch_after(k_bin, (unsigned)((cap + kBinChunk - 1) / kBinChunk), kBinThreads, 0, st,
         d_ids, d_offsets, d_nvalid, d_tiles, ntx, wrap_x, (uint32_t)cap, d_keys, d_vals, d_hist,
         end_bit, d_err, (const uint32_t *)owner.p, (int64_t)(owner.bytes / 4), d_ranges, ntiles);
     SG_LAUNCHED();
@@ -888,6 +892,7 @@ k_ranges(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K,
          const float4 *__restrict__ rects, int ntx, float inv_ntx, uint32_t *__restrict__ mask,
          const uint32_t *__restrict__ err)
 {
+    after_previous();
     const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRangePer;
     const int64_t K = *d_K;
     if (i0 >= K || *err) return;
@@ -927,10 +932,10 @@ sg_status tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max
     if (K_max == 0) return SG_OK;
     const unsigned grid = (unsigned)((K_max + 256 * kRangePer - 1) / (256 * kRangePer));
     if (d_words)
-        k_ranges<true><<<grid, 256, 0, st>>>(d_keys, d_K, d_ranges, d_ids, d_rects, ntx,
+        launch_after(k_ranges<true>, grid, 256, 0, st, d_keys, d_K, d_ranges, d_ids, d_rects, ntx,
                                              1.f / (float)ntx, d_words, d_err);
     else
-        k_ranges<false><<<grid, 256, 0, st>>>(d_keys, d_K, d_ranges, nullptr, nullptr, 0, 0.f,
+        launch_after(k_ranges<false>, grid, 256, 0, st, d_keys, d_K, d_ranges, nullptr, nullptr, 0, 0.f,
                                               nullptr, d_err);
     SG_LAUNCHED();
     return SG_OK;
@@ -954,6 +959,7 @@ k_ranges_lidar(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d
                const LidarItemRays *__restrict__ tab, uint32_t *__restrict__ lmask,
                const uint32_t *__restrict__ err)
 {
+    after_previous();
     const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRangePer;
     const int64_t K = *d_K;
     if (i0 >= K || *err) return;
@@ -1026,7 +1032,7 @@ sg_status lidar_tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t
 {
     if (K_max == 0) return SG_OK;
     const unsigned grid = (unsigned)((K_max + 256 * kRangePer - 1) / (256 * kRangePer));
-    k_ranges_lidar<<<grid, 256, 0, st>>>(
+    launch_after(k_ranges_lidar, grid, 256, 0, st,
         d_keys, d_K, lmask_stride, d_ranges, d_ids, d_rects, L.d_tile_items, L.d_item_ray_tab,
         d_lmask, d_err);
     SG_LAUNCHED();
@@ -1038,6 +1044,7 @@ sg_status lidar_tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t
 __global__ void k_clamp_pairs(uint32_t *__restrict__ d_K, uint32_t cap,
                               uint32_t *__restrict__ d_dropped)
 {
+    after_previous();
     const uint32_t K = *d_K;
     *d_dropped = K > cap ? K - cap : 0u;
     if (K > cap) *d_K = cap;
@@ -1045,7 +1052,7 @@ __global__ void k_clamp_pairs(uint32_t *__restrict__ d_K, uint32_t cap,
 
 sg_status clamp_pairs(uint32_t *d_K, int64_t cap, uint32_t *d_dropped, cudaStream_t st)
 {
-    k_clamp_pairs<<<1, 1, 0, st>>>(d_K, (uint32_t)cap, d_dropped);
+    launch_after(k_clamp_pairs, 1, 1, 0, st, d_K, (uint32_t)cap, d_dropped);
     SG_LAUNCHED();
     return SG_OK;
 }
