@@ -8,7 +8,7 @@
 
 #include <atomic>
 #include <new>
-
+#include <thread>
 #include <vector>
 
 #include "internal.h"
@@ -266,6 +266,7 @@ static sg_status frame_prepare(Frame &fr, int64_t n, int64_t nrays, int64_t ntil
             set_error("pinned allocation failed");
             return SG_ERR_OOM;
         }
+        memset(fr.h_scalars, 0, 512);     // no render has sequence number 0
         fr.h_desc = (RenderDesc *)((char *)fr.h_scalars + 256);
     }
     if (!fr.ev_count && cudaEventCreateWithFlags(&fr.ev_count, cudaEventDisableTiming) != cudaSuccess) {
@@ -305,14 +306,18 @@ static sg_status sort_and_count(Frame &fr, int64_t n, cudaStream_t st)
     uint32_t *dk[2] = {(uint32_t *)fr.dkeys[0].p, (uint32_t *)fr.dkeys[1].p};
     uint32_t *dv[2] = {(uint32_t *)fr.dvals[0].p, (uint32_t *)fr.dvals[1].p};
     int rb = 0;
+    fr.count_told = fr.k_cap == 0 && n > 0;
+    if (fr.count_told && ++fr.count_seq == 0) fr.count_seq = 1;
     sg_status s = depth_stage((const uint32_t *)fr.count.p, (const float *)fr.depth.p, n, dk, dv,
-                              sc, (uint32_t *)fr.offsets.p, fr, st, &rb);
+                              sc, (uint32_t *)fr.offsets.p, fr, st, &rb,
+                              fr.count_told ? fr.count_seq : 0u);
     if (s != SG_OK) return s;
     fr.depth_buf = rb;
     tmark(fr, 2, st);
     if (fr.k_cap > 0) return clamp_pairs(sc + 1, fr.k_cap, sc + 3, st);
-    // the counts and the status word in one copy
-    SG_CUDA(cudaMemcpyAsync(fr.h_scalars, sc, 4 * (kScalStatus + 1), cudaMemcpyDeviceToHost, st));
+    // the counts and the status word in one copy, unless the kernel has sent them
+    if (!fr.count_told)
+        SG_CUDA(cudaMemcpyAsync(fr.h_scalars, sc, 4 * (kScalStatus + 1), cudaMemcpyDeviceToHost, st));
     SG_CUDA(cudaEventRecord(fr.ev_count, st));
     return SG_OK;
 }
@@ -326,6 +331,34 @@ static const char *status_cause(uint32_t w)
     return "a look-back wait of the sort gave up";
 }
 
+// Wait until the counts of the render are in h_scalars.  k_pair_offsets writes
+// them there itself and the host polls the sequence number: a copy and an event
+// behind the kernel and waking up from its wait cost 10 us more (64x64 97 -> 88
+// us a render, 641x479 156 -> 149, street sweep 729 -> 717).  The event, asked
+// now and then, ends the wait if the kernel failed.
+static sg_status wait_count(Frame &fr)
+{
+    if (!fr.count_told) {
+        SG_CUDA(cudaEventSynchronize(fr.ev_count));
+        return SG_OK;
+    }
+    for (uint32_t spin = 1;; ++spin) {
+        if (__atomic_load_n(fr.h_scalars + kHostCountSeq, __ATOMIC_ACQUIRE) == fr.count_seq)
+            return SG_OK;
+        if (spin % 4096 != 0) continue;
+        const cudaError_t e = cudaEventQuery(fr.ev_count);
+        if (e == cudaErrorNotReady) {
+            std::this_thread::yield();
+            continue;
+        }
+        if (e != cudaSuccess) return cuda_status(e, "waiting for the pair count");
+        if (__atomic_load_n(fr.h_scalars + kHostCountSeq, __ATOMIC_ACQUIRE) == fr.count_seq)
+            return SG_OK;
+        set_error("internal: the pair count did not reach the host");
+        return SG_ERR_CUDA;
+    }
+}
+
 // bin_and_sort: waits for the pair count (exact mode), which sizes the pair
 // buffers, then binning, tile sort and ranges; in capacity mode nothing
 // waits and the scalars are copied to h_scalars at the end for the caller
@@ -335,10 +368,11 @@ static sg_status bin_and_sort(Frame &fr, int64_t n, int ntx, int64_t ntiles, int
 {
     uint32_t *sc = (uint32_t *)fr.scalars.p;
     int64_t K = 0;
+    sg_status s;
     if (fr.k_cap > 0) {
         K = fr.k_cap;
     } else {
-        SG_CUDA(cudaEventSynchronize(fr.ev_count));
+        if ((s = wait_count(fr)) != SG_OK) return s;
         if (fr.h_scalars[kScalStatus]) {
             set_error("%s before the pair count (device status word set)",
                       status_cause(fr.h_scalars[kScalStatus]));
@@ -351,7 +385,6 @@ static sg_status bin_and_sort(Frame &fr, int64_t n, int ntx, int64_t ntiles, int
         }
     }
     fr.n_pairs = K;
-    sg_status s;
     for (int i = 0; i < 2; ++i) {
         if ((s = ensure(fr.pkeys[i], sizeof(uint32_t) * (K > 0 ? K : 1))) != SG_OK) return s;
         if ((s = ensure(fr.pvals[i], sizeof(uint32_t) * (K > 0 ? K : 1))) != SG_OK) return s;

@@ -285,6 +285,8 @@ struct Frame {
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     float ms[4] = {0, 0, 0, 0};
     cudaEvent_t ev_count = nullptr;  // exact mode: the pair count has reached h_scalars
+    uint32_t count_seq = 0;         // sequence number of the last render that counts (0: none)
+    bool count_told = false;        // k_pair_offsets writes its counts to h_scalars itself
     Buf host_stage[3];               // device results of a render with host outputs
     cudaStream_t copy_st = nullptr;  // their copies to the host run here, off the view's stream
     cudaEvent_t ev_rendered = nullptr, ev_copied = nullptr;
@@ -316,6 +318,9 @@ constexpr uint32_t kStatusBulkCopy = 2u;
 // Pinned-mirror slots (frame h_scalars) of the status word read after the
 // render: by sg_frame_status, and with the host-output copies.
 constexpr int kHostStatusQuery = 12, kHostStatusOutputs = 13;
+// The pinned slot that k_pair_offsets sets to the render's sequence number once
+// the counts and the status word are there.
+constexpr int kHostCountSeq = 14;
 
 // Upper bounds of the compositing work-item buffers.  A unit (a camera
 // tile, or a LiDAR work item of up to 32 rays of one tile) whose list holds
@@ -407,7 +412,7 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n, cons
 // = the pair total.  Its scratch (fr.hist) was zeroed by the projection.
 sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, uint32_t *keys[2],
                       uint32_t *vals[2], uint32_t *d_scal, uint32_t *d_offsets, Frame &fr,
-                      cudaStream_t st, int *result_buf);
+                      cudaStream_t st, int *result_buf, uint32_t host_seq = 0);
 // With d_hist (in the tile sort's zeroed scratch), k_bin also counts the
 // digits of the tile sort over end_bit bits, for radix_sort_pairs.  d_err: the
 // frame's status word (no pair is written once it is set).  It also empties

@@ -519,13 +519,26 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
     }
 }
 
+// The counts and the status word so far to the frame's pinned words (host; NULL:
+// nobody waits for them), the sequence number last.
+__device__ __forceinline__ void tell_host(volatile uint32_t *host, uint32_t nvalid, uint32_t pairs,
+                                          uint32_t status, uint32_t seq)
+{
+    if (!host) return;
+    host[0] = nvalid;
+    host[1] = pairs;
+    host[kScalStatus] = status;
+    __threadfence_system();
+    host[kHostCountSeq] = seq;
+}
+
 template <int kOffChunks>
 __global__ void __launch_bounds__(kChainThreads)
 k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ count, int64_t n,
                const uint32_t *__restrict__ d_nvalid, uint32_t *__restrict__ offsets,
                uint32_t *__restrict__ d_total, unsigned long long *__restrict__ lb,
                uint32_t *__restrict__ ticket, uint32_t *__restrict__ err,
-               uint32_t *__restrict__ owner, int64_t owner_cap)
+               uint32_t *__restrict__ owner, int64_t owner_cap, volatile uint32_t *host, uint32_t seq)
 {
     after_previous();
     constexpr int kOffTile = kOffChunks * kChainThreads;
@@ -536,7 +549,10 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
     const int64_t tile = S.tile;
     const int64_t ntiles = (nv + kOffTile - 1) / kOffTile;
     if (nv == 0) {
-        if (tile == 0 && threadIdx.x == 0) *d_total = 0u;
+        if (tile == 0 && threadIdx.x == 0) {
+            *d_total = 0u;
+            tell_host(host, 0u, 0u, *(volatile uint32_t *)err, seq);
+        }
         return;
     }
     if (tile >= ntiles) return;   // so is every later tile: nobody waits for this one
@@ -576,7 +592,9 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
     if (threadIdx.x == 0 && tile == ntiles - 1) {
         // saturated, so that a total of 2^32 pairs or more reads as an overflow
         const unsigned long long tot = excl + total;
-        *d_total = tot > 0xffffffffull ? 0xffffffffu : (uint32_t)tot;
+        const uint32_t sat = tot > 0xffffffffull ? 0xffffffffu : (uint32_t)tot;
+        *d_total = sat;
+        tell_host(host, (uint32_t)nv, sat, *(volatile uint32_t *)err, seq);
     }
     const uint32_t pre = (uint32_t)excl + before;
 #pragma unroll
@@ -600,7 +618,7 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
 
 sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, uint32_t *keys[2],
                       uint32_t *vals[2], uint32_t *d_scal, uint32_t *d_offsets, Frame &fr,
-                      cudaStream_t st, int *result_buf)
+                      cudaStream_t st, int *result_buf, uint32_t host_seq)
 {
     *result_buf = 0;
     fr.tscratch_zeroed = 0;
@@ -639,7 +657,8 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     auto k_off = small ? k_pair_offsets<kOffSmall> : k_pair_offsets<kOffLarge>;
     launch_after(k_off, (unsigned)((n + off_tile - 1) / off_tile), kChainThreads, 0, st,
         vals[*result_buf], d_count, n, d_scal, d_offsets, d_scal + 1, chain + 2 + ntiles,
-        tickets + 1, err, (uint32_t *)fr.owner.p, (int64_t)(fr.owner.bytes / 4));
+        tickets + 1, err, (uint32_t *)fr.owner.p, (int64_t)(fr.owner.bytes / 4),
+        host_seq ? (volatile uint32_t *)fr.h_scalars : nullptr, host_seq);
     SG_LAUNCHED();
     return SG_OK;
 }
