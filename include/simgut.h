@@ -433,6 +433,14 @@ sg_status sg_backward_camera(sg_scene scene, sg_frame frame, const float *d_g_rg
 sg_status sg_backward_lidar(sg_scene scene, sg_frame frame, const float *d_g_range,
                             const float *d_g_intensity, const float *d_g_drop,
                             const float *d_g_alpha, const sg_grads *grads, void *stream);
+/* The same gradients, written over whatever the arrays hold (every element,
+ * 0 where a Gaussian has none), so that the caller need not zero them. */
+sg_status sg_backward_camera_write(sg_scene scene, sg_frame frame, const float *d_g_rgb,
+                                   const float *d_g_alpha, const float *d_g_depth,
+                                   const sg_grads *grads, void *stream);
+sg_status sg_backward_lidar_write(sg_scene scene, sg_frame frame, const float *d_g_range,
+                                  const float *d_g_intensity, const float *d_g_drop,
+                                  const float *d_g_alpha, const sg_grads *grads, void *stream);
 
 /* ----------------------------------------------------------------------
  * Request server (continuous batching).  Scenes and sensors are created as

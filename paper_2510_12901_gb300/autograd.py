@@ -3,7 +3,7 @@
 ``render_camera(params, scene, cam, c2w)`` and ``render_lidar(...)`` copy the
 parameter tensors into the library's resident scene (sg_update_scene),
 render through the C-ABI and return outputs whose backward calls
-sg_backward_camera / sg_backward_lidar.  Gradients flow to ``means``,
+sg_backward_camera_write / sg_backward_lidar_write.  Gradients flow to ``means``,
 ``log_scales``, ``quats``, ``opacity`` and ``features``; the unscented
 projection only selects tiles and carries no gradient (Sec. 3.2).
 """
@@ -33,17 +33,18 @@ class _RenderCamera(torch.autograd.Function):
         sg.sg_render_camera(scene.handle, cam.handle, c2w, opts, frame.handle, rgb.data_ptr(),
                             alpha.data_ptr(), depth.data_ptr(), stream)
         ctx.scene, ctx.frame = scene, frame
+        ctx.set_materialize_grads(False)    # an output without a gradient: NULL, not zeros
         ctx.shapes = [t.shape for t in ts]
         return rgb, alpha, depth
 
     @staticmethod
     def backward(ctx, g_rgb, g_alpha, g_depth):
-        dev = g_rgb.device if g_rgb is not None else g_alpha.device
-        grads = [torch.zeros(s, device=dev) for s in ctx.shapes]
+        ref = next(g for g in (g_rgb, g_alpha, g_depth) if g is not None)
+        grads = [torch.empty(s, device=ref.device) for s in ctx.shapes]
         gs = sg.sg_grads(*[g.data_ptr() for g in grads])
         ups = [None if g is None else g.contiguous() for g in (g_rgb, g_alpha, g_depth)]
-        sg.sg_backward_camera(ctx.scene.handle, ctx.frame.handle, *[_ptr(u) for u in ups], gs,
-                              torch.cuda.current_stream().cuda_stream)
+        sg.sg_backward_camera_write(ctx.scene.handle, ctx.frame.handle, *[_ptr(u) for u in ups],
+                                    gs, torch.cuda.current_stream().cuda_stream)
         return (*grads, None, None, None, None, None)
 
 
@@ -58,17 +59,18 @@ class _RenderLidar(torch.autograd.Function):
         sg.sg_render_lidar(scene.handle, lid.handle, poses.data_ptr(), opts, frame.handle,
                            *[o.data_ptr() for o in outs], stream)
         ctx.scene, ctx.frame, ctx.poses = scene, frame, poses
+        ctx.set_materialize_grads(False)
         ctx.shapes = [t.shape for t in ts]
         return tuple(outs)
 
     @staticmethod
     def backward(ctx, g_range, g_int, g_drop, g_alpha):
         ref = next(g for g in (g_range, g_int, g_drop, g_alpha) if g is not None)
-        grads = [torch.zeros(s, device=ref.device) for s in ctx.shapes]
+        grads = [torch.empty(s, device=ref.device) for s in ctx.shapes]
         gs = sg.sg_grads(*[g.data_ptr() for g in grads])
         ups = [None if g is None else g.contiguous() for g in (g_range, g_int, g_drop, g_alpha)]
-        sg.sg_backward_lidar(ctx.scene.handle, ctx.frame.handle, *[_ptr(u) for u in ups], gs,
-                             torch.cuda.current_stream().cuda_stream)
+        sg.sg_backward_lidar_write(ctx.scene.handle, ctx.frame.handle, *[_ptr(u) for u in ups],
+                                   gs, torch.cuda.current_stream().cuda_stream)
         return (*grads, None, None, None, None, None)
 
 

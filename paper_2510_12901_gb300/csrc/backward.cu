@@ -733,6 +733,23 @@ __device__ __forceinline__ void sh_basis_grad(float x, float y, float z,
 
 constexpr int kPgThreads = 128;     // Gaussians per block of k_param_grads
 
+// Write zeros (s NULL) or the block's rows of C floats, staged at s + row *
+// stride, to out (rows g0 .. g0 + ng - 1 of [n, C]).
+template <int C>
+__device__ __forceinline__ void put_rows(float *__restrict__ out, int64_t g0, int ng,
+                                         const float *s, int stride)
+{
+    if (!out) return;
+    float *p = out + g0 * C;
+    const int tot = ng * C;
+    const int v4 = ((uintptr_t)out & 15u) == 0 ? tot / 4 : 0;   // then p is aligned, too
+    auto at = [&](int i) { return s ? s[(i / C) * stride + i % C] : 0.f; };
+    for (int j = threadIdx.x; j < v4; j += kPgThreads)
+        reinterpret_cast<float4 *>(p)[j] =
+            make_float4(at(4 * j), at(4 * j + 1), at(4 * j + 2), at(4 * j + 3));
+    for (int j = 4 * v4 + threadIdx.x; j < tot; j += kPgThreads) p[j] = at(j);
+}
+
 // Add the block's rows of C floats, staged at s + row * stride, to out (rows
 // g0 .. g0 + ng - 1 of [n, C]); a group of four floats is skipped if no row in
 // it has a gradient (any: a bit a row).
@@ -777,8 +794,10 @@ __device__ __forceinline__ void add_rows(float *__restrict__ out, int64_t g0, in
 // rows, staged in shared memory and added with 16-byte accesses: one thread
 // adding its own 192-byte row 4 bytes at a time, with the SH planes read twice
 // and the basis in local memory, took 365 us for 1M Gaussians, now 182 (LiDAR
-// features, 2M: 136 -> 96).
-template <int kDeg>
+// features, 2M: 136 -> 96).  kWrite: the arrays' old contents do not count and
+// every row is written, nothing read: 95 and 68 us, and the caller's fills (39 and
+// 22 us) are gone.
+template <int kDeg, bool kWrite>
 __global__ void __launch_bounds__(kPgThreads)
 k_param_grads(const float *__restrict__ planes, int64_t pitch, int64_t n, int lidar, float ox,
               float oy, float oz, const GRec *__restrict__ rec, const float *__restrict__ poses,
@@ -808,7 +827,16 @@ k_param_grads(const float *__restrict__ planes, int64_t pitch, int64_t n, int li
                      a2.z != 0.f || a2.w != 0.f || a3 != 0.f;
     const uint32_t bits = __ballot_sync(0xffffffffu, any);
     if ((t & 31) == 0) s_any[t >> 5] = bits;
-    if (!__syncthreads_or(any)) return;
+    if (!__syncthreads_or(any)) {
+        if constexpr (kWrite) {
+            put_rows<F>(gf, g0, ng, nullptr, 0);
+            put_rows<3>(gm, g0, ng, nullptr, 0);
+            put_rows<3>(gls, g0, ng, nullptr, 0);
+            put_rows<4>(gq, g0, ng, nullptr, 0);
+            put_rows<1>(gop, g0, ng, nullptr, 0);
+        }
+        return;
+    }
     float *fo = s_f + t * fs, *po = s_p + t * 11;     // means 3, log-scales 3, quaternion 4, opacity
     if (!any) {
 #pragma unroll
@@ -976,21 +1004,36 @@ k_param_grads(const float *__restrict__ planes, int64_t pitch, int64_t n, int li
         po[0] = gmu[0]; po[1] = gmu[1]; po[2] = gmu[2];
     }
     __syncthreads();
-    add_rows<F>(gf, g0, ng, s_f, fs, s_any);
-    add_rows<3>(gm, g0, ng, s_p, 11, s_any);
-    add_rows<3>(gls, g0, ng, s_p + 3, 11, s_any);
-    add_rows<4>(gq, g0, ng, s_p + 6, 11, s_any);
-    add_rows<1>(gop, g0, ng, s_p + 10, 11, s_any);
+    if constexpr (kWrite) {
+        put_rows<F>(gf, g0, ng, s_f, fs);
+        put_rows<3>(gm, g0, ng, s_p, 11);
+        put_rows<3>(gls, g0, ng, s_p + 3, 11);
+        put_rows<4>(gq, g0, ng, s_p + 6, 11);
+        put_rows<1>(gop, g0, ng, s_p + 10, 11);
+    } else {
+        add_rows<F>(gf, g0, ng, s_f, fs, s_any);
+        add_rows<3>(gm, g0, ng, s_p, 11, s_any);
+        add_rows<3>(gls, g0, ng, s_p + 3, 11, s_any);
+        add_rows<4>(gq, g0, ng, s_p + 6, 11, s_any);
+        add_rows<1>(gop, g0, ng, s_p + 10, 11, s_any);
+    }
+}
+
+template <bool kWrite>
+static auto param_kernel(const Scene &sc)
+{
+    if (!sh_features(sc.feature_kind)) return k_param_grads<-1, kWrite>;
+    return sc.sh_degree == 0   ? k_param_grads<0, kWrite>
+           : sc.sh_degree == 1 ? k_param_grads<1, kWrite>
+           : sc.sh_degree == 2 ? k_param_grads<2, kWrite>
+                               : k_param_grads<3, kWrite>;
 }
 
 static sg_status finish(const Scene &sc, Frame &fr, const float o[3], float beam,
-                        const sg_grads &g, cudaStream_t st)
+                        const sg_grads &g, bool write, cudaStream_t st)
 {
     if (sc.n == 0) return SG_OK;
-    auto kern = k_param_grads<-1>;
-    if (sh_features(sc.feature_kind))
-        kern = sc.sh_degree == 0 ? k_param_grads<0> : sc.sh_degree == 1 ? k_param_grads<1>
-               : sc.sh_degree == 2 ? k_param_grads<2> : k_param_grads<3>;
+    auto kern = write ? param_kernel<true>(sc) : param_kernel<false>(sc);
     launch_after(kern, (unsigned)((sc.n + kPgThreads - 1) / kPgThreads), kPgThreads, 0, st,
         sc.d_planes, sc.pitch, sc.n, sc.feature_kind == SG_FEATURES_LIDAR_SH ? 1 : 0, o[0], o[1],
         o[2], (const GRec *)fr.rec.p, fr.d_lidar_poses, actor_params(sc), beam,
@@ -1038,7 +1081,7 @@ static sg_status persistent_grid(const void *kern, int warps, int64_t max_items,
 
 sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const float *g_rgb,
                           const float *g_alpha, const float *g_depth, const sg_grads &g,
-                          cudaStream_t st)
+                          bool write, cudaStream_t st)
 {
     if (fr.seg_len != kSegLen) {
         set_error("sg_backward_camera: the frame's render used another list segment length");
@@ -1066,7 +1109,7 @@ sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const f
             (const uint32_t *)fr.n_contrib.p, g_rgb, g_alpha, g_depth, (float *)fr.gacc.p);
         SG_LAUNCHED();
         const float o[3] = {0.f, 0.f, 0.f};
-        return finish(sc, fr, o, 0.f, g, st);
+        return finish(sc, fr, o, 0.f, g, write, st);
     }
     if ((s = persistent_grid((const void *)k_backward_camera, kBwWarps, ws.max_items, grid)) != SG_OK)
         return s;
@@ -1080,12 +1123,12 @@ sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr, const f
         g_depth, (float *)fr.gacc.p);
     SG_LAUNCHED();
     const float o[3] = {fr.c2w[3], fr.c2w[7], fr.c2w[11]};
-    return finish(sc, fr, o, 0.f, g, st);
+    return finish(sc, fr, o, 0.f, g, write, st);
 }
 
 sg_status backward_lidar(const Scene &sc, const Lidar &L, Frame &fr, const float *g_range,
                          const float *g_int, const float *g_drop, const float *g_alpha,
-                         const sg_grads &g, cudaStream_t st)
+                         const sg_grads &g, bool write, cudaStream_t st)
 {
     sg_status s = clear_sums(fr, sc.n, st);
     if (s != SG_OK) return s;
@@ -1111,7 +1154,7 @@ sg_status backward_lidar(const Scene &sc, const Lidar &L, Frame &fr, const float
         SG_LAUNCHED();
     }
     const float o[3] = {0.f, 0.f, 0.f};
-    return finish(sc, fr, o, fr.opts.beam_divergence, g, st);
+    return finish(sc, fr, o, fr.opts.beam_divergence, g, write, st);
 }
 
 }  // namespace sg

@@ -1172,9 +1172,11 @@ sg_status sg_frame_stats(sg_frame frame, int64_t *n_pairs, int64_t *n_tiles, int
     return SG_OK;
 }
 
-sg_status sg_backward_camera(sg_scene scene, sg_frame frame, const float *d_g_rgb,
-                             const float *d_g_alpha, const float *d_g_depth,
-                             const sg_grads *grads, void *stream)
+}  // extern "C"
+
+static sg_status call_backward_camera(sg_scene scene, sg_frame frame, const float *d_g_rgb,
+                                      const float *d_g_alpha, const float *d_g_depth,
+                                      const sg_grads *grads, bool write, void *stream)
 {
     if (!scene || !frame || !grads) { set_error("NULL argument"); return SG_ERR_INVALID; }
     Frame &f = frame->f;
@@ -1188,12 +1190,13 @@ sg_status sg_backward_camera(sg_scene scene, sg_frame frame, const float *d_g_rg
         return SG_ERR_INVALID;
     }
     return backward_camera(scene->s, ((sg_camera)f.sensor)->c, f, d_g_rgb, d_g_alpha, d_g_depth,
-                           *grads, (cudaStream_t)stream);
+                           *grads, write, (cudaStream_t)stream);
 }
 
-sg_status sg_backward_lidar(sg_scene scene, sg_frame frame, const float *d_g_range,
-                            const float *d_g_intensity, const float *d_g_drop,
-                            const float *d_g_alpha, const sg_grads *grads, void *stream)
+static sg_status call_backward_lidar(sg_scene scene, sg_frame frame, const float *d_g_range,
+                                     const float *d_g_intensity, const float *d_g_drop,
+                                     const float *d_g_alpha, const sg_grads *grads, bool write,
+                                     void *stream)
 {
     if (!scene || !frame || !grads) { set_error("NULL argument"); return SG_ERR_INVALID; }
     Frame &f = frame->f;
@@ -1206,8 +1209,40 @@ sg_status sg_backward_lidar(sg_scene scene, sg_frame frame, const float *d_g_ran
                   "(sg_frame_set_backward_state)");
         return SG_ERR_INVALID;
     }
-    return backward_lidar(scene->s, ((sg_lidar)f.sensor)->l, f, d_g_range, d_g_intensity,
-                          d_g_drop, d_g_alpha, *grads, (cudaStream_t)stream);
+    return backward_lidar(scene->s, ((sg_lidar)f.sensor)->l, f, d_g_range, d_g_intensity, d_g_drop,
+                          d_g_alpha, *grads, write, (cudaStream_t)stream);
+}
+
+extern "C" {
+
+sg_status sg_backward_camera(sg_scene scene, sg_frame frame, const float *d_g_rgb,
+                             const float *d_g_alpha, const float *d_g_depth,
+                             const sg_grads *grads, void *stream)
+{
+    return call_backward_camera(scene, frame, d_g_rgb, d_g_alpha, d_g_depth, grads, false, stream);
+}
+
+sg_status sg_backward_lidar(sg_scene scene, sg_frame frame, const float *d_g_range,
+                            const float *d_g_intensity, const float *d_g_drop,
+                            const float *d_g_alpha, const sg_grads *grads, void *stream)
+{
+    return call_backward_lidar(scene, frame, d_g_range, d_g_intensity, d_g_drop, d_g_alpha, grads,
+                               false, stream);
+}
+
+sg_status sg_backward_camera_write(sg_scene scene, sg_frame frame, const float *d_g_rgb,
+                                   const float *d_g_alpha, const float *d_g_depth,
+                                   const sg_grads *grads, void *stream)
+{
+    return call_backward_camera(scene, frame, d_g_rgb, d_g_alpha, d_g_depth, grads, true, stream);
+}
+
+sg_status sg_backward_lidar_write(sg_scene scene, sg_frame frame, const float *d_g_range,
+                                  const float *d_g_intensity, const float *d_g_drop,
+                                  const float *d_g_alpha, const sg_grads *grads, void *stream)
+{
+    return call_backward_lidar(scene, frame, d_g_range, d_g_intensity, d_g_drop, d_g_alpha, grads,
+                               true, stream);
 }
 
 }  // extern "C"

@@ -478,10 +478,10 @@ sg_status build_lidar(Lidar &L);
 // backward.cu
 sg_status backward_camera(const Scene &sc, const Camera &cam, Frame &fr,
                           const float *g_rgb, const float *g_alpha, const float *g_depth,
-                          const sg_grads &g, cudaStream_t st);
+                          const sg_grads &g, bool write, cudaStream_t st);
 sg_status backward_lidar(const Scene &sc, const Lidar &L, Frame &fr, const float *g_range,
                          const float *g_int, const float *g_drop, const float *g_alpha,
-                         const sg_grads &g, cudaStream_t st);
+                         const sg_grads &g, bool write, cudaStream_t st);
 
 }  // namespace sg
 

@@ -125,6 +125,8 @@ _SIGNATURES = {
                                           C.POINTER(sg_render_opts), _P, _P, _P, _P]),
     "sg_backward_camera": (C.c_int, [_H, _H, _P, _P, _P, C.POINTER(sg_grads), _P]),
     "sg_backward_lidar": (C.c_int, [_H, _H, _P, _P, _P, _P, C.POINTER(sg_grads), _P]),
+    "sg_backward_camera_write": (C.c_int, [_H, _H, _P, _P, _P, C.POINTER(sg_grads), _P]),
+    "sg_backward_lidar_write": (C.c_int, [_H, _H, _P, _P, _P, _P, C.POINTER(sg_grads), _P]),
     "sg_frame_field": (C.c_int, [_H, C.c_int, C.POINTER(C.c_void_p), C.POINTER(C.c_int64)]),
     "sg_frame_stats": (C.c_int, [_H, C.POINTER(C.c_int64), C.POINTER(C.c_int64),
                                  C.POINTER(C.c_int64)]),
@@ -327,6 +329,17 @@ def sg_backward_camera(scene, frame, d_g_rgb, d_g_alpha, d_g_depth, grads, strea
 def sg_backward_lidar(scene, frame, d_g_range, d_g_int, d_g_drop, d_g_alpha, grads, stream=0):
     _check(load().sg_backward_lidar(scene, frame, _P(d_g_range), _P(d_g_int), _P(d_g_drop),
                                     _P(d_g_alpha), C.byref(grads), _P(stream)))
+
+
+def sg_backward_camera_write(scene, frame, d_g_rgb, d_g_alpha, d_g_depth, grads, stream=0):
+    _check(load().sg_backward_camera_write(scene, frame, _P(d_g_rgb), _P(d_g_alpha),
+                                           _P(d_g_depth), C.byref(grads), _P(stream)))
+
+
+def sg_backward_lidar_write(scene, frame, d_g_range, d_g_int, d_g_drop, d_g_alpha, grads,
+                            stream=0):
+    _check(load().sg_backward_lidar_write(scene, frame, _P(d_g_range), _P(d_g_int), _P(d_g_drop),
+                                          _P(d_g_alpha), C.byref(grads), _P(stream)))
 
 
 def sg_frame_field(frame, field):
