@@ -286,9 +286,12 @@ static void tmark(Frame &fr, int i, cudaStream_t st)
     if (fr.timing) cudaEventRecord(fr.ev[i], st);
 }
 
-// The render's RenderDesc (written to fr.h_desc by the caller) to the device.
-static sg_status upload_desc(Frame &fr, cudaStream_t st)
+// The render's RenderDesc (written to fr.h_desc by the caller) to the device,
+// unless the projection of n Gaussians takes it by value.
+static sg_status upload_desc(Frame &fr, int64_t n, cudaStream_t st)
 {
+    fr.desc_direct = fr.k_cap == 0 && n > 0;
+    if (fr.desc_direct) return SG_OK;
     SG_CUDA(cudaMemcpyAsync(fr.desc.p, fr.h_desc, sizeof(RenderDesc), cudaMemcpyHostToDevice, st));
     return SG_OK;
 }
@@ -334,29 +337,30 @@ static const char *status_cause(uint32_t w)
 // Wait until the counts of the render are in h_scalars.  k_pair_offsets writes
 // them there itself and the host polls the sequence number: a copy and an event
 // behind the kernel and waking up from its wait cost 10 us more (64x64 97 -> 88
-// us a render, 641x479 156 -> 149, street sweep 729 -> 717).  The event, asked
-// now and then, ends the wait if the kernel failed.
-static sg_status wait_count(Frame &fr)
+// us a render, 641x479 156 -> 149, street sweep 729 -> 717).  The event (or the
+// stream, ev NULL), asked now and then, ends the wait if the kernel failed.
+sg_status poll_count(const uint32_t *h, uint32_t seq, cudaEvent_t ev, cudaStream_t st)
 {
-    if (!fr.count_told) {
-        SG_CUDA(cudaEventSynchronize(fr.ev_count));
-        return SG_OK;
-    }
     for (uint32_t spin = 1;; ++spin) {
-        if (__atomic_load_n(fr.h_scalars + kHostCountSeq, __ATOMIC_ACQUIRE) == fr.count_seq)
-            return SG_OK;
+        if (__atomic_load_n(h + kHostCountSeq, __ATOMIC_ACQUIRE) == seq) return SG_OK;
         if (spin % 4096 != 0) continue;
-        const cudaError_t e = cudaEventQuery(fr.ev_count);
+        const cudaError_t e = ev ? cudaEventQuery(ev) : cudaStreamQuery(st);
         if (e == cudaErrorNotReady) {
             std::this_thread::yield();
             continue;
         }
         if (e != cudaSuccess) return cuda_status(e, "waiting for the pair count");
-        if (__atomic_load_n(fr.h_scalars + kHostCountSeq, __ATOMIC_ACQUIRE) == fr.count_seq)
-            return SG_OK;
+        if (__atomic_load_n(h + kHostCountSeq, __ATOMIC_ACQUIRE) == seq) return SG_OK;
         set_error("internal: the pair count did not reach the host");
         return SG_ERR_CUDA;
     }
+}
+
+static sg_status wait_count(Frame &fr)
+{
+    if (fr.count_told) return poll_count(fr.h_scalars, fr.count_seq, fr.ev_count, 0);
+    SG_CUDA(cudaEventSynchronize(fr.ev_count));
+    return SG_OK;
 }
 
 // bin_and_sort: waits for the pair count (exact mode), which sizes the pair
@@ -470,7 +474,7 @@ static sg_status camera_begin(sg_scene scene, sg_camera cam, const float h_c2w[1
     D.out[2] = d_depth;
     D.out[3] = nullptr;
     if (fr.timing) cudaEventRecord(fr.ev[0], st);
-    if ((s = upload_desc(fr, st)) != SG_OK) return s;
+    if ((s = upload_desc(fr, sc.n, st)) != SG_OK) return s;
     if ((s = project_camera(sc, c, *opts, fr, st, d_row_c2w != nullptr)) != SG_OK) return s;
     if (fr.timing) cudaEventRecord(fr.ev[1], st);
     return sort_and_count(fr, sc.n, st);
@@ -670,7 +674,14 @@ sg_status sg_create_camera(int model, int width, int height, float fx, float fy,
     c.fx = fx; c.fy = fy; c.cx = cx; c.cy = cy;
     for (int i = 0; i < 4; ++i) c.k[i] = (model == SG_CAMERA_FISHEYE && k) ? k[i] : 0.f;
     sg_status s = build_camera(c);
+    if (s == SG_OK && host_malloc(&c.h_count, 64) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("pinned allocation failed");
+        s = SG_ERR_OOM;
+    }
+    if (s == SG_OK) memset(c.h_count, 0, 64);
     if (s != SG_OK) {
+        host_free(c.h_count);
         dev_free(c.d_pix);
         dev_free(c.d_tile_dir);
         dev_free(c.d_pix2);
@@ -686,6 +697,7 @@ void sg_destroy_camera(sg_camera cam)
 {
     if (!cam) return;
     cudaDeviceSynchronize();   // renders still queued may read its ray tables
+    host_free(cam->c.h_count);
     dev_free(cam->c.d_pix);
     dev_free(cam->c.d_tile_dir);
     dev_free(cam->c.d_pix2);
@@ -1035,7 +1047,7 @@ sg_status sg_render_lidar(sg_scene scene, sg_lidar lidar, const float *d_col_c2w
     D.out[2] = d_drop;
     D.out[3] = d_alpha;
     if (fr.timing) cudaEventRecord(fr.ev[0], st);
-    if ((s = upload_desc(fr, st)) != SG_OK) return s;
+    if ((s = upload_desc(fr, sc.n, st)) != SG_OK) return s;
     if ((s = project_lidar(sc, L, *opts, fr, st)) != SG_OK) return s;
     if (fr.timing) cudaEventRecord(fr.ev[1], st);
     if ((s = sort_and_bin(fr, sc.n, L.n_theta, nt, 1, st)) != SG_OK) return s;

@@ -160,6 +160,10 @@ struct Camera {
     float4 *d_pix2 = nullptr;
     float *d_tile_basis = nullptr;
     bool tangent_ok = false;
+    // pinned words for the pair count of the allocation-free render, whose calls
+    // never overlap (kHostCountSeq), and the last sequence number
+    uint32_t *h_count = nullptr;
+    uint32_t count_seq = 0;
 };
 
 struct LidarItem {       // one warp of LiDAR rendering
@@ -221,9 +225,13 @@ struct __align__(16) GRec {
 
 // ------------------------------------------------------------------ frame
 // Per-render parameters that change from one render to the next, kept in
-// device memory (copied from pinned host memory at the start of each render)
-// so that a captured launch sequence can be replayed for a new pose and new
-// output buffers.  The kernels read the pose and the output pointers here.
+// device memory; the kernels read the pose and the output pointers there.  In
+// capacity mode they are copied from pinned host memory at the start of a
+// render, so that a captured launch sequence can be replayed for a new pose and
+// new output buffers.  Otherwise the projection gets them by value and writes
+// them there for the kernels after it (desc_direct): the copy and the wait for
+// it took 6 us of every render (64x64 88 -> 82, 641x479 152 -> 144, street sweep
+// 722 -> 716).
 struct RenderDesc {
     float c2w[12];          // camera renders: row-major [R | t]
     const float *poses;     // LiDAR renders: per-column c2w [n_cols, 12] (device)
@@ -264,7 +272,8 @@ struct Frame {
                       // [8] status: a look-back wait gave up (kScalStatus)
     Buf desc;         // RenderDesc of the current render (device)
     uint32_t *h_scalars = nullptr;  // pinned: scalars mirror (64 B), then the RenderDesc
-    RenderDesc *h_desc = nullptr;   // pinned staging of desc
+    RenderDesc *h_desc = nullptr;   // staging of desc (pinned)
+    bool desc_direct = false;       // the projection takes *h_desc by value
     // capacity mode: > 0 = the pair buffers hold this many pairs and no
     // step waits for the pair count (pairs beyond it are dropped and counted)
     int64_t k_cap = 0;
@@ -406,10 +415,14 @@ sg_status tile_scratch(int64_t n_max, int passes, Frame &fr, cudaStream_t st, ui
 sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n, const uint32_t *d_n,
                            int begin_bit, int end_bit, uint32_t *scratch, uint32_t *d_err,
                            cudaStream_t st, int *result_buf, int site, bool keep_keys = true);
+// capi.cu: wait until the pinned words h hold the counts of the render `seq`.
+sg_status poll_count(const uint32_t *h, uint32_t seq, cudaEvent_t ev, cudaStream_t st);
 // The depth stage: the Gaussians with a non-zero tile count sorted by depth
 // (keys/vals[*result_buf]: depth bits, ids), d_scal[0] = their number,
 // d_offsets = exclusive scan of their tile counts in that order, d_scal[1]
 // = the pair total.  Its scratch (fr.hist) was zeroed by the projection.
+// host_seq: also write the counts and the status word to fr.h_scalars, with this
+// sequence number (0: do not).
 sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, uint32_t *keys[2],
                       uint32_t *vals[2], uint32_t *d_scal, uint32_t *d_offsets, Frame &fr,
                       cudaStream_t st, int *result_buf, uint32_t host_seq = 0);

@@ -163,8 +163,6 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
     // the stages of sg_render_camera: project, depth sort, offsets, pair
     // count, binning, tile sort, ranges, compositing
     const int64_t n = sc.n;
-    // the descriptor goes from pageable host memory: the copy has taken its
-    // source by the time cudaMemcpyAsync returns
     RenderDesc D;
     memcpy(D.c2w, h_c2w, sizeof(D.c2w));
     D.poses = nullptr;
@@ -172,19 +170,32 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
     D.out[1] = d_alpha;
     D.out[2] = d_depth;
     D.out[3] = nullptr;
-    SG_CUDA(cudaMemcpyAsync(fr.desc.p, &D, sizeof(D), cudaMemcpyHostToDevice, st));
+    fr.h_desc = &D;
+    fr.desc_direct = n > 0;
+    // (from pageable memory: the copy has taken its source when the call returns)
+    if (n <= 0) SG_CUDA(cudaMemcpyAsync(fr.desc.p, &D, sizeof(D), cudaMemcpyHostToDevice, st));
     if ((s = project_camera(sc, c, *opts, fr, st)) != SG_OK) return s;
     uint32_t *scal = (uint32_t *)fr.scalars.p;
     uint32_t *dk[2] = {(uint32_t *)fr.dkeys[0].p, (uint32_t *)fr.dkeys[1].p};
     uint32_t *dv[2] = {(uint32_t *)fr.dvals[0].p, (uint32_t *)fr.dvals[1].p};
     int rb = 0;
+    // the pair count comes back through the camera's pinned words
+    uint32_t seq = 0;
+    if (n > 0) {
+        seq = ++cam->c.count_seq;
+        if (seq == 0) seq = cam->c.count_seq = 1;
+    }
+    fr.h_scalars = cam->c.h_count;
     if ((s = depth_stage((const uint32_t *)fr.count.p, (const float *)fr.depth.p, n, dk, dv, scal,
-                         (uint32_t *)fr.offsets.p, fr, st, &rb)) != SG_OK)
+                         (uint32_t *)fr.offsets.p, fr, st, &rb, seq)) != SG_OK)
         return s;
-    // the counts and the status word (pageable: the copy is synchronous here)
-    uint32_t hs[kScalStatus + 1] = {};
-    SG_CUDA(cudaMemcpyAsync(hs, scal, sizeof(hs), cudaMemcpyDeviceToHost, st));
-    SG_CUDA(cudaStreamSynchronize(st));
+    // the counts and the status word
+    const uint32_t *hs = cam->c.h_count;
+    const uint32_t none[kScalStatus + 1] = {};
+    if (seq == 0)       // no Gaussians
+        hs = none;
+    else if ((s = poll_count(hs, seq, nullptr, st)) != SG_OK)
+        return s;
     if (hs[kScalStatus]) {
         set_error("sg_render_camera_static: a bounded device wait (sort look-back or projection bulk copy) gave up");
         return SG_ERR_TIMEOUT;

@@ -290,9 +290,8 @@ __device__ __forceinline__ int cam_row_point(const CamParams &C, const float *po
 template <bool kRS>
 __global__ void __launch_bounds__(256, SG_PROJ_MINB)
 k_project_camera(const float *__restrict__ planes, int64_t pitch, int64_t n, int feature_kind,
-                 int sh_degree, ActorParams A, CamParams C, const RenderDesc *__restrict__ D,
-                 UTParams U,
-                 GRec *__restrict__ rec,
+                 int sh_degree, ActorParams A, CamParams C, RenderDesc *__restrict__ D,
+                 const __grid_constant__ RenderDesc direct, int is_direct, UTParams U, GRec *__restrict__ rec,
                  float4 *__restrict__ rect_out, int4 *__restrict__ tiles_out,
                  float *__restrict__ depth_out, uint32_t *__restrict__ count_out,
                  float2 *__restrict__ mean_out, float4 *__restrict__ cov_out,
@@ -306,7 +305,8 @@ k_project_camera(const float *__restrict__ planes, int64_t pitch, int64_t n, int
     __shared__ uint64_t s_bar;
     const int n_stage =
         feature_kind == SG_FEATURES_SH ? 3 * (sh_degree + 1) * (sh_degree + 1) : 0;
-    if (threadIdx.x < 12) s_c2w[threadIdx.x] = D->c2w[threadIdx.x];
+    if (threadIdx.x < 12)
+        s_c2w[threadIdx.x] = is_direct ? direct.c2w[threadIdx.x] : D->c2w[threadIdx.x];
     if (threadIdx.x == 0 && n_stage) mbar_init(&s_bar);
     __syncthreads();
     const int64_t g0 = (int64_t)blockIdx.x * blockDim.x;
@@ -321,9 +321,12 @@ k_project_camera(const float *__restrict__ planes, int64_t pitch, int64_t n, int
                           &s_bar);
     }
     int64_t g = g0 + threadIdx.x;
-    if (g == 0) *status = 0u;     // a new render: no device wait has given up
+    if (g == 0) {
+        *status = 0u;             // a new render: no device wait has given up
+        if (is_direct) *D = direct;
+    }
     if (g >= n) return;           // (thread 0 of a block always has a Gaussian)
-    const float *poses = kRS ? D->poses : nullptr;
+    const float *poses = kRS ? (is_direct ? direct.poses : D->poses) : nullptr;
     Activated a = activate(planes, pitch, g);
     to_world(A, g, a);
     // the mean's pose: the camera's, or that of the row that sees the mean
@@ -454,7 +457,8 @@ sg_status project_camera(const Scene &sc, const Camera &cam, const sg_render_opt
     }
     kern<<<grid, 256, smem, st>>>(
         sc.d_planes, sc.pitch, sc.n, sc.feature_kind, sc.sh_degree, actor_params(sc), C,
-        (const RenderDesc *)fr.desc.p, U, (GRec *)fr.rec.p,
+        (RenderDesc *)fr.desc.p, fr.desc_direct ? *fr.h_desc : RenderDesc{}, fr.desc_direct ? 1 : 0,
+        U, (GRec *)fr.rec.p,
         (float4 *)fr.rect.p, (int4 *)fr.tiles.p, (float *)fr.depth.p, (uint32_t *)fr.count.p,
         (float2 *)fr.mean2d.p, (float4 *)fr.cov2d.p, (uint32_t *)fr.scalars.p + kScalStatus,
         (uint4 *)fr.hist.p, depth_stage_words(sc.n) / 4);
@@ -655,8 +659,9 @@ __device__ __forceinline__ void cholesky3(const float C[9], float Lc[9])
 template <bool kSH, bool kBeam>
 __global__ void __launch_bounds__(256, 4)
 k_project_lidar(const float *__restrict__ planes, int64_t pitch, int64_t n, int sh_degree,
-                ActorParams A, LidParams Lp, const RenderDesc *__restrict__ D, UTParams U,
-                int cull, GRec *__restrict__ rec, float4 *__restrict__ rect_out,
+                ActorParams A, LidParams Lp, RenderDesc *__restrict__ D,
+                const __grid_constant__ RenderDesc direct,
+                int is_direct, UTParams U, int cull, GRec *__restrict__ rec, float4 *__restrict__ rect_out,
                 int4 *__restrict__ tiles_out, float *__restrict__ depth_out,
                 uint32_t *__restrict__ count_out, float2 *__restrict__ mean_out,
                 float4 *__restrict__ cov_out, uint32_t *__restrict__ status,
@@ -664,10 +669,13 @@ k_project_lidar(const float *__restrict__ planes, int64_t pitch, int64_t n, int 
 {
     zero_scratch(zero, nzero);
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g == 0) *status = 0u;     // a new render: no look-back wait has given up
+    if (g == 0) {
+        *status = 0u;     // a new render: no look-back wait has given up
+        if (is_direct) *D = direct;
+    }
     if (g >= n) return;
     LidParams L = Lp;
-    L.poses = D->poses;
+    L.poses = is_direct ? direct.poses : D->poses;
     Activated a = activate(planes, pitch, g);
     to_world(A, g, a);
     float xs0[3], az0;               // chi_0 = mu, also the depth key
@@ -821,7 +829,8 @@ sg_status project_lidar(const Scene &sc, const Lidar &Ld, const sg_render_opts &
                    : (beam ? k_project_lidar<false, true> : k_project_lidar<false, false>);
     kern<<<grid, 256, 0, st>>>(
         sc.d_planes, sc.pitch, sc.n, sc.sh_degree, actor_params(sc), L,
-        (const RenderDesc *)fr.desc.p, U, o.cull,
+        (RenderDesc *)fr.desc.p, fr.desc_direct ? *fr.h_desc : RenderDesc{}, fr.desc_direct ? 1 : 0,
+        U, o.cull,
         (GRec *)fr.rec.p, (float4 *)fr.rect.p,
         (int4 *)fr.tiles.p, (float *)fr.depth.p, (uint32_t *)fr.count.p, (float2 *)fr.mean2d.p,
         (float4 *)fr.cov2d.p, (uint32_t *)fr.scalars.p + kScalStatus, (uint4 *)fr.hist.p,
