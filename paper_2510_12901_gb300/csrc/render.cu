@@ -320,7 +320,7 @@ sg_status launch_work_items(Frame &fr, const WorkSize &ws, const Lidar *lidar, i
 
 // Camera compositing, persistent and warp-independent.  A work item is one
 // 8x4 pixel sub-block of a 16x16 tile and one segment of that tile's list
-// (k_camera_items); items are taken in order of decreasing tile-list length
+// (k_work_items); items are taken in order of decreasing tile-list length
 // through an atomic counter, so the densest tiles start first and their
 // sub-blocks and segments run on different SMs.  A warp reads its segment's
 // sub-block masks 32 at a time, keeps (in list order) the entries whose
