@@ -616,6 +616,157 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
     }
 }
 
+// The whole depth stage of a scene of at most kSmallN Gaussians, in one block:
+// compaction in id order, four stable 8-bit passes over the depth bits in shared
+// memory, and the offsets, as the kernels above make them.  Bound by the latency
+// of its steps (a pass: digits of a warp's 128 keys matched 32 at a time, counts
+// of 32 warps scanned, one scatter).  One launch for six: 27 -> 16 us with their
+// gaps at 4096 Gaussians (64x64 view 82 -> 71 us).  A thread holds four entries,
+// which fills a block at 4096; the look-back passes spread what is more over the
+// SMs.
+constexpr int kSmallThreads = 1024, kSmallPer = 4, kSmallN = kSmallThreads * kSmallPer;
+constexpr size_t kSmallZero = 64 * 1024;
+
+__global__ void __launch_bounds__(kSmallThreads)
+k_depth_small(const uint32_t *__restrict__ count, const float *__restrict__ depth, int n,
+              uint32_t *__restrict__ vals, uint32_t *__restrict__ d_nvalid,
+              uint32_t *__restrict__ offsets, uint32_t *__restrict__ d_total,
+              const uint32_t *__restrict__ err, uint32_t *__restrict__ owner, int64_t owner_cap,
+              volatile uint32_t *host, uint32_t seq, uint4 *__restrict__ zero, int64_t nzero)
+{
+    after_previous();
+    constexpr uint32_t full = 0xffffffffu;
+    __shared__ uint32_t s_key[kSmallN];
+    __shared__ uint16_t s_val[kSmallN];
+    // a warp's keys of a digit; rows 2 longer: the four threads of a digit read rows 8
+    // apart, from banks of their own
+    __shared__ __align__(4) uint16_t s_cnt[32][258];
+    __shared__ uint32_t s_base[256], s_w[32];
+    for (int64_t i = threadIdx.x; i < nzero; i += kSmallThreads) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, first = warp * 32 * kSmallPer + lane;
+    const uint32_t below = (1u << lane) - 1u;
+    {
+        uint32_t bal[kSmallPer], key[kSmallPer], wtot = 0u;
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            const int i = first + 32 * r;
+            bal[r] = __ballot_sync(full, i < n && count[i] > 0u);
+            key[r] = i < n ? __float_as_uint(depth[i]) : 0u;
+            wtot += __popc(bal[r]);
+        }
+        if (lane == 0) s_w[warp] = wtot;
+        __syncthreads();
+        uint32_t pos = __reduce_add_sync(full, lane < warp ? s_w[lane] : 0u);
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            if ((bal[r] >> lane) & 1u) {
+                const uint32_t q = pos + __popc(bal[r] & below);
+                s_key[q] = key[r];
+                s_val[q] = (uint16_t)(first + 32 * r);
+            }
+            pos += __popc(bal[r]);
+        }
+    }
+    const int nv = (int)__reduce_add_sync(full, s_w[lane]);
+    __syncthreads();
+    for (int p = 0; p < 4; ++p) {
+        uint32_t key[kSmallPer], val[kSmallPer], rank[kSmallPer];
+        for (int i = lane; i < 128; i += 32) reinterpret_cast<uint32_t *>(s_cnt[warp])[i] = 0u;
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            const int i = first + 32 * r;
+            const bool live = i < nv;
+            key[r] = live ? s_key[i] : 0u;
+            val[r] = live ? s_val[i] : 0u;
+            const uint32_t d = (key[r] >> (8 * p)) & 255u;
+            const uint32_t peers = __match_any_sync(full, live ? d : 256u);
+            const uint32_t had = s_cnt[warp][d];
+            __syncwarp();
+            if (live && lane == __ffs(peers) - 1) s_cnt[warp][d] = (uint16_t)(had + __popc(peers));
+            __syncwarp();
+            rank[r] = had + __popc(peers & below);
+        }
+        __syncthreads();
+        // per digit, the keys of earlier warps: four threads a digit, eight warps each
+        const int digit = t >> 2, part = t & 3;
+        uint32_t sum = 0u;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sum += s_cnt[8 * part + q][digit];
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(full, inc, o, 4);
+            if (part >= o) inc += x;
+        }
+        uint32_t run = inc - sum;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const uint32_t c = s_cnt[8 * part + q][digit];
+            s_cnt[8 * part + q][digit] = (uint16_t)run;
+            run += c;
+        }
+        // the digits' first positions: the last of the four threads has the total
+        const uint32_t tot = part == 3 ? inc : 0u;
+        const uint32_t di = warp_incl_scan(tot);
+        if (lane == 31) s_w[warp] = di;
+        __syncthreads();
+        const uint32_t pre = __reduce_add_sync(full, lane < warp ? s_w[lane] : 0u);
+        if (part == 3) s_base[digit] = pre + di - tot;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            if (first + 32 * r >= nv) continue;
+            const uint32_t d = (key[r] >> (8 * p)) & 255u;
+            const uint32_t q = s_base[d] + s_cnt[warp][d] + rank[r];
+            s_key[q] = key[r];
+            s_val[q] = (uint16_t)val[r];
+        }
+        __syncthreads();
+    }
+    // the offsets, as k_pair_offsets
+    uint32_t c[kSmallPer], run = 0u;
+#pragma unroll
+    for (int r = 0; r < kSmallPer; ++r) {
+        const int i = first + 32 * r;
+        const uint32_t id = i < nv ? s_val[i] : 0u;
+        const uint32_t v = i < nv ? count[id] : 0u;
+        if (i < nv) vals[i] = id;
+        const uint32_t inc = warp_incl_scan(v);
+        c[r] = run + inc - v;
+        run += __shfl_sync(full, inc, 31);
+    }
+    if (lane == 0) s_w[warp] = run;
+    __syncthreads();
+    unsigned long long total = 0;
+    uint32_t pre = 0;
+    for (int w = 0; w < 32; ++w) {
+        pre += w < warp ? s_w[w] : 0u;
+        total += s_w[w];
+    }
+#pragma unroll
+    for (int r = 0; r < kSmallPer; ++r) {
+        const int i = first + 32 * r;
+        uint32_t next = __shfl_down_sync(full, c[r], 1);
+        const uint32_t chunk_end =
+            r + 1 < kSmallPer ? __shfl_sync(full, c[r + 1 < kSmallPer ? r + 1 : r], 0) : run;
+        if (lane == 31) next = chunk_end;
+        if (i < nv) {
+            const uint64_t off = pre + c[r], end = off + (next - c[r]);
+            offsets[i] = (uint32_t)off;
+            for (uint64_t b = (off + kBinChunk - 1) / kBinChunk;
+                 b * kBinChunk < end && (int64_t)b < owner_cap; ++b)
+                owner[b] = (uint32_t)i;
+        }
+    }
+    if (t == 0) {
+        const uint32_t sat = total > 0xffffffffull ? 0xffffffffu : (uint32_t)total;
+        *d_nvalid = (uint32_t)nv;
+        *d_total = sat;
+        tell_host(host, (uint32_t)nv, sat, *(const volatile uint32_t *)err, seq);
+    }
+}
+
 sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, uint32_t *keys[2],
                       uint32_t *vals[2], uint32_t *d_scal, uint32_t *d_offsets, Frame &fr,
                       cudaStream_t st, int *result_buf, uint32_t host_seq)
@@ -643,6 +794,18 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     unsigned long long *chain = (unsigned long long *)(hist + radix_scratch_words(n, 4));
     uint32_t *tickets = (uint32_t *)chain;                 // [0] compaction, [1] offsets
     uint32_t *err = (uint32_t *)fr.scalars.p + kScalStatus;
+    if (n <= kSmallN) {
+        // one block zeroes what a scene of this size needs of the tile sort's
+        // scratch, not all that a larger render has left
+        const size_t zero = fr.tscratch.bytes < kSmallZero ? fr.tscratch.bytes : kSmallZero;
+        launch_after(k_depth_small, 1, kSmallThreads, 0, st, d_count, d_depth, (int)n, vals[0], d_scal,
+                     d_offsets, d_scal + 1, err, (uint32_t *)fr.owner.p, (int64_t)(fr.owner.bytes / 4),
+                     host_seq ? (volatile uint32_t *)fr.h_scalars : nullptr, host_seq,
+                     (uint4 *)fr.tscratch.p, (int64_t)(zero / 16));
+        SG_LAUNCHED();
+        fr.tscratch_zeroed = zero / 16 * 16;
+        return SG_OK;
+    }
     launch_after(k_compact_depth, (unsigned)ntiles, kChainThreads, 0, st,
         d_count, d_depth, n, ntiles, keys[0], vals[0], d_scal, hist, chain + 2, tickets, err,
         (uint4 *)fr.tscratch.p, (int64_t)(fr.tscratch.bytes / 16));
