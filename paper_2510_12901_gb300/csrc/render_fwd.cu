@@ -29,11 +29,20 @@
 namespace sg {
 
 constexpr int kFwdWarps = 4;        // warps per block of the persistent grid
-// blocks per SM the register budget is set for (64 registers; a few bytes of
-// the merge spill).  Measured (1920x1080 pinhole of 2M Gaussians / 641x479
-// fisheye of 100k): 6 blocks 651 / 43, 7 blocks 643 / 46, 8 blocks 624 / 48, 9
-// blocks 656 / 54 us.
-constexpr int kFwdBlocks = 8;
+// Blocks per SM (4 and 6: 80 registers; 8: 64, a few bytes of the merge spill).
+// Few warps walk faster, and below a few million pairs the launch ends with the
+// dense tiles' chain of merges and re-walks; many hide more latency.  Measured, 4
+// / 6 / 8 blocks in us: 641x479 of 150k Gaussians (0.16M pairs) 32 / 34 / 38,
+// 1024x768 of 500k (0.68M) 137 / 150 / 177, 1280x960 of 333k (0.42M) 104 / 104 /
+// 124, 1920x1080 of 333k (0.69M) 193 / 156 / 188, of 1M (2.0M) 408 / 339 / 374, of
+// 1.5M (3.0M) 582 / 492 / 482, of 2M (3.9M) 763 / 651 / 625; 1920x1280 fisheye of
+// 1M (1.5M) 322 / 264 / 304, of 1.5M (2.2M) 438 / 364 / 377.  Frames in capacity
+// mode are a server's, whose renders overlap on several streams and fill each
+// other's ends: 12 requests 1595 with 8 blocks, 1655 with the rule for one view.
+constexpr int fwd_blocks(int n_tiles, int64_t n_pairs, bool capacity)
+{
+    return capacity ? 8 : n_tiles < 4000 ? 4 : n_pairs < 2700000 ? 6 : 8;
+}
 // List entries a warp scans at a time: kFwdPer per lane.  Those that reach a
 // live ray of the sub-block (about a third on the street views) go to a queue
 // and are staged 32 at a time, so that the staging pass, one entry per lane,
@@ -353,8 +362,8 @@ __device__ __forceinline__ void fwd_put(float4 *pq, const FwdAcc &a, bool stoppe
     pq[1] = make_float4(a.Z, a.T, 0.f, stopped ? 1.f : 0.f);
 }
 
-template <uint32_t kSeg>
-__global__ void __launch_bounds__(32 * kFwdWarps, kFwdBlocks)
+template <uint32_t kSeg, int kBlocks>
+__global__ void __launch_bounds__(32 * kFwdWarps, kBlocks)
 k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
                     const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
                     const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
@@ -481,20 +490,6 @@ k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *_
     }
 }
 
-static int fwd_blocks_per_sm()
-{
-    static int cached = 0;
-    if (!cached) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_render_camera_fwd<kFwdSeg>,
-                                                          32 * kFwdWarps, 0) != cudaSuccess ||
-            nb < 1)
-            nb = 4;
-        cached = nb;
-    }
-    return cached;
-}
-
 bool camera_forward_only(const Camera &cam, const Frame &fr)
 {
     return !fr.keep_state && fr.seg_len == kSegLen && cam.tangent_ok;
@@ -527,10 +522,11 @@ sg_status render_camera_fwd(const Camera &cam, const sg_render_opts &o, Frame &f
     SG_CUDA(cudaGetDevice(&dev));
     SG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t cap = (ws.max_items + kFwdWarps - 1) / kFwdWarps;
-    int64_t grid = (int64_t)sms * fwd_blocks_per_sm();
+    const int nb = fwd_blocks(nt, K, fr.k_cap > 0);
+    int64_t grid = (int64_t)sms * nb;
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
-    launch_after(k_render_camera_fwd<kFwdSeg>, (unsigned)grid, 32 * kFwdWarps, 0, st,
+    launch_after(nb > 6 ? k_render_camera_fwd<kFwdSeg, 8> : k_render_camera_fwd<kFwdSeg, 6>, (unsigned)grid, 32 * kFwdWarps, 0, st,
         P, (const GRec *)fr.rec.p, ids, (const uint2 *)fr.ranges.p, items, tile_info, counts,
         (const uint32_t *)fr.submask.p, counter, arrive, (float4 *)fr.partials.p, cam.d_pix2,
         cam.d_tile_dir, cam.d_tile_basis, (const RenderDesc *)fr.desc.p);
