@@ -36,12 +36,14 @@ constexpr int kFwdWarps = 4;        // warps per block of the persistent grid
 // 1024x768 of 500k (0.68M) 137 / 150 / 177, 1280x960 of 333k (0.42M) 104 / 104 /
 // 124, 1920x1080 of 333k (0.69M) 193 / 156 / 188, of 1M (2.0M) 408 / 339 / 374, of
 // 1.5M (3.0M) 582 / 492 / 482, of 2M (3.9M) 763 / 651 / 625; 1920x1280 fisheye of
-// 1M (1.5M) 322 / 264 / 304, of 1.5M (2.2M) 438 / 364 / 377.  Frames in capacity
-// mode are a server's, whose renders overlap on several streams and fill each
-// other's ends: 12 requests 1595 with 8 blocks, 1655 with the rule for one view.
-constexpr int fwd_blocks(int n_tiles, int64_t n_pairs, bool capacity)
+// 1M (1.5M) 322 / 264 / 304, of 1.5M (2.2M) 438 / 364 / 377.  Renders that
+// overlap with others fill each other's ends, and take 8: the views of one call
+// (both street views of 1M in steps queued one after another 4636 Mrays/s, 4392
+// with the rule for one view) and frames in capacity mode, which are a server's (12
+// requests 1595 and 1655 us).
+constexpr int fwd_blocks(int n_tiles, int64_t n_pairs, bool overlaps)
 {
-    return capacity ? 8 : n_tiles < 4000 ? 4 : n_pairs < 2700000 ? 6 : 8;
+    return overlaps ? 8 : n_tiles < 4000 ? 4 : n_pairs < 2700000 ? 6 : 8;
 }
 // List entries a warp scans at a time: kFwdPer per lane.  Those that reach a
 // live ray of the sub-block (about a third on the street views) go to a queue
@@ -522,7 +524,7 @@ sg_status render_camera_fwd(const Camera &cam, const sg_render_opts &o, Frame &f
     SG_CUDA(cudaGetDevice(&dev));
     SG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t cap = (ws.max_items + kFwdWarps - 1) / kFwdWarps;
-    const int nb = fwd_blocks(nt, K, fr.k_cap > 0);
+    const int nb = fwd_blocks(nt, K, fr.k_cap > 0 || fr.one_of_many);
     int64_t grid = (int64_t)sms * nb;
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
