@@ -20,6 +20,18 @@ def _ptr(t):
     return 0 if t is None else t.data_ptr()
 
 
+def _gradients(ctx, ups, write):
+    """The five parameter gradients, written by write(upstream pointers, sg_grads).  The
+    engine also runs the node when no output has a gradient (a later function returned
+    None for all of them): they are 0 then."""
+    if all(g is None for g in ups):
+        return [torch.zeros(s, device=ctx.device) for s in ctx.shapes]
+    grads = [torch.empty(s, device=ctx.device) for s in ctx.shapes]
+    ups = [None if g is None else g.contiguous() for g in ups]
+    write([_ptr(u) for u in ups], sg.sg_grads(*[g.data_ptr() for g in grads]))
+    return grads
+
+
 class _RenderCamera(torch.autograd.Function):
     @staticmethod
     def forward(ctx, means, log_scales, quats, opacity, features, scene, cam, c2w, opts, frame):
@@ -34,17 +46,14 @@ class _RenderCamera(torch.autograd.Function):
                             alpha.data_ptr(), depth.data_ptr(), stream)
         ctx.scene, ctx.frame = scene, frame
         ctx.set_materialize_grads(False)    # an output without a gradient: NULL, not zeros
-        ctx.shapes = [t.shape for t in ts]
+        ctx.shapes, ctx.device = [t.shape for t in ts], means.device
         return rgb, alpha, depth
 
     @staticmethod
     def backward(ctx, g_rgb, g_alpha, g_depth):
-        ref = next(g for g in (g_rgb, g_alpha, g_depth) if g is not None)
-        grads = [torch.empty(s, device=ref.device) for s in ctx.shapes]
-        gs = sg.sg_grads(*[g.data_ptr() for g in grads])
-        ups = [None if g is None else g.contiguous() for g in (g_rgb, g_alpha, g_depth)]
-        sg.sg_backward_camera_write(ctx.scene.handle, ctx.frame.handle, *[_ptr(u) for u in ups],
-                                    gs, torch.cuda.current_stream().cuda_stream)
+        grads = _gradients(ctx, (g_rgb, g_alpha, g_depth), lambda ups, gs:
+                           sg.sg_backward_camera_write(ctx.scene.handle, ctx.frame.handle, *ups, gs,
+                                                       torch.cuda.current_stream().cuda_stream))
         return (*grads, None, None, None, None, None)
 
 
@@ -60,17 +69,14 @@ class _RenderLidar(torch.autograd.Function):
                            *[o.data_ptr() for o in outs], stream)
         ctx.scene, ctx.frame, ctx.poses = scene, frame, poses
         ctx.set_materialize_grads(False)
-        ctx.shapes = [t.shape for t in ts]
+        ctx.shapes, ctx.device = [t.shape for t in ts], means.device
         return tuple(outs)
 
     @staticmethod
     def backward(ctx, g_range, g_int, g_drop, g_alpha):
-        ref = next(g for g in (g_range, g_int, g_drop, g_alpha) if g is not None)
-        grads = [torch.empty(s, device=ref.device) for s in ctx.shapes]
-        gs = sg.sg_grads(*[g.data_ptr() for g in grads])
-        ups = [None if g is None else g.contiguous() for g in (g_range, g_int, g_drop, g_alpha)]
-        sg.sg_backward_lidar_write(ctx.scene.handle, ctx.frame.handle, *[_ptr(u) for u in ups],
-                                   gs, torch.cuda.current_stream().cuda_stream)
+        grads = _gradients(ctx, (g_range, g_int, g_drop, g_alpha), lambda ups, gs:
+                           sg.sg_backward_lidar_write(ctx.scene.handle, ctx.frame.handle, *ups, gs,
+                                                      torch.cuda.current_stream().cuda_stream))
         return (*grads, None, None, None, None, None)
 
 
