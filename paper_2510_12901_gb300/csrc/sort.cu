@@ -532,6 +532,20 @@ __device__ __forceinline__ void tell_host(volatile uint32_t *host, uint32_t nval
     host[kHostCountSeq] = seq;
 }
 
+// Entry i's pairs [off, off + n): its offset, and the binning blocks whose first
+// pair is one of them.  Offsets of 2^32 and more, which only a render that drops
+// pairs can reach (its capacity is below 2^31), are stored as 2^32 - 1: wrapped
+// ones would decrease, and binning takes them to be sorted.
+__device__ __forceinline__ void put_offset(int64_t i, unsigned long long off, uint32_t n,
+                                           uint32_t *__restrict__ offsets,
+                                           uint32_t *__restrict__ owner, int64_t owner_cap)
+{
+    offsets[i] = off < 0xffffffffull ? (uint32_t)off : 0xffffffffu;
+    for (unsigned long long b = (off + kBinChunk - 1) / kBinChunk;
+         b * kBinChunk < off + n && (int64_t)b < owner_cap; ++b)
+        owner[b] = (uint32_t)i;
+}
+
 template <int kOffChunks>
 __global__ void __launch_bounds__(kChainThreads)
 k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ count, int64_t n,
@@ -578,8 +592,7 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
     }
     if (lane == 0) S.warp[warp] = run;
     __syncthreads();
-    uint32_t before = 0;
-    unsigned long long total = 0;
+    unsigned long long before = 0, total = 0;
 #pragma unroll
     for (int w = 0; w < kChainWarps; ++w) {
         const uint32_t x = S.warp[w];
@@ -596,7 +609,7 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
         *d_total = sat;
         tell_host(host, (uint32_t)nv, sat, *(volatile uint32_t *)err, seq);
     }
-    const uint32_t pre = (uint32_t)excl + before;
+    const unsigned long long pre = excl + before;
 #pragma unroll
     for (int r = 0; r < kOffChunks; ++r) {
         const int64_t i = wbase + r * 32 + lane;
@@ -605,14 +618,7 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
         const uint32_t chunk_end =
             r + 1 < kOffChunks ? __shfl_sync(0xffffffffu, c[r + 1 < kOffChunks ? r + 1 : r], 0) : run;
         if (lane == 31) next = chunk_end;
-        if (i < nv) {
-            const uint64_t off = pre + c[r], end = off + (next - c[r]);
-            offsets[i] = (uint32_t)off;
-            // the binning blocks whose first pair is one of them
-            for (uint64_t b = (off + kBinChunk - 1) / kBinChunk;
-                 b * kBinChunk < end && (int64_t)b < owner_cap; ++b)
-                owner[b] = (uint32_t)i;
-        }
+        if (i < nv) put_offset(i, pre + c[r], next - c[r], offsets, owner, owner_cap);
     }
 }
 
@@ -738,8 +744,7 @@ k_depth_small(const uint32_t *__restrict__ count, const float *__restrict__ dept
     }
     if (lane == 0) s_w[warp] = run;
     __syncthreads();
-    unsigned long long total = 0;
-    uint32_t pre = 0;
+    unsigned long long total = 0, pre = 0;
     for (int w = 0; w < 32; ++w) {
         pre += w < warp ? s_w[w] : 0u;
         total += s_w[w];
@@ -751,13 +756,7 @@ k_depth_small(const uint32_t *__restrict__ count, const float *__restrict__ dept
         const uint32_t chunk_end =
             r + 1 < kSmallPer ? __shfl_sync(full, c[r + 1 < kSmallPer ? r + 1 : r], 0) : run;
         if (lane == 31) next = chunk_end;
-        if (i < nv) {
-            const uint64_t off = pre + c[r], end = off + (next - c[r]);
-            offsets[i] = (uint32_t)off;
-            for (uint64_t b = (off + kBinChunk - 1) / kBinChunk;
-                 b * kBinChunk < end && (int64_t)b < owner_cap; ++b)
-                owner[b] = (uint32_t)i;
-        }
+        if (i < nv) put_offset(i, pre + c[r], next - c[r], offsets, owner, owner_cap);
     }
     if (t == 0) {
         const uint32_t sat = total > 0xffffffffull ? 0xffffffffu : (uint32_t)total;
@@ -886,7 +885,7 @@ k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
     if (p0 >= K || nvalid == 0 || *err) return;
     const int64_t p1 = min(K, p0 + kBinChunk);
     // the owner of p0: the largest k with offsets[k] <= p0 (offsets[0] = 0,
-    // strictly increasing: every valid Gaussian has a pair)
+    // strictly increasing below 2^32 - 1: every valid Gaussian has a pair)
     int64_t k0 = 0;
     if ((int64_t)blockIdx.x < owner_cap) {
         k0 = owner[blockIdx.x];
