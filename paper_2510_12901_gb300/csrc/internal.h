@@ -392,8 +392,8 @@ constexpr int64_t radix_scratch_words(int64_t n_max, int passes)
     return 2 * 256 * (int64_t)passes + 16 + (int64_t)passes * (tiles > 0 ? tiles : 1) * 256;
 }
 // The depth stage's scratch (fr.hist): the radix scratch of its 4 passes,
-// then two tickets and a 64-bit look-back word per tile of kChainTile
-// entries for each of its two chained scans.
+// then four words (two tickets, the offset tiles done) and a 64-bit look-back
+// word per tile of kChainTile entries for each of its two chained scans.
 constexpr int kChainTile = 2048;
 constexpr int64_t depth_stage_words(int64_t n)
 {

@@ -519,7 +519,7 @@ k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ de
     }
 }
 
-// The counts and the status word so far to the frame's pinned words (host; NULL:
+// The counts and the status word to the frame's pinned words (host; NULL:
 // nobody waits for them), the sequence number last.
 __device__ __forceinline__ void tell_host(volatile uint32_t *host, uint32_t nvalid, uint32_t pairs,
                                           uint32_t status, uint32_t seq)
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(kChainThreads)
 k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ count, int64_t n,
                const uint32_t *__restrict__ d_nvalid, uint32_t *__restrict__ offsets,
                uint32_t *__restrict__ d_total, unsigned long long *__restrict__ lb,
-               uint32_t *__restrict__ ticket, uint32_t *__restrict__ err,
+               uint32_t *__restrict__ ticket, uint32_t *__restrict__ done, uint32_t *__restrict__ err,
                uint32_t *__restrict__ owner, int64_t owner_cap, volatile uint32_t *host, uint32_t seq)
 {
     after_previous();
@@ -602,12 +602,23 @@ k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ co
     const bool publish = tile != held_tile(SG_LOOKBACK_OFFSETS);
     chain_publish(lb, tile, total, publish);
     const unsigned long long excl = chain_lookback(lb, tile, total, publish, err, S);
-    if (threadIdx.x == 0 && tile == ntiles - 1) {
-        // saturated, so that a total of 2^32 pairs or more reads as an overflow
-        const unsigned long long tot = excl + total;
-        const uint32_t sat = tot > 0xffffffffull ? 0xffffffffu : (uint32_t)tot;
-        *d_total = sat;
-        tell_host(host, (uint32_t)nv, sat, *(volatile uint32_t *)err, seq);
+    if (threadIdx.x == 0) {
+        if (tile == ntiles - 1) {
+            // saturated, so that a total of 2^32 pairs or more reads as an overflow
+            const unsigned long long tot = excl + total;
+            *d_total = tot > 0xffffffffull ? 0xffffffffu : (uint32_t)tot;
+        }
+        // The tile whose wait ends last tells the host: a wait that gave up set
+        // the status word before its tile counted itself here, so the host learns
+        // of every one with the count.
+        if (host) {
+            __threadfence();
+            if (atomicAdd(done, 1u) == (uint32_t)ntiles - 1u) {
+                __threadfence();
+                tell_host(host, (uint32_t)nv, *(volatile uint32_t *)d_total,
+                          *(volatile uint32_t *)err, seq);
+            }
+        }
     }
     const unsigned long long pre = excl + before;
 #pragma unroll
@@ -780,8 +791,9 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
         set_error("depth sort of %lld Gaussians exceeds 2^30", (long long)n);
         return SG_ERR_OVERFLOW;
     }
-    // after the radix scratch, zeroed with it: two tickets, then one 64-bit
-    // word per tile for each of the two chained scans
+    // after the radix scratch, zeroed with it: two tickets and the number of
+    // offset tiles done (four words), then one 64-bit word per tile for each of
+    // the two chained scans
     const int64_t ntiles = (n + kChainTile - 1) / kChainTile;
     if (fr.hist.bytes < sizeof(uint32_t) * (size_t)depth_stage_words(n)) {
         set_error("internal: depth stage scratch missing");
@@ -791,7 +803,7 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     sg_status s;
     static_assert(radix_scratch_words(1, 4) % 2 == 0, "64-bit chain words stay aligned");
     unsigned long long *chain = (unsigned long long *)(hist + radix_scratch_words(n, 4));
-    uint32_t *tickets = (uint32_t *)chain;                 // [0] compaction, [1] offsets
+    uint32_t *tickets = (uint32_t *)chain;      // [0] compaction, [1] offsets, [2] offsets done
     uint32_t *err = (uint32_t *)fr.scalars.p + kScalStatus;
     if (n <= kSmallN) {
         // one block zeroes what a scene of this size needs of the tile sort's
@@ -819,7 +831,7 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
     auto k_off = small ? k_pair_offsets<kOffSmall> : k_pair_offsets<kOffLarge>;
     launch_after(k_off, (unsigned)((n + off_tile - 1) / off_tile), kChainThreads, 0, st,
         vals[*result_buf], d_count, n, d_scal, d_offsets, d_scal + 1, chain + 2 + ntiles,
-        tickets + 1, err, (uint32_t *)fr.owner.p, (int64_t)(fr.owner.bytes / 4),
+        tickets + 1, tickets + 2, err, (uint32_t *)fr.owner.p, (int64_t)(fr.owner.bytes / 4),
         host_seq ? (volatile uint32_t *)fr.h_scalars : nullptr, host_seq);
     SG_LAUNCHED();
     return SG_OK;
