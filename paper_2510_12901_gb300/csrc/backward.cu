@@ -24,16 +24,15 @@
 // dL/dD^2, b = (dL/dtau) / |den|^2 and u = a q - b den,
 //   dL/dM = S M^-T,  S = sum (u q^T - b q den^T)  (symmetric),
 //   dL/dmu = -M^T sum u:
-// 13 sums a Gaussian (6 of S, 3 of u, sum x / sigma for dL/dsigma, 3 of the
-// features) that need neither M^-1 nor the ray's direction.  A last
+// 13 sums a Gaussian (6 of S, 3 of u, dL/dsigma, 3 of the features) that need neither M^-1 nor the ray's direction.  A last
 // per-Gaussian kernel maps them to the raw parameters (M = S^-1 R^T, R of the
 // normalised quaternion, SH colour at the direction from the camera to the
 // mean).
 //
 // Two phases per 16 staged entries.  Lanes are rays first: each walks the
 // entries in list order, as the forward, and leaves two numbers per pair in
-// shared memory, w = alpha T and x = alpha dL/dalpha (0 where alpha is clamped
-// or the pair does not composite).  Then lanes are entries (two lanes each,
+// shared memory, w = alpha T and y = rho dL/dalpha, which is the pair's
+// dL/dsigma (both 0 where the pair does not composite, y where alpha is clamped).  Then lanes are entries (two lanes each,
 // half of the rays a lane): each evaluates its pairs' num and den again and
 // adds the 13 terms in registers.  One shuffle a sum joins the two halves and
 // four 16-byte atomics a Gaussian add them to its row.  The kernels are bound
@@ -62,23 +61,23 @@ struct RayGrad {
     float T, U, Ut;  // transmittance and gQ . Q before the entry, gQ . Q of the ray
 };
 
-// Front-to-back step of one composited entry with features q: returns (w, x).
+// Front-to-back step of one composited entry with features q: returns (w, y).
 __device__ __forceinline__ float2 ray_step(RayGrad &r, const PairEval &pe, const float q[3])
 {
     const float w = pe.alpha * r.T;
     const float gq = r.gQ[0] * q[0] + r.gQ[1] * q[1] + r.gQ[2] * q[2] + r.gQ[3] * pe.tau + r.gQ[4];
     const float Ua = r.U + gq * w, om = 1.f - pe.alpha;
-    const float dLda = gq * r.T - __fdividef(r.Ut - Ua, om);
+    const float dLda = gq * r.T - (r.Ut - Ua) / om;
     r.U = Ua;
     r.T = r.T * om;
-    return make_float2(w, pe.clamped ? 0.f : dLda * pe.alpha);
+    return make_float2(w, pe.clamped ? 0.f : dLda * pe.rho);
 }
 
 // The sums of one Gaussian.
 struct GaussSums {
     float S[6];      // 00 01 02 11 12 22
     float u[3];
-    float x;
+    float y;
     float F[3];
 };
 
@@ -88,29 +87,30 @@ __device__ __forceinline__ void clear(GaussSums &g)
     for (int k = 0; k < 6; ++k) g.S[k] = 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) g.u[k] = g.F[k] = 0.f;
-    g.x = 0.f;
+    g.y = 0.f;
 }
 
-// Add one pair: num scaled by 1 / nscale, den, (w, x) and the ray's upstream
-// (gF, gZ).
+// Add one pair: num scaled by 1 / nscale, den, sigma, (w, y) and the ray's
+// upstream (gF, gZ).
 __device__ __forceinline__ void add_pair(GaussSums &g, const float n[3], const float e[3],
-                                         float nscale, float2 wx, const float gF[3], float gZ)
+                                         float nscale, float sigma, float2 wy, const float gF[3],
+                                         float gZ)
 {
     const float inv = __fdividef(1.f, e[0] * e[0] + e[1] * e[1] + e[2] * e[2]);
     const float c = inv * nscale;
     const float q[3] = {(n[1] * e[2] - n[2] * e[1]) * c, (n[2] * e[0] - n[0] * e[2]) * c,
                         (n[0] * e[1] - n[1] * e[0]) * c};
-    // a = 2 dL/dD^2 = -x (dalpha/dD^2 = -alpha / 2); b = gZ w / |den|^2
-    const float b = gZ * wx.x * inv;
+    // a = 2 dL/dD^2 = -sigma y (dalpha/dD^2 = -sigma rho / 2); b = gZ w / |den|^2
+    const float x = sigma * wy.y, b = gZ * wy.x * inv;
     float u[3], bq[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        u[k] = -(wx.y * q[k] + b * e[k]);
+        u[k] = -(x * q[k] + b * e[k]);
         bq[k] = b * q[k];
         g.u[k] += u[k];
-        g.F[k] += gF[k] * wx.x;
+        g.F[k] += gF[k] * wy.x;
     }
-    g.x += wx.y;
+    g.y += wy.y;
     g.S[0] += u[0] * q[0] - bq[0] * e[0];
     g.S[1] += u[0] * q[1] - bq[0] * e[1];
     g.S[2] += u[0] * q[2] - bq[0] * e[2];
@@ -120,9 +120,9 @@ __device__ __forceinline__ void add_pair(GaussSums &g, const float n[3], const f
 }
 
 // Join the halves of an entry's rays (lanes L and L ^ 16) and add the sums to
-// the Gaussian's row: S 0..5, u 6..8, sum x / sigma 9, F 10..12.  Every lane
-// calls it; `use`: the entry has a composited pair.
-__device__ __forceinline__ void add_sums(GaussSums &g, float sigma, bool use, float *row)
+// the Gaussian's row: S 0..5, u 6..8, sum y 9, F 10..12.  Every lane calls it;
+// `use`: the entry has a composited pair.
+__device__ __forceinline__ void add_sums(GaussSums &g, bool use, float *row)
 {
 #pragma unroll
     for (int k = 0; k < 6; ++k) g.S[k] += __shfl_xor_sync(0xffffffffu, g.S[k], 16);
@@ -131,11 +131,11 @@ __device__ __forceinline__ void add_sums(GaussSums &g, float sigma, bool use, fl
         g.u[k] += __shfl_xor_sync(0xffffffffu, g.u[k], 16);
         g.F[k] += __shfl_xor_sync(0xffffffffu, g.F[k], 16);
     }
-    g.x += __shfl_xor_sync(0xffffffffu, g.x, 16);
+    g.y += __shfl_xor_sync(0xffffffffu, g.y, 16);
     if (!use) return;
     if (threadIdx.x & 16) {
         atomicAdd(reinterpret_cast<float4 *>(row) + 2,
-                  make_float4(g.u[2], __fdividef(g.x, sigma), g.F[0], g.F[1]));
+                  make_float4(g.u[2], g.y, g.F[0], g.F[1]));
         atomicAdd(row + 12, g.F[2]);
     } else {
         atomicAdd(reinterpret_cast<float4 *>(row), make_float4(g.S[0], g.S[1], g.S[2], g.S[3]));
@@ -185,7 +185,7 @@ constexpr int kBwPass = 2;
 // ------------------------------------------------------------------ camera
 struct BwCam {                     // a warp's shared memory
     float4 e[8][32];               // staged entries (cam_entry's planes 0..7)
-    float2 wx[kBwBatch][33];       // (w, x) per (entry, ray); rows an odd number of banks apart
+    float2 wy[kBwBatch][33];       // (w, y) per (entry, ray); rows an odd number of banks apart
     float4 ray[2][32];             // (dd, gZ), (gF, 0)
     EntryQueue<kBwQueue> q;
     uint32_t pos[32], lanes[32], gid[32];
@@ -229,13 +229,13 @@ __device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose
 #pragma unroll
             for (int k = 0; k < kBwPass; ++k) {
                 const int i = min(b0 + j0 + k, n - 1);
-                float2 wx = make_float2(0.f, 0.f);
+                float2 wy = make_float2(0.f, 0.f);
                 if (ok[k]) {
                     const float4 col = S.e[7][i];
                     const float q[3] = {col.x, col.y, col.z};
-                    wx = ray_step(r, pe[k], q);
+                    wy = ray_step(r, pe[k], q);
                 }
-                if (kBwPass == 1 || j0 + k < kBwBatch) S.wx[j0 + k][lane] = wx;
+                if (kBwPass == 1 || j0 + k < kBwBatch) S.wy[j0 + k][lane] = wy;
                 used |= (__any_sync(0xffffffffu, ok[k]) ? 1u : 0u) << (j0 + k);
             }
         }
@@ -249,11 +249,12 @@ __device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose
         const int il = use ? i : b0;
         const float4 e0 = S.e[0][il], e1 = S.e[1][il], e2 = S.e[2][il];
         const float4 e3 = S.e[3][il], e4 = S.e[4][il], e5 = S.e[5][il];
+        const float sigma = S.e[6][il].w;
 #pragma unroll 8
         for (int k = 0; k < 16; ++k) {
             const float4 d = S.ray[0][r0 + k], f = S.ray[1][r0 + k];
-            const float2 wx = use ? S.wx[j][r0 + k] : make_float2(0.f, 0.f);
-            if (wx.x == 0.f) continue;      // not composited
+            const float2 wy = use ? S.wy[j][r0 + k] : make_float2(0.f, 0.f);
+            if (wy.x == 0.f) continue;      // not composited
             const float2 xx = make_float2(d.x, d.x), yy = make_float2(d.y, d.y);
             const float2 zz = make_float2(d.z, d.z);
             const float2 v0 = fma2(hi2(e3), zz, fma2(lo2(e3), yy, fma2(hi2(e0), xx, lo2(e0))));
@@ -261,9 +262,9 @@ __device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose
             const float2 v2 = fma2(hi2(e5), zz, fma2(lo2(e5), yy, fma2(hi2(e2), xx, lo2(e2))));
             const float num[3] = {v0.x, v1.x, v2.x}, den[3] = {v0.y, v1.y, v2.y};
             const float gF[3] = {f.x, f.y, f.z};
-            add_pair(g, num, den, 1.f / kResponseScale, wx, gF, d.w);
+            add_pair(g, num, den, 1.f / kResponseScale, sigma, wy, gF, d.w);
         }
-        add_sums(g, S.e[6][il].w, use, gacc + (int64_t)S.gid[il] * kG);
+        add_sums(g, use, gacc + (int64_t)S.gid[il] * kG);
         __syncwarp();
     }
 }
@@ -365,7 +366,7 @@ k_backward_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__r
 // slots.
 struct BwPosed {                   // a warp's shared memory
     float4 s[(3 * 32 + kBwBatch * kLidEntryStride + 31) / 32][32];
-    float2 wx[kBwBatch][33];
+    float2 wy[kBwBatch][33];
     float4 ray[3][32];             // (dd, gZ), (d, slot), (gF, 0)
     EntryQueue<kBwQueue> q;
     uint32_t pos[kBwBatch], lanes[kBwBatch], gid[kBwBatch];
@@ -391,9 +392,9 @@ __device__ __forceinline__ void posed_stage(const GRec *__restrict__ rec, BwPose
 
 // Phase 2 of one pair: entry j, ray k (rows of M in m).
 __device__ __forceinline__ void posed_pair(GaussSums &g, BwPosed &S, int j, int k, const float4 m[3],
-                                           float2 wx)
+                                           float2 wy)
 {
-    if (wx.x == 0.f) return;     // not composited
+    if (wy.x == 0.f) return;     // not composited
     const float4 a = S.ray[0][k], d = S.ray[1][k], f = S.ray[2][k];
     const int sl = __float_as_int(d.w);
     const float4 q0 = lid_col(S.s, j, 0, sl), q1 = lid_col(S.s, j, 1, sl), q2 = lid_col(S.s, j, 2, sl);
@@ -404,7 +405,7 @@ __device__ __forceinline__ void posed_pair(GaussSums &g, BwPosed &S, int j, int 
 #pragma unroll
     for (int i = 0; i < 3; ++i) den[i] = m[i].x * d.x + m[i].y * d.y + m[i].z * d.z;
     const float gF[3] = {f.x, f.y, f.z};
-    add_pair(g, num, den, 1.f, wx, gF, a.w);
+    add_pair(g, num, den, 1.f, m[0].w, wy, gF, a.w);
 }
 
 // ------------------------------------------------------------------ rolling shutter
@@ -495,12 +496,12 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
                     bool ok = lidar_pair_in(S.s, j, sb, (S.lanes[j] >> lane) & 1u, dd, d,
                                             P.alpha_min, P.alpha_max, pe);
                     ok = ok && S.pos[j] <= last;
-                    float2 wx = make_float2(0.f, 0.f);
+                    float2 wy = make_float2(0.f, 0.f);
                     if (ok) {
                         const float q[3] = {S.s[1][j].w, S.s[2][j].w, lid_u(S.s, j, sb).w};
-                        wx = ray_step(r, pe, q);
+                        wy = ray_step(r, pe, q);
                     }
-                    S.wx[j][lane] = wx;
+                    S.wy[j][lane] = wy;
                     used |= (__any_sync(0xffffffffu, ok) ? 1u : 0u) << j;
                 }
                 __syncwarp();
@@ -514,8 +515,8 @@ k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *
 #pragma unroll 2
                 for (int k = 0; k < 16; ++k)
                     posed_pair(g, S, jl, r0 + k, m,
-                               use ? S.wx[j][r0 + k] : make_float2(0.f, 0.f));
-                add_sums(g, m[0].w, use, gacc + (int64_t)S.gid[jl] * kG);
+                               use ? S.wy[j][r0 + k] : make_float2(0.f, 0.f));
+                add_sums(g, use, gacc + (int64_t)S.gid[jl] * kG);
             }
         }
         __syncwarp();
@@ -645,13 +646,13 @@ k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
 #pragma unroll
                     for (int k = 0; k < kBwPass; ++k) {
                         const int j = jj[k];
-                        float2 wx = make_float2(0.f, 0.f);
+                        float2 wy = make_float2(0.f, 0.f);
                         if (ok[k]) {
                             const float q[3] = {S.s[1][j].w, S.s[2][j].w, lid_u(S.s, j, sb).w};
-                            wx = ray_step(r, pe[k], q);
+                            wy = ray_step(r, pe[k], q);
                             used |= 1u << j;
                         }
-                        if (in[k]) S.wx[j][lane] = wx;
+                        if (in[k]) S.wy[j][lane] = wy;
                     }
                 }
                 used = __reduce_or_sync(0xffffffffu, used);
@@ -667,10 +668,10 @@ k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
                 while (rays) {
                     const int k = r0 + __ffs(rays) - 1;
                     rays &= rays - 1u;
-                    posed_pair(g, S, jl, k, m, S.wx[jl][k]);
+                    posed_pair(g, S, jl, k, m, S.wy[jl][k]);
                 }
                 __syncwarp();
-                add_sums(g, m[0].w, use, gacc + (int64_t)S.gid[jl] * kG);
+                add_sums(g, use, gacc + (int64_t)S.gid[jl] * kG);
             }
         }
     }
