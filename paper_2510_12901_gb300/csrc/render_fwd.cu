@@ -30,20 +30,28 @@ namespace sg {
 
 constexpr int kFwdWarps = 4;        // warps per block of the persistent grid
 // Blocks per SM (4 and 6: 80 registers; 8: 64, a few bytes of the merge spill).
-// Few warps walk faster, and below a few million pairs the launch ends with the
-// dense tiles' chain of merges and re-walks; many hide more latency.  Measured, 4
-// / 6 / 8 blocks in us: 641x479 of 150k Gaussians (0.16M pairs) 32 / 34 / 38,
-// 1024x768 of 500k (0.68M) 137 / 150 / 177, 1280x960 of 333k (0.42M) 104 / 104 /
-// 124, 1920x1080 of 333k (0.69M) 193 / 156 / 188, of 1M (2.0M) 408 / 339 / 374, of
-// 1.5M (3.0M) 582 / 492 / 482, of 2M (3.9M) 763 / 651 / 625; 1920x1280 fisheye of
-// 1M (1.5M) 322 / 264 / 304, of 1.5M (2.2M) 438 / 364 / 377.  Renders that
-// overlap with others fill each other's ends, and take 8: the views of one call
-// (both street views of 1M in steps queued one after another 4636 Mrays/s, 4392
-// with the rule for one view) and frames in capacity mode, which are a server's (12
-// requests 1595 and 1655 us).
-constexpr int fwd_blocks(int n_tiles, int64_t n_pairs, bool overlaps)
+// Few warps walk faster, and with few pairs the launch ends with the dense tiles'
+// chain of merges and re-walks, the longer the fewer tiles there are; many warps
+// hide more latency, which counts the more pairs there are.  Measured, 4 / 6 / 8
+// blocks in us, pinhole street views, by pairs:
+//   320x240    0.97M 224 / 238 / 267   3.9M 742 / 748 / 867     7.8M 834 / 793 / 871
+//   640x480    1.1M 203 / 224 / 260    2.3M 298 / 333 / 375     4.5M 605 / 559 / 669
+//              9.0M 1158 / 955 / 904
+//   800x600    1.2M 199 / 218 / 263    2.5M 337 / 335 / 388     4.9M 713 / 595 / 670
+//   1024x768   1.4M 226 / 239 / 275    2.7M 429 / 360 / 407     5.5M 902 / 756 / 724
+//   1280x720   0.45M 111 / 119 / 132   1.5M 259 / 251 / 293     6.0M 1041 / 881 / 842
+//   1280x960   0.42M 104 / 104 / 124   3.1M 541 / 456 / 476     6.3M 1136 / 960 / 915
+//   1600x900   1.7M 335 / 289 / 340    3.4M 629 / 534 / 525
+//   1920x1080  0.69M 193 / 156 / 188   2.0M 408 / 339 / 374     3.0M 582 / 492 / 482
+// Renders that overlap with others fill each other's ends, and take 8: views of
+// one call on streams of their own (both street views of 1M in steps queued one
+// after another 4636 Mrays/s, 4392 with the rule for one view) and frames in
+// capacity mode, which are a server's (12 requests 1595 and 1655 us).
+constexpr int fwd_blocks(int64_t n_tiles, int64_t n_pairs, bool overlaps)
 {
-    return overlaps ? 8 : n_tiles < 4000 ? 4 : n_pairs < 2700000 ? 6 : 8;
+    if (overlaps) return 8;
+    if (n_tiles < 4000 && n_pairs < 4500000 && n_pairs * n_tiles < 4500000000LL) return 4;
+    return n_pairs < (n_tiles < 2000 ? 7000000 : n_tiles < 5000 ? 4300000 : 2700000) ? 6 : 8;
 }
 // List entries a warp scans at a time: kFwdPer per lane.  Those that reach a
 // live ray of the sub-block (about a third on the street views) go to a queue
