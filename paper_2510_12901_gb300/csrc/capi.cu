@@ -444,7 +444,7 @@ static sg_status sort_and_bin(Frame &fr, int64_t n, int ntx, int64_t ntiles, int
 static sg_status camera_begin(sg_scene scene, sg_camera cam, const float h_c2w[12],
                               const sg_render_opts *opts, sg_frame frame, float *d_rgb,
                               float *d_alpha, float *d_depth, cudaStream_t st,
-                              const float *d_row_c2w = nullptr, bool one_of_many = false)
+                              const float *d_row_c2w = nullptr, bool beside_others = false)
 {
     if (!scene || !cam || !frame || !h_c2w) { set_error("NULL handle or pose"); return SG_ERR_INVALID; }
     if (!opts_ok(opts)) return SG_ERR_INVALID;
@@ -461,7 +461,7 @@ static sg_status camera_begin(sg_scene scene, sg_camera cam, const float h_c2w[1
     sg_status s = frame_prepare(fr, sc.n, nr, nt);
     if (s != SG_OK) return s;
     fr.kind = d_row_c2w ? 2 : 0;
-    fr.one_of_many = one_of_many;
+    fr.beside_others = beside_others;
     fr.scene = scene;
     fr.sensor = cam;
     fr.opts = *opts;
@@ -945,8 +945,11 @@ sg_status sg_render_cameras(sg_scene scene, int n_views, const sg_camera_view *v
             set_error("view %d: a rolling-shutter view cannot use an allocation-free frame", i);
             return SG_ERR_INVALID;
         }
+        // views on one stream follow one another
+        bool beside = false;
+        for (int j = 0; j < n_views; ++j) beside = beside || views[j].stream != v.stream;
         s = camera_begin(scene, v.camera, v.c2w, opts, v.frame, out[0], out[1], out[2],
-                         (cudaStream_t)v.stream, v.row_c2w, n_views > 1);
+                         (cudaStream_t)v.stream, v.row_c2w, beside);
         if (s != SG_OK) return s;
     }
     for (int i = 0; i < n_views; ++i) {

@@ -274,7 +274,7 @@ struct Frame {
     uint32_t *h_scalars = nullptr;  // pinned: scalars mirror (64 B), then the RenderDesc
     RenderDesc *h_desc = nullptr;   // staging of desc (pinned)
     bool desc_direct = false;       // the projection takes *h_desc by value
-    bool one_of_many = false;       // the call renders other views beside this one
+    bool beside_others = false;     // the call renders views on other streams beside this one
     // capacity mode: > 0 = the pair buffers hold this many pairs and no
     // step waits for the pair count (pairs beyond it are dropped and counted)
     int64_t k_cap = 0;

@@ -46,7 +46,9 @@ constexpr int kFwdWarps = 4;        // warps per block of the persistent grid
 // Renders that overlap with others fill each other's ends, and take 8: views of
 // one call on streams of their own (both street views of 1M in steps queued one
 // after another 4636 Mrays/s, 4392 with the rule for one view) and frames in
-// capacity mode, which are a server's (12 requests 1595 and 1655 us).
+// capacity mode, which are a server's (12 requests 1595 and 1655 us).  Views that
+// follow one another on one stream take the rule for one view (the same two views
+// 1177 us with 8 blocks, 1113 with the rule).
 constexpr int fwd_blocks(int64_t n_tiles, int64_t n_pairs, bool overlaps)
 {
     if (overlaps) return 8;
@@ -532,7 +534,7 @@ sg_status render_camera_fwd(const Camera &cam, const sg_render_opts &o, Frame &f
     SG_CUDA(cudaGetDevice(&dev));
     SG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t cap = (ws.max_items + kFwdWarps - 1) / kFwdWarps;
-    const int nb = fwd_blocks(nt, K, fr.k_cap > 0 || fr.one_of_many);
+    const int nb = fwd_blocks(nt, K, fr.k_cap > 0 || fr.beside_others);
     int64_t grid = (int64_t)sms * nb;
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
