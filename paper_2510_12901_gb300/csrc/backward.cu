@@ -270,16 +270,16 @@ __device__ __forceinline__ void bw_batch(const CamRender &P, const CamPose &pose
 }
 
 __global__ void __launch_bounds__(32 * kBwWarps, kBwCamBlocks)
-k_backward_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
-                  const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
-                  const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
-                  const uint32_t *__restrict__ crw, uint32_t *__restrict__ counter,
-                  const float4 *__restrict__ partials, const float4 *__restrict__ pix,
-                  const double *__restrict__ tile_dir, const RenderDesc *__restrict__ D,
-                  const float4 *__restrict__ ray_state, const float4 *__restrict__ ray_feat,
-                  const uint32_t *__restrict__ n_contrib, const float *__restrict__ g_rgb,
-                  const float *__restrict__ g_alpha, const float *__restrict__ g_depth,
-                  float *__restrict__ gacc)
+k_backward_camera(CamRender P, const GRec *rec, const uint32_t *ids,
+                  const uint2 *ranges, const uint2 *items,
+                  const uint2 *tile_info, const uint32_t *counts,
+                  const uint32_t *crw, uint32_t *counter,
+                  const float4 *partials, const float4 *__restrict__ pix,
+                  const double *__restrict__ tile_dir, const RenderDesc *D,
+                  const float4 *ray_state, const float4 *ray_feat,
+                  const uint32_t *n_contrib, const float *g_rgb,
+                  const float *g_alpha, const float *g_depth,
+                  float *gacc)
 {
     after_previous();
     __shared__ BwCam s_all[kBwWarps];
@@ -411,16 +411,16 @@ __device__ __forceinline__ void posed_pair(GaussSums &g, BwPosed &S, int j, int 
 // ------------------------------------------------------------------ rolling shutter
 // The camera backward with a pose per pixel row.
 __global__ void __launch_bounds__(32 * kBwWarpsPosed)
-k_backward_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
-                     const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
-                     const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
-                     const uint32_t *__restrict__ crw, uint32_t *__restrict__ counter,
-                     const float4 *__restrict__ partials, const float4 *__restrict__ pix,
+k_backward_camera_rs(CamRender P, const GRec *rec, const uint32_t *ids,
+                     const uint2 *ranges, const uint2 *items,
+                     const uint2 *tile_info, const uint32_t *counts,
+                     const uint32_t *crw, uint32_t *counter,
+                     const float4 *partials, const float4 *__restrict__ pix,
                      const double *__restrict__ tile_dir, const float *__restrict__ poses,
-                     const float4 *__restrict__ ray_state, const float4 *__restrict__ ray_feat,
-                     const uint32_t *__restrict__ n_contrib, const float *__restrict__ g_rgb,
-                     const float *__restrict__ g_alpha, const float *__restrict__ g_depth,
-                     float *__restrict__ gacc)
+                     const float4 *ray_state, const float4 *ray_feat,
+                     const uint32_t *n_contrib, const float *g_rgb,
+                     const float *g_alpha, const float *g_depth,
+                     float *gacc)
 {
     after_previous();
     __shared__ BwPosed s_all[kBwWarpsPosed];
@@ -531,16 +531,16 @@ __global__ void __launch_bounds__(32 * kBwWarpsPosed)
 k_backward_lidar(LidRender P, const LidarItem *__restrict__ items,
                  const uint32_t *__restrict__ item_rays, const float4 *__restrict__ ray_e,
                  const double *__restrict__ item_u, const float *__restrict__ poses,
-                 const uint2 *__restrict__ tile_items, const uint32_t *__restrict__ lmask,
-                 int64_t lmask_stride, const GRec *__restrict__ rec,
-                 const uint32_t *__restrict__ ids,
-                 const uint2 *__restrict__ ranges, const uint2 *__restrict__ work,
-                 const uint2 *__restrict__ unit_info, const uint32_t *__restrict__ counts,
-                 uint32_t *__restrict__ counter, const float4 *__restrict__ partials,
-                 const float4 *__restrict__ ray_state, const float4 *__restrict__ ray_feat,
-                 const uint32_t *__restrict__ n_contrib, const float *__restrict__ g_range,
-                 const float *__restrict__ g_int, const float *__restrict__ g_drop,
-                 const float *__restrict__ g_alpha, float *__restrict__ gacc)
+                 const uint2 *__restrict__ tile_items, const uint32_t *lmask,
+                 int64_t lmask_stride, const GRec *rec,
+                 const uint32_t *ids,
+                 const uint2 *ranges, const uint2 *work,
+                 const uint2 *unit_info, const uint32_t *counts,
+                 uint32_t *counter, const float4 *partials,
+                 const float4 *ray_state, const float4 *ray_feat,
+                 const uint32_t *n_contrib, const float *g_range,
+                 const float *g_int, const float *g_drop,
+                 const float *g_alpha, float *gacc)
 {
     after_previous();
     __shared__ BwPosed s_all[kBwWarpsPosed];
@@ -816,10 +816,10 @@ __device__ __forceinline__ void add_rows(float *__restrict__ out, int64_t g0, in
 template <int kDeg, bool kWrite>
 __global__ void __launch_bounds__(kPgThreads)
 k_param_grads(const float *__restrict__ planes, int64_t pitch, int64_t n, int lidar, float ox,
-              float oy, float oz, const GRec *__restrict__ rec, const float *__restrict__ poses,
-              ActorParams A, float beam, int posed_origin, float *__restrict__ gacc,
-              float *__restrict__ gm, float *__restrict__ gls, float *__restrict__ gq,
-              float *__restrict__ gop, float *__restrict__ gf)
+              float oy, float oz, const GRec *rec, const float *__restrict__ poses,
+              ActorParams A, float beam, int posed_origin, float *gacc,
+              float *gm, float *gls, float *gq,
+              float *gop, float *gf)
 {
     after_previous();
     constexpr int nc = kDeg < 0 ? 1 : (kDeg + 1) * (kDeg + 1), F = 3 * nc;

@@ -103,7 +103,12 @@ inline void launch_after(void (*kern)(P...), unsigned grid, unsigned block, size
 }
 
 #ifdef __CUDACC__
-// The first statement of a kernel launched by launch_after.
+// The first statement of a kernel launched by launch_after.  Before it returns the
+// stream's previous kernel may still write, so nothing that kernel writes is read
+// above it.  The asm's memory clobber says so to the compiler, but not of memory
+// that a parameter promises nobody else changes: of such a kernel's parameters
+// only what it writes and does not read, and tables made before the render's
+// first kernel, are __restrict__.
 __device__ __forceinline__ void after_previous()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

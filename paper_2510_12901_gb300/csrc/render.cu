@@ -182,7 +182,7 @@ constexpr int kWorkOneTiles = kWorkThreads * kWorkChunks;
 constexpr int kWorkShare = 256, kWorkPerWarp = kWorkShare / (kWorkThreads / 32);
 
 __global__ void __launch_bounds__(kWorkThreads)
-k_work_items(const uint2 *__restrict__ ranges, const uint2 *__restrict__ tile_items, int n_tiles,
+k_work_items(const uint2 *ranges, const uint2 *__restrict__ tile_items, int n_tiles,
              int subs, uint32_t seg_len, uint32_t *__restrict__ counts,
              uint32_t *__restrict__ counter, uint2 *__restrict__ unit_info,
              uint2 *__restrict__ items, uint32_t *__restrict__ arrive)
@@ -463,13 +463,13 @@ __device__ __forceinline__ CamAcc get_state(float4 u, float4 v)
 
 template <uint32_t kSeg>
 __global__ void __launch_bounds__(32 * kCamWarps, kCamBlocks)
-k_render_camera(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
-                const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
-                const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
-                const uint32_t *__restrict__ crw, uint32_t *__restrict__ counter,
-                uint32_t *__restrict__ arrive, float4 *__restrict__ partials,
+k_render_camera(CamRender P, const GRec *rec, const uint32_t *ids,
+                const uint2 *ranges, const uint2 *items,
+                const uint2 *tile_info, const uint32_t *counts,
+                const uint32_t *crw, uint32_t *counter,
+                uint32_t *arrive, float4 *partials,
                 const float4 *__restrict__ pix, const double *__restrict__ tile_dir,
-                const RenderDesc *__restrict__ D, float4 *__restrict__ ray_state,
+                const RenderDesc *D, float4 *__restrict__ ray_state,
                 float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
     after_previous();
@@ -727,13 +727,13 @@ __device__ __forceinline__ void cam_rs_ray(const float *__restrict__ poses,
 constexpr int kRsWarps = 4;        // warps per block
 template <uint32_t kSeg>
 __global__ void __launch_bounds__(32 * kRsWarps)
-k_render_camera_rs(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
-                   const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
-                   const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
-                   const uint32_t *__restrict__ crw, uint32_t *__restrict__ counter,
-                   uint32_t *__restrict__ arrive, float4 *__restrict__ partials,
+k_render_camera_rs(CamRender P, const GRec *rec, const uint32_t *ids,
+                   const uint2 *ranges, const uint2 *items,
+                   const uint2 *tile_info, const uint32_t *counts,
+                   const uint32_t *crw, uint32_t *counter,
+                   uint32_t *arrive, float4 *partials,
                    const float4 *__restrict__ pix, const double *__restrict__ tile_dir,
-                   const RenderDesc *__restrict__ D, float4 *__restrict__ ray_state,
+                   const RenderDesc *D, float4 *__restrict__ ray_state,
                    float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
     after_previous();
@@ -1025,13 +1025,13 @@ __global__ void __launch_bounds__(32 * kLidarWarps)
 k_render_lidar(LidRender P, const LidarItem *__restrict__ items,
                const uint32_t *__restrict__ item_rays, const float4 *__restrict__ ray_e,
                const double *__restrict__ item_u, const uint2 *__restrict__ tile_items,
-               const uint32_t *__restrict__ lmask, int64_t lmask_stride,
-               const GRec *__restrict__ rec,
-               const uint32_t *__restrict__ ids, const uint2 *__restrict__ ranges,
-               const uint2 *__restrict__ work, const uint2 *__restrict__ unit_info,
-               const uint32_t *__restrict__ counts, uint32_t *__restrict__ counter,
-               uint32_t *__restrict__ arrive, float4 *__restrict__ partials, FixList F,
-               const RenderDesc *__restrict__ D, float4 *__restrict__ ray_state,
+               const uint32_t *lmask, int64_t lmask_stride,
+               const GRec *rec,
+               const uint32_t *ids, const uint2 *ranges,
+               const uint2 *work, const uint2 *unit_info,
+               const uint32_t *counts, uint32_t *counter,
+               uint32_t *arrive, float4 *partials, FixList F,
+               const RenderDesc *D, float4 *__restrict__ ray_state,
                float4 *__restrict__ ray_feat, uint32_t *__restrict__ n_contrib)
 {
     after_previous();

@@ -376,13 +376,13 @@ __device__ __forceinline__ void fwd_put(float4 *pq, const FwdAcc &a, bool stoppe
 
 template <uint32_t kSeg, int kBlocks>
 __global__ void __launch_bounds__(32 * kFwdWarps, kBlocks)
-k_render_camera_fwd(CamRender P, const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
-                    const uint2 *__restrict__ ranges, const uint2 *__restrict__ items,
-                    const uint2 *__restrict__ tile_info, const uint32_t *__restrict__ counts,
-                    const uint32_t *__restrict__ crw, uint32_t *__restrict__ counter,
-                    uint32_t *__restrict__ arrive, float4 *__restrict__ partials,
+k_render_camera_fwd(CamRender P, const GRec *rec, const uint32_t *ids,
+                    const uint2 *ranges, const uint2 *items,
+                    const uint2 *tile_info, const uint32_t *counts,
+                    const uint32_t *crw, uint32_t *counter,
+                    uint32_t *arrive, float4 *partials,
                     const float4 *__restrict__ pix2, const double *__restrict__ tile_dir,
-                    const float *__restrict__ tile_basis, const RenderDesc *__restrict__ D)
+                    const float *__restrict__ tile_basis, const RenderDesc *D)
 {
     after_previous();
     __shared__ float4 s_all[kFwdWarps][7][kFwdStage];

@@ -254,12 +254,12 @@ __global__ void __launch_bounds__(32 * kLfWarps, kLfBlocks)
 k_render_lidar_fwd(LidRender P, const LidarItem *__restrict__ items,
                    const uint32_t *__restrict__ item_rays, const float2 *__restrict__ ray_tau,
                    const double *__restrict__ item_ref, const uint2 *__restrict__ tile_items,
-                   const uint32_t *__restrict__ lmask, int64_t lmask_stride,
-                   const GRec *__restrict__ rec, const uint32_t *__restrict__ ids,
-                   const uint2 *__restrict__ ranges, const uint2 *__restrict__ work,
-                   const uint2 *__restrict__ unit_info, const uint32_t *__restrict__ counts,
-                   uint32_t *__restrict__ counter, uint32_t *__restrict__ arrive,
-                   float4 *__restrict__ partials, FixList F, const RenderDesc *__restrict__ D)
+                   const uint32_t *lmask, int64_t lmask_stride,
+                   const GRec *rec, const uint32_t *ids,
+                   const uint2 *ranges, const uint2 *work,
+                   const uint2 *unit_info, const uint32_t *counts,
+                   uint32_t *counter, uint32_t *arrive,
+                   float4 *partials, FixList F, const RenderDesc *D)
 {
     after_previous();
     __shared__ LfShared s_all[kLfWarps];

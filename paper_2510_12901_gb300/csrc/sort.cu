@@ -147,11 +147,11 @@ __device__ __forceinline__ bool published(const uint4 &w)
 }
 
 __global__ void __launch_bounds__(kRadixThreads, 2)
-k_onesweep(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
+k_onesweep(const uint32_t *keys_in, const uint32_t *vals_in,
            uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out,
-           const uint32_t *__restrict__ d_n, int shift, uint32_t mask,
-           const uint32_t *__restrict__ hist, uint32_t *__restrict__ lookback,
-           uint32_t *__restrict__ ticket, uint32_t *__restrict__ err, int site)
+           const uint32_t *d_n, int shift, uint32_t mask,
+           const uint32_t *hist, uint32_t *lookback,
+           uint32_t *ticket, uint32_t *err, int site)
 {
     after_previous();
     // the warps' digit counts, then the look-back groups' sums
@@ -450,11 +450,11 @@ __device__ __forceinline__ unsigned long long chain_lookback(unsigned long long 
 }
 
 __global__ void __launch_bounds__(kChainThreads)
-k_compact_depth(const uint32_t *__restrict__ count, const float *__restrict__ depth, int64_t n,
+k_compact_depth(const uint32_t *count, const float *depth, int64_t n,
                 int64_t ntiles, uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
-                uint32_t *__restrict__ d_nvalid, uint32_t *__restrict__ hist,
-                unsigned long long *__restrict__ lb, uint32_t *__restrict__ ticket,
-                uint32_t *__restrict__ err, uint4 *__restrict__ zero, int64_t nzero)
+                uint32_t *__restrict__ d_nvalid, uint32_t *hist,
+                unsigned long long *lb, uint32_t *ticket,
+                uint32_t *err, uint4 *__restrict__ zero, int64_t nzero)
 {
     after_previous();
     __shared__ uint32_t s_h[4][256];
@@ -548,10 +548,10 @@ __device__ __forceinline__ void put_offset(int64_t i, unsigned long long off, ui
 
 template <int kOffChunks>
 __global__ void __launch_bounds__(kChainThreads)
-k_pair_offsets(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ count, int64_t n,
-               const uint32_t *__restrict__ d_nvalid, uint32_t *__restrict__ offsets,
-               uint32_t *__restrict__ d_total, unsigned long long *__restrict__ lb,
-               uint32_t *__restrict__ ticket, uint32_t *__restrict__ done, uint32_t *__restrict__ err,
+k_pair_offsets(const uint32_t *ids, const uint32_t *count, int64_t n,
+               const uint32_t *d_nvalid, uint32_t *__restrict__ offsets,
+               uint32_t *d_total, unsigned long long *lb,
+               uint32_t *ticket, uint32_t *done, uint32_t *err,
                uint32_t *__restrict__ owner, int64_t owner_cap, volatile uint32_t *host, uint32_t seq)
 {
     after_previous();
@@ -645,10 +645,10 @@ constexpr int kSmallThreads = 1024, kSmallPer = 4, kSmallN = kSmallThreads * kSm
 constexpr size_t kSmallZero = 64 * 1024;
 
 __global__ void __launch_bounds__(kSmallThreads)
-k_depth_small(const uint32_t *__restrict__ count, const float *__restrict__ depth, int n,
+k_depth_small(const uint32_t *count, const float *depth, int n,
               uint32_t *__restrict__ vals, uint32_t *__restrict__ d_nvalid,
               uint32_t *__restrict__ offsets, uint32_t *__restrict__ d_total,
-              const uint32_t *__restrict__ err, uint32_t *__restrict__ owner, int64_t owner_cap,
+              const uint32_t *err, uint32_t *__restrict__ owner, int64_t owner_cap,
               volatile uint32_t *host, uint32_t seq, uint4 *__restrict__ zero, int64_t nzero)
 {
     after_previous();
@@ -867,11 +867,11 @@ __device__ __forceinline__ int pmod_i(int a, int n)
 }
 
 __global__ void __launch_bounds__(kBinThreads)
-k_bin(const uint32_t *__restrict__ ids, const uint32_t *__restrict__ offsets,
-      const uint32_t *__restrict__ d_scal, const int4 *__restrict__ tiles, int ntx, int wrap_x,
+k_bin(const uint32_t *ids, const uint32_t *offsets,
+      const uint32_t *d_scal, const int4 *tiles, int ntx, int wrap_x,
       uint32_t cap, uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
-      uint32_t *__restrict__ hist, int end_bit, const uint32_t *__restrict__ err,
-      const uint32_t *__restrict__ owner, int64_t owner_cap, uint2 *__restrict__ ranges,
+      uint32_t *hist, int end_bit, const uint32_t *err,
+      const uint32_t *owner, int64_t owner_cap, uint2 *__restrict__ ranges,
       int64_t ntiles)
 {
     after_previous();
@@ -1080,10 +1080,10 @@ __device__ __forceinline__ void write_ranges(const uint32_t *__restrict__ keys, 
 
 template <bool kMask>
 __global__ void __launch_bounds__(256)
-k_ranges(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K,
-         uint2 *__restrict__ ranges, const uint32_t *__restrict__ ids,
-         const float4 *__restrict__ rects, int ntx, float inv_ntx, uint32_t *__restrict__ mask,
-         const uint32_t *__restrict__ err)
+k_ranges(const uint32_t *keys, const uint32_t *d_K,
+         uint2 *__restrict__ ranges, const uint32_t *ids,
+         const float4 *rects, int ntx, float inv_ntx, uint32_t *__restrict__ mask,
+         const uint32_t *err)
 {
     after_previous();
     const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRangePer;
@@ -1146,11 +1146,11 @@ sg_status tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t K_max
 // them.  Measured (2M Gaussians, 3.7M pairs): one pair a thread 43 us, now 36
 // (38 with the table read word by word).
 __global__ void __launch_bounds__(256)
-k_ranges_lidar(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ d_K, int64_t stride,
-               uint2 *__restrict__ ranges, const uint32_t *__restrict__ ids,
-               const float4 *__restrict__ rects, const uint2 *__restrict__ tile_items,
+k_ranges_lidar(const uint32_t *keys, const uint32_t *d_K, int64_t stride,
+               uint2 *__restrict__ ranges, const uint32_t *ids,
+               const float4 *rects, const uint2 *__restrict__ tile_items,
                const LidarItemRays *__restrict__ tab, uint32_t *__restrict__ lmask,
-               const uint32_t *__restrict__ err)
+               const uint32_t *err)
 {
     after_previous();
     const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kRangePer;
@@ -1234,7 +1234,7 @@ sg_status lidar_tile_ranges(const uint32_t *d_keys, const uint32_t *d_K, int64_t
 
 // Capacity mode: keep at most `cap` pairs; d_K is clamped to it and the
 // number of pairs beyond it is stored in d_dropped (0 when all fit).
-__global__ void k_clamp_pairs(uint32_t *__restrict__ d_K, uint32_t cap,
+__global__ void k_clamp_pairs(uint32_t *d_K, uint32_t cap,
                               uint32_t *__restrict__ d_dropped)
 {
     after_previous();
