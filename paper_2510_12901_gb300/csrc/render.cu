@@ -596,7 +596,10 @@ sg_status render_camera(const Camera &cam, const sg_render_opts &o, Frame &fr, c
         return SG_ERR_INVALID;
     }
     if (camera_forward_only(cam, fr)) return render_camera_fwd(cam, o, fr, st);
-    const CamRender P = cam_render_params(cam, o);
+    CamRender P = cam_render_params(cam, o);
+    int dev = 0;
+    SG_CUDA(cudaGetDevice(&dev));
+    SG_CUDA(cudaDeviceGetAttribute(&P.sms, cudaDevAttrMultiProcessorCount, dev));
     const int nt = cam.ntx * cam.nty;
     const int64_t K = fr.n_pairs;
     const WorkSize ws = work_size(nt, K, fr.seg_len, 8);
@@ -618,8 +621,8 @@ sg_status render_camera(const Camera &cam, const sg_render_opts &o, Frame &fr, c
     const uint32_t *ids = (const uint32_t *)fr.pvals[fr.pair_buf].p;
     const int64_t cap = ws.max_items;      // a block an item: warp_takes_part picks
     const bool dflt = fr.seg_len == kSegLen;
-    int64_t grid = (int64_t)sm_count() * (dflt ? cam_blocks_per_sm<kSegLen>()
-                                        : cam_blocks_per_sm<kSegLenStatic>());
+    int64_t grid = (int64_t)P.sms * (dflt ? cam_blocks_per_sm<kSegLen>()
+                                          : cam_blocks_per_sm<kSegLenStatic>());
     grid = grid < cap ? grid : cap;
     if (grid < 1) grid = 1;
     auto kern = dflt ? k_render_camera<kSegLen> : k_render_camera<kSegLenStatic>;

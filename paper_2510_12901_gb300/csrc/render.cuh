@@ -7,7 +7,8 @@
 namespace sg {
 
 struct CamRender {
-    int W, H, ntx, sms;
+    int W, H, ntx;
+    int sms;                // SMs of the device (k_render_camera)
     float alpha_min, alpha_max, t_min;
 };
 
@@ -39,15 +40,6 @@ struct LidRender {
     float alpha_min, alpha_max, t_min;
 };
 
-inline int sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        sms = 152;
-    return sms;
-}
-
 // The warps of a persistent grid take their first items as they start, all of
 // an SM's at once, so with fewer items than warps the first SMs get more of
 // them.  A warp takes part only if it is among the first n_items when the warps
@@ -67,7 +59,7 @@ inline CamRender cam_render_params(const Camera &cam, const sg_render_opts &o)
     P.W = cam.width;
     P.H = cam.height;
     P.ntx = cam.ntx;
-    P.sms = sm_count();
+    P.sms = 0;
     P.alpha_min = o.alpha_min;
     P.alpha_max = o.alpha_max;
     P.t_min = o.t_min;
