@@ -1134,9 +1134,9 @@ sg_status sg_workspace_bytes(sg_scene scene, int sensor_kind, int64_t n_rays, si
     const size_t g[] = {sizeof(GRec), 16, 16, 4, 4, 8, 16, 4, 4, 4, 4, 4};
     for (size_t by : g) b += grown(by * (size_t)n);
     b += grown(sizeof(uint32_t) * (size_t)bin_owner_words(n));
-    // per ray: state, features, contributor count; per unit: ranges, order
+    // per ray: state, features, contributor count; per unit: ranges
     b += grown(16 * (size_t)nr) * 2 + grown(4 * (size_t)nr);
-    b += grown(8 * (size_t)units) + grown(4 * (size_t)units);
+    b += grown(8 * (size_t)units);
     // pairs: keys and ids (x2), camera column/row masks or LiDAR ray masks
     b += 4 * grown(4 * (size_t)K) + grown(4 * (size_t)K * per_tile);
     // sort scratch: the depth stage's and the tile sort's

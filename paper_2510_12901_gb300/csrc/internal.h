@@ -259,7 +259,7 @@ struct Frame {
     size_t tscratch_zeroed = 0;
     // pairs; LiDAR: per (work item of the pair's tile, pair) the 32-bit mask
     // of the item's rays inside the Gaussian's box, planes of lmask_stride
-    Buf pkeys[2], pvals[2], ranges, order, submask, lmask;
+    Buf pkeys[2], pvals[2], ranges, submask, lmask;
     int64_t lmask_stride = 0;
     // camera work items: per-tile (segments, first partial slot), items,
     // arrival counters of long tiles; per-pixel partials of their segments
@@ -512,7 +512,7 @@ template <class Fn> inline void for_each_buf(Frame &f, Fn fn)
 {
     Buf *bufs[] = {&f.rec, &f.rect, &f.tiles, &f.depth, &f.count, &f.mean2d, &f.cov2d,
                    &f.dkeys[0], &f.dkeys[1], &f.dvals[0], &f.dvals[1], &f.offsets, &f.hist, &f.owner, &f.tscratch,
-                   &f.pkeys[0], &f.pkeys[1], &f.pvals[0], &f.pvals[1], &f.ranges, &f.order, &f.submask,
+                   &f.pkeys[0], &f.pkeys[1], &f.pvals[0], &f.pvals[1], &f.ranges, &f.submask,
                    &f.lmask, &f.camwork,
                    &f.partials, &f.ray_state, &f.n_contrib, &f.ray_feat, &f.gacc, &f.scalars,
                    &f.desc, &f.host_stage[0], &f.host_stage[1], &f.host_stage[2]};

@@ -37,7 +37,7 @@ constexpr size_t kStBytes = kStRec + 3 * kStG16 + kStG8 +       // rec, rect, ti
                             al(4 * bin_owner_words(kStMaxGauss)) + // binning blocks' owners
                             4 * kStP4 +                          // pair keys/values x2
                             kStHist + kStTile +                  // sort scratch
-                            al(8 * kStMaxTiles) + al(4 * kStMaxTiles) +  // ranges, order
+                            al(8 * kStMaxTiles) +                // ranges
                             2 * al(16 * kStMaxRays) + al(4 * kStMaxRays) + // ray state, features,
                                                                          // contributors
                             kStP4 +                                      // column/row words
@@ -143,7 +143,6 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
     carve(fr.hist, cur, kStHist);
     carve(fr.tscratch, cur, kStTile);
     carve(fr.ranges, cur, al(8 * kStMaxTiles));
-    carve(fr.order, cur, al(4 * kStMaxTiles));
     carve(fr.ray_state, cur, al(16 * kStMaxRays));
     carve(fr.ray_feat, cur, al(16 * kStMaxRays));
     carve(fr.n_contrib, cur, al(4 * kStMaxRays));

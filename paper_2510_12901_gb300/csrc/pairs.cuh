@@ -70,10 +70,7 @@ __device__ __forceinline__ void cam_entry(const GRec &r, const float o[3], const
 }
 
 struct PairEval {
-    float n[3];      // num = cof(M)(v x d)
-    float e[3];      // den = M d
-    float inv;       // 1 / |den|^2 (fast reciprocal, within 2 ulp)
-    float D2, tau, rho, alpha;
+    float tau, rho, alpha;
     bool clamped;    // alpha hit alpha_max
 };
 
@@ -84,8 +81,7 @@ struct PairEval {
 // two multiplies of exp(-D^2 / 2).  Returns false when the entry does not
 // composite at this ray (outside the box, behind the origin, or below
 // alpha_min).  The forward and the backward both decide through this
-// function, so they take the same decisions; pe gets the unscaled num and
-// D^2 for the gradients.  Branch-free: every value is computed and the tests
+// function, so they take the same decisions.  Branch-free: every value is computed and the tests
 // combined at the end, so that evaluations of consecutive entries overlap.
 constexpr float kResponseScale = 0.84932180028801904f;   // sqrt(log2(e) / 2)
 
@@ -112,21 +108,13 @@ __device__ __forceinline__ bool cam_pair_scaled(const float4 e0, const float4 e1
     const float2 r1 = fma2(hi2(e4), zz, fma2(lo2(e4), yy, fma2(hi2(e1), xx, lo2(e1))));
     const float2 r2 = fma2(hi2(e5), zz, fma2(lo2(e5), yy, fma2(hi2(e2), xx, lo2(e2))));
     const float2 sq = fma2(r2, r2, fma2(r0, r0, mul2(r1, r1)));     // |num|^2, |den|^2
-    pe.e[0] = r0.y;
-    pe.e[1] = r1.y;
-    pe.e[2] = r2.y;
-    pe.inv = __fdividef(1.f, sq.y);
-    pe.tau = (mv.x * pe.e[0] + mv.y * pe.e[1] + mv.z * pe.e[2]) * pe.inv;
-    const float d2s = sq.x * pe.inv;
+    const float inv = __fdividef(1.f, sq.y);     // within 2 ulp
+    pe.tau = (mv.x * r0.y + mv.y * r1.y + mv.z * r2.y) * inv;
+    const float d2s = sq.x * inv;
     pe.rho = ex2_approx(-d2s);
     const float a = mv.w * pe.rho;
     pe.clamped = a > alpha_max;
     pe.alpha = fminf(a, alpha_max);
-    constexpr float kInv = 1.f / kResponseScale;
-    pe.n[0] = r0.x * kInv;
-    pe.n[1] = r1.x * kInv;
-    pe.n[2] = r2.x * kInv;
-    pe.D2 = d2s * (kInv * kInv);
     return in_box && pe.tau > 0.f && pe.alpha >= alpha_min;
 }
 
@@ -221,21 +209,19 @@ __device__ __forceinline__ bool lidar_pair_in(float4 (*s)[32], int j, int sb, bo
     const int sl = (sb - 3) >> 2;
     const float4 q0 = lid_col(s, j, 0, sl), q1 = lid_col(s, j, 1, sl), q2 = lid_col(s, j, 2, sl),
                  u = lid_col(s, j, 3, sl);
-    pe.n[0] = __fmaf_rn(q0.z, dd[2], __fmaf_rn(q0.y, dd[1], __fmaf_rn(q0.x, dd[0], q0.w)));
-    pe.n[1] = __fmaf_rn(q1.z, dd[2], __fmaf_rn(q1.y, dd[1], __fmaf_rn(q1.x, dd[0], q1.w)));
-    pe.n[2] = __fmaf_rn(q2.z, dd[2], __fmaf_rn(q2.y, dd[1], __fmaf_rn(q2.x, dd[0], q2.w)));
-    pe.e[0] = __fmaf_rn(m0.z, d[2], __fmaf_rn(m0.y, d[1], __fmul_rn(m0.x, d[0])));
-    pe.e[1] = __fmaf_rn(m1.z, d[2], __fmaf_rn(m1.y, d[1], __fmul_rn(m1.x, d[0])));
-    pe.e[2] = __fmaf_rn(m2.z, d[2], __fmaf_rn(m2.y, d[1], __fmul_rn(m2.x, d[0])));
-    const float ee = __fmaf_rn(pe.e[2], pe.e[2],
-                               __fmaf_rn(pe.e[1], pe.e[1], __fmul_rn(pe.e[0], pe.e[0])));
-    pe.inv = __fdividef(1.f, ee);
-    const float nn = __fmaf_rn(pe.n[2], pe.n[2],
-                               __fmaf_rn(pe.n[1], pe.n[1], __fmul_rn(pe.n[0], pe.n[0])));
-    pe.D2 = __fmul_rn(nn, pe.inv);
-    const float ue = __fmaf_rn(u.z, pe.e[2], __fmaf_rn(u.y, pe.e[1], __fmul_rn(u.x, pe.e[0])));
-    pe.tau = __fmul_rn(ue, pe.inv);
-    pe.rho = __expf(__fmul_rn(-0.5f, pe.D2));
+    const float n0 = __fmaf_rn(q0.z, dd[2], __fmaf_rn(q0.y, dd[1], __fmaf_rn(q0.x, dd[0], q0.w)));
+    const float n1 = __fmaf_rn(q1.z, dd[2], __fmaf_rn(q1.y, dd[1], __fmaf_rn(q1.x, dd[0], q1.w)));
+    const float n2 = __fmaf_rn(q2.z, dd[2], __fmaf_rn(q2.y, dd[1], __fmaf_rn(q2.x, dd[0], q2.w)));
+    const float e0 = __fmaf_rn(m0.z, d[2], __fmaf_rn(m0.y, d[1], __fmul_rn(m0.x, d[0])));
+    const float e1 = __fmaf_rn(m1.z, d[2], __fmaf_rn(m1.y, d[1], __fmul_rn(m1.x, d[0])));
+    const float e2 = __fmaf_rn(m2.z, d[2], __fmaf_rn(m2.y, d[1], __fmul_rn(m2.x, d[0])));
+    const float ee = __fmaf_rn(e2, e2, __fmaf_rn(e1, e1, __fmul_rn(e0, e0)));
+    const float inv = __fdividef(1.f, ee);
+    const float nn = __fmaf_rn(n2, n2, __fmaf_rn(n1, n1, __fmul_rn(n0, n0)));
+    const float D2 = __fmul_rn(nn, inv);
+    const float ue = __fmaf_rn(u.z, e2, __fmaf_rn(u.y, e1, __fmul_rn(u.x, e0)));
+    pe.tau = __fmul_rn(ue, inv);
+    pe.rho = __expf(__fmul_rn(-0.5f, D2));
     const float a = __fmul_rn(m0.w, pe.rho);
     pe.clamped = a > alpha_max;
     pe.alpha = fminf(a, alpha_max);

@@ -40,36 +40,6 @@ static uint32_t *saved_contrib(Frame &fr)
     return fr.keep_state ? (uint32_t *)fr.n_contrib.p : nullptr;
 }
 
-// Exclusive sum over a block of 1024 threads; every thread calls it.
-__device__ __forceinline__ uint32_t block_excl_scan_1024(uint32_t v, uint32_t *s_w, uint32_t &total)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t inc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    if (lane == 31) s_w[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        uint32_t x = s_w[lane];
-        uint32_t xi = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t t = __shfl_up_sync(0xffffffffu, xi, o);
-            if (lane >= o) xi += t;
-        }
-        s_w[lane] = xi - x;
-        if (lane == 31) s_w[32] = xi;
-    }
-    __syncthreads();
-    const uint32_t r = s_w[w] + inc - v;
-    total = s_w[32];
-    __syncthreads();
-    return r;
-}
-
 // Work items of the compositing.  A unit is a camera tile (units = tiles)
 // or a LiDAR work item (up to 32 rays of one tile, unit_tile[u].tile).
 // Units are taken in (coarsely) decreasing list length, so the longest start
@@ -603,8 +573,7 @@ sg_status render_camera(const Camera &cam, const sg_render_opts &o, Frame &fr, c
     const int nt = cam.ntx * cam.nty;
     const int64_t K = fr.n_pairs;
     const WorkSize ws = work_size(nt, K, fr.seg_len, 8);
-    sg_status s = ensure(fr.order, sizeof(uint32_t) * (nt > 0 ? nt : 1));
-    if (s == SG_OK) s = ensure(fr.camwork, ws.work_bytes);
+    sg_status s = ensure(fr.camwork, ws.work_bytes);
     if (s == SG_OK) s = ensure(fr.partials, ws.partial_bytes);
     if (s == SG_OK && fr.submask.bytes < 4 * (size_t)(K > 0 ? K : 1)) {
         set_error("internal: sub-block masks of the camera list missing");
@@ -842,8 +811,7 @@ sg_status render_camera_rs(const Camera &cam, const sg_render_opts &o, Frame &fr
     const int nt = cam.ntx * cam.nty;
     const int64_t K = fr.n_pairs;
     const WorkSize ws = work_size(nt, K, fr.seg_len, 8);
-    sg_status s = ensure(fr.order, sizeof(uint32_t) * (nt > 0 ? nt : 1));
-    if (s == SG_OK) s = ensure(fr.camwork, ws.work_bytes);
+    sg_status s = ensure(fr.camwork, ws.work_bytes);
     if (s == SG_OK) s = ensure(fr.partials, ws.partial_bytes);
     if (s == SG_OK && fr.submask.bytes < 4 * (size_t)(K > 0 ? K : 1)) {
         set_error("internal: sub-block masks of the camera list missing");
@@ -1178,8 +1146,7 @@ sg_status render_lidar(const Lidar &L, const sg_render_opts &o, Frame &fr, cudaS
     // items that share a tile each walk its list: the entries of all units
     // add up to at most max_items_per_tile x K
     const WorkSize ws = work_size(L.n_items, K * L.max_items_per_tile, kSegLen, 1);
-    sg_status s = ensure(fr.order, sizeof(uint32_t) * (size_t)L.n_items);
-    if (s == SG_OK) s = ensure(fr.camwork, ws.work_bytes);
+    sg_status s = ensure(fr.camwork, ws.work_bytes);
     if (s == SG_OK) s = ensure(fr.partials, ws.partial_bytes);
     if (s != SG_OK) return s;
     if ((s = launch_work_items(fr, ws, &L, L.n_theta * L.nphi, L.n_items, 1, kSegLen, st)) != SG_OK) return s;

@@ -514,8 +514,7 @@ sg_status render_camera_fwd(const Camera &cam, const sg_render_opts &o, Frame &f
     const int nt = cam.ntx * cam.nty;
     const int64_t K = fr.n_pairs;
     const WorkSize ws = work_size(nt, K, kFwdSeg, 8);
-    sg_status s = ensure(fr.order, sizeof(uint32_t) * (nt > 0 ? nt : 1));
-    if (s == SG_OK) s = ensure(fr.camwork, ws.work_bytes);
+    sg_status s = ensure(fr.camwork, ws.work_bytes);
     if (s == SG_OK) s = ensure(fr.partials, ws.partial_bytes);
     if (s == SG_OK && fr.submask.bytes < 4 * (size_t)(K > 0 ? K : 1)) {
         set_error("internal: sub-block masks of the camera list missing");

@@ -412,8 +412,7 @@ sg_status render_lidar_fwd(const Lidar &L, const sg_render_opts &o, Frame &fr, c
     if (L.n_items == 0) return SG_OK;
     const int64_t K = fr.n_pairs;
     const WorkSize ws = work_size(L.n_items, K * L.max_items_per_tile, kLfSeg, 1);
-    sg_status s = ensure(fr.order, sizeof(uint32_t) * (size_t)L.n_items);
-    if (s == SG_OK) s = ensure(fr.camwork, ws.work_bytes);
+    sg_status s = ensure(fr.camwork, ws.work_bytes);
     if (s == SG_OK) s = ensure(fr.partials, ws.partial_bytes);
     if (s != SG_OK) return s;
     if ((s = launch_work_items(fr, ws, &L, L.n_theta * L.nphi, L.n_items, 1, kLfSeg, st)) != SG_OK)

@@ -31,21 +31,6 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v)
 }
 
 // ------------------------------------------------------------------ radix sort
-// Lanes of the warp holding the same 8-bit digit as this one, among lanes
-// with a key (valid): one ballot per bit, each lane keeping the lanes that
-// agree with it on that bit.  A lane without a key is in no lane's set.
-__device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid)
-{
-    uint32_t peers = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const bool bit = (d >> b) & 1u;
-        const uint32_t bb = __ballot_sync(0xffffffffu, bit);
-        peers &= bit ? bb : ~bb;
-    }
-    return peers;
-}
-
 // Stable LSD radix sort of (key, value) pairs, digits of at most 8 bits, one
 // kernel per digit pass with decoupled look-back (the "onesweep" scheme):
 //   1. the kernel that writes the keys counts the digits of every pass
