@@ -397,8 +397,9 @@ sg_status sg_frame_sync_outputs(sg_frame frame);
  * no state is kept for a backward pass.  The first call on a device looks
  * up the array's device address (cudaGetSymbolAddress) with that device
  * current; make that first call before any stream capture.  All calls
- * share the one array: calls that overlap on the GPU (other threads or
- * streams of the same device) race and must be serialised by the caller.
+ * share the one array, and the host words that bring the pair count back:
+ * calls that overlap (other threads or streams of the same device) race and
+ * must be serialised by the caller.
  * Nothing in the array needs clearing between calls: every stage writes the
  * parts it later reads.  Like sg_render_camera, the call waits once for the
  * pair count; SG_ERR_TIMEOUT when a look-back wait of the depth sort gave

@@ -675,14 +675,8 @@ sg_status sg_create_camera(int model, int width, int height, float fx, float fy,
     c.fx = fx; c.fy = fy; c.cx = cx; c.cy = cy;
     for (int i = 0; i < 4; ++i) c.k[i] = (model == SG_CAMERA_FISHEYE && k) ? k[i] : 0.f;
     sg_status s = build_camera(c);
-    if (s == SG_OK && host_malloc(&c.h_count, 64) != cudaSuccess) {
-        cudaGetLastError();
-        set_error("pinned allocation failed");
-        s = SG_ERR_OOM;
-    }
-    if (s == SG_OK) memset(c.h_count, 0, 64);
+    if (s == SG_OK) s = static_words_ready();
     if (s != SG_OK) {
-        host_free(c.h_count);
         dev_free(c.d_pix);
         dev_free(c.d_tile_dir);
         dev_free(c.d_pix2);
@@ -698,7 +692,6 @@ void sg_destroy_camera(sg_camera cam)
 {
     if (!cam) return;
     cudaDeviceSynchronize();   // renders still queued may read its ray tables
-    host_free(cam->c.h_count);
     dev_free(cam->c.d_pix);
     dev_free(cam->c.d_tile_dir);
     dev_free(cam->c.d_pix2);

@@ -165,10 +165,6 @@ struct Camera {
     float4 *d_pix2 = nullptr;
     float *d_tile_basis = nullptr;
     bool tangent_ok = false;
-    // pinned words for the pair count of the allocation-free render, whose calls
-    // never overlap (kHostCountSeq), and the last sequence number
-    uint32_t *h_count = nullptr;
-    uint32_t count_seq = 0;
 };
 
 struct LidarItem {       // one warp of LiDAR rendering
@@ -492,6 +488,8 @@ sg_status render_lidar_fwd(const Lidar &L, const sg_render_opts &o, Frame &fr,
 
 // sensors.cu
 sg_status build_camera(Camera &cam);
+// noalloc.cu: the pinned words of the allocation-free render, made once
+sg_status static_words_ready();
 sg_status build_lidar(Lidar &L);
 
 // backward.cu

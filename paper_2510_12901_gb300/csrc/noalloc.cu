@@ -52,7 +52,33 @@ static __device__ __align__(256) unsigned char g_static_ws[kStBytes];
 static std::mutex g_ws_mu;
 static void *g_ws_addr[128];
 
-static sg_status static_workspace(unsigned char **out)
+// Pinned words through which the pair count of a call reaches the host
+// (kHostCountSeq), a line for each device, and the device's last sequence
+// number: like the array, they serve one call at a time.  Made with the first
+// camera, since the call itself may not allocate, and kept; a line of its own
+// for every camera made creating one 5 to 20 us longer (64x64 65 -> 70 us).
+constexpr size_t kWordsLine = 64;
+static uint32_t *g_words;
+static uint32_t g_words_seq[128];
+
+sg_status static_words_ready()
+{
+    std::lock_guard<std::mutex> lk(g_ws_mu);
+    if (g_words) return SG_OK;
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, 128 * kWordsLine, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("pinned allocation failed");
+        return SG_ERR_OOM;
+    }
+    note_alloc();
+    memset(p, 0, 128 * kWordsLine);      // no call has sequence number 0
+    g_words = (uint32_t *)p;
+    return SG_OK;
+}
+
+// The array's address, the device's pinned words and its sequence number.
+static sg_status static_workspace(unsigned char **out, uint32_t **words, uint32_t **seq)
 {
     int dev = 0;
     SG_CUDA(cudaGetDevice(&dev));
@@ -68,6 +94,8 @@ static sg_status static_workspace(unsigned char **out)
         g_ws_addr[dev] = p;
     }
     *out = (unsigned char *)g_ws_addr[dev];
+    *words = g_words + dev * (kWordsLine / sizeof(uint32_t));
+    *seq = &g_words_seq[dev];
     return SG_OK;
 }
 
@@ -115,7 +143,8 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
             return SG_ERR_INVALID;
         }
     unsigned char *base = nullptr;
-    sg_status s = static_workspace(&base);
+    uint32_t *words = nullptr, *last_seq = nullptr;
+    sg_status s = static_workspace(&base, &words, &last_seq);
     if (s != SG_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
 
@@ -178,18 +207,18 @@ extern "C" sg_status sg_render_camera_static(sg_scene scene, sg_camera cam,
     uint32_t *dk[2] = {(uint32_t *)fr.dkeys[0].p, (uint32_t *)fr.dkeys[1].p};
     uint32_t *dv[2] = {(uint32_t *)fr.dvals[0].p, (uint32_t *)fr.dvals[1].p};
     int rb = 0;
-    // the pair count comes back through the camera's pinned words
+    // the pair count comes back through the device's pinned words
     uint32_t seq = 0;
     if (n > 0) {
-        seq = ++cam->c.count_seq;
-        if (seq == 0) seq = cam->c.count_seq = 1;
+        seq = ++*last_seq;
+        if (seq == 0) seq = *last_seq = 1;
     }
-    fr.h_scalars = cam->c.h_count;
+    fr.h_scalars = words;
     if ((s = depth_stage((const uint32_t *)fr.count.p, (const float *)fr.depth.p, n, dk, dv, scal,
                          (uint32_t *)fr.offsets.p, fr, st, &rb, seq)) != SG_OK)
         return s;
     // the counts and the status word
-    const uint32_t *hs = cam->c.h_count;
+    const uint32_t *hs = words;
     const uint32_t none[kScalStatus + 1] = {};
     if (seq == 0)       // no Gaussians
         hs = none;
