@@ -260,7 +260,9 @@ sg_status sg_frame_workspace_bytes(sg_frame frame, size_t *bytes);
  * max_spins: polling rounds a look-back wait makes before it gives up
  * (0 = the default, about a second).  hold_site / hold_tile: the kernel
  * kind and the tile (ticket) whose published counts are withheld, so that
- * the next tile's wait is certain to run out (hold_site 0: none).  Every
+ * the next tile's wait is certain to run out (hold_site 0: none).  The depth
+ * stage of a scene of at most 4096 Gaussians is one block that waits for
+ * nothing: its three sites have no effect there.  Every
  * wait stays bounded and every access in bounds.  The values live in the
  * current device's memory (so that replays of captured CUDA graphs see
  * them); the call synchronises that device first.  Set them back with

@@ -40,7 +40,10 @@
 // warp), 16 shuffles with their selects and 16 atomics, and forming p and d
 // per pair (three divisions) took about 280 instructions an entry, the second
 // evaluation takes 75.  Measured: the 1M-Gaussian fisheye view 826 -> 594 us,
-// the 2M-Gaussian LiDAR sweep 620 -> 410 us.
+// the 2M-Gaussian LiDAR sweep 620 -> 410 us; two entries a pass (kBwPass) 583 and
+// 382.  Both divide a ray's remainder as IEEE 754 rounds it and get dL/dsigma
+// without a division, as the one-phase form did: 602 and 396 us (approximate
+// divisions, within 2 ulp, gave the 583 and 382).
 #include <math.h>
 
 #include "pairs.cuh"
@@ -177,9 +180,9 @@ __device__ __forceinline__ void start_ray(RayGrad &r, const float4 *slot, const 
 }
 
 // Entries that the lanes as rays evaluate before they take the steps in turn:
-// the evaluations overlap (1M-Gaussian fisheye view: 1 entry 601, 2 586 us; the
-// camera's last step, 16 rays an entry, unrolled by 8 583; street sweep of 2M: 1
-// entry 407, 2 382, 3 382 us).
+// the evaluations overlap (with approximate divisions, 1M-Gaussian fisheye view: 1
+// entry 601, 2 586 us; the camera's last step, 16 rays an entry, unrolled by 8 583;
+// street sweep of 2M: 1 entry 407, 2 382, 3 382 us).
 constexpr int kBwPass = 2;
 
 // ------------------------------------------------------------------ camera

@@ -300,7 +300,8 @@ static sg_status upload_desc(Frame &fr, int64_t n, cudaStream_t st)
 // several renders on their own streams can each have their pair count on
 // the way before any of them waits for one.
 // sort_and_count: depth sort, offsets and the pair count.  In exact mode the
-// count is copied to h_scalars and ev_count recorded; in capacity mode
+// depth stage writes the count to h_scalars itself (count_told; a scene without
+// Gaussians has it copied) and ev_count is recorded behind it; in capacity mode
 // (fr.k_cap > 0) the count stays on the device, clamped to k_cap (the excess
 // in scalars[3]).
 static sg_status sort_and_count(Frame &fr, int64_t n, cudaStream_t st)
@@ -334,8 +335,8 @@ static const char *status_cause(uint32_t w)
     return "a look-back wait of the sort gave up";
 }
 
-// Wait until the counts of the render are in h_scalars.  k_pair_offsets writes
-// them there itself and the host polls the sequence number: a copy and an event
+// Wait until the counts of the render are in h_scalars.  k_pair_offsets (or
+// k_depth_small) writes them there itself and the host polls the sequence number: a copy and an event
 // behind the kernel and waking up from its wait cost 10 us more (64x64 97 -> 88
 // us a render, 641x479 156 -> 149, street sweep 729 -> 717).  The event (or the
 // stream, ev NULL), asked now and then, ends the wait if the kernel failed.
