@@ -353,8 +353,9 @@ sg_status radix_sort_pairs(uint32_t *keys[2], uint32_t *vals[2], int64_t n_max,
 // each, about 5 us at 1.5M) and take tiles of 8192 above 256k Gaussians, whose
 // shorter look-back chain is worth more than the fuller chip (at 1M 12 us; 4096
 // 16, 2048 19), and of 2048 below, where the chain is short (150k: the stage 52
-// us, 56 with 8192); counting the tiles done, in exact mode, adds 1 to 1.5 us.  One warp walks back, 32 words a round: 128 words a round or
-// all warps reading took 11 -> 12 and 14 -> 17 us.
+// us, 56 with 8192); counting the tiles done, in exact mode, adds 1 to 1.5 us.
+// One warp walks back, 32 words a round: 128 words a round or all warps reading
+// took 11 -> 12 and 14 -> 17 us.
 constexpr int kChainThreads = 256;
 constexpr int kChainWarps = kChainThreads / 32;
 constexpr int kChainChunks = kChainTile / kChainThreads;   // 32-entry chunks per warp
@@ -835,7 +836,7 @@ sg_status depth_stage(const uint32_t *d_count, const float *d_depth, int64_t n, 
 // depth-ordered expansion (C = kBinChunk; pair p belongs to the valid
 // Gaussian k with offsets[k] <= p < offsets[k + 1]).  The owner of its first
 // pair is in the table that k_pair_offsets wrote (beyond the table, a
-// cooperative search over the offsets, 256 samples per round).  The block
+// cooperative search over the offsets, 512 samples per round).  The block
 // loads the at most C + 1 Gaussians its pairs can belong to, marks each one's
 // first pair, and a running maximum over the pairs gives every pair its
 // owner; a thread takes four consecutive pairs and writes them as 16 bytes.
